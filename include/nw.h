@@ -459,6 +459,16 @@ nw_status nw_debug_enumerate_query_pairs(const uint32_t *q_lengths, uint32_t nq,
                                          uint32_t nd, uint32_t ta, uint32_t *q, uint32_t *d, uint64_t cap,
                                          uint64_t *count);
 
+/* Host-only: the pairs of the bit-parallel alignment kernel's plan, as the
+ * two functions above give them for the DPX kernel's.  With nq == 0: the
+ * all-pairs plan (or shard `shard` of `nshards`) over words of lengths
+ * lengths[0..n); otherwise the (query, word) pairs of query words of lengths
+ * q_lengths[0..nq) against them.  `ta` A words per task (0: as the calls
+ * choose it). */
+nw_status nw_debug_enumerate_bit_pairs(const uint32_t *q_lengths, uint32_t nq, const uint32_t *lengths, uint32_t n,
+                                       uint32_t shard, uint32_t nshards, uint32_t ta, uint32_t *a, uint32_t *b,
+                                       uint64_t cap, uint64_t *count);
+
 /* Host-only: the tables behind NW_RANK_NORMALISED for scores [lo, hi].
  * *nranks receives the number of distinct weights s/m (rank 0 = smallest);
  * when it is <= cap_ranks, also writes

@@ -55,9 +55,11 @@ nw_status load_impl(nw_ctx* c, const uint8_t* codes, const uint32_t* offsets, ui
     d->score_lo = lo;
     d->score_hi = hi;
     plan_all_pairs(d->ws.bk, kDefaultTA, d->plan);
-    st = ctx_alloc(c, d->d_segs, sizeof(Seg) * std::max<size_t>(1, d->plan.segs.size()), "segment plan");
-    if (st == NW_OK && !d->plan.segs.empty()) {
-      cudaError_t e = cudaMemcpyAsync(d->d_segs.p, d->plan.segs.data(), sizeof(Seg) * d->plan.segs.size(),
+    if (d->ss.bit_m) bit_plan_sized(d->bits, [&](uint32_t ta, BitPlan& p) { bit_pairs(d->ws.bk, ta, 0, p); });
+    const std::vector<Seg>& segs = d->ss.bit_m ? d->bits.segs : d->plan.segs;
+    st = ctx_alloc(c, d->d_segs, sizeof(Seg) * std::max<size_t>(1, segs.size()), "segment plan");
+    if (st == NW_OK && !segs.empty()) {
+      cudaError_t e = cudaMemcpyAsync(d->d_segs.p, segs.data(), sizeof(Seg) * segs.size(),
                                       cudaMemcpyHostToDevice, c->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
       if (e != cudaSuccess) st = cuda_fail(c, e, "uploading the segment plan");
@@ -274,11 +276,7 @@ nw_status matrix_impl(nw_dict* d, int8_t* out, uint64_t chunk_bytes, uint32_t fl
     base.hist_mode = kHistNone;
     base.err = d_err;
     SideView side{d->ws.perm.as<uint32_t>(), nullptr, nullptr};
-    const uint32_t* a_enc[3] = {d->ws.a_enc.as<uint32_t>(), nullptr, nullptr};
-    const uint4* b_rec[3] = {d->ws.b_rec.as<uint4>(), nullptr, nullptr};
-    const SideView* views[3] = {&side, nullptr, nullptr};
-    NW_TRY(run_plan(c, c->stream, d->plan, d->d_segs.as<Seg>(), base, d_counters, 0, 1, tm, ro, a_enc, views,
-                    b_rec, views));
+    NW_TRY(run_dict(d, base, side, d_counters, 0, 1, tm, ro));
     if (!dev) {
       NW_CK(cudaMemcpyAsync(out + lo, dst, hi - lo, cudaMemcpyDeviceToHost, s));
       if (chunked) NW_CK(cudaStreamSynchronize(s));  // the chunk buffer is reused
@@ -469,9 +467,13 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   const int32_t key_lo = lo - 1;
   if ((uint64_t)(hi - key_lo) >= (1ull << (32 - ib)))
     return set_err(c, NW_ERANGE, "score range with %u dictionary words does not fit 32-bit list keys", n);
+  const bool bits = d->ss.bit_m > 0;
   Plan plan;
   plan_query(q.bk, d->ws.bk, kDefaultTA, plan, kQueryMinTasks);
-  NW_TRY(ctx_ensure(c, c->ws_segs, sizeof(Seg) * std::max<size_t>(1, plan.segs.size()), "query segments"));
+  BitPlan bplan;
+  if (bits) bit_plan_sized(bplan, [&](uint32_t ta, BitPlan& p) { bit_queries(q.bk, d->ws.bk, ta, 0, p); });
+  const std::vector<Seg>& segs = bits ? bplan.segs : plan.segs;
+  NW_TRY(ctx_ensure(c, c->ws_segs, sizeof(Seg) * std::max<size_t>(1, segs.size()), "query segments"));
   NW_TRY(ctx_ensure(c, c->ws_slots, sizeof(uint32_t) * (size_t)nq * k, "list slots"));
   NW_TRY(ctx_ensure(c, c->ws_thr, sizeof(uint32_t) * (size_t)nq, "list thresholds"));
   NW_TRY(ctx_ensure(c, c->ws_small, 64 + sizeof(unsigned long long) * (plan.launches.size() + 1), "task counters"));
@@ -489,8 +491,8 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   Timer tm{c};
   cudaEvent_t e_all = nullptr;
   tm.begin(false, e_all);
-  if (!plan.segs.empty())
-    NW_CK(cudaMemcpyAsync(c->ws_segs.p, plan.segs.data(), sizeof(Seg) * plan.segs.size(), cudaMemcpyHostToDevice, s));
+  if (!segs.empty())
+    NW_CK(cudaMemcpyAsync(c->ws_segs.p, segs.data(), sizeof(Seg) * segs.size(), cudaMemcpyHostToDevice, s));
   NW_CK(cudaMemsetAsync(c->ws_small.p, 0, c->ws_small.bytes, s));
   NW_CK(cudaMemsetAsync(c->ws_slots.p, 0, sizeof(uint32_t) * (size_t)nq * k, s));
   NW_CK(cudaMemsetAsync(c->ws_thr.p, 0, sizeof(uint32_t) * (size_t)nq, s));
@@ -512,13 +514,21 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   base.err = d_err;
   SideView qside{q.perm.as<uint32_t>(), c->ws_slots.as<uint32_t>(), c->ws_thr.as<uint32_t>()};
   SideView dside{d->ws.perm.as<uint32_t>(), nullptr, nullptr};
-  const uint32_t* a_enc[3] = {nullptr, q.a_enc.as<uint32_t>(), d->ws.a_enc.as<uint32_t>()};
-  const uint4* b_rec[3] = {nullptr, d->ws.b_rec.as<uint4>(), q.b_rec.as<uint4>()};
-  const SideView* A_views[3] = {nullptr, &qside, &dside};
-  const SideView* B_views[3] = {nullptr, &dside, &qside};
   RunOut ro;
-  NW_TRY(run_plan(c, c->stream, plan, c->ws_segs.as<Seg>(), base, d_counters, 0, 1, tm, ro, a_enc, A_views,
-                  b_rec, B_views));
+  if (bits) {
+    BitParams P = bit_params(base, d_counters);
+    P.local[0] = bit_terms(d, q, d->ws, qside, dside, key_lo, ib);
+    P.local[0].serial_a = 1u;  // query words are the A side
+    P.local[1] = bit_terms(d, d->ws, q, dside, qside, key_lo, ib);
+    NW_TRY(run_bits(c, s, d->ss.bit_m, d->ss.bit_x, kEpiLists, d->alphabet, bplan, c->ws_segs.as<Seg>(), P, tm, ro));
+  } else {
+    const uint32_t* a_enc[3] = {nullptr, q.a_enc.as<uint32_t>(), d->ws.a_enc.as<uint32_t>()};
+    const uint4* b_rec[3] = {nullptr, d->ws.b_rec.as<uint4>(), q.b_rec.as<uint4>()};
+    const SideView* A_views[3] = {nullptr, &qside, &dside};
+    const SideView* B_views[3] = {nullptr, &dside, &qside};
+    NW_TRY(run_plan(c, c->stream, plan, c->ws_segs.as<Seg>(), base, d_counters, 0, 1, tm, ro, a_enc, A_views,
+                    b_rec, B_views));
+  }
   cudaEvent_t e_fin = nullptr;
   tm.begin(false, e_fin);
   NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), nq, k, q.perm.as<uint32_t>(), ib, base.imask, key_lo, out_idx,
@@ -711,6 +721,60 @@ nw_status nw_debug_enumerate_query_pairs(const uint32_t* q_lengths, uint32_t nq,
   return NW_OK;
 }
 
+nw_status nw_debug_enumerate_bit_pairs(const uint32_t* q_lengths, uint32_t nq, const uint32_t* lengths, uint32_t n,
+                                       uint32_t shard, uint32_t nshards, uint32_t ta, uint32_t* a, uint32_t* b,
+                                       uint64_t cap, uint64_t* count) {
+  if (!lengths || !count || nshards == 0 || shard >= nshards || (nq && !q_lengths)) return NW_EINVAL;
+  if ((cap && (!a || !b)) || (nq && nshards != 1)) return NW_EINVAL;
+  Buckets bk[2];
+  std::vector<uint32_t> perm[2];
+  const uint32_t* len[2] = {lengths, q_lengths};
+  const uint32_t cnts[2] = {n, nq};
+  for (int s = 0; s < 2; ++s) {
+    bk[s] = Buckets{};
+    for (uint32_t i = 0; i < cnts[s]; ++i) {
+      if (len[s][i] > (uint32_t)kMaxLen) return NW_EINVAL;
+      ++bk[s].count[len[s][i]];
+    }
+    fill_buckets(bk[s]);
+    perm[s].assign(cnts[s], 0);
+    std::vector<uint32_t> fill(kBuckets, 0);
+    for (uint32_t i = 0; i < cnts[s]; ++i) perm[s][bk[s].start[len[s][i]] + fill[len[s][i]]++] = i;
+  }
+  BitPlan plan;
+  auto make = [&](uint32_t t, BitPlan& p) {
+    if (nq) {
+      bit_queries(bk[1], bk[0], t, 0, p);
+    } else if (nshards == 1) {
+      bit_pairs(bk[0], t, 0, p);
+    } else {
+      Plan full;
+      plan_all_pairs(bk[0], kDefaultTA, full);
+      bit_shard(bk[0], full, shard, nshards, t, p);
+    }
+  };
+  if (ta) make(ta, plan); else bit_plan_sized(plan, make);
+  uint64_t cnt = 0;
+  for (uint64_t t = 0; t < plan.ntasks; ++t) {
+    const Seg& S = plan.segs[find_seg(plan.segs.data(), (uint32_t)plan.segs.size(), t)];
+    const TaskGeom g = task_geom(S, t, plan.ta, 32u * (uint32_t)bit_words_per_lane((int)S.lb));
+    // terms 0: the queries (if any) are the A words; terms 1: they are the B words
+    const std::vector<uint32_t>& pa = perm[nq && S.dict == 0 ? 1 : 0];
+    const std::vector<uint32_t>& pb = perm[S.dict == 1 ? 1 : 0];
+    for (uint32_t x = g.a0; x < g.a1; ++x)
+      for (uint32_t y = g.b0; y < g.bend; ++y) {
+        if (!pair_valid(g, x, y)) continue;
+        if (cnt < cap) {
+          a[cnt] = S.dict == 1 ? pb[y] : pa[x];
+          b[cnt] = S.dict == 1 ? pa[x] : pb[y];
+        }
+        ++cnt;
+      }
+  }
+  *count = cnt;
+  return NW_OK;
+}
+
 nw_status nw_debug_fail_alloc(nw_ctx* c, uint32_t countdown) {
   if (!c) return NW_EINVAL;
   c->fail_countdown = countdown;
@@ -825,13 +889,9 @@ nw_status topk_into_scratch(nw_dict* d, ScratchProvider provide, uint32_t k, uin
   P.stats = d_stats;
   P.err = async ? d_err_async : d_err;
   SideView side{d->ws.perm.as<uint32_t>(), d_slots, d_thr};
-  const uint32_t* a_enc[3] = {d->ws.a_enc.as<uint32_t>(), nullptr, nullptr};
-  const uint4* b_rec[3] = {d->ws.b_rec.as<uint4>(), nullptr, nullptr};
-  const SideView* views[3] = {&side, nullptr, nullptr};
   Timer tm{c};
   RunOut ro;
-  NW_TRY(run_plan(c, c->stream, d->plan, d->d_segs.as<Seg>(), P, d_counters, 0, 1, tm, ro, a_enc, views, b_rec,
-                  views));
+  NW_TRY(run_dict(d, P, side, d_counters, 0, 1, tm, ro));
   NW_CK(launch_finalize(d_slots, n, k, d->ws.perm.as<uint32_t>(), ib, P.imask, key_lo, nbr_idx, nbr_score, s));
   if (hist) {
     NW_CK(cudaMemcpyAsync(hist, d_hist, sizeof(int64_t) * need_bins, cudaMemcpyDeviceToDevice, s));

@@ -223,7 +223,8 @@ __device__ __forceinline__ uint64_t upper_offset(uint64_t i, uint64_t j, uint64_
 // shared array (bin b of lane l at b*32 + l), so the shared atomics of a warp
 // never collide; kHistSmem: one shared array per warp; kHistGlobal: global
 // atomics.  `bin` is the score minus the histogram's lowest score.
-__device__ __forceinline__ void hist_add(const DpParams& P, uint32_t* wh, int lane, int bin) {
+template <class PT>
+__device__ __forceinline__ void hist_add(const PT& P, uint32_t* wh, int lane, int bin) {
   const uint32_t bi = (uint32_t)bin;
   if (bi >= P.nbins) { atomicOr(P.err, kErrHistRange); return; }
   if (P.hist_mode == kHistLane) atomicAdd(wh + bi * 32u + (uint32_t)lane, 1u);
@@ -231,7 +232,8 @@ __device__ __forceinline__ void hist_add(const DpParams& P, uint32_t* wh, int la
   else atomicAdd(P.hist + bi, 1ull);
 }
 
-__device__ __forceinline__ void hist_flush(const DpParams& P, uint32_t* wh, int lane) {
+template <class PT>
+__device__ __forceinline__ void hist_flush(const PT& P, uint32_t* wh, int lane) {
   __syncwarp();
   if (P.hist_mode == kHistLane) {
     for (uint32_t b = lane; b < P.nbins; b += 32) {
@@ -281,8 +283,8 @@ struct TaskTerms {
 // List key of a pair with score s whose longer word has m symbols: the raw
 // score, or the rank of s/m in the normalised ranking, above the partner's
 // reversed index (higher key = better neighbour).
-__device__ __forceinline__ uint32_t list_key(const DpParams& P, const TaskTerms& T, int s, int m,
-                                             uint32_t partner) {
+template <class PT, class TT>
+__device__ __forceinline__ uint32_t list_key(const PT& P, const TT& T, int s, int m, uint32_t partner) {
   const uint32_t v = P.norm_rank ? (uint32_t)P.norm_rank[(s - P.norm_lo) * kBuckets + m] + 1u
                                  : (uint32_t)(s - T.key_lo);
   return (v << T.ib) | (T.imask - partner);
@@ -294,7 +296,8 @@ __device__ __forceinline__ uint32_t list_key(const DpParams& P, const TaskTerms&
 // threshold's own score; with normalised keys, the smallest score whose s/m
 // has the threshold's rank (a lower rank makes a key below any key of that
 // rank, whatever the partner).
-__device__ __forceinline__ int g_bound(const DpParams& P, const TaskTerms& T, uint32_t thr_key, int m, int pconst) {
+template <class PT, class TT>
+__device__ __forceinline__ int g_bound(const PT& P, const TT& T, uint32_t thr_key, int m, int pconst) {
   if (thr_key == 0u) return INT_MIN;
   if (P.norm_rank) return (int)P.norm_smin[((thr_key >> T.ib) - 1u) * kBuckets + m] - pconst;
   return (int)(thr_key >> T.ib) + T.key_lo - pconst;

@@ -1,4 +1,5 @@
-// Maps a length LB to its alignment kernel across the instantiation units.
+// Maps a length LB, and reduced steps (m, x), to their alignment kernels across
+// the instantiation units.
 #include "nw_launch.h"
 
 namespace nw {
@@ -13,5 +14,16 @@ const void* dp_kernel(int LB, int epi, bool tab) {
   if (LB <= 20) return dp_kernel_range_11(LB, epi, tab);
   if (LB <= 30) return dp_kernel_range_21(LB, epi, tab);
   return dp_kernel_range_31(LB, epi, tab);
+}
+
+#define NW_BIT_ALL(F) F(1, 0) F(2, 1) F(3, 1) F(3, 2) F(4, 1) F(4, 3) F(5, 1) F(5, 2) F(5, 3) F(5, 4)
+#define NW_BIT_DECL(m, x) const void* bit_kernel_##m##_##x(int epi);
+NW_BIT_ALL(NW_BIT_DECL)
+
+const void* bit_kernel(int m, int x, int epi) {
+#define NW_BIT_CASE(a, b) \
+  if (m == a && x == b) return bit_kernel_##a##_##b(epi);
+  NW_BIT_ALL(NW_BIT_CASE)
+  return nullptr;
 }
 }  // namespace nw

@@ -62,6 +62,14 @@ struct Plan {
   uint64_t pairs = 0, cells = 0;
 };
 
+// The plan of one bit-parallel launch: every length pair in one segment list.
+struct BitPlan {
+  std::vector<Seg> segs;
+  uint32_t ta = 0;      // A words per task
+  uint64_t ntasks = 0;
+  uint32_t max_la = 0;  // longest A word
+};
+
 }  // namespace
 
 struct nw_ctx {
@@ -97,7 +105,8 @@ struct nw_dict {
   uint32_t alphabet = 0;
   int32_t score_lo = 0, score_hi = 0;
   Plan plan;
-  DevBuf d_segs;
+  BitPlan bits;        // used instead of plan's launches when ss.bit_m > 0
+  DevBuf d_segs;       // the segments of the plan in use
   bool subst = false;  // scored with a full similarity matrix (d_tab)
   DevBuf d_tab;        // kTabDim x kTabDim s'+ table
   uint64_t serial = 0;  // unique per loaded dictionary (caches keyed on it)
@@ -204,6 +213,22 @@ uint32_t pack16(int32_t v) {
   return h | (h << 16);
 }
 
+// The reduced steps of the bit-parallel kernel: s'_m and max(s'_x, 0) over
+// their gcd.  match == mismatch (every cell gains the same) and s'_m = 0 keep
+// the DPX kernel, as do steps above kBitMaxStep: a row takes about m^2 logic
+// operations for 64 columns against 2 m for 2 cells there.
+void bit_steps(ShiftedScoring& s) {
+  const int m = s.sm, x = std::max(s.sx, 0);
+  s.bit_m = s.bit_x = s.bit_coef = 0;
+  if (m <= 0 || x >= m) return;
+  int g = m, h = x;
+  while (h) { const int r = g % h; g = h; h = r; }
+  if (m / g > kBitMaxStep) return;
+  s.bit_m = m / g;
+  s.bit_x = x / g;
+  s.bit_coef = g;
+}
+
 nw_status make_shifted(nw_ctx* c, const nw_scoring& s, uint32_t alphabet, ShiftedScoring& out) {
   if (std::abs(s.match) > 1024 || std::abs(s.mismatch) > 1024 || std::abs(s.gap) > 1024)
     return set_err(c, NW_EINVAL, "scoring values must lie in [-1024, 1024]");
@@ -222,6 +247,7 @@ nw_status make_shifted(nw_ctx* c, const nw_scoring& s, uint32_t alphabet, Shifte
   out.shift = shift;
   out.C1 = pack16(sm + 1);
   out.C2 = pack16(std::max(sx, 0));  // a negative mismatch term never wins (see nw_dp.cuh)
+  bit_steps(out);
   return NW_OK;
 }
 
@@ -336,6 +362,143 @@ void plan_all_pairs(const Buckets& bk, uint32_t TA, Plan& out) {
     }
   }
   order_launches(out);
+}
+
+// ---- plans of the bit-parallel kernel
+
+// Estimated SM sub-partition cycles (per warp) of nA words of length a against
+// nB words of length b in the lanes: a row costs ~70 cycles for the lane's
+// words, an A word ~40, each of the lane's words ~12 to score and file, and
+// each task ~1500 to build its match masks.
+uint64_t bit_cost(uint64_t nA, int a, uint64_t nB, int b, uint32_t ta) {
+  const uint64_t K = (uint64_t)bit_words_per_lane(b);
+  const uint64_t chunks = cdiv(nB, 32 * K), kk = std::min<uint64_t>(K, cdiv(nB, 32));
+  return chunks * (nA * ((uint64_t)a * 70 + 40 + 12 * kk) + cdiv(nA, ta) * 1500);
+}
+
+// One rectangle of pairs for the bit-parallel kernel: words [a0, a1) of bucket
+// La of A (relative to the bucket) against [b0, b1) of bucket LB of B.
+struct BitRect {
+  int La, LB;
+  uint32_t a0, a1, b0, b1;
+  bool tri;
+  uint32_t dict;
+};
+
+void bit_add(BitPlan& p, const Buckets& A, const Buckets& B, const BitRect& r) {
+  if (r.a0 >= r.a1 || r.b0 >= r.b1) return;
+  Seg s{};
+  s.a_beg = A.start[r.La] + r.a0;
+  s.a_end = A.start[r.La] + r.a1;
+  s.b_beg = B.start[r.LB] + r.b0;
+  s.b_end = B.start[r.LB] + r.b1;
+  s.aenc_base = A.aenc_base[r.La] + r.a0 * (uint32_t)r.La;
+  s.brec_base = B.aenc_base[r.LB] + r.b0 * (uint32_t)r.LB;
+  s.la = (uint16_t)r.La;
+  s.lb = (uint32_t)r.LB;
+  s.tri = r.tri ? 1 : 0;
+  s.dict = r.dict;
+  s.nca = (uint32_t)cdiv(r.a1 - r.a0, p.ta);
+  s.task0 = p.ntasks;
+  p.ntasks += (uint64_t)s.nca * cdiv(r.b1 - r.b0, 32u * (uint32_t)bit_words_per_lane(r.LB));
+  p.max_la = std::max(p.max_la, (uint32_t)r.La);
+  p.segs.push_back(s);
+}
+
+// Every unordered pair of one set, once.  Same-length pairs are cut into
+// strips of ta A words against the words from the strip on; pairs of two
+// lengths take the cheaper of the two orientations.  Length differences come
+// in increasing order: a word's best neighbours mostly have nearly its
+// length, so its list bound rises before the many low-scoring pairs arrive.
+void bit_pairs(const Buckets& bk, uint32_t ta, uint32_t dict, BitPlan& p) {
+  p.ta = ta;
+  for (int diff = 0; diff < kBuckets; ++diff) {
+    for (int L = diff; L < kBuckets; ++L) {
+      const int s = L - diff;
+      const uint32_t nL = bk.count[L], ns = bk.count[s];
+      if (!nL || !ns) continue;
+      if (diff == 0) {
+        for (uint32_t a = 0; a + 1 < nL; a += ta)
+          bit_add(p, bk, bk, {L, L, a, std::min(nL, a + ta), a, nL, true, dict});
+      } else if (bit_cost(ns, s, nL, L, ta) <= bit_cost(nL, L, ns, s, ta)) {
+        bit_add(p, bk, bk, {s, L, 0, ns, 0, nL, false, dict});
+      } else {
+        bit_add(p, bk, bk, {L, s, 0, nL, 0, ns, false, dict});
+      }
+    }
+  }
+}
+
+// Every (query, dictionary word) pair, once: terms dict0 where the queries
+// are the A words, dict0 + 1 where they are the lanes' words.
+void bit_queries(const Buckets& qb, const Buckets& db, uint32_t ta, uint32_t dict0, BitPlan& p) {
+  p.ta = ta;
+  for (int diff = 0; diff < kBuckets; ++diff)
+    for (int lq = 0; lq < kBuckets; ++lq)
+      for (int sign = -1; sign <= 1; sign += 2) {
+        const int ld = lq + sign * diff;
+        if (ld < 0 || ld >= kBuckets || (diff == 0 && sign > 0)) continue;
+        const uint32_t nq = qb.count[lq], nd = db.count[ld];
+        if (!nq || !nd) continue;
+        if (bit_cost(nq, lq, nd, ld, ta) <= bit_cost(nd, ld, nq, lq, ta))
+          bit_add(p, qb, db, {lq, ld, 0, nq, 0, nd, false, dict0});
+        else
+          bit_add(p, db, qb, {ld, lq, 0, nd, 0, nq, false, dict0 + 1});
+      }
+}
+
+// The chunk of A words per task: 256, halved down to 16 while the plan has
+// fewer tasks than kBitMinTasks (several per resident block of a full GPU).
+constexpr uint64_t kBitMinTasks = 12288;
+constexpr uint32_t kBitMinTA = 16;
+template <class Make>
+void bit_plan_sized(BitPlan& p, Make make) {
+  for (uint32_t ta = kDefaultTA;; ta /= 2) {
+    p = BitPlan{};
+    make(ta, p);
+    if (p.ntasks >= kBitMinTasks || ta <= kBitMinTA) return;
+  }
+}
+
+// The pairs that shard `shard` of `nshards` of the DPX plan holds (each
+// launch's task list cut into contiguous ranges), as rectangles of the same
+// buckets.  Shards keep this partition whatever kernel scores them, so
+// shards saved by one build combine with another's.
+void bit_shard(const Buckets& bk, const Plan& plan, uint32_t shard, uint32_t nshards, uint32_t ta, BitPlan& p) {
+  p.ta = ta;
+  for (const LaunchPlan& lp : plan.launches) {
+    const uint64_t lo = lp.ntasks * shard / nshards, hi = lp.ntasks * (shard + 1) / nshards;
+    for (uint32_t x = 0; x < lp.nsegs; ++x) {
+      const Seg& S = plan.segs[lp.seg_first + x];
+      const uint32_t ncb = (uint32_t)cdiv(S.b_end - S.b_beg, kWarpB);
+      const uint64_t t0 = S.task0, t1 = S.task0 + (uint64_t)S.nca * ncb;
+      const uint64_t a = std::max(lo, t0), b = std::min(hi, t1);
+      if (a >= b) continue;
+      // tasks [a, b) of the segment: chunk coordinates (ca fastest)
+      auto rect = [&](uint32_t ca0, uint32_t ca1, uint32_t cb0, uint32_t cb1) {
+        if (ca0 >= ca1 || cb0 >= cb1) return;
+        const uint32_t nA = S.a_end - S.a_beg, nB = S.b_end - S.b_beg, ao = S.a_beg - bk.start[S.la],
+                       bo = S.b_beg - bk.start[lp.LB];
+        BitRect r{(int)S.la, lp.LB, ao + std::min(nA, ca0 * kDefaultTA), ao + std::min(nA, ca1 * kDefaultTA),
+                  bo + std::min(nB, cb0 * (uint32_t)kWarpB), bo + std::min(nB, cb1 * (uint32_t)kWarpB), S.tri != 0, 0u};
+        if (!r.tri && bit_cost(r.b1 - r.b0, r.LB, r.a1 - r.a0, r.La, ta) < bit_cost(r.a1 - r.a0, r.La, r.b1 - r.b0, r.LB, ta)) {
+          std::swap(r.La, r.LB);
+          std::swap(r.a0, r.b0);
+          std::swap(r.a1, r.b1);
+        }
+        bit_add(p, bk, bk, r);
+      };
+      const uint32_t l0 = (uint32_t)((a - t0) / S.nca), c0 = (uint32_t)((a - t0) % S.nca);
+      const uint32_t l1 = (uint32_t)((b - t0) / S.nca), c1 = (uint32_t)((b - t0) % S.nca);
+      if (l0 == l1) {
+        rect(c0, c1, l0, l0 + 1);
+      } else {
+        rect(c0, S.nca, l0, l0 + 1);
+        rect(0, S.nca, l0 + 1, l1);
+        rect(0, c1, l1, l1 + 1);
+      }
+    }
+  }
 }
 
 // Tasks a query launch should have at least (a few per warp of a full GPU)
@@ -677,6 +840,111 @@ nw_status run_plan(nw_ctx* c, cudaStream_t stream, const Plan& plan, const Seg* 
   return NW_OK;
 }
 
+// One side of a bit-parallel launch's terms: scoring and key layout of `d`.
+BitTerms bit_terms(const nw_dict* d, const WordSet& a, const WordSet& b, SideView A, SideView B, int32_t key_lo,
+                   uint32_t ib) {
+  BitTerms T{};
+  T.a_sym = a.a_enc.as<uint32_t>();
+  T.b_sym = b.a_enc.as<uint32_t>();
+  T.A = A;
+  T.B = B;
+  T.shift = d->ss.shift;
+  T.alphabet = d->alphabet;
+  T.coef = (uint32_t)d->ss.bit_coef;
+  T.match = d->sc.match;
+  T.mismatch = d->sc.mismatch;
+  T.gap = d->sc.gap;
+  T.key_lo = key_lo;
+  T.ib = ib;
+  T.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
+  return T;
+}
+
+// Launches the bit-parallel kernel of steps (m, x) over a plan.  `P` brings
+// the terms, epilogue settings and counter; `alphabet` is the largest of the
+// launch's sets.
+nw_status run_bits(nw_ctx* c, cudaStream_t stream, int m, int x, int epi, uint32_t alphabet, const BitPlan& plan,
+                   const Seg* d_segs, BitParams P, Timer& tm, RunOut& ro, uint32_t bps = 0) {
+  if (plan.ntasks == 0) return NW_OK;
+  P.segs = d_segs;
+  P.nsegs = (uint32_t)plan.segs.size();
+  P.TA = plan.ta;
+  P.ntasks = plan.ntasks;
+  P.sub = std::max<uint32_t>(1, std::min<uint32_t>(kBitSub, plan.ta / kBitWarps));
+  P.mask_bytes = alphabet * kMaskRow;
+  P.stage_words = (P.sub * plan.max_la + 2 + 3) & ~3u;
+  P.dbg_insert_limit = c->dbg_insert_iters >= 0 ? (uint32_t)c->dbg_insert_iters + 1u : 0u;
+  const void* fn = bit_kernel(m, x, epi);
+  if (!fn) return set_err(c, NW_EINVAL, "no kernel for steps (%d, %d)", m, x);
+  const size_t hist_b = epi == kEpiListsLaneHist || epi == kEpiLists ? hist_smem_bytes(P.hist_mode, P.nbins) * kBitWarps / kWarpsPerBlock : 0;
+  const size_t smem = P.mask_bytes + hist_b + (size_t)kBitWarps * P.stage_words * sizeof(uint32_t);
+  NW_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int occ = 0;
+  NW_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBitBlock, smem));
+  if (occ < 1) occ = 1;
+  if (bps && occ > (int)bps) occ = (int)bps;
+  const uint64_t grid = std::min<uint64_t>((uint64_t)c->sm_count * occ, plan.ntasks);
+  void* args[] = {&P};
+  cudaEvent_t e0 = nullptr;
+  tm.begin(true, e0);
+  NW_CK(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kBitBlock), args, smem, stream));
+  tm.end(true, e0);
+  ++ro.dp_launches;
+  return NW_OK;
+}
+
+// The settings of a DPX launch that the bit-parallel kernel shares.
+BitParams bit_params(const DpParams& b, unsigned long long* counter) {
+  BitParams P{};
+  P.counter = counter;
+  P.mat = b.mat;
+  P.n = b.n;
+  P.mat_lo = b.mat_lo;
+  P.mat_hi = b.mat_hi;
+  P.k = b.k;
+  P.hist_mode = b.hist_mode;
+  P.hist = b.hist;
+  P.hist_lo = b.hist_lo;
+  P.nbins = b.nbins;
+  P.stats = b.stats;
+  P.err = b.err;
+  P.norm_rank = b.norm_rank;
+  P.norm_smin = b.norm_smin;
+  P.norm_lo = b.norm_lo;
+  return P;
+}
+
+int epi_for(int mode, int hist_mode) {
+  return mode == kModeMatrix ? kEpiMatrix : (hist_mode == kHistLane ? kEpiListsLaneHist : kEpiLists);
+}
+
+// The whole pair set of a dictionary (or one shard of it, through the
+// context's segment workspace) by whichever kernel its scoring takes.
+nw_status run_dict(nw_dict* d, const DpParams& base, SideView side, unsigned long long* counters, uint32_t shard,
+                   uint32_t nshards, Timer& tm, RunOut& ro) {
+  nw_ctx* c = d->ctx;
+  if (d->ss.bit_m == 0) {
+    const uint32_t* a_enc[3] = {d->ws.a_enc.as<uint32_t>(), nullptr, nullptr};
+    const uint4* b_rec[3] = {d->ws.b_rec.as<uint4>(), nullptr, nullptr};
+    const SideView* views[3] = {&side, nullptr, nullptr};
+    return run_plan(c, c->stream, d->plan, d->d_segs.as<Seg>(), base, counters, shard, nshards, tm, ro, a_enc, views,
+                    b_rec, views);
+  }
+  BitParams P = bit_params(base, counters);
+  P.local[0] = bit_terms(d, d->ws, d->ws, side, side, base.key_lo, base.ib);
+  const int epi = epi_for(base.mode, base.hist_mode);
+  if (nshards == 1)
+    return run_bits(c, c->stream, d->ss.bit_m, d->ss.bit_x, epi, d->alphabet, d->bits, d->d_segs.as<Seg>(), P, tm, ro);
+  BitPlan bp;
+  bit_plan_sized(bp, [&](uint32_t ta, BitPlan& p) { bit_shard(d->ws.bk, d->plan, shard, nshards, ta, p); });
+  NW_TRY(ctx_ensure(c, c->ws_segs, sizeof(Seg) * std::max<size_t>(1, bp.segs.size()), "shard segments"));
+  if (!bp.segs.empty()) {
+    NW_CK(cudaMemcpyAsync(c->ws_segs.p, bp.segs.data(), sizeof(Seg) * bp.segs.size(), cudaMemcpyHostToDevice, c->stream));
+    NW_CK(cudaStreamSynchronize(c->stream));  // the host list goes out of scope
+  }
+  return run_bits(c, c->stream, d->ss.bit_m, d->ss.bit_x, epi, d->alphabet, bp, c->ws_segs.as<Seg>(), P, tm, ro);
+}
+
 nw_status check_device_flags(nw_ctx* c, const uint32_t* d_small) {
   uint32_t err = 0;
   NW_CK(cudaMemcpyAsync(&err, d_small, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
@@ -784,12 +1052,8 @@ nw_status topk_impl(nw_dict* d, uint32_t shard, uint32_t nshards, uint32_t k, ui
     d_frac = reinterpret_cast<const int16_t*>(c->ws_norm.as<char>() + o_frac);
   }
   SideView side{d->ws.perm.as<uint32_t>(), c->ws_slots.as<uint32_t>(), c->ws_thr.as<uint32_t>()};
-  const uint32_t* a_enc[3] = {d->ws.a_enc.as<uint32_t>(), nullptr, nullptr};
-  const uint4* b_rec[3] = {d->ws.b_rec.as<uint4>(), nullptr, nullptr};
-  const SideView* views[3] = {&side, nullptr, nullptr};
   RunOut ro;
-  NW_TRY(run_plan(c, c->stream, d->plan, d->d_segs.as<Seg>(), base, d_counters, shard, nshards, tm, ro, a_enc,
-                  views, b_rec, views));
+  NW_TRY(run_dict(d, base, side, d_counters, shard, nshards, tm, ro));
   cudaEvent_t e_fin = nullptr;
   tm.begin(false, e_fin);
   NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), n, k, d->ws.perm.as<uint32_t>(), ib, base.imask, key_lo,

@@ -68,6 +68,8 @@ struct Seg {
   uint16_t tri;
   uint32_t nca;         // A chunks (tasks = nca * ceil((b_end - b_beg) / kWarpB))
   uint32_t dict;        // terms of the segment in a batched launch (else 0)
+  uint32_t lb;          // bit-parallel launches: the B words' length (brec_base is then the
+                        // index of b_beg's first symbol in the B set's symbols)
   uint64_t task0;       // first task of the segment within its launch
 };
 
@@ -109,15 +111,17 @@ __host__ __device__ __forceinline__ uint32_t find_seg(const Seg* segs, uint32_t 
   return lo;
 }
 
-__host__ __device__ __forceinline__ TaskGeom task_geom(const Seg& S, uint64_t t, uint32_t TA) {
+// B words come in chunks of `chunk` (the whole segment's chunks end at b_end)
+__host__ __device__ __forceinline__ TaskGeom task_geom(const Seg& S, uint64_t t, uint32_t TA,
+                                                       uint32_t chunk = (uint32_t)kWarpB) {
   TaskGeom g;
   uint64_t local = t - S.task0;
   g.ca = (uint32_t)(local % S.nca);
   g.cb = (uint32_t)(local / S.nca);
   g.a0 = S.a_beg + g.ca * TA;
   g.a1 = S.a_end < g.a0 + TA ? S.a_end : g.a0 + TA;
-  g.b0 = S.b_beg + g.cb * (uint32_t)kWarpB;
-  g.bend = S.b_end < g.b0 + (uint32_t)kWarpB ? S.b_end : g.b0 + (uint32_t)kWarpB;
+  g.b0 = S.b_beg + g.cb * chunk;
+  g.bend = S.b_end < g.b0 + chunk ? S.b_end : g.b0 + chunk;
   g.tri = S.tri != 0;
   if (g.tri && g.a1 > g.bend - 1) g.a1 = g.bend - 1;  // some b > a must exist
   if (g.a1 < g.a0) g.a1 = g.a0;
@@ -256,6 +260,66 @@ struct ShiftedScoring {
   int32_t sm, sx;   // s'_m = match - 2*gap, s'_x = mismatch - 2*gap
   uint32_t shift;   // code shift of the XOR encoding
   uint32_t C1, C2;  // packed 16x2 constants
+  int32_t bit_m, bit_x, bit_coef;  // reduced steps of the bit-parallel kernel (bit_m = 0: none) and their gcd
+};
+
+// ---- bit-parallel alignment (nw_bits.cuh) ----
+
+constexpr int kBitBlock = 128;
+constexpr int kBitWarps = kBitBlock / 32;
+constexpr uint32_t kMaskRow = 256;   // bytes of one code's match masks: 32 lanes x 64 columns
+constexpr uint32_t kBitSub = 16;     // A words a warp stages at a time (at most 32)
+constexpr int kBitMaxStep = 5;       // largest reduced match step with a kernel
+
+// Words of length b held in a lane's 64 columns, and the columns each gets
+// (fixed by that number, so that the score extraction knows every field at
+// compile time).  More than eight words of fewer than eight symbols would
+// fit; the planner puts such words on the A side instead.
+__host__ __device__ constexpr int bit_words_per_lane(int b) {
+  return b <= 8 ? 8 : b == 9 ? 7 : b == 10 ? 6 : b <= 12 ? 5 : b <= 16 ? 4 : b <= 21 ? 3 : b <= 32 ? 2 : 1;
+}
+__host__ __device__ constexpr int bit_pitch(int K) {
+  return K == 8 ? 8 : K == 7 ? 9 : K == 6 ? 10 : K == 5 ? 12 : K == 4 ? 16 : K == 3 ? 21 : K == 2 ? 32 : 64;
+}
+
+// Word sets, lists and scoring of one kind of segment (indexed by Seg::dict).
+struct BitTerms {
+  const uint32_t* a_sym;  // a_enc of the A side's set
+  const uint32_t* b_sym;  // a_enc of the B side's set
+  SideView A, B;
+  uint32_t shift;         // code shift of the symbols
+  uint32_t alphabet;
+  uint32_t coef;          // gcd of the steps: G = coef * (sum of the reduced steps)
+  uint32_t serial_a;      // nonzero: one A word's list offers go through the warp one at a time
+  int32_t match, mismatch, gap, key_lo;
+  uint32_t ib, imask;
+};
+
+struct BitParams {
+  const Seg* segs;
+  uint32_t nsegs;
+  uint32_t TA;
+  uint64_t ntasks;
+  unsigned long long* counter;    // zeroed before the launch
+  BitTerms local[2];              // terms of segments 0 and 1 (single-dictionary launches)
+  const BitTerms* terms;          // batched launches: terms by segment (device)
+  uint32_t sub;                   // A words a warp takes at a time (1 .. kBitSub)
+  uint32_t mask_bytes;            // shared memory of the match masks
+  uint32_t stage_words;           // shared words a warp stages symbols in
+  int8_t* mat;                    // as in DpParams from here on
+  uint64_t n;
+  uint64_t mat_lo, mat_hi;
+  uint32_t k;
+  int32_t hist_mode;
+  unsigned long long* hist;
+  int32_t hist_lo;
+  uint32_t nbins;
+  unsigned long long* stats;
+  uint32_t* err;
+  const uint16_t* norm_rank;
+  const int16_t* norm_smin;
+  int32_t norm_lo;
+  uint32_t dbg_insert_limit;
 };
 
 }  // namespace nw

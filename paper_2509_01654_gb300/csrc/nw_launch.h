@@ -12,6 +12,11 @@ namespace nw {
 // scoring (tab: substitution table); nullptr if there is none
 const void* dp_kernel(int LB, int epi, bool tab = false);
 
+// bit-parallel alignment kernel for the reduced steps (m, x) and epilogue
+// kind; nullptr if there is none (kernels exist for gcd(m, x) = 1, x < m <=
+// kBitMaxStep)
+const void* bit_kernel(int m, int x, int epi);
+
 // ingest: stable bucketing by length and encoding of a word set
 cudaError_t launch_ingest_count(const uint8_t* codes, const uint32_t* offsets, uint32_t n,
                                 uint32_t alphabet, uint32_t* block_counts, uint32_t* err,

@@ -32,7 +32,8 @@ EXPORTED = [
     "nw_load_dictionary", "nw_dict_info_get", "nw_dict_free", "nw_all_pairs_matrix",
     "nw_all_pairs_topk", "nw_all_pairs_topk_shard", "nw_topk_merge", "nw_topk_merge_device", "nw_score_pairs",
     "nw_query",
-    "nw_measure_int_rates", "nw_debug_enumerate_pairs", "nw_debug_enumerate_query_pairs", "nw_debug_fail_alloc",
+    "nw_measure_int_rates", "nw_debug_enumerate_pairs", "nw_debug_enumerate_query_pairs", "nw_debug_enumerate_bit_pairs",
+    "nw_debug_fail_alloc",
     "nw_debug_set_bounds",
     "nw_all_pairs_topk_noalloc",
     "nw_server_create", "nw_server_submit", "nw_server_wait", "nw_server_last_error", "nw_server_destroy",
@@ -155,6 +156,7 @@ def load_library(path: str = LIB_PATH):
     L.nw_measure_int_rates.argtypes = [vp, ctypes.c_double, ctypes.POINTER(IntRates)]
     L.nw_debug_enumerate_pairs.argtypes = [vp, u32, u32, u32, vp, vp, u64, ctypes.POINTER(u64)]
     L.nw_debug_enumerate_query_pairs.argtypes = [vp, u32, vp, u32, u32, vp, vp, u64, ctypes.POINTER(u64)]
+    L.nw_debug_enumerate_bit_pairs.argtypes = [vp, u32, vp, u32, u32, u32, u32, vp, vp, u64, ctypes.POINTER(u64)]
     L.nw_debug_fail_alloc.argtypes = [vp, u32]
     L.nw_debug_set_bounds.argtypes = [vp, i32, ctypes.c_int64, u32]
     L.nw_debug_norm_tables.argtypes = [ctypes.POINTER(Scoring), i32, i32, vp, vp, vp, u32, ctypes.POINTER(u32)]
@@ -498,6 +500,24 @@ def debug_enumerate_query_pairs(q_lengths, d_lengths, ta: int = 0):
     if st != NW_OK:
         raise NwError(st, "nw_debug_enumerate_query_pairs failed")
     return q[:cnt.value], d[:cnt.value]
+
+
+def debug_enumerate_bit_pairs(lengths, q_lengths=None, shard: int = 0, nshards: int = 1, ta: int = 0):
+    """The original-index pairs of the bit-parallel kernel's plan, in task order: (a, b) of one set, or
+    (query, word) with query lengths."""
+    L = load_library()
+    wl = np.ascontiguousarray(lengths, dtype=np.uint32)
+    ql = np.ascontiguousarray(q_lengths if q_lengths is not None else [], dtype=np.uint32)
+    out, cnt = (None, None), ctypes.c_uint64(0)
+    for _ in range(2):  # count, then fill
+        st = L.nw_debug_enumerate_bit_pairs(ql.ctypes.data, ql.size, wl.ctypes.data, wl.size, shard, nshards, ta,
+                                            *(None if o is None else o.ctypes.data for o in out),
+                                            0 if out[0] is None else cnt.value, ctypes.byref(cnt))
+        if st != NW_OK:
+            raise NwError(st, "nw_debug_enumerate_bit_pairs failed")
+        if out[0] is None:
+            out = (np.empty(max(1, cnt.value), np.uint32), np.empty(max(1, cnt.value), np.uint32))
+    return out[0][:cnt.value], out[1][:cnt.value]
 
 
 def debug_enumerate_pairs(lengths, shard: int = 0, nshards: int = 1):

@@ -1,0 +1,63 @@
+"""The bit-parallel alignment kernel against the oracle, bit for bit: every step class it is built for, every number of
+words per lane (word lengths 0 to 40), chunk edges, and the largest alphabet."""
+import numpy as np
+import pytest
+
+from paper_2509_01654_gb300 import nw, synth
+
+pytestmark = pytest.mark.gpu
+
+# one scoring of each class of reduced steps (match - 2 gap, mismatch - 2 gap) / gcd, the last two beyond the kernel
+SCORINGS = [(1, -2, -1), (0, -1, -1), (1, -1, -1), (1, -2, -4), (2, -1, -1), (0, -1, -2), (3, -1, -1), (1, -2, -2),
+            (1, -1, -2), (1, 0, -2), (2, -2, -2), (1, -1, -3), (1, 1, -1)]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2509_01654_gb300 import build
+    build.build()
+    with nw.Context(0) as c:
+        yield c
+
+
+def _words(lengths, alphabet, seed):
+    r = np.random.default_rng(seed)
+    offs = np.zeros(len(lengths) + 1, np.uint32)
+    offs[1:] = np.cumsum(lengths)
+    return synth.WordList(r.integers(0, alphabet, int(offs[-1])).astype(np.uint8), offs, alphabet)
+
+
+def _check(ctx, oracle, w, sc, k):
+    d = ctx.load_dictionary(w.codes, w.offsets, w.alphabet, sc)
+    idx, score, hist, lo = d.all_pairs_topk(k)
+    wi, ws = oracle.topk_rows(w, np.arange(w.n), k, sc)
+    ws = np.where(ws == oracle.MISSING_SCORE, nw.MISSING_SCORE, ws)
+    assert np.array_equal(idx, wi) and np.array_equal(score.astype(np.int32), ws)
+    assert np.array_equal(hist, oracle.histogram(w, sc, lo, hist.size))
+    return d
+
+
+@pytest.mark.parametrize("sc", SCORINGS)
+def test_every_step_class_and_length(ctx, oracle_mod, sc):
+    lengths = np.concatenate([np.arange(41), np.random.default_rng(1).integers(0, 41, 400)])
+    w = _words(lengths, 4, 2)
+    d = _check(ctx, oracle_mod, w, sc, 7)
+    q = _words(np.random.default_rng(3).integers(0, 41, 90), 4, 4)
+    qi, qs = d.query(q.codes, q.offsets, 7)
+    oi, os_ = oracle_mod.query_topk(q, w, 7, sc)
+    assert np.array_equal(qi, oi) and np.array_equal(qs.astype(np.int32), os_)
+    d.free()
+
+
+# the last word of a lane's field, of a chunk (32 words a lane slot) and of a strip
+@pytest.mark.parametrize("length,n", [(8, 255), (8, 257), (9, 225), (12, 161), (21, 97), (32, 65), (33, 33), (40, 300)])
+def test_single_length_chunk_edges(ctx, oracle_mod, length, n):
+    _check(ctx, oracle_mod, _words([length] * n, 3, n), (1, -1, -1), 5).free()
+
+
+def test_largest_alphabet_and_matrix(ctx, oracle_mod):
+    w = _words(np.random.default_rng(5).integers(0, 26, 500), 256, 6)
+    d = _check(ctx, oracle_mod, w, (1, -1, -1), 128)
+    assert np.array_equal(d.all_pairs_matrix().astype(np.int32), oracle_mod.all_pairs(w, (1, -1, -1)))
+    assert np.array_equal(d.all_pairs_matrix_chunked(10007).astype(np.int32), oracle_mod.all_pairs(w, (1, -1, -1)))
+    d.free()
