@@ -518,7 +518,6 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   if (bits) {
     BitParams P = bit_params(base, d_counters);
     P.local[0] = bit_terms(d, q, d->ws, qside, dside, key_lo, ib);
-    P.local[0].serial_a = 1u;  // query words are the A side
     P.local[1] = bit_terms(d, d->ws, q, dside, qside, key_lo, ib);
     NW_TRY(run_bits(c, s, d->ss.bit_m, d->ss.bit_x, kEpiLists, d->alphabet, bplan, c->ws_segs.as<Seg>(), P, tm, ro));
   } else {

@@ -119,11 +119,50 @@ __device__ __forceinline__ void bit_row(B64 (&H)[MM], const B64 M, const B64 NL)
   for (int a = 0; a < MM; ++a) H[a] = N[a];
 }
 
-// The planes recoded to binary digits: h = sum over d of 2^d * D[d].
+// Planes a row's state takes: thermometer planes, except for the steps (3, 1)
+// of the paper's scoring, which keep h as two binary digits (below).
+__host__ __device__ constexpr int bit_planes(int m, int x) { return m == 3 && x == 1 ? 2 : m; }
+
+// One row of the steps (3, 1) on the binary digits H[0] + 2 H[1] of h.  The
+// cell's c = max(s, h', v') is 1, 2 or 3: c >= 2 is C2 = M | h' >= 2 | v' >= 2,
+// and c is odd unless it is 2.  v' = 3 and v' >= 2 come from the two carry
+// chains above; the parities of v and h follow from c = v + h' = h + v' alone,
+// without a plane for v >= 1: 14 logic operations and three additions, against
+// 16 on thermometer planes.
+template <bool Split>
+__device__ __forceinline__ void bit_row31(B64 (&H)[2], const B64 M, const B64 NL) {
+  const B64 h0 = H[0], h1 = H[1];
+  const B64 z = ~h1 & ~h0 & NL;                    // h' = 0
+  const B64 g3 = M & z;
+  const B64 U3 = add64<Split>(z, g3) ^ (z & ~M);   // v' = 3
+  const B64 r = M | U3;
+  const B64 g2 = r & ~h1 & NL;                     // c = 3 and h' <= 1
+  const B64 U2 = add64<Split>(g2 | z, g2) ^ (z & ~g2);  // v' >= 2
+  const B64 C2 = M | h1 | U2;
+  const B64 odd = r | ((h1 & h0) | ~C2);           // c = 1 or 3
+  const B64 v0 = (odd ^ h0) & NL;                  // v odd
+  const B64 u0 = add64<Split>(v0, v0);             // v' odd
+  H[0] = odd ^ u0;
+  H[1] = C2 ^ U2 ^ (~odd & u0);
+}
+// The first row (h' = 0): v is 3 from a match on and 1 before it, so c is odd,
+// v' is odd past a word's first column, and h = c - v'.
+template <bool Split>
+__device__ __forceinline__ void bit_row31_first(B64 (&H)[2], const B64 M, const B64 NL) {
+  const B64 g3 = M & NL;
+  const B64 U3 = add64<Split>(NL, g3) ^ (NL & ~M);
+  H[0] = ~add64<Split>(NL, NL);
+  H[1] = M & ~U3;
+}
+
+// The state recoded to binary digits: h = sum over d of 2^d * D[d].
 __host__ __device__ constexpr int bit_digits(int m) { return m == 1 ? 1 : (m <= 3 ? 2 : 3); }
-template <int MM>
-__device__ __forceinline__ void bit_digit_planes(const B64 (&H)[MM], B64 (&D)[bit_digits(MM)]) {
-  if constexpr (MM == 1) {
+template <int MM, int XX>
+__device__ __forceinline__ void bit_digit_planes(const B64 (&H)[bit_planes(MM, XX)], B64 (&D)[bit_digits(MM)]) {
+  if constexpr (MM == 3 && XX == 1) {
+    D[0] = H[0];
+    D[1] = H[1];
+  } else if constexpr (MM == 1) {
     D[0] = H[0];
   } else if constexpr (MM == 2) {
     D[0] = H[0] & ~H[1];
@@ -140,6 +179,23 @@ __device__ __forceinline__ void bit_digit_planes(const B64 (&H)[MM], B64 (&D)[bi
     D[1] = H[1] & ~H[3];
     D[2] = H[3];
   }
+}
+
+// row 1 from nothing, and any later row
+template <int MM, int XX, bool Split>
+__device__ __forceinline__ void bit_first(B64 (&H)[bit_planes(MM, XX)], const B64 M, const B64 NL) {
+  if constexpr (MM == 3 && XX == 1) {
+    bit_row31_first<Split>(H, M, NL);
+  } else {
+#pragma unroll
+    for (int a = 0; a < MM; ++a) H[a] = {0u, 0u};  // folds most of the row away
+    bit_row<MM, XX, Split>(H, M, NL);
+  }
+}
+template <int MM, int XX, bool Split>
+__device__ __forceinline__ void bit_next(B64 (&H)[bit_planes(MM, XX)], const B64 M, const B64 NL) {
+  if constexpr (MM == 3 && XX == 1) bit_row31<Split>(H, M, NL);
+  else bit_row<MM, XX, Split>(H, M, NL);
 }
 
 // bits of a word's field [w * pitch, (w + 1) * pitch) in the two halves
@@ -176,15 +232,6 @@ __device__ __forceinline__ void bit_scores(const B64 (&D)[bit_digits(MM)], B64 F
   }
 }
 
-// value i of a register array by a run-time index
-template <int N>
-__device__ __forceinline__ uint32_t pick(const uint32_t (&v)[N], int i) {
-  uint32_t r = v[0];
-#pragma unroll
-  for (int x = 1; x < N; ++x) r = x == i ? v[x] : r;
-  return r;
-}
-
 // what a task's warps share
 struct BitTask {
   TaskGeom g;
@@ -195,28 +242,74 @@ struct BitTask {
   bool check;             // same bucket, chunks overlap: test a < b
 };
 
+// Candidate queue.  A pair that may enter a list is rare late in a launch and
+// common early, and filing it takes several dependent trips to L2.  The lanes
+// only append such pairs to their warp's queue; once 32 are waiting, each lane
+// files one, so the trips overlap 32-fold.  (Filing each pair in the lane that
+// found it took 126 of 584 ms at 600k words, half of the time at 100k.)
+// An entry: G << 16 | A word (from g.a0) << 8 | B word (from g.b0); G < 2^15,
+// a task has at most 256 words on either side.
+constexpr uint32_t kBitQueue = 64;  // entries: up to 31 waiting plus a warp's 32
+
+// Files n <= 32 queued pairs in their words' lists; returns the lane's inserts.
+__device__ __forceinline__ uint32_t bit_drain(const BitParams& P, const BitTerms& T, const BitTask& Q,
+                                           const uint32_t* queue, uint32_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const int max_iters = P.dbg_insert_limit ? (int)(P.dbg_insert_limit - 1u) : kInsertMaxIters;
+  const bool have = lane < n;
+  const uint32_t e = have ? queue[lane] : 0u;
+  const uint32_t a = Q.g.a0 + ((e >> 8) & 0xffu), b = Q.g.b0 + (e & 0xffu);
+  const int s = (int)(e >> 16) + T.gap * (Q.la + Q.lb);
+  const uint32_t oa = have ? __ldg(T.A.perm + a) : 0u, ob = have ? __ldg(T.B.perm + b) : 0u;
+  uint32_t inserts = 0u;
+  if (T.B.slots && have) {  // word b takes the A word as a neighbour
+    const uint32_t key = list_key(P, T, s, Q.mx, oa);
+    if (key > __ldcg(T.B.thr + b))
+      list_offer(T.B.slots + (size_t)b * P.k, T.B.thr + b, P.k, key, P.err, inserts, max_iters);
+  }
+  if (T.A.slots) {
+    // the A word takes word b.  Several lanes may hold the same A word: one
+    // lane of each such group offers at a time and the others are tested again
+    // against the bound it leaves, so the lanes never race on one list
+    uint32_t key = 0u;
+    if (have) {
+      key = list_key(P, T, s, Q.mx, ob);
+      if (key <= __ldcg(T.A.thr + a)) key = 0u;
+    }
+    const uint32_t group = __match_any_sync(0xffffffffu, a);
+    uint32_t todo;
+    while ((todo = __ballot_sync(0xffffffffu, key != 0u)) != 0u) {
+      if ((uint32_t)(__ffs(todo & group) - 1) == lane) {
+        list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, key, P.err, inserts, max_iters);
+        key = 0u;
+      }
+      __syncwarp();
+      if (key != 0u && key <= __ldcg(T.A.thr + a)) key = 0u;
+    }
+  }
+  return inserts;
+}
+
 // The A words of one task against the lane's K words (b = b0 + 32 w + lane).
 template <int MM, int XX, int EPI, int K>
 __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, const BitTask& Q,
-                                         const unsigned char* masks, uint32_t* wh, uint32_t* sA, uint32_t& inserts,
-                                         int max_iters) {
+                                         const unsigned char* masks, uint32_t* wh, uint16_t* sA, uint32_t* queue,
+                                         uint32_t& inserts) {
   constexpr int PITCH = bit_pitch(K);
   constexpr bool kSplit = PITCH == 8 || PITCH == 16 || PITCH == 32;
   constexpr bool kLists = EPI != kEpiMatrix;
   constexpr bool kHist = EPI == kEpiListsLaneHist;
   constexpr int KP = (K + 1) / 2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const TaskGeom& g = Q.g;
+  const TaskGeom g = Q.g;
   const int pconst = T.gap * (Q.la + Q.lb);  // score = G + pconst
-  const bool listsA = kLists && T.A.slots != nullptr;
-  const bool listsB = kLists && T.B.slots != nullptr;
-  const bool serialA = !kHist && listsA && T.serial_a != 0u;
+  const bool check = Q.check;
   const int la = Q.la;
 
   // columns of the lane's words: all of them, and all but each word's last
   B64 FM{0u, 0u}, NL{0u, 0u};
   {
-    const uint64_t f = Q.lb >= 64 ? ~0ull : ((1ull << Q.lb) - 1ull);
+    const uint64_t f = (1ull << Q.lb) - 1ull;
     uint64_t fm = 0, nl = 0;
 #pragma unroll
     for (int w = 0; w < K; ++w) {
@@ -229,19 +322,29 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
   uint32_t vmask = 0u;  // bit w: word w exists
 #pragma unroll
   for (int w = 0; w < K; ++w) vmask |= (g.b0 + 32u * w + lane < g.bend ? 1u : 0u) << w;
-  const bool full = __all_sync(0xffffffffu, vmask == (1u << K) - 1u) && !Q.check;
+  const bool full = __all_sync(0xffffffffu, vmask == (1u << K) - 1u) && !check;
 
-  // B-side list bounds in G, packed for the prefilter (see neg_bound16)
+  // list bounds in G, packed for the prefilter (see neg_bound16): the lane's
+  // B words, and A word c0 + lane of the words staged last
   uint32_t nB2[KP];
+  uint32_t my_nA2 = 0u;
+  auto load_bounds_B = [&]() {
 #pragma unroll
-  for (int i = 0; i < KP; ++i) {
-    int t[2] = {INT_MAX, INT_MAX};
+    for (int i = 0; i < KP; ++i) {
+      int t[2] = {INT_MAX, INT_MAX};
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (listsB && ((vmask >> (2 * i + h)) & 1u))
-        t[h] = g_bound(P, T, __ldcg(T.B.thr + g.b0 + 32u * (2 * i + h) + lane), Q.mx, pconst);
-    nB2[i] = neg_bound2(t[0], t[1]);
-  }
+      for (int h = 0; h < 2; ++h)
+        if (T.B.slots && ((vmask >> (2 * i + h)) & 1u))
+          t[h] = g_bound(P, T, __ldcg(T.B.thr + g.b0 + 32u * (2 * i + h) + lane), Q.mx, pconst);
+      nB2[i] = neg_bound2(t[0], t[1]);
+    }
+  };
+  auto load_bound_A = [&](uint32_t c0, uint32_t nA) {
+    const int t = T.A.slots && (uint32_t)lane < nA ? g_bound(P, T, __ldcg(T.A.thr + c0 + lane), Q.mx, pconst) : INT_MAX;
+    my_nA2 = neg_bound2(t, t);
+  };
+  if constexpr (kLists) load_bounds_B();
+  uint32_t waiting = 0u;  // queued candidates (warp-uniform)
   uint32_t ob[EPI == kEpiMatrix ? K : 1];
   if constexpr (EPI == kEpiMatrix) {
 #pragma unroll
@@ -255,52 +358,45 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
   for (uint32_t c0 = g.a0 + (uint32_t)warp * sub; c0 < g.a1; c0 += kBitWarps * sub) {
     const uint32_t nA = g.a1 - c0 < sub ? g.a1 - c0 : sub;
     // the symbols of nA consecutive A words are one run of T.a_sym: stage
-    // their table offsets (two zero entries beyond for the reads ahead)
+    // their codes (two zero entries beyond for the reads ahead)
     __syncwarp();
-    const uint32_t total = nA * (uint32_t)la;
-    const uint32_t* src = T.a_sym + Q.a_base + (size_t)(c0 - g.a0) * (uint32_t)la;
-    const uint32_t shift = T.shift;
-    for (uint32_t i = lane; i < total + 2u; i += 32u)
-      sA[i] = i < total ? ((__ldg(src + i) & 0xffffu) >> shift) * kMaskRow : 0u;
-    const uint32_t my_a = c0 + (uint32_t)lane;
-    const bool have = (uint32_t)lane < nA;
-    const uint32_t my_orig = (EPI == kEpiMatrix && have) ? __ldg(T.A.perm + my_a) : 0u;
-    uint32_t my_nA2 = 0u;
-    if constexpr (kLists) {
-      const int t = listsA && have ? g_bound(P, T, __ldcg(T.A.thr + my_a), Q.mx, pconst) : INT_MAX;
-      my_nA2 = neg_bound2(t, t);
+    {
+      const uint32_t total = nA * (uint32_t)la;
+      const uint32_t* src = T.a_sym + Q.a_base + (size_t)(c0 - g.a0) * (uint32_t)la;
+      const uint32_t shift = T.shift;
+      for (uint32_t i = lane; i < total + 2u; i += 32u)
+        sA[i] = i < total ? (uint16_t)((__ldg(src + i) & 0xffffu) >> shift) : (uint16_t)0;
     }
+    const uint32_t my_orig = (EPI == kEpiMatrix && (uint32_t)lane < nA) ? __ldg(T.A.perm + c0 + lane) : 0u;
+    if constexpr (kLists) load_bound_A(c0, nA);
     __syncwarp();
 
     const unsigned char* mrow = masks + lane * 8;
-    const uint32_t* sp = sA;
-    uint2 mv = *reinterpret_cast<const uint2*>(mrow + sp[0]);
+    const uint16_t* sp = sA;
+    uint2 mv = *reinterpret_cast<const uint2*>(mrow + sp[0] * kMaskRow);
     uint32_t o1 = sp[1];
+    auto next_mask = [&]() {  // the row's mask; the next one's read is issued
+      const B64 M{mv.x, mv.y};
+      mv = *reinterpret_cast<const uint2*>(mrow + o1 * kMaskRow);
+      o1 = sp[2];
+      ++sp;
+      return M;
+    };
     for (uint32_t w0 = 0; w0 < nA; ++w0) {
       const uint32_t a = c0 + w0;
-      B64 H[MM];
-#pragma unroll
-      for (int x = 0; x < MM; ++x) H[x] = {0u, 0u};
+      B64 H[bit_planes(MM, XX)];
       if (la > 0) {
-        // the first row (H = 0) folds to a few operations
-        {
-          const B64 M{mv.x, mv.y};
-          mv = *reinterpret_cast<const uint2*>(mrow + o1);
-          o1 = sp[2];
-          ++sp;
-          bit_row<MM, XX, kSplit>(H, M, NL);
-        }
-#pragma unroll 2
-        for (int r = 1; r < la; ++r) {
-          const B64 M{mv.x, mv.y};
-          mv = *reinterpret_cast<const uint2*>(mrow + o1);
-          o1 = sp[2];
-          ++sp;
-          bit_row<MM, XX, kSplit>(H, M, NL);
-        }
+        bit_first<MM, XX, kSplit>(H, next_mask(), NL);
+        // (unrolled by 1, 2, 4: 388, 394, 398 ms at 600k words; eight bodies
+        // share the instruction cache)
+#pragma unroll 1
+        for (int r = 1; r < la; ++r) bit_next<MM, XX, kSplit>(H, next_mask(), NL);
+      } else {
+#pragma unroll
+        for (int x = 0; x < bit_planes(MM, XX); ++x) H[x] = {0u, 0u};
       }
       B64 D[bit_digits(MM)];
-      bit_digit_planes<MM>(H, D);
+      bit_digit_planes<MM, XX>(H, D);
       int gv[K];
       bit_scores<MM, K>(D, FM, coef, gv);
 
@@ -308,129 +404,131 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
         const uint32_t oa = __shfl_sync(0xffffffffu, my_orig, (int)w0);
 #pragma unroll
         for (int w = 0; w < K; ++w) {
-          if (!((vmask >> w) & 1u) || (Q.check && a >= g.b0 + 32u * w + lane)) continue;
+          if (!((vmask >> w) & 1u) || (check && a >= g.b0 + 32u * w + lane)) continue;
           const uint64_t i = oa < ob[w] ? oa : ob[w], j = oa < ob[w] ? ob[w] : oa;
           const uint64_t off = upper_offset(i, j, P.n);
           if (off >= P.mat_lo && off < P.mat_hi) P.mat[off] = (int8_t)(gv[w] + pconst);
         }
       } else {
         if constexpr (kHist) {
+          // lane columns: a warp's additions never collide
           if (full) {
 #pragma unroll
-            for (int w = 0; w < K; ++w) hcol[32 * gv[w]] += 1u;
+            for (int w = 0; w < K; ++w) atomicAdd(hcol + 32 * gv[w], 1u);
           } else {
 #pragma unroll
             for (int w = 0; w < K; ++w)
-              if (((vmask >> w) & 1u) && (!Q.check || a < g.b0 + 32u * w + lane)) hcol[32 * gv[w]] += 1u;
+              if (((vmask >> w) & 1u) && (!check || a < g.b0 + 32u * w + lane)) atomicAdd(hcol + 32 * gv[w], 1u);
           }
         } else if (EPI == kEpiLists && P.hist_mode != kHistNone) {
 #pragma unroll
           for (int w = 0; w < K; ++w)
-            if (((vmask >> w) & 1u) && (!Q.check || a < g.b0 + 32u * w + lane))
+            if (((vmask >> w) & 1u) && (!check || a < g.b0 + 32u * w + lane))
               hist_add(P, wh, lane, gv[w] + pconst - P.hist_lo);
         }
+        // prefilter: non-zero when some word's G reaches its own list's bound,
+        // or the largest G reaches the A word's
         uint32_t res[KP];
 #pragma unroll
-        for (int i = 0; i < KP; ++i) res[i] = (uint32_t)gv[2 * i] + (2 * i + 1 < K ? (uint32_t)gv[2 * i + 1 < K ? 2 * i + 1 : 0] * 65536u : 0u);
+        for (int i = 0; i < KP; ++i)
+          res[i] = (uint32_t)gv[2 * i] + (2 * i + 1 < K ? (uint32_t)gv[2 * i + 1 < K ? 2 * i + 1 : 0] * 65536u : 0u);
         const uint32_t nA2 = __shfl_sync(0xffffffffu, my_nA2, (int)w0);
-        uint32_t any = 0u;
+        uint32_t top = res[0], any = __viaddmax_s16x2_relu(res[0], nB2[0], 0u);
 #pragma unroll
-        for (int i = 0; i < KP; ++i) any |= __viaddmax_s16x2_relu(res[i], __vmaxs2(nB2[i], nA2), 0u);
-        uint32_t amask = 0u;  // words this lane offers to the A word's list (serial offers)
-        if (any) {
-          const uint32_t thrA = listsA ? __ldcg(T.A.thr + a) : 0u;
-          const uint32_t oa = __ldg(T.A.perm + a);
+        for (int i = 1; i < KP; ++i) {
+          top = __vmaxs2(top, res[i]);
+          any = __viaddmax_s16x2(res[i], nB2[i], any);
+        }
+        any = __viaddmax_s16x2(top, nA2, any);
+        if (__any_sync(0xffffffffu, any != 0u)) {
+          uint32_t cand = 0u;  // bit w: word w is a candidate
+#pragma unroll
           for (int w = 0; w < K; ++w) {
-            const uint32_t b = g.b0 + 32u * (uint32_t)w + (uint32_t)lane;
-            if (!((vmask >> w) & 1u) || (Q.check && a >= b)) continue;
-            const uint32_t rv = pick<KP>(res, w >> 1), nv = pick<KP>(nB2, w >> 1);
-            const int G = (int)((w & 1) ? rv >> 16 : rv & 0xffffu);
-            const int nb = (int)(int16_t)((w & 1) ? nv >> 16 : nv & 0xffffu);
-            const int s = G + pconst;
-            if (listsB && G + nb > 0) {  // word b takes the A word as a neighbour
-              const uint32_t key = list_key(P, T, s, Q.mx, oa);
-              uint32_t nm = __ldcg(T.B.thr + b);
-              if (key > nm)
-                nm = list_offer(T.B.slots + (size_t)b * P.k, T.B.thr + b, P.k, key, P.err, inserts, max_iters);
-              const uint32_t nn = neg_bound16(g_bound(P, T, nm, Q.mx, pconst));
-              const uint32_t keep = (w & 1) ? (nv & 0xffffu) | (nn << 16) : (nv & 0xffff0000u) | nn;
+            // the packed test again, one half at a time on plain integers
+            const uint32_t n2 = __vmaxs2(nB2[w >> 1], nA2);
+            const int nb = (w & 1) ? (int)n2 >> 16 : (int)(int16_t)n2;
+            const bool in = gv[w] + nb > 0 && (!check || a < g.b0 + 32u * w + lane);
+            cand |= (in ? 1u : 0u) << w;
+          }
+          cand &= vmask;
+          bool filed = false;
+          uint32_t m;
+          while ((m = __ballot_sync(0xffffffffu, cand != 0u)) != 0u) {
+            if (cand) {
+              const int w = __ffs(cand) - 1;
+              uint32_t G = res[0];
 #pragma unroll
-              for (int i = 0; i < KP; ++i)
-                if (i == (w >> 1)) nB2[i] = keep;
+              for (int i = 1; i < KP; ++i) G = (w >> 1) == i ? res[i] : G;
+              G = (w & 1) ? G >> 16 : G & 0xffffu;
+              queue[waiting + __popc(m & ((1u << lane) - 1u))] =
+                  (G << 16) | ((a - g.a0) << 8) | (32u * (uint32_t)w + (uint32_t)lane);
+              cand &= cand - 1u;
             }
-            if (listsA) {  // the A word takes word b as a neighbour
-              const uint32_t ob1 = __ldg(T.B.perm + b);
-              const uint32_t key = list_key(P, T, s, Q.mx, ob1);
-              if (key > thrA) {
-                if (serialA) amask |= 1u << w;
-                else list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, key, P.err, inserts, max_iters);
-              }
+            waiting += __popc(m);
+            if (waiting >= 32u) {
+              __syncwarp();
+              inserts += bit_drain(P, T, Q, queue, 32u);
+              waiting -= 32u;
+              const uint32_t v = (uint32_t)lane < waiting ? queue[32 + lane] : 0u;
+              __syncwarp();
+              queue[lane] = v;
+              __syncwarp();
+              filed = true;
             }
           }
-        }
-        if (serialA) {
-          // many lanes may hold keys for the same A word's list: the warp
-          // offers them one at a time from the best down, each against the
-          // bound the previous offer returned (the lanes never race on that
-          // list, and a list that is already full costs one offer)
-          uint32_t thrW = 0u;
-          while (__any_sync(0xffffffffu, amask != 0u)) {
-            uint32_t best = 0u;
-            int bw = -1;
-            for (int w = 0; w < K; ++w)
-              if ((amask >> w) & 1u) {
-                const uint32_t rv = pick<KP>(res, w >> 1);
-                const int s = (int)((w & 1) ? rv >> 16 : rv & 0xffffu) + pconst;
-                const uint32_t key = list_key(P, T, s, Q.mx, __ldg(T.B.perm + g.b0 + 32u * (uint32_t)w + lane));
-                if (key <= thrW) amask &= ~(1u << w);
-                else if (key > best) { best = key; bw = w; }
-              }
-            const uint32_t m = __reduce_max_sync(0xffffffffu, best);
-            if (m == 0u) break;  // every key fell below the list's bound
-            const int src = __ffs(__ballot_sync(0xffffffffu, best == m)) - 1;
-            uint32_t nm = 0u;
-            if (lane == src) {
-              nm = list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, m, P.err, inserts, max_iters);
-              amask &= ~(1u << bw);
-            }
-            nm = __shfl_sync(0xffffffffu, nm, src);
-            thrW = nm > thrW ? nm : thrW;
+          if (filed) {
+            load_bounds_B();
+            load_bound_A(c0, nA);
           }
         }
       }
     }
   }
+  if constexpr (kLists) {
+    if (waiting) {
+      __syncwarp();
+      inserts += bit_drain(P, T, Q, queue, waiting);
+    }
+  }
 }
 
-// blocks per SM the kernel is compiled for
-constexpr int kBitMinBlocks = 6;
+// Blocks per SM the kernel is compiled for: 5 leave the row loop and the
+// epilogue ~100 registers a thread.  600k words: 4 blocks 407 ms, 5 blocks
+// 394, 6 blocks 408, 8 blocks 414 (the row loop unrolled twice).
+constexpr int kBitMinBlocks = 5;
 
 template <int MM, int XX, int EPI>
-__global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const BitParams P) {
+__global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const __grid_constant__ BitParams P) {
   extern __shared__ __align__(16) unsigned char s_bits[];
   __shared__ unsigned long long s_task[2];
   __shared__ uint32_t s_seg[2];
+  __shared__ uint32_t s_queue[kBitWarps][kBitQueue];
   // the task's terms and geometry live in shared memory: most of them are
   // read on the rare paths only, and registers are what bounds the block count
   __shared__ BitTerms T;
   __shared__ BitTask Q;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // dynamic shared memory: match masks, histogram (lane columns shared by the
+  // block, or one array per warp), staged A symbols
   constexpr bool kHist = EPI == kEpiListsLaneHist;
-  const bool smem_hist = kHist || (EPI == kEpiLists && P.hist_mode == kHistSmem);
-  const uint32_t wstride = kHist ? P.nbins * 32u : (smem_hist ? P.nbins : 0u);
+  const bool warp_hist = EPI == kEpiLists && P.hist_mode == kHistSmem;
+  const uint32_t hist_words = kHist ? P.nbins * 32u : (warp_hist ? P.nbins * kBitWarps : 0u);
   unsigned char* masks = s_bits;
-  uint32_t* wh = reinterpret_cast<uint32_t*>(s_bits + P.mask_bytes) + (size_t)warp * wstride;
-  uint32_t* sA = reinterpret_cast<uint32_t*>(s_bits + P.mask_bytes) + (size_t)kBitWarps * wstride +
-                 (size_t)warp * P.stage_words;
-  if (smem_hist)
-    for (uint32_t q = lane; q < wstride; q += 32) wh[q] = 0u;
-  uint64_t wpairs = 0;
+  uint32_t* hist0 = reinterpret_cast<uint32_t*>(s_bits + P.mask_bytes);
+  uint32_t* wh = hist0 + (warp_hist ? (size_t)warp * P.nbins : 0);
+  uint16_t* sA = reinterpret_cast<uint16_t*>(hist0 + hist_words) + (size_t)warp * P.stage_syms;
+  for (uint32_t q = (uint32_t)tid; q < hist_words; q += kBitBlock) hist0[q] = 0u;
+  uint64_t hpairs = 0;
   uint32_t inserts = 0;
-  const int max_iters = P.dbg_insert_limit ? (int)(P.dbg_insert_limit - 1u) : kInsertMaxIters;
   auto fetch = [&](int buf) {  // thread 0: the next task and its segment
     const unsigned long long t = atomicAdd(P.counter, 1ull);
     s_task[buf] = t;
     s_seg[buf] = t < P.ntasks ? find_seg(P.segs, P.nsegs, t) : 0u;
+  };
+  auto flush = [&]() {  // block-uniform
+    __syncthreads();
+    if (warp_hist || (kHist && warp == 0)) hist_flush(P, wh, lane);
+    __syncthreads();
   };
   if (tid == 0) fetch(0);
   for (int buf = 0;; buf ^= 1) {
@@ -474,14 +572,13 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
           for (int j = 0; j < lb; ++j) {
             const uint32_t c = (__ldg(src + j) & 0xffffu) >> shift;
             const int bit = at + j;
-            atomicOr(reinterpret_cast<uint32_t*>(masks + c * (uint32_t)kMaskRow) + lane * 2 + (bit >> 5), 1u << (bit & 31));
+            atomicOr(reinterpret_cast<uint32_t*>(masks + c * kMaskRow) + lane * 2 + (bit >> 5), 1u << (bit & 31));
           }
         }
       }
     }
     if ((EPI == kEpiLists || kHist) && P.hist_mode != kHistNone) {
-      // every bin this task can produce lies inside the histogram (proven
-      // bounds; the launch's plan holds only length pairs that the bins cover)
+      // every bin this task can produce lies inside the histogram (proven bounds)
       int lo, hi;
       pair_score_bounds(T.match, T.mismatch, T.gap, Q.la < Q.lb ? Q.la : Q.lb, Q.mx, lo, hi);
       if (lo < P.hist_lo || hi - P.hist_lo >= (int)P.nbins) {
@@ -491,24 +588,24 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
     }
     __syncthreads();
     switch (K) {
-      case 8: bit_task<MM, XX, EPI, 8>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      case 7: bit_task<MM, XX, EPI, 7>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      case 6: bit_task<MM, XX, EPI, 6>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      case 5: bit_task<MM, XX, EPI, 5>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      case 4: bit_task<MM, XX, EPI, 4>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      case 3: bit_task<MM, XX, EPI, 3>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      case 2: bit_task<MM, XX, EPI, 2>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
-      default: bit_task<MM, XX, EPI, 1>(P, T, Q, masks, wh, sA, inserts, max_iters); break;
+      case 8: bit_task<MM, XX, EPI, 8>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      case 7: bit_task<MM, XX, EPI, 7>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      case 6: bit_task<MM, XX, EPI, 6>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      case 5: bit_task<MM, XX, EPI, 5>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      case 4: bit_task<MM, XX, EPI, 4>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      case 3: bit_task<MM, XX, EPI, 3>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      case 2: bit_task<MM, XX, EPI, 2>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
+      default: bit_task<MM, XX, EPI, 1>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
     }
-    if (smem_hist) {  // 32-bit shared counters: flush long before they could wrap
-      wpairs += (uint64_t)(Q.g.a1 - Q.g.a0) * (32u * (uint32_t)K);
-      if (wpairs >= (1ull << 30)) {
-        hist_flush(P, wh, lane);
-        wpairs = 0;
+    if (hist_words) {  // 32-bit shared counters: flush long before they could wrap
+      hpairs += (uint64_t)(Q.g.a1 - Q.g.a0) * (32u * (uint32_t)K);
+      if (hpairs >= (1ull << 30)) {
+        flush();
+        hpairs = 0;
       }
     }
   }
-  if (smem_hist) hist_flush(P, wh, lane);
+  if (hist_words) flush();
   if (P.stats) {
     for (int o = 16; o > 0; o >>= 1) inserts += __shfl_xor_sync(0xffffffffu, inserts, o);
     if (lane == 0 && inserts) atomicAdd(P.stats, (unsigned long long)inserts);

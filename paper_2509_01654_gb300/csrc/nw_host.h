@@ -872,12 +872,14 @@ nw_status run_bits(nw_ctx* c, cudaStream_t stream, int m, int x, int epi, uint32
   P.ntasks = plan.ntasks;
   P.sub = std::max<uint32_t>(1, std::min<uint32_t>(kBitSub, plan.ta / kBitWarps));
   P.mask_bytes = alphabet * kMaskRow;
-  P.stage_words = (P.sub * plan.max_la + 2 + 3) & ~3u;
+  P.stage_syms = (P.sub * plan.max_la + 2 + 7) & ~7u;
   P.dbg_insert_limit = c->dbg_insert_iters >= 0 ? (uint32_t)c->dbg_insert_iters + 1u : 0u;
   const void* fn = bit_kernel(m, x, epi);
   if (!fn) return set_err(c, NW_EINVAL, "no kernel for steps (%d, %d)", m, x);
-  const size_t hist_b = epi == kEpiListsLaneHist || epi == kEpiLists ? hist_smem_bytes(P.hist_mode, P.nbins) * kBitWarps / kWarpsPerBlock : 0;
-  const size_t smem = P.mask_bytes + hist_b + (size_t)kBitWarps * P.stage_words * sizeof(uint32_t);
+  const size_t hist_words = epi == kEpiListsLaneHist                                ? (size_t)P.nbins * 32
+                            : epi == kEpiLists && P.hist_mode == kHistSmem ? (size_t)P.nbins * kBitWarps
+                                                                                    : 0;
+  const size_t smem = P.mask_bytes + hist_words * sizeof(uint32_t) + (size_t)kBitWarps * P.stage_syms * sizeof(uint16_t);
   NW_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int occ = 0;
   NW_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBitBlock, smem));

@@ -268,7 +268,7 @@ struct ShiftedScoring {
 constexpr int kBitBlock = 128;
 constexpr int kBitWarps = kBitBlock / 32;
 constexpr uint32_t kMaskRow = 256;   // bytes of one code's match masks: 32 lanes x 64 columns
-constexpr uint32_t kBitSub = 16;     // A words a warp stages at a time (at most 32)
+constexpr uint32_t kBitSub = 32;     // A words a warp stages at a time (at most 32)
 constexpr int kBitMaxStep = 5;       // largest reduced match step with a kernel
 
 // Words of length b held in a lane's 64 columns, and the columns each gets
@@ -290,7 +290,6 @@ struct BitTerms {
   uint32_t shift;         // code shift of the symbols
   uint32_t alphabet;
   uint32_t coef;          // gcd of the steps: G = coef * (sum of the reduced steps)
-  uint32_t serial_a;      // nonzero: one A word's list offers go through the warp one at a time
   int32_t match, mismatch, gap, key_lo;
   uint32_t ib, imask;
 };
@@ -305,7 +304,7 @@ struct BitParams {
   const BitTerms* terms;          // batched launches: terms by segment (device)
   uint32_t sub;                   // A words a warp takes at a time (1 .. kBitSub)
   uint32_t mask_bytes;            // shared memory of the match masks
-  uint32_t stage_words;           // shared words a warp stages symbols in
+  uint32_t stage_syms;            // symbols a warp has room to stage
   int8_t* mat;                    // as in DpParams from here on
   uint64_t n;
   uint64_t mat_lo, mat_hi;
