@@ -272,10 +272,11 @@ typedef struct {
                                 * dictionary's own lists are not computed */
 } nw_batch_dict;
 
-/* nw_batch_create flag: time tile-shape candidates per launch.  Per longer
- * length, the A words per task are chosen from {64, 128, 256}, then the
- * resident blocks per SM from {2, 3, as many as fit} at that size, by timing
- * whole launches on the batch.  (A task's B chunk is 64 words: two words per
+/* nw_batch_create flag: time tile-shape candidates per launch.  Per range of
+ * ten longer lengths, the A words per task of the DPX kernel's launch are
+ * chosen from {64, 128, 256}, then the resident blocks per SM from {2, 3, as
+ * many as fit} at that size, by timing whole launches on the batch.  (The
+ * bit-parallel kernel's launches follow a rule on their number of tasks.)  (A task's B chunk is 64 words: two words per
  * lane in the kernel's int16x2 registers, fixed at compile time.)  The
  * choices are cached for the life of the process, keyed by the device's SM
  * count, k, and every dictionary's and query set's length histogram, scoring

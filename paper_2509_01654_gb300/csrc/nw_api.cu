@@ -54,9 +54,10 @@ nw_status load_impl(nw_ctx* c, const uint8_t* codes, const uint32_t* offsets, ui
     if (lo > hi) lo = hi = 0;  // fewer than two words
     d->score_lo = lo;
     d->score_hi = hi;
-    plan_all_pairs(d->ws.bk, kDefaultTA, d->plan);
-    if (d->ss.bit_m) bit_plan_sized(d->bits, [&](uint32_t ta, BitPlan& p) { bit_pairs(d->ws.bk, ta, 0, p); });
-    const std::vector<Seg>& segs = d->ss.bit_m ? d->bits.segs : d->plan.segs;
+    Rects rects;
+    rects_all(d->ws.bk, 0, rects);
+    make_plan(std::move(rects), d->ss, alphabet, 0, d->plan);
+    const std::vector<Seg>& segs = d->plan.segs;
     st = ctx_alloc(c, d->d_segs, sizeof(Seg) * std::max<size_t>(1, segs.size()), "segment plan");
     if (st == NW_OK && !segs.empty()) {
       cudaError_t e = cudaMemcpyAsync(d->d_segs.p, segs.data(), sizeof(Seg) * segs.size(),
@@ -249,7 +250,7 @@ nw_status matrix_impl(nw_dict* d, int8_t* out, uint64_t chunk_bytes, uint32_t fl
     NW_TRY(ctx_ensure(c, c->ws_mat, step, "score matrix"));
     dst = c->ws_mat.as<int8_t>();
   }
-  NW_TRY(ctx_ensure(c, c->ws_small, 64 + sizeof(unsigned long long) * (d->plan.launches.size() + 1), "task counters"));
+  NW_TRY(ctx_ensure(c, c->ws_small, kCounterBytes, "task counters"));
   uint32_t* d_err = c->ws_small.as<uint32_t>();
   unsigned long long* d_counters = reinterpret_cast<unsigned long long*>(c->ws_small.as<char>() + 64);
   Timer tm{c};
@@ -260,23 +261,17 @@ nw_status matrix_impl(nw_dict* d, int8_t* out, uint64_t chunk_bytes, uint32_t fl
   for (uint64_t lo = 0; lo < E; lo += step) {
     const uint64_t hi = std::min(E, lo + step);
     if (lo > 0) NW_CK(cudaMemsetAsync(d_counters, 0, sizeof(unsigned long long) * d->plan.launches.size(), s));
-    DpParams base{};
-    base.TA = kDefaultTA;
-    base.C1 = d->ss.C1;
-    base.C2 = d->ss.C2;
-    base.match = d->sc.match;
-    base.mismatch = d->sc.mismatch;
-    base.gap = d->sc.gap;
+    AlignParams base{};
     base.sim_tab = dict_tab(d);
-    base.mode = kModeMatrix;
     base.mat = dst - lo;  // entry `off` of the chunk [lo, hi) lands at dst[off - lo]
     base.n = n;
     base.mat_lo = lo;
     base.mat_hi = hi;
     base.hist_mode = kHistNone;
     base.err = d_err;
-    SideView side{d->ws.perm.as<uint32_t>(), nullptr, nullptr};
-    NW_TRY(run_dict(d, base, side, d_counters, 0, 1, tm, ro));
+    const SideView side{d->ws.perm.as<uint32_t>(), nullptr, nullptr};
+    base.local[0] = make_terms(d, d->ws, d->ws, side, side, 0, 1);
+    NW_TRY(run_dict(d, kEpiMatrix, base, d_counters, 0, 1, tm, ro));
     if (!dev) {
       NW_CK(cudaMemcpyAsync(out + lo, dst, hi - lo, cudaMemcpyDeviceToHost, s));
       if (chunked) NW_CK(cudaStreamSynchronize(s));  // the chunk buffer is reused
@@ -467,16 +462,15 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   const int32_t key_lo = lo - 1;
   if ((uint64_t)(hi - key_lo) >= (1ull << (32 - ib)))
     return set_err(c, NW_ERANGE, "score range with %u dictionary words does not fit 32-bit list keys", n);
-  const bool bits = d->ss.bit_m > 0;
+  Rects rects;
+  rects_queries(q.bk, d->ws.bk, 0, rects);
   Plan plan;
-  plan_query(q.bk, d->ws.bk, kDefaultTA, plan, kQueryMinTasks);
-  BitPlan bplan;
-  if (bits) bit_plan_sized(bplan, [&](uint32_t ta, BitPlan& p) { bit_queries(q.bk, d->ws.bk, ta, 0, p); });
-  const std::vector<Seg>& segs = bits ? bplan.segs : plan.segs;
+  make_plan(std::move(rects), d->ss, d->alphabet, 0, plan);
+  const std::vector<Seg>& segs = plan.segs;
   NW_TRY(ctx_ensure(c, c->ws_segs, sizeof(Seg) * std::max<size_t>(1, segs.size()), "query segments"));
   NW_TRY(ctx_ensure(c, c->ws_slots, sizeof(uint32_t) * (size_t)nq * k, "list slots"));
   NW_TRY(ctx_ensure(c, c->ws_thr, sizeof(uint32_t) * (size_t)nq, "list thresholds"));
-  NW_TRY(ctx_ensure(c, c->ws_small, 64 + sizeof(unsigned long long) * (plan.launches.size() + 1), "task counters"));
+  NW_TRY(ctx_ensure(c, c->ws_small, kCounterBytes, "task counters"));
   uint32_t* out_idx = nbr_idx;
   int16_t* out_score = nbr_score;
   if (!dev) {
@@ -496,41 +490,21 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   NW_CK(cudaMemsetAsync(c->ws_small.p, 0, c->ws_small.bytes, s));
   NW_CK(cudaMemsetAsync(c->ws_slots.p, 0, sizeof(uint32_t) * (size_t)nq * k, s));
   NW_CK(cudaMemsetAsync(c->ws_thr.p, 0, sizeof(uint32_t) * (size_t)nq, s));
-  DpParams base{};
-  base.TA = kDefaultTA;
-  base.C1 = d->ss.C1;
-  base.C2 = d->ss.C2;
-  base.match = d->sc.match;
-  base.mismatch = d->sc.mismatch;
-  base.gap = d->sc.gap;
+  AlignParams base{};
   base.sim_tab = dict_tab(d);
-  base.mode = kModeLists;
   base.k = k;
-  base.ib = ib;
-  base.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
-  base.key_lo = key_lo;
   base.hist_mode = kHistNone;
   base.stats = d_stats;
   base.err = d_err;
   SideView qside{q.perm.as<uint32_t>(), c->ws_slots.as<uint32_t>(), c->ws_thr.as<uint32_t>()};
   SideView dside{d->ws.perm.as<uint32_t>(), nullptr, nullptr};
+  base.local[0] = make_terms(d, q, d->ws, qside, dside, key_lo, ib);
+  base.local[1] = make_terms(d, d->ws, q, dside, qside, key_lo, ib);
   RunOut ro;
-  if (bits) {
-    BitParams P = bit_params(base, d_counters);
-    P.local[0] = bit_terms(d, q, d->ws, qside, dside, key_lo, ib);
-    P.local[1] = bit_terms(d, d->ws, q, dside, qside, key_lo, ib);
-    NW_TRY(run_bits(c, s, d->ss.bit_m, d->ss.bit_x, kEpiLists, d->alphabet, bplan, c->ws_segs.as<Seg>(), P, tm, ro));
-  } else {
-    const uint32_t* a_enc[3] = {nullptr, q.a_enc.as<uint32_t>(), d->ws.a_enc.as<uint32_t>()};
-    const uint4* b_rec[3] = {nullptr, d->ws.b_rec.as<uint4>(), q.b_rec.as<uint4>()};
-    const SideView* A_views[3] = {nullptr, &qside, &dside};
-    const SideView* B_views[3] = {nullptr, &dside, &qside};
-    NW_TRY(run_plan(c, c->stream, plan, c->ws_segs.as<Seg>(), base, d_counters, 0, 1, tm, ro, a_enc, A_views,
-                    b_rec, B_views));
-  }
+  NW_TRY(run_plan(c, s, plan, c->ws_segs.as<Seg>(), kEpiLists, base, d_counters, tm, ro));
   cudaEvent_t e_fin = nullptr;
   tm.begin(false, e_fin);
-  NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), nq, k, q.perm.as<uint32_t>(), ib, base.imask, key_lo, out_idx,
+  NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), nq, k, q.perm.as<uint32_t>(), ib, base.local[0].imask, key_lo, out_idx,
                         out_score, s));
   tm.end(false, e_fin);
   if (!dev) {
@@ -633,6 +607,28 @@ nw_status nw_debug_norm_tables(const nw_scoring* sc, int32_t lo, int32_t hi, uin
   return NW_OK;
 }
 
+}  // extern "C"
+
+namespace {
+// f(segment, A position, B position) for every pair of a plan, in task order
+template <class F>
+void for_each_pair(const Plan& plan, F f) {
+  for (const Launch& l : plan.launches) {
+    const Seg* segs = plan.segs.data() + l.seg_first;
+    for (uint64_t t = 0; t < l.ntasks; ++t) {
+      const Seg& S = segs[find_seg(segs, l.nsegs, t)];
+      const TaskGeom g = l.range < 0 ? task_geom(S, t, l.ta, 32u * (uint32_t)bit_words_per_lane((int)S.lb))
+                                     : task_geom(S, t, l.ta);
+      for (uint32_t x = g.a0; x < g.a1; ++x)
+        for (uint32_t y = g.b0; y < g.bend; ++y)
+          if (pair_valid(g, x, y)) f(S, x, y);
+    }
+  }
+}
+}  // namespace
+
+extern "C" {
+
 nw_status nw_debug_enumerate_pairs(const uint32_t* lengths, uint32_t n, uint32_t shard, uint32_t nshards, uint32_t* a,
                                    uint32_t* b, uint64_t cap, uint64_t* count) {
   if (!lengths || !count || nshards == 0 || shard >= nshards) return NW_EINVAL;
@@ -645,30 +641,19 @@ nw_status nw_debug_enumerate_pairs(const uint32_t* lengths, uint32_t n, uint32_t
   fill_buckets(bk);
   std::vector<uint32_t> perm(n), fill(kBuckets, 0);
   for (uint32_t i = 0; i < n; ++i) perm[bk.start[lengths[i]] + fill[lengths[i]]++] = i;  // stable by length
+  Rects rects;
+  if (nshards == 1) rects_all(bk, 0, rects);
+  else rects_shard(bk, shard, nshards, rects);
   Plan plan;
-  plan_all_pairs(bk, kDefaultTA, plan);
+  make_plan(std::move(rects), ShiftedScoring{}, 0, 0, plan);
   uint64_t cnt = 0;
-  for (const LaunchPlan& lp : plan.launches) {
-    const uint64_t lo = lp.ntasks * shard / nshards, hi = lp.ntasks * (shard + 1) / nshards;
-    const Seg* segs = plan.segs.data() + lp.seg_first;
-    for (uint64_t t = lo; t < hi; ++t) {
-      const Seg& S = segs[find_seg(segs, lp.nsegs, t)];
-      const TaskGeom g = task_geom(S, t, kDefaultTA);
-      for (uint32_t x = g.a0; x < g.a1; ++x) {
-        for (uint32_t lane = 0; lane < 32; ++lane) {
-          for (uint32_t h = 0; h < 2; ++h) {
-            const uint32_t y = g.b0 + 2 * lane + h;
-            if (!pair_valid(g, x, y)) continue;
-            if (cnt < cap) {
-              a[cnt] = perm[x];
-              b[cnt] = perm[y];
-            }
-            ++cnt;
-          }
-        }
-      }
+  for_each_pair(plan, [&](const Seg&, uint32_t x, uint32_t y) {
+    if (cnt < cap) {
+      a[cnt] = perm[x];
+      b[cnt] = perm[y];
     }
-  }
+    ++cnt;
+  });
   *count = cnt;
   return NW_OK;
 }
@@ -694,28 +679,19 @@ nw_status nw_debug_enumerate_query_pairs(const uint32_t* q_lengths, uint32_t nq,
   Buckets qb, db;
   std::vector<uint32_t> qperm, dperm;
   if (!bucket(q_lengths, nq, qb, qperm) || !bucket(d_lengths, nd, db, dperm)) return NW_EINVAL;
-  const uint32_t TA = ta ? ta : kDefaultTA;
+  Rects rects;
+  rects_queries(qb, db, 0, rects);
   Plan plan;
-  plan_query(qb, db, TA, plan, kQueryMinTasks);
+  make_plan(std::move(rects), ShiftedScoring{}, 0, ta, plan);
   uint64_t cnt = 0;
-  for (const LaunchPlan& lp : plan.launches) {
-    const Seg* segs = plan.segs.data() + lp.seg_first;
-    for (uint64_t t = 0; t < lp.ntasks; ++t) {
-      const Seg& S = segs[find_seg(segs, lp.nsegs, t)];
-      const TaskGeom g = task_geom(S, t, lp.ta ? lp.ta : TA);
-      for (uint32_t x = g.a0; x < g.a1; ++x) {
-        for (uint32_t y = g.b0; y < g.bend; ++y) {
-          if (!pair_valid(g, x, y)) continue;
-          // role 1: queries are the A words; role 2: queries are the B words
-          if (cnt < cap) {
-            q[cnt] = lp.role == 1 ? qperm[x] : qperm[y];
-            d[cnt] = lp.role == 1 ? dperm[y] : dperm[x];
-          }
-          ++cnt;
-        }
-      }
+  for_each_pair(plan, [&](const Seg& S, uint32_t x, uint32_t y) {
+    // terms 0: queries are the A words; terms 1: they are the B words
+    if (cnt < cap) {
+      q[cnt] = S.dict == 0 ? qperm[x] : qperm[y];
+      d[cnt] = S.dict == 0 ? dperm[y] : dperm[x];
     }
-  }
+    ++cnt;
+  });
   *count = cnt;
   return NW_OK;
 }
@@ -740,36 +716,24 @@ nw_status nw_debug_enumerate_bit_pairs(const uint32_t* q_lengths, uint32_t nq, c
     std::vector<uint32_t> fill(kBuckets, 0);
     for (uint32_t i = 0; i < cnts[s]; ++i) perm[s][bk[s].start[len[s][i]] + fill[len[s][i]]++] = i;
   }
-  BitPlan plan;
-  auto make = [&](uint32_t t, BitPlan& p) {
-    if (nq) {
-      bit_queries(bk[1], bk[0], t, 0, p);
-    } else if (nshards == 1) {
-      bit_pairs(bk[0], t, 0, p);
-    } else {
-      Plan full;
-      plan_all_pairs(bk[0], kDefaultTA, full);
-      bit_shard(bk[0], full, shard, nshards, t, p);
-    }
-  };
-  if (ta) make(ta, plan); else bit_plan_sized(plan, make);
+  Rects rects;
+  if (nq) rects_queries(bk[1], bk[0], 0, rects);
+  else if (nshards == 1) rects_all(bk[0], 0, rects);
+  else rects_shard(bk[0], shard, nshards, rects);
+  ShiftedScoring ss{};
+  ss.bit_m = 3;
+  ss.bit_x = ss.bit_coef = 1;
+  Plan plan;
+  make_plan(std::move(rects), ss, 40, ta, plan);
   uint64_t cnt = 0;
-  for (uint64_t t = 0; t < plan.ntasks; ++t) {
-    const Seg& S = plan.segs[find_seg(plan.segs.data(), (uint32_t)plan.segs.size(), t)];
-    const TaskGeom g = task_geom(S, t, plan.ta, 32u * (uint32_t)bit_words_per_lane((int)S.lb));
+  for_each_pair(plan, [&](const Seg& S, uint32_t x, uint32_t y) {
     // terms 0: the queries (if any) are the A words; terms 1: they are the B words
-    const std::vector<uint32_t>& pa = perm[nq && S.dict == 0 ? 1 : 0];
-    const std::vector<uint32_t>& pb = perm[S.dict == 1 ? 1 : 0];
-    for (uint32_t x = g.a0; x < g.a1; ++x)
-      for (uint32_t y = g.b0; y < g.bend; ++y) {
-        if (!pair_valid(g, x, y)) continue;
-        if (cnt < cap) {
-          a[cnt] = S.dict == 1 ? pb[y] : pa[x];
-          b[cnt] = S.dict == 1 ? pa[x] : pb[y];
-        }
-        ++cnt;
-      }
-  }
+    if (cnt < cap) {
+      a[cnt] = nq == 0 ? perm[0][x] : (S.dict == 0 ? perm[1][x] : perm[1][y]);
+      b[cnt] = nq == 0 ? perm[0][y] : (S.dict == 0 ? perm[0][y] : perm[0][x]);
+    }
+    ++cnt;
+  });
   *count = cnt;
   return NW_OK;
 }
@@ -823,14 +787,12 @@ nw_status topk_into_scratch(nw_dict* d, ScratchProvider provide, uint32_t k, uin
                    d->score_hi, n);
 
   // scratch layout: [error flag, insert count, task counters | 2 KiB][thresholds][list slots][histogram]
-  const size_t nlaunch = d->plan.launches.size();
   auto up256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t off_thr = 2048;
   const size_t off_slots = off_thr + up256(sizeof(uint32_t) * (size_t)n);
   const size_t off_hist = off_slots + up256(sizeof(uint32_t) * (size_t)n * k);
   const size_t need = off_hist + (hist ? up256(sizeof(unsigned long long) * need_bins) : 0);
-  if (64 + sizeof(unsigned long long) * (nlaunch + 1) > off_thr)
-    return set_err(c, NW_ERANGE, "too many launches for the scratch header");
+  static_assert(kCounterBytes <= 2048, "the counters fit the scratch header");
   void* base = nullptr;
   size_t cap = 0;
   const char* why = "";
@@ -869,18 +831,8 @@ nw_status topk_into_scratch(nw_dict* d, ScratchProvider provide, uint32_t k, uin
   NW_CK(cudaMemsetAsync(d_slots, 0, sizeof(uint32_t) * (size_t)n * k, s));
   if (hist) NW_CK(cudaMemsetAsync(d_hist, 0, sizeof(unsigned long long) * need_bins, s));
 
-  DpParams P{};
-  P.TA = kDefaultTA;
-  P.C1 = d->ss.C1;
-  P.C2 = d->ss.C2;
-  P.match = d->sc.match;
-  P.mismatch = d->sc.mismatch;
-  P.gap = d->sc.gap;
-  P.mode = kModeLists;
+  AlignParams P{};
   P.k = k;
-  P.ib = ib;
-  P.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
-  P.key_lo = key_lo;
   P.hist_mode = !hist ? kHistNone : hist_mode_for(need_bins);
   P.hist = d_hist;
   P.hist_lo = d->score_lo;
@@ -888,10 +840,11 @@ nw_status topk_into_scratch(nw_dict* d, ScratchProvider provide, uint32_t k, uin
   P.stats = d_stats;
   P.err = async ? d_err_async : d_err;
   SideView side{d->ws.perm.as<uint32_t>(), d_slots, d_thr};
+  P.local[0] = make_terms(d, d->ws, d->ws, side, side, key_lo, ib);
   Timer tm{c};
   RunOut ro;
-  NW_TRY(run_dict(d, P, side, d_counters, 0, 1, tm, ro));
-  NW_CK(launch_finalize(d_slots, n, k, d->ws.perm.as<uint32_t>(), ib, P.imask, key_lo, nbr_idx, nbr_score, s));
+  NW_TRY(run_dict(d, lists_epi(P.hist_mode), P, d_counters, 0, 1, tm, ro));
+  NW_CK(launch_finalize(d_slots, n, k, d->ws.perm.as<uint32_t>(), ib, P.local[0].imask, key_lo, nbr_idx, nbr_score, s));
   if (hist) {
     NW_CK(cudaMemcpyAsync(hist, d_hist, sizeof(int64_t) * need_bins, cudaMemcpyDeviceToDevice, s));
     if (nbins > need_bins) NW_CK(cudaMemsetAsync(hist + need_bins, 0, sizeof(int64_t) * (nbins - need_bins), s));

@@ -3,15 +3,16 @@
 //
 // Every dictionary is loaded as usual (its own word set, scoring and score
 // bounds), and its query set is ingested with the dictionary's alphabet and
-// code shift.  The pair plans of all dictionaries and query sets are merged
-// by longer length: the launch for length LB walks the LB segments of every
-// dictionary and query set, each segment tagged with its terms (3d for
-// dictionary d's own pairs, 3d + 1 for its queries as A words, 3d + 2 for its
-// queries as B words), and the kernel (epilogue kEpiBatchLists) reads those
-// terms' word sets, lists and scoring per task.  The A-chunk size of each
-// launch is a tile-shape parameter that the autotuner picks by timing
-// candidates on the batch.  The whole reduction is captured once into a CUDA
-// graph and replayed by nw_batch_run / nw_batch_run_queries.
+// code shift.  The pair lists of all dictionaries and query sets are planned
+// together, each rectangle tagged with its terms (3d for dictionary d's own
+// pairs, 3d + 1 for its queries as A words, 3d + 2 for its queries as B words);
+// the kernels (epilogue kEpiBatchLists) read those terms' word sets, lists and
+// scoring per task.  Dictionaries whose scoring the bit-parallel kernel takes
+// share one launch per step class, on a second stream; the others share one
+// DPX launch per range of longer lengths, whose A-chunk size is a tile-shape
+// parameter that the autotuner picks by timing candidates on the batch.  The
+// whole reduction is captured once into a CUDA graph and replayed by
+// nw_batch_run / nw_batch_run_queries.
 #include <chrono>
 #include <map>
 #include <mutex>
@@ -21,12 +22,17 @@
 struct nw_batch {
   nw_ctx* ctx = nullptr;
   cudaStream_t stream = nullptr;  // the batch's own stream (capture needs a non-legacy stream)
+  cudaStream_t side = nullptr;    // the bit-parallel launches run here, forked from and joined to `stream`
+  cudaEvent_t forked = nullptr, joined = nullptr;
   std::vector<nw_dict*> dicts;
   std::vector<WordSet> qsets;     // each dictionary's query set (n = 0: none)
   std::vector<uint8_t> self;      // 1: the dictionary's own lists are computed
   uint32_t k = 0;
-  uint32_t ta_by_lb[kBuckets] = {0};
-  uint32_t bps_by_lb[kBuckets] = {0};  // resident blocks per SM at most (0: as many as fit)
+  Rects dp_rects;                      // the DPX launches' pairs, ordered
+  uint32_t ta[kDpRanges] = {0};        // their A words per task, by range of longer lengths
+  uint32_t bps[kDpRanges] = {0};       // resident blocks per SM at most (0: as many as fit)
+  bool has_len[kBuckets] = {false};    // longer lengths with pairs, and of which in DPX launches
+  bool dp_len[kBuckets] = {false};
   bool tune_cached = false;
   Plan plan;
   std::vector<size_t> list_off;   // first list of each dictionary's own lists in the combined arrays
@@ -49,68 +55,13 @@ constexpr uint32_t kTaCandidates[] = {64, 128, 256};
 // (role 1) or B words (role 2).
 uint32_t term_index(size_t d, int role) { return (uint32_t)(3 * d + role); }
 
-// Every dictionary's own plan and every query set's plan (launches of roles 1
-// and 2), made with A chunks of `ta` words.
-struct DictPlans {
-  std::vector<Plan> self, query;
-};
-
-DictPlans dict_plans(const nw_batch* B, uint32_t ta) {
-  DictPlans p;
-  p.self.resize(B->dicts.size());
-  p.query.resize(B->dicts.size());
-  for (size_t d = 0; d < B->dicts.size(); ++d) {
-    if (B->self[d]) plan_all_pairs(B->dicts[d]->ws.bk, ta, p.self[d]);
-    if (B->qsets[d].n) plan_query(B->qsets[d].bk, B->dicts[d]->ws.bk, ta, p.query[d]);
-  }
-  return p;
-}
-
-// The segments of every dictionary and query set whose longer length is LB,
-// taken from plans made with A chunks of `ta` words, appended as one launch
-// (task0 rebased, terms tagged).
-void append_launch(const nw_batch* B, const DictPlans& plans, int LB, uint32_t ta, Plan& out, uint32_t bps = 0) {
-  LaunchPlan lp;
-  lp.LB = LB;
-  lp.role = 0;
-  lp.ta = ta;
-  lp.bps = bps;
-  lp.seg_first = (uint32_t)out.segs.size();
-  uint64_t task = 0;
-  for (size_t d = 0; d < B->dicts.size(); ++d) {
-    for (const Plan* p : {&plans.self[d], &plans.query[d]}) {
-      for (const LaunchPlan& q : p->launches) {
-        if (q.LB != LB) continue;
-        for (uint32_t s = 0; s < q.nsegs; ++s) {
-          Seg g = p->segs[q.seg_first + s];
-          g.task0 += task;
-          g.dict = term_index(d, q.role);
-          out.segs.push_back(g);
-        }
-        task += q.ntasks;
-        lp.pairs += q.pairs;
-        lp.cells += q.cells;
-      }
-    }
-  }
-  lp.nsegs = (uint32_t)out.segs.size() - lp.seg_first;
-  lp.ntasks = task;
-  if (lp.nsegs) {
-    out.pairs += lp.pairs;
-    out.cells += lp.cells;
-    out.launches.push_back(lp);
-  }
-}
-
-DpParams batch_params(nw_batch* B) {
-  DpParams P{};
-  P.TA = kDefaultTA;
-  P.mode = kModeLists;
+AlignParams batch_params(nw_batch* B) {
+  AlignParams P{};
   P.k = B->k;
   P.hist_mode = kHistNone;
   P.stats = reinterpret_cast<unsigned long long*>(B->d_small.as<char>() + 8);
   P.err = B->d_small.as<uint32_t>();
-  P.terms = B->d_terms.as<DictTerms>();
+  P.terms = B->d_terms.as<Terms>();
   return P;
 }
 
@@ -123,28 +74,34 @@ nw_status upload_plan(nw_batch* B, const Plan& plan) {
   return NW_OK;
 }
 
-// List resets and the alignment launches of `plan` (shard `shard` of
-// `nshards` of each launch's tasks) on the batch's stream.
-nw_status issue_lists(nw_batch* B, const Plan& plan, uint32_t shard = 0, uint32_t nshards = 1) {
+// List resets and the alignment launches of `plan`: the DPX launches on the
+// batch's stream, the bit-parallel ones beside them on its side stream.
+nw_status issue_lists(nw_batch* B, const Plan& plan) {
   nw_ctx* c = B->ctx;
   cudaStream_t s = B->stream;
   NW_CK(cudaMemsetAsync(B->d_small.p, 0, B->d_small.bytes, s));
   NW_CK(cudaMemsetAsync(B->d_slots.p, 0, sizeof(uint32_t) * B->nlists * B->k, s));
   NW_CK(cudaMemsetAsync(B->d_thr.p, 0, sizeof(uint32_t) * B->nlists, s));
-  const DpParams P = batch_params(B);
-  SideView none{nullptr, nullptr, nullptr};
-  const uint32_t* a_enc[3] = {nullptr, nullptr, nullptr};
-  const uint4* b_rec[3] = {nullptr, nullptr, nullptr};
-  const SideView* views[3] = {&none, &none, &none};
   const bool saved = c->profiling;
   c->profiling = false;
+  struct Restore {
+    nw_ctx* c;
+    bool v;
+    ~Restore() { c->profiling = v; }
+  } restore{c, saved};
   Timer tm{c};
   RunOut ro;
-  const nw_status st = run_plan(c, s, plan, B->d_segs.as<Seg>(), P,
-                                reinterpret_cast<unsigned long long*>(B->d_small.as<char>() + 64), shard, nshards,
-                                tm, ro,
-                                a_enc, views, b_rec, views);
-  c->profiling = saved;
+  NW_CK(cudaEventRecord(B->forked, s));
+  NW_CK(cudaStreamWaitEvent(B->side, B->forked, 0));
+  nw_status st = NW_OK;
+  for (size_t i = 0; i < plan.launches.size() && st == NW_OK; ++i) {
+    AlignParams P = batch_params(B);
+    P.counter = reinterpret_cast<unsigned long long*>(B->d_small.as<char>() + 64) + i;
+    st = run_launch(c, plan.launches[i].range < 0 ? B->side : s, plan.launches[i], B->d_segs.as<Seg>(), kEpiBatchLists,
+                    P, tm, ro);
+  }
+  NW_CK(cudaEventRecord(B->joined, B->side));
+  NW_CK(cudaStreamWaitEvent(s, B->joined, 0));
   return st;
 }
 
@@ -173,8 +130,8 @@ nw_status issue_finalize(nw_batch* B) {
 // The autotuner's choices, kept for the life of the process and keyed by the
 // batch's shape (tune_key): a batch of the same shape is not timed again.
 struct TunedShape {
-  uint32_t ta[kBuckets];
-  uint32_t bps[kBuckets];
+  uint32_t ta[kDpRanges];
+  uint32_t bps[kDpRanges];
 };
 std::mutex& tune_mutex() {
   static std::mutex m;
@@ -215,7 +172,7 @@ uint64_t tune_key(const nw_batch* B) {
 
 constexpr uint32_t kBpsCandidates[] = {3, 2};
 
-// Per launch length: the fastest A-chunk candidate, then the fastest cap on
+// Per DPX launch: the fastest A-chunk candidate, then the fastest cap on
 // resident blocks per SM at that chunk (whole launches timed on the batch).
 nw_status autotune(nw_batch* B) {
   nw_ctx* c = B->ctx;
@@ -224,8 +181,8 @@ nw_status autotune(nw_batch* B) {
     std::lock_guard<std::mutex> lk(tune_mutex());
     auto it = tune_cache().find(key);
     if (it != tune_cache().end()) {
-      std::copy(it->second.ta, it->second.ta + kBuckets, B->ta_by_lb);
-      std::copy(it->second.bps, it->second.bps + kBuckets, B->bps_by_lb);
+      std::copy(it->second.ta, it->second.ta + kDpRanges, B->ta);
+      std::copy(it->second.bps, it->second.bps + kDpRanges, B->bps);
       B->tune_cached = true;
       B->tune_ms = 0;
       return NW_OK;
@@ -240,12 +197,10 @@ nw_status autotune(nw_batch* B) {
     ~EvFree() { cudaEventDestroy(a); cudaEventDestroy(b); }
   } evfree{e0, e1};
   constexpr size_t kNta = sizeof(kTaCandidates) / sizeof(kTaCandidates[0]);
-  std::vector<DictPlans> plans;
-  for (uint32_t ta : kTaCandidates) plans.push_back(dict_plans(B, ta));
-  // one timed launch of length LB with chunk candidate ci and cap bps; false if the length has no pairs
-  auto time_launch = [&](int LB, size_t ci, uint32_t bps, bool& warm, float& ms) -> nw_status {
+  // one timed launch of range r with chunk candidate ci and cap bps; ms < 0 if the range has no pairs
+  auto time_launch = [&](int r, size_t ci, uint32_t bps, bool& warm, float& ms) -> nw_status {
     Plan p;
-    append_launch(B, plans[ci], LB, kTaCandidates[ci], p, bps);
+    plan_dp(B->dp_rects, kTaCandidates[ci], p, r, bps);
     ms = -1.f;
     if (p.launches.empty()) return NW_OK;
     NW_TRY(upload_plan(B, p));
@@ -260,34 +215,34 @@ nw_status autotune(nw_batch* B) {
     NW_CK(cudaEventElapsedTime(&ms, e0, e1));
     return NW_OK;
   };
-  for (int LB = 0; LB < kBuckets; ++LB) {
+  for (int r = 0; r < kDpRanges; ++r) {
     float best = 0;
     size_t best_ci = kNta;
     bool warm = false;
     for (size_t ci = 0; ci < kNta; ++ci) {
       float ms;
-      NW_TRY(time_launch(LB, ci, 0, warm, ms));
+      NW_TRY(time_launch(r, ci, 0, warm, ms));
       if (ms < 0) break;
       if (best_ci == kNta || ms < best) {
         best = ms;
         best_ci = ci;
       }
     }
-    if (best_ci == kNta) continue;  // lengths without pairs keep the defaults
-    B->ta_by_lb[LB] = kTaCandidates[best_ci];
+    if (best_ci == kNta) continue;  // ranges without pairs keep the defaults
+    B->ta[r] = kTaCandidates[best_ci];
     for (uint32_t bps : kBpsCandidates) {
       float ms;
-      NW_TRY(time_launch(LB, best_ci, bps, warm, ms));
+      NW_TRY(time_launch(r, best_ci, bps, warm, ms));
       if (ms >= 0 && ms < best) {
         best = ms;
-        B->bps_by_lb[LB] = bps;
+        B->bps[r] = bps;
       }
     }
   }
   B->tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   TunedShape t;
-  std::copy(B->ta_by_lb, B->ta_by_lb + kBuckets, t.ta);
-  std::copy(B->bps_by_lb, B->bps_by_lb + kBuckets, t.bps);
+  std::copy(B->ta, B->ta + kDpRanges, t.ta);
+  std::copy(B->bps, B->bps + kDpRanges, t.bps);
   std::lock_guard<std::mutex> lk(tune_mutex());
   tune_cache()[key] = t;
   return NW_OK;
@@ -352,8 +307,15 @@ nw_status create_impl(nw_batch* B, const nw_batch_dict* dicts, uint32_t ndicts, 
   NW_TRY(ctx_alloc(c, B->d_thr, sizeof(uint32_t) * L, "batch list bounds"));
   NW_TRY(ctx_alloc(c, B->d_out_idx, sizeof(uint32_t) * L * B->k, "batch output indices"));
   NW_TRY(ctx_alloc(c, B->d_out_score, sizeof(int16_t) * L * B->k, "batch output scores"));
-  NW_TRY(ctx_alloc(c, B->d_small, 64 + sizeof(unsigned long long) * (kBuckets + 2), "batch counters"));
-  std::vector<DictTerms> terms(std::max<size_t>(1, 3 * B->dicts.size()));
+  NW_TRY(ctx_alloc(c, B->d_small, kCounterBytes, "batch counters"));
+  std::vector<Terms> terms(std::max<size_t>(1, 3 * B->dicts.size()));
+  // the pairs: DPX dictionaries together, the others by step class
+  struct Group {
+    int m, x;
+    uint32_t alphabet;
+    Rects rects;
+  };
+  std::vector<Group> groups;
   for (size_t d = 0; d < B->dicts.size(); ++d) {
     const nw_dict* D = B->dicts[d];
     const WordSet& Q = B->qsets[d];
@@ -363,50 +325,47 @@ nw_status create_impl(nw_batch* B, const nw_batch_dict* dicts, uint32_t ndicts, 
     const SideView dict_nolists{D->ws.perm.as<uint32_t>(), nullptr, nullptr};
     const SideView query_side{Q.perm.as<uint32_t>(), B->d_slots.as<uint32_t>() + B->qlist_off[d] * B->k,
                               B->d_thr.as<uint32_t>() + B->qlist_off[d]};
-    for (int role = 0; role < 3; ++role) {
-      DictTerms& T = terms[term_index(d, role)];
-      T.a_enc = role == 1 ? Q.a_enc.as<uint32_t>() : D->ws.a_enc.as<uint32_t>();
-      T.b_rec = role == 2 ? Q.b_rec.as<uint4>() : D->ws.b_rec.as<uint4>();
-      T.A = role == 0 ? dict_side : (role == 1 ? query_side : dict_nolists);
-      T.B = role == 0 ? dict_side : (role == 1 ? dict_nolists : query_side);
-      T.C1 = D->ss.C1;
-      T.C2 = D->ss.C2;
-      T.match = D->sc.match;
-      T.mismatch = D->sc.mismatch;
-      T.gap = D->sc.gap;
-      T.key_lo = role == 0 ? D->score_lo - 1 : B->q_key_lo[d];
-      T.ib = ib;
-      T.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
+    terms[term_index(d, 0)] = make_terms(D, D->ws, D->ws, dict_side, dict_side, D->score_lo - 1, ib);
+    terms[term_index(d, 1)] = make_terms(D, Q, D->ws, query_side, dict_nolists, B->q_key_lo[d], ib);
+    terms[term_index(d, 2)] = make_terms(D, D->ws, Q, dict_nolists, query_side, B->q_key_lo[d], ib);
+    Rects* rects = &B->dp_rects;
+    if (D->ss.bit_m) {
+      auto g = std::find_if(groups.begin(), groups.end(),
+                            [&](const Group& x) { return x.m == D->ss.bit_m && x.x == D->ss.bit_x; });
+      if (g == groups.end()) g = groups.insert(g, Group{D->ss.bit_m, D->ss.bit_x, 0, {}});
+      g->alphabet = std::max(g->alphabet, D->alphabet);
+      rects = &g->rects;
     }
-    if (Q.n) {
-      Plan qp;
-      plan_query(Q.bk, D->ws.bk, kDefaultTA, qp);
-      B->query_pairs += qp.pairs;
-      B->query_cells += qp.cells;
-    }
+    Rects own, queries;
+    if (B->self[d]) rects_all(D->ws.bk, term_index(d, 0), own);
+    if (Q.n) rects_queries(Q.bk, D->ws.bk, term_index(d, 1), queries);
+    count_rects(queries, B->query_pairs, B->query_cells);
+    for (const Rects* list : {&own, &queries})
+      for (const Rect& r : *list) {
+        rects->push_back(r);
+        B->has_len[r.LB] = true;
+        if (!D->ss.bit_m) B->dp_len[r.LB] = true;
+      }
   }
-  NW_TRY(ctx_alloc(c, B->d_terms, sizeof(DictTerms) * terms.size(), "batch terms"));
-  NW_CK(cudaMemcpyAsync(B->d_terms.p, terms.data(), sizeof(DictTerms) * terms.size(), cudaMemcpyHostToDevice,
-                        B->stream));
+  NW_TRY(ctx_alloc(c, B->d_terms, sizeof(Terms) * terms.size(), "batch terms"));
+  NW_CK(cudaMemcpyAsync(B->d_terms.p, terms.data(), sizeof(Terms) * terms.size(), cudaMemcpyHostToDevice, B->stream));
 
-  for (int LB = 0; LB < kBuckets; ++LB) B->ta_by_lb[LB] = kDefaultTA;
+  order_rects(B->dp_rects);
+  for (uint32_t& t : B->ta) t = kDefaultTA;
   if (flags & NW_BATCH_AUTOTUNE) NW_TRY(autotune(B));
   B->plan = Plan{};
-  {
-    std::vector<uint32_t> tas;  // the distinct chunk sizes chosen, each planned once
-    for (int LB = 0; LB < kBuckets; ++LB)
-      if (std::find(tas.begin(), tas.end(), B->ta_by_lb[LB]) == tas.end()) tas.push_back(B->ta_by_lb[LB]);
-    std::vector<DictPlans> plans;
-    for (uint32_t ta : tas) plans.push_back(dict_plans(B, ta));
-    for (int LB = 0; LB < kBuckets; ++LB) {
-      const size_t ci = std::find(tas.begin(), tas.end(), B->ta_by_lb[LB]) - tas.begin();
-      append_launch(B, plans[ci], LB, B->ta_by_lb[LB], B->plan, B->bps_by_lb[LB]);
+  for (int r = 0; r < kDpRanges; ++r) plan_dp(B->dp_rects, B->ta[r], B->plan, r, B->bps[r]);
+  count_rects(B->dp_rects, B->plan.pairs, B->plan.cells);
+  for (Group& g : groups) {
+    order_rects(g.rects);
+    Plan p;
+    sized(p, kBitMinTasks, [&](uint32_t ta, Plan& q) { plan_bits(g.rects, g.m, g.x, g.alphabet, ta, q); });
+    for (Launch& l : p.launches) {
+      l.seg_first += (uint32_t)B->plan.segs.size();
+      B->plan.launches.push_back(l);
     }
-  }
-  for (int LB = 0; LB < kBuckets; ++LB) {
-    bool present = false;
-    for (const LaunchPlan& lp : B->plan.launches) present |= lp.LB == LB;
-    if (!present) B->ta_by_lb[LB] = B->bps_by_lb[LB] = 0;
+    B->plan.segs.insert(B->plan.segs.end(), p.segs.begin(), p.segs.end());
+    count_rects(g.rects, B->plan.pairs, B->plan.cells);
   }
   NW_TRY(upload_plan(B, B->plan));
   // one uncaptured run sets the kernels' shared-memory attributes
@@ -438,6 +397,12 @@ void destroy_impl(nw_batch* B) {
     ctx_free(c, *b);
   for (WordSet& Q : B->qsets) free_wordset(c, Q);
   for (nw_dict* D : B->dicts) nw_dict_free(D);
+  if (B->side) {
+    cudaStreamSynchronize(B->side);
+    cudaStreamDestroy(B->side);
+  }
+  if (B->forked) cudaEventDestroy(B->forked);
+  if (B->joined) cudaEventDestroy(B->joined);
   if (B->stream) cudaStreamDestroy(B->stream);
   delete B;
 }
@@ -458,7 +423,10 @@ nw_status nw_batch_create(nw_ctx* ctx, const nw_batch_dict* dicts, uint32_t ndic
   B->ctx = ctx;
   B->k = k;
   nw_status st = NW_OK;
-  if (cudaStreamCreateWithFlags(&B->stream, cudaStreamNonBlocking) != cudaSuccess)
+  if (cudaStreamCreateWithFlags(&B->stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&B->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&B->forked, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&B->joined, cudaEventDisableTiming) != cudaSuccess)
     st = cuda_fail(ctx, cudaGetLastError(), "cudaStreamCreateWithFlags");
   if (st == NW_OK) st = create_impl(B, dicts, ndicts, flags);
   if (st != NW_OK) {
@@ -517,8 +485,11 @@ nw_status nw_batch_info_get(const nw_batch* B, nw_batch_info* out) {
   i.pairs = B->plan.pairs;
   i.cells = B->plan.cells;
   i.tune_ms = B->tune_ms;
-  for (int L = 0; L < kBuckets; ++L) i.words_per_task[L] = B->ta_by_lb[L];
-  for (int L = 0; L < kBuckets; ++L) i.blocks_per_sm[L] = B->bps_by_lb[L];
+  // lengths met in bit-parallel launches alone: the size their chunks start from
+  for (int L = 0; L < kBuckets; ++L) {
+    i.words_per_task[L] = B->dp_len[L] ? B->ta[dp_range_of(L)] : (B->has_len[L] ? kDefaultTA : 0);
+    i.blocks_per_sm[L] = B->dp_len[L] ? B->bps[dp_range_of(L)] : 0;
+  }
   i.tune_cached = B->tune_cached ? 1u : 0u;
   i.query_words = B->query_words;
   i.query_pairs = B->query_pairs;

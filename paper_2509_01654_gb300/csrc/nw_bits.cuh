@@ -232,67 +232,9 @@ __device__ __forceinline__ void bit_scores(const B64 (&D)[bit_digits(MM)], B64 F
   }
 }
 
-// what a task's warps share
-struct BitTask {
-  TaskGeom g;
-  int K;                  // words per lane
-  int la, lb, mx;         // mx: the longer of the two
-  uint32_t a_base;        // index of A word g.a0's first symbol in T.a_sym
-  uint32_t b_base;        // index of B word g.b0's first symbol in T.b_sym
-  bool check;             // same bucket, chunks overlap: test a < b
-};
-
-// Candidate queue.  A pair that may enter a list is rare late in a launch and
-// common early, and filing it takes several dependent trips to L2.  The lanes
-// only append such pairs to their warp's queue; once 32 are waiting, each lane
-// files one, so the trips overlap 32-fold.  (Filing each pair in the lane that
-// found it took 126 of 584 ms at 600k words, half of the time at 100k.)
-// An entry: G << 16 | A word (from g.a0) << 8 | B word (from g.b0); G < 2^15,
-// a task has at most 256 words on either side.
-constexpr uint32_t kBitQueue = 64;  // entries: up to 31 waiting plus a warp's 32
-
-// Files n <= 32 queued pairs in their words' lists; returns the lane's inserts.
-__device__ __forceinline__ uint32_t bit_drain(const BitParams& P, const BitTerms& T, const BitTask& Q,
-                                           const uint32_t* queue, uint32_t n) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const int max_iters = P.dbg_insert_limit ? (int)(P.dbg_insert_limit - 1u) : kInsertMaxIters;
-  const bool have = lane < n;
-  const uint32_t e = have ? queue[lane] : 0u;
-  const uint32_t a = Q.g.a0 + ((e >> 8) & 0xffu), b = Q.g.b0 + (e & 0xffu);
-  const int s = (int)(e >> 16) + T.gap * (Q.la + Q.lb);
-  const uint32_t oa = have ? __ldg(T.A.perm + a) : 0u, ob = have ? __ldg(T.B.perm + b) : 0u;
-  uint32_t inserts = 0u;
-  if (T.B.slots && have) {  // word b takes the A word as a neighbour
-    const uint32_t key = list_key(P, T, s, Q.mx, oa);
-    if (key > __ldcg(T.B.thr + b))
-      list_offer(T.B.slots + (size_t)b * P.k, T.B.thr + b, P.k, key, P.err, inserts, max_iters);
-  }
-  if (T.A.slots) {
-    // the A word takes word b.  Several lanes may hold the same A word: one
-    // lane of each such group offers at a time and the others are tested again
-    // against the bound it leaves, so the lanes never race on one list
-    uint32_t key = 0u;
-    if (have) {
-      key = list_key(P, T, s, Q.mx, ob);
-      if (key <= __ldcg(T.A.thr + a)) key = 0u;
-    }
-    const uint32_t group = __match_any_sync(0xffffffffu, a);
-    uint32_t todo;
-    while ((todo = __ballot_sync(0xffffffffu, key != 0u)) != 0u) {
-      if ((uint32_t)(__ffs(todo & group) - 1) == lane) {
-        list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, key, P.err, inserts, max_iters);
-        key = 0u;
-      }
-      __syncwarp();
-      if (key != 0u && key <= __ldcg(T.A.thr + a)) key = 0u;
-    }
-  }
-  return inserts;
-}
-
 // The A words of one task against the lane's K words (b = b0 + 32 w + lane).
 template <int MM, int XX, int EPI, int K>
-__device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, const BitTask& Q,
+__device__ __forceinline__ void bit_task(const AlignParams& P, const Terms& T, const AlignTask& Q,
                                          const unsigned char* masks, uint32_t* wh, uint16_t* sA, uint32_t* queue,
                                          uint32_t& inserts) {
   constexpr int PITCH = bit_pitch(K);
@@ -424,7 +366,7 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
 #pragma unroll
           for (int w = 0; w < K; ++w)
             if (((vmask >> w) & 1u) && (!check || a < g.b0 + 32u * w + lane))
-              hist_add(P, wh, lane, gv[w] + pconst - P.hist_lo);
+              hist_add(P, wh, gv[w] + pconst - P.hist_lo);
         }
         // prefilter: non-zero when some word's G reaches its own list's bound,
         // or the largest G reaches the A word's
@@ -452,29 +394,15 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
           }
           cand &= vmask;
           bool filed = false;
-          uint32_t m;
-          while ((m = __ballot_sync(0xffffffffu, cand != 0u)) != 0u) {
-            if (cand) {
-              const int w = __ffs(cand) - 1;
-              uint32_t G = res[0];
+          while (__any_sync(0xffffffffu, cand != 0u)) {
+            const int w = __ffs(cand) - 1;  // (-1: nothing left, the entry is not used)
+            uint32_t G = res[0];
 #pragma unroll
-              for (int i = 1; i < KP; ++i) G = (w >> 1) == i ? res[i] : G;
-              G = (w & 1) ? G >> 16 : G & 0xffffu;
-              queue[waiting + __popc(m & ((1u << lane) - 1u))] =
-                  (G << 16) | ((a - g.a0) << 8) | (32u * (uint32_t)w + (uint32_t)lane);
-              cand &= cand - 1u;
-            }
-            waiting += __popc(m);
-            if (waiting >= 32u) {
-              __syncwarp();
-              inserts += bit_drain(P, T, Q, queue, 32u);
-              waiting -= 32u;
-              const uint32_t v = (uint32_t)lane < waiting ? queue[32 + lane] : 0u;
-              __syncwarp();
-              queue[lane] = v;
-              __syncwarp();
-              filed = true;
-            }
+            for (int i = 1; i < KP; ++i) G = (w >> 1) == i ? res[i] : G;
+            G = (w & 1) ? G >> 16 : G & 0xffffu;
+            filed |= queue_candidate(P, T, Q, queue, waiting, inserts, cand != 0u,
+                                     (G << 16) | ((a - g.a0) << 8) | (32u * (uint32_t)w + (uint32_t)lane));
+            cand &= cand - 1u;
           }
           if (filed) {
             load_bounds_B();
@@ -487,7 +415,7 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
   if constexpr (kLists) {
     if (waiting) {
       __syncwarp();
-      inserts += bit_drain(P, T, Q, queue, waiting);
+      inserts += file_candidates(P, T, Q, queue, waiting);
     }
   }
 }
@@ -498,15 +426,15 @@ __device__ __forceinline__ void bit_task(const BitParams& P, const BitTerms& T, 
 constexpr int kBitMinBlocks = 5;
 
 template <int MM, int XX, int EPI>
-__global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const __grid_constant__ BitParams P) {
+__global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const __grid_constant__ AlignParams P) {
   extern __shared__ __align__(16) unsigned char s_bits[];
   __shared__ unsigned long long s_task[2];
   __shared__ uint32_t s_seg[2];
-  __shared__ uint32_t s_queue[kBitWarps][kBitQueue];
+  __shared__ uint32_t s_queue[kBitWarps][kQueueEntries];
   // the task's terms and geometry live in shared memory: most of them are
   // read on the rare paths only, and registers are what bounds the block count
-  __shared__ BitTerms T;
-  __shared__ BitTask Q;
+  __shared__ Terms T;
+  __shared__ AlignTask Q;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // dynamic shared memory: match masks, histogram (lane columns shared by the
   // block, or one array per warp), staged A symbols
@@ -525,11 +453,6 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
     s_task[buf] = t;
     s_seg[buf] = t < P.ntasks ? find_seg(P.segs, P.nsegs, t) : 0u;
   };
-  auto flush = [&]() {  // block-uniform
-    __syncthreads();
-    if (warp_hist || (kHist && warp == 0)) hist_flush(P, wh, lane);
-    __syncthreads();
-  };
   if (tid == 0) fetch(0);
   for (int buf = 0;; buf ^= 1) {
     __syncthreads();  // the task is known, and the masks are no longer in use
@@ -539,7 +462,7 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
     {
       const uint32_t d = S->dict;
       const uint32_t* src = reinterpret_cast<const uint32_t*>(EPI == kEpiBatchLists ? P.terms + d : P.local + d);
-      if (tid < (int)(sizeof(BitTerms) / 4)) reinterpret_cast<uint32_t*>(&T)[tid] = src[tid];
+      if (tid < (int)(sizeof(Terms) / 4)) reinterpret_cast<uint32_t*>(&T)[tid] = src[tid];
     }
     if (tid == kBitBlock - 1) {
       const int K = bit_words_per_lane((int)S->lb);
@@ -549,7 +472,7 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
       Q.lb = (int)S->lb;
       Q.mx = Q.la > Q.lb ? Q.la : Q.lb;
       Q.a_base = S->aenc_base + (Q.g.a0 - S->a_beg) * (uint32_t)Q.la;
-      Q.b_base = S->brec_base + (Q.g.b0 - S->b_beg) * (uint32_t)Q.lb;
+      Q.b_base = S->b_base + (Q.g.b0 - S->b_beg) * (uint32_t)Q.lb;
       Q.check = Q.g.tri && Q.g.a1 > Q.g.b0;
     }
     if (tid == 0) fetch(buf ^ 1);  // read after the barrier at the next task's start
@@ -577,14 +500,9 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
         }
       }
     }
-    if ((EPI == kEpiLists || kHist) && P.hist_mode != kHistNone) {
-      // every bin this task can produce lies inside the histogram (proven bounds)
-      int lo, hi;
-      pair_score_bounds(T.match, T.mismatch, T.gap, Q.la < Q.lb ? Q.la : Q.lb, Q.mx, lo, hi);
-      if (lo < P.hist_lo || hi - P.hist_lo >= (int)P.nbins) {
-        if (tid == 0) atomicOr(P.err, kErrHistRange);
-        continue;  // block-uniform
-      }
+    if ((EPI == kEpiLists || kHist) && P.hist_mode != kHistNone && !hist_covers(P, T, Q)) {
+      if (tid == 0) atomicOr(P.err, kErrHistRange);
+      continue;  // block-uniform
     }
     __syncthreads();
     switch (K) {
@@ -597,15 +515,18 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
       case 2: bit_task<MM, XX, EPI, 2>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
       default: bit_task<MM, XX, EPI, 1>(P, T, Q, masks, wh, sA, s_queue[warp], inserts); break;
     }
-    if (hist_words) {  // 32-bit shared counters: flush long before they could wrap
-      hpairs += (uint64_t)(Q.g.a1 - Q.g.a0) * (32u * (uint32_t)K);
-      if (hpairs >= (1ull << 30)) {
-        flush();
+    if (hist_words) {
+      hpairs += (uint64_t)(Q.g.a1 - Q.g.a0) * (32u * (uint32_t)K);  // (more than the warp's share)
+      if (hpairs >= kHistFlushPairs) {
+        hist_flush(P, wh, lane);
         hpairs = 0;
       }
     }
   }
-  if (hist_words) flush();
+  if (hist_words) {
+    __syncthreads();
+    if (warp_hist || warp == 0) hist_flush(P, wh, lane);
+  }
   if (P.stats) {
     for (int o = 16; o > 0; o >>= 1) inserts += __shfl_xor_sync(0xffffffffu, inserts, o);
     if (lane == 0 && inserts) atomicAdd(P.stats, (unsigned long long)inserts);

@@ -1,5 +1,8 @@
-// nw_dp.cuh -- the all-pairs alignment kernel (sm_103a), templated on the
-// length LB of the longer word of every pair it scores.
+// nw_dp.cuh -- the DPX alignment kernel (sm_103a), whose inner loop is unrolled
+// for the length LB of the longer word of a pair, and the list and histogram
+// updates it shares with the bit-parallel kernel (nw_bits.cuh).  It scores
+// substitution-matrix dictionaries and the match / mismatch scorings that the
+// bit-parallel kernel does not take.
 //
 // Recurrence.  Algorithm 1 of the paper fills H[i][j] = max(H[i-1][j-1] +
 // sim(A[i-1], B[j-1]), H[i-1][j] + p, H[i][j-1] + p) from H[i][0] = p*i and
@@ -124,7 +127,12 @@ __device__ __forceinline__ uint32_t dp_word(const uint32_t* __restrict__ arow, i
 
 // The same DP with the A word's symbols in shared memory, symbol i at
 // acol[32 * i] (the staging layout of the all-pairs kernel; every lane reads
-// the same address, so each load is a broadcast).
+// the same address, so each load is a broadcast).  One row per iteration: a
+// body of R rows is about 64 R LB bytes of instructions, and the warps of an
+// SM sub-partition are at different places of it.  With four rows, LB = 31..40
+// spent 10 of 13 stall cycles per issue waiting for instructions; 4, 2 and 1
+// rows took 10.7, 9.5 and 8.9 ms for a batch of 16 dictionaries (lengths
+// 1..40), and 1 row was also the fastest for 20k and 200k words of 1..25.
 template <int LB, bool TAB = false>
 __device__ __forceinline__ uint32_t dp_word_staged(const uint32_t* acol, int la, const BRow<LB>& b, uint32_t C1,
                                                    uint32_t C2, const uint16_t* tab = nullptr) {
@@ -134,28 +142,8 @@ __device__ __forceinline__ uint32_t dp_word_staged(const uint32_t* acol, int la,
     if (la == 0) return 0u;
     uint32_t G[LB];
     dp_row_first<LB, TAB>(G, acol[0], b, C1, C2, tab);
-    int i = 1;
-    // four rows per iteration: their dependency chains interleave as a
-    // wavefront, and the loop control is paid once per four rows
 #pragma unroll 1
-    for (; i + 3 < la; i += 4) {
-      const uint32_t a0 = acol[32 * i];
-      const uint32_t a1 = acol[32 * (i + 1)];
-      const uint32_t a2 = acol[32 * (i + 2)];
-      const uint32_t a3 = acol[32 * (i + 3)];
-      dp_row<LB, TAB>(G, a0, b, C1, C2, tab);
-      dp_row<LB, TAB>(G, a1, b, C1, C2, tab);
-      dp_row<LB, TAB>(G, a2, b, C1, C2, tab);
-      dp_row<LB, TAB>(G, a3, b, C1, C2, tab);
-    }
-    if (i + 1 < la) {
-      const uint32_t a0 = acol[32 * i];
-      const uint32_t a1 = acol[32 * (i + 1)];
-      dp_row<LB, TAB>(G, a0, b, C1, C2, tab);
-      dp_row<LB, TAB>(G, a1, b, C1, C2, tab);
-      i += 2;
-    }
-    if (i < la) dp_row<LB, TAB>(G, acol[32 * i], b, C1, C2, tab);
+    for (int i = 1; i < la; ++i) dp_row<LB, TAB>(G, acol[32 * i], b, C1, C2, tab);
     return G[LB - 1];
   }
 }
@@ -219,41 +207,36 @@ __device__ __forceinline__ uint64_t upper_offset(uint64_t i, uint64_t j, uint64_
   return i * (2 * n - i - 1) / 2 + (j - i - 1);
 }
 
-// Histogram accumulation.  kHistLane: every lane owns a column of the warp's
-// shared array (bin b of lane l at b*32 + l), so the shared atomics of a warp
-// never collide; kHistSmem: one shared array per warp; kHistGlobal: global
-// atomics.  `bin` is the score minus the histogram's lowest score.
-template <class PT>
-__device__ __forceinline__ void hist_add(const PT& P, uint32_t* wh, int lane, int bin) {
+// Histogram accumulation.  kHistLane: every lane owns a column of the block's
+// shared array (bin b of lane l at b*32 + l), so the shared additions of a
+// warp never collide; kHistSmem: one shared array per warp; kHistGlobal:
+// global atomics.  `bin` is the score minus the histogram's lowest score.
+__device__ __forceinline__ void hist_add(const AlignParams& P, uint32_t* wh, int bin) {
   const uint32_t bi = (uint32_t)bin;
   if (bi >= P.nbins) { atomicOr(P.err, kErrHistRange); return; }
-  if (P.hist_mode == kHistLane) atomicAdd(wh + bi * 32u + (uint32_t)lane, 1u);
-  else if (P.hist_mode == kHistSmem) atomicAdd(wh + bi, 1u);
+  if (P.hist_mode == kHistSmem) atomicAdd(wh + bi, 1u);
   else atomicAdd(P.hist + bi, 1ull);
 }
 
-template <class PT>
-__device__ __forceinline__ void hist_flush(const PT& P, uint32_t* wh, int lane) {
-  __syncwarp();
+// Moves the shared counters (lane columns, or a warp's array) to the
+// histogram, taking each by exchange: other warps may be adding meanwhile.
+__device__ __forceinline__ void hist_flush(const AlignParams& P, uint32_t* wh, int lane) {
   if (P.hist_mode == kHistLane) {
     for (uint32_t b = lane; b < P.nbins; b += 32) {
       uint32_t c = 0;
-      for (int l = 0; l < 32; ++l) {
-        const uint32_t q = b * 32u + (uint32_t)((l + lane) & 31);  // rotated: no bank conflicts
-        c += wh[q];
-      }
+      for (int l = 0; l < 32; ++l) c += atomicExch(wh + b * 32u + (uint32_t)((l + lane) & 31), 0u);  // rotated: no bank conflicts
       if (c) atomicAdd(P.hist + b, (unsigned long long)c);
     }
-    __syncwarp();
-    for (uint32_t q = lane; q < P.nbins * 32u; q += 32) wh[q] = 0u;
   } else {
     for (uint32_t b = lane; b < P.nbins; b += 32) {
-      const uint32_t c = wh[b];
-      if (c) { atomicAdd(P.hist + b, (unsigned long long)c); wh[b] = 0u; }
+      const uint32_t c = atomicExch(wh + b, 0u);
+      if (c) atomicAdd(P.hist + b, (unsigned long long)c);
     }
   }
-  __syncwarp();
 }
+// A warp flushes after this many of its pairs: eight warps' pairs, all in one
+// lane column and bin, still fit the 32-bit counters and their 32-lane sum.
+constexpr uint64_t kHistFlushPairs = 1ull << 28;
 
 // Lowest and highest score any pair of lengths la <= lb can reach: the
 // all-gap alignment and the alignment with min(la, lb) diagonal columns bound
@@ -269,22 +252,18 @@ __device__ __forceinline__ void pair_score_bounds(int match, int mismatch, int g
   hi = allgap > diag_hi ? allgap : diag_hi;
 }
 
-// Word sets, lists and scoring of one task: the kernel parameters, or in a
-// batched launch the terms of the segment (its dictionary or query set).
-struct TaskTerms {
-  const uint32_t* a_enc;
-  const uint4* b_rec;
-  SideView A, B;
-  uint32_t C1, C2;
-  int32_t match, mismatch, gap, key_lo;
-  uint32_t ib, imask;
-};
+// Every bin a task can produce lies inside the histogram (checked once per
+// task against the proven score bounds instead of per pair).
+__device__ __forceinline__ bool hist_covers(const AlignParams& P, const Terms& T, const AlignTask& Q) {
+  int lo, hi;
+  pair_score_bounds(T.match, T.mismatch, T.gap, Q.la < Q.lb ? Q.la : Q.lb, Q.mx, lo, hi);
+  return lo >= P.hist_lo && hi - P.hist_lo < (int)P.nbins;
+}
 
 // List key of a pair with score s whose longer word has m symbols: the raw
 // score, or the rank of s/m in the normalised ranking, above the partner's
 // reversed index (higher key = better neighbour).
-template <class PT, class TT>
-__device__ __forceinline__ uint32_t list_key(const PT& P, const TT& T, int s, int m, uint32_t partner) {
+__device__ __forceinline__ uint32_t list_key(const AlignParams& P, const Terms& T, int s, int m, uint32_t partner) {
   const uint32_t v = P.norm_rank ? (uint32_t)P.norm_rank[(s - P.norm_lo) * kBuckets + m] + 1u
                                  : (uint32_t)(s - T.key_lo);
   return (v << T.ib) | (T.imask - partner);
@@ -296,8 +275,7 @@ __device__ __forceinline__ uint32_t list_key(const PT& P, const TT& T, int s, in
 // threshold's own score; with normalised keys, the smallest score whose s/m
 // has the threshold's rank (a lower rank makes a key below any key of that
 // rank, whatever the partner).
-template <class PT, class TT>
-__device__ __forceinline__ int g_bound(const PT& P, const TT& T, uint32_t thr_key, int m, int pconst) {
+__device__ __forceinline__ int g_bound(const AlignParams& P, const Terms& T, uint32_t thr_key, int m, int pconst) {
   if (thr_key == 0u) return INT_MIN;
   if (P.norm_rank) return (int)P.norm_smin[((thr_key >> T.ib) - 1u) * kBuckets + m] - pconst;
   return (int)(thr_key >> T.ib) + T.key_lo - pconst;
@@ -306,7 +284,7 @@ __device__ __forceinline__ int g_bound(const PT& P, const TT& T, uint32_t thr_ke
 // Packed candidate prefilter.  A G-space bound t (a pair is a candidate for
 // a list when G >= t) is held as 1 - t, clamped so that t = 0 admits every G
 // (G >= 0) and t = 0x7fff none (G <= 819 * 40 < 0x7fff: the host bounds
-// s'_m * NW_MAX_WORD_LEN by 32767).  For the lane's two results packed in res,
+// s'_m * NW_MAX_WORD_LEN by 32767).  For two results packed in res,
 // viaddmax_relu(res, 1 - t, 0) is non-zero in a half exactly when G >= t there.
 __device__ __forceinline__ uint32_t neg_bound16(int t) {
   const int c = t < 0 ? 0 : (t > 0x7fff ? 0x7fff : t);
@@ -316,255 +294,276 @@ __device__ __forceinline__ uint32_t neg_bound2(int t_lo, int t_hi) {
   return neg_bound16(t_lo) | (neg_bound16(t_hi) << 16);
 }
 
-// The all-pairs kernel.  TAB selects substitution-matrix scoring (the table
-// is copied to shared memory after the staging area).  EPI selects the
-// per-pair epilogue at compile time:
+// Candidate queue.  A pair that may enter a list is rare late in a launch and
+// common early, and filing it takes several dependent trips to L2.  The lanes
+// only append such pairs to their warp's queue; once 32 are waiting, each lane
+// files one, so the trips overlap 32-fold.  (Filing each pair in the lane that
+// found it took 126 of 584 ms at 600k words in the bit-parallel kernel, and
+// half of its time at 100k.)  An entry: G << 16 | A word (from g.a0) << 8 |
+// B word (from g.b0); G < 2^15, a task has at most 256 words on either side.
+//
+// Files n <= 32 queued pairs in their words' lists; returns the lane's inserts.
+__device__ __forceinline__ uint32_t file_candidates(const AlignParams& P, const Terms& T, const AlignTask& Q,
+                                                    const uint32_t* queue, uint32_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const int max_iters = P.dbg_insert_limit ? (int)(P.dbg_insert_limit - 1u) : kInsertMaxIters;
+  const bool have = lane < n;
+  const uint32_t e = have ? queue[lane] : 0u;
+  const uint32_t a = Q.g.a0 + ((e >> 8) & 0xffu), b = Q.g.b0 + (e & 0xffu);
+  const int s = (int)(e >> 16) + T.gap * (Q.la + Q.lb);
+  const uint32_t oa = have ? __ldg(T.A.perm + a) : 0u, ob = have ? __ldg(T.B.perm + b) : 0u;
+  uint32_t inserts = 0u;
+  if (T.B.slots && have) {  // word b takes the A word as a neighbour
+    const uint32_t key = list_key(P, T, s, Q.mx, oa);
+    if (key > __ldcg(T.B.thr + b))
+      list_offer(T.B.slots + (size_t)b * P.k, T.B.thr + b, P.k, key, P.err, inserts, max_iters);
+  }
+  if (T.A.slots) {
+    // the A word takes word b.  Several lanes may hold the same A word: one
+    // lane of each such group offers at a time and the others are tested again
+    // against the bound it leaves, so the lanes never race on one list
+    uint32_t key = 0u;
+    if (have) {
+      key = list_key(P, T, s, Q.mx, ob);
+      if (key <= __ldcg(T.A.thr + a)) key = 0u;
+    }
+    const uint32_t group = __match_any_sync(0xffffffffu, a);
+    uint32_t todo;
+    while ((todo = __ballot_sync(0xffffffffu, key != 0u)) != 0u) {
+      if ((uint32_t)(__ffs(todo & group) - 1) == lane) {
+        list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, key, P.err, inserts, max_iters);
+        key = 0u;
+      }
+      __syncwarp();
+      if (key != 0u && key <= __ldcg(T.A.thr + a)) key = 0u;
+    }
+  }
+  return inserts;
+}
+
+// Appends the lanes' candidates (`have`) to the queue and files the first 32
+// once as many are waiting; true if it filed (the lists' bounds have moved).
+__device__ __forceinline__ bool queue_candidate(const AlignParams& P, const Terms& T, const AlignTask& Q,
+                                                uint32_t* queue, uint32_t& waiting, uint32_t& inserts, bool have,
+                                                uint32_t entry) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t m = __ballot_sync(0xffffffffu, have);
+  if (have) queue[waiting + __popc(m & ((1u << lane) - 1u))] = entry;
+  waiting += __popc(m);
+  if (waiting < 32u) return false;
+  __syncwarp();
+  inserts += file_candidates(P, T, Q, queue, 32u);
+  waiting -= 32u;
+  const uint32_t v = lane < waiting ? queue[32 + lane] : 0u;
+  __syncwarp();
+  queue[lane] = v;
+  __syncwarp();
+  return true;
+}
+
+// One task: the A words of a chunk against the lane's two B words of length
+// LB.  TAB selects substitution-matrix scoring; EPI the per-pair epilogue:
 // kEpiMatrix writes the int8 upper triangle, kEpiLists updates neighbour lists
-// (and a shared or global histogram), kEpiListsLaneHist updates lists and the
-// per-lane shared histogram columns, kEpiBatchLists updates the lists named
-// by the segment's terms (a dictionary's own lists, or a query set's lists
-// against a dictionary) in a launch spanning many dictionaries.
-template <int LB, int EPI, bool TAB = false>
-__global__ void __launch_bounds__(kBlock, dp_min_blocks(LB)) nw_dp_kernel(const DpParams P) {
-  extern __shared__ uint32_t s_dyn[];
-  const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
+// (and a shared or global histogram), kEpiListsLaneHist lists and the lane
+// columns of the shared histogram, kEpiBatchLists the lists named by the
+// segment's terms in a launch spanning many dictionaries.
+template <int LB, int EPI, bool TAB>
+__device__ __forceinline__ void dp_task(const AlignParams& P, const Terms& T, const AlignTask& Q, uint32_t* wh,
+                                        uint32_t* sA, const uint16_t* sTab, uint32_t* queue, uint32_t& inserts) {
   constexpr bool kLists = EPI != kEpiMatrix;
-  const bool smem_hist = EPI == kEpiListsLaneHist || (EPI == kEpiLists && P.hist_mode == kHistSmem);
-  const uint32_t wstride = EPI == kEpiListsLaneHist ? P.nbins * 32u : (smem_hist ? P.nbins : 0u);
-  uint32_t* wh = s_dyn + (size_t)wib * wstride;
-  // this warp's staging area: symbol i of the chunk's word w at sA[32 * i + w],
-  // followed by the 32 words' list bounds (raw keys) at sT[w]
-  uint32_t* sA = s_dyn + (size_t)kWarpsPerBlock * wstride + (size_t)wib * 32u * (uint32_t)(LB + 1);
-  uint32_t* sT = sA + 32u * (uint32_t)LB;
+  const int lane = threadIdx.x & 31;
+  const TaskGeom g = Q.g;
+  const int la = Q.la;
+  const int pconst = T.gap * (la + LB);  // score = G + pconst
+  const bool check = Q.check;
+  const uint32_t C1 = T.C1, C2 = T.C2;
+  const uint32_t blo = g.b0 + 2u * lane, bhi = blo + 1u;
+  const bool vlo = blo < g.bend, vhi = bhi < g.bend;
+
+  BRow<LB> brow;
+  if constexpr (LB > 0) {
+#pragma unroll
+    for (int j = 0; j < LB; ++j) brow.v[j] = 0xffffffffu;
+    if (vlo) load_brow<LB>(T.b_rec + Q.b_base + (size_t)lane * (ceil4(LB) / 4), brow);
+    if constexpr (TAB) {
+      // records hold ~code per half (unshifted codes): back to codes, and
+      // code 0 for halves without a word (their results are discarded)
+      const uint32_t keep = (vlo ? 0x0000ffffu : 0u) | (vhi ? 0xffff0000u : 0u);
+#pragma unroll
+      for (int j = 0; j < LB; ++j) brow.v[j] = ~brow.v[j] & keep;
+    }
+  }
+  uint32_t ob_lo = 0u, ob_hi = 0u;
+  if constexpr (EPI == kEpiMatrix) {
+    ob_lo = vlo ? __ldg(T.B.perm + blo) : 0u;
+    ob_hi = vhi ? __ldg(T.B.perm + bhi) : 0u;
+  }
+  uint32_t* hcol = wh + (ptrdiff_t)lane + (ptrdiff_t)(pconst - P.hist_lo) * 32;  // lane column shifted so bin = G
+
+  // packed list bounds of the lane's words, and of A word c0 + lane
+  uint32_t nB2 = 0u, my_nA2 = 0u, waiting = 0u;
+  auto load_bounds_B = [&]() {
+    nB2 = neg_bound2(T.B.slots && vlo ? g_bound(P, T, __ldcg(T.B.thr + blo), LB, pconst) : INT_MAX,
+                     T.B.slots && vhi ? g_bound(P, T, __ldcg(T.B.thr + bhi), LB, pconst) : INT_MAX);
+  };
+  auto load_bound_A = [&](uint32_t c0, uint32_t nA) {
+    const int t = T.A.slots && (uint32_t)lane < nA ? g_bound(P, T, __ldcg(T.A.thr + c0 + lane), LB, pconst) : INT_MAX;
+    my_nA2 = neg_bound2(t, t);
+  };
+  if constexpr (kLists) load_bounds_B();
+
+  for (uint32_t c0 = g.a0; c0 < g.a1; c0 += 32u) {
+    // Stage 32 A words: lane l copies word c0 + l (la symbols); the warp then
+    // reads symbols as shared-memory broadcasts and the G-space bound by shuffle.
+    const uint32_t nA = g.a1 - c0 < 32u ? g.a1 - c0 : 32u;
+    const bool have = (uint32_t)lane < nA;
+    const uint32_t my_orig = (EPI == kEpiMatrix && have) ? __ldg(T.A.perm + c0 + lane) : 0u;
+    if constexpr (kLists) load_bound_A(c0, nA);
+    __syncwarp();
+    if (have) {
+      // asynchronous 4-byte copies: the word's symbol loads are in flight together
+      const uint32_t* src = T.a_sym + Q.a_base + (size_t)(c0 - g.a0 + (uint32_t)lane) * (uint32_t)la;
+      for (int i = 0; i < la; ++i) cp_async4(sA + 32 * i + lane, src + i);
+    }
+    cp_async_wait_all();
+    __syncwarp();
+
+    for (uint32_t w = 0; w < nA; ++w) {
+      const uint32_t a = c0 + w;
+      const uint32_t res = dp_word_staged<LB, TAB>(sA + w, la, brow, C1, C2, sTab);
+      const int g_lo = (int)(res & 0xffffu);  // G >= 0
+      const int g_hi = (int)(res >> 16);
+      const bool ok_lo = vlo && (!check || a < blo), ok_hi = vhi && (!check || a < bhi);
+      if constexpr (EPI == kEpiMatrix) {
+        const uint32_t oa = __shfl_sync(0xffffffffu, my_orig, (int)w);
+        if (ok_lo) {
+          const uint64_t i = oa < ob_lo ? oa : ob_lo, j = oa < ob_lo ? ob_lo : oa;
+          const uint64_t off = upper_offset(i, j, P.n);
+          if (off >= P.mat_lo && off < P.mat_hi) P.mat[off] = (int8_t)(g_lo + pconst);
+        }
+        if (ok_hi) {
+          const uint64_t i = oa < ob_hi ? oa : ob_hi, j = oa < ob_hi ? ob_hi : oa;
+          const uint64_t off = upper_offset(i, j, P.n);
+          if (off >= P.mat_lo && off < P.mat_hi) P.mat[off] = (int8_t)(g_hi + pconst);
+        }
+      } else {
+        if constexpr (EPI == kEpiListsLaneHist) {
+          if (ok_lo) atomicAdd(hcol + 32 * g_lo, 1u);
+          if (ok_hi) atomicAdd(hcol + 32 * g_hi, 1u);
+        } else if (EPI == kEpiLists && P.hist_mode != kHistNone) {
+          if (ok_lo) hist_add(P, wh, g_lo + pconst - P.hist_lo);
+          if (ok_hi) hist_add(P, wh, g_hi + pconst - P.hist_lo);
+        }
+        // both halves against the lower of their two lists' bounds
+        const uint32_t n2 = __vmaxs2(nB2, __shfl_sync(0xffffffffu, my_nA2, (int)w));
+        if (__any_sync(0xffffffffu, __viaddmax_s16x2_relu(res, n2, 0u) != 0u)) {
+          const uint32_t at = ((a - g.a0) << 8) | (2u * (uint32_t)lane);
+          bool filed = false;
+#pragma unroll 1
+          for (int h = 0; h < 2; ++h) {
+            const int G = h ? g_hi : g_lo, nb = h ? (int)n2 >> 16 : (int)(int16_t)n2;
+            const bool in = (h ? ok_hi : ok_lo) && G + nb > 0;
+            if (!__any_sync(0xffffffffu, in)) continue;
+            filed |= queue_candidate(P, T, Q, queue, waiting, inserts, in, ((uint32_t)G << 16) | (at + (uint32_t)h));
+          }
+          if (filed) {
+            load_bounds_B();
+            load_bound_A(c0, nA);
+          }
+        }
+      }
+    }
+  }
+  if constexpr (kLists) {
+    if (waiting) {
+      __syncwarp();
+      inserts += file_candidates(P, T, Q, queue, waiting);
+    }
+  }
+}
+
+template <int LB, int HI, int EPI, bool TAB>
+__device__ __forceinline__ void dp_dispatch(int lb, const AlignParams& P, const Terms& T, const AlignTask& Q,
+                                            uint32_t* wh, uint32_t* sA, const uint16_t* sTab, uint32_t* queue,
+                                            uint32_t& inserts) {
+  if (lb == LB) {
+    dp_task<LB, EPI, TAB>(P, T, Q, wh, sA, sTab, queue, inserts);
+  } else if constexpr (LB < HI) {
+    dp_dispatch<LB + 1, HI, EPI, TAB>(lb, P, T, Q, wh, sA, sTab, queue, inserts);
+  }
+}
+
+// All pairs of a plan whose longer word has LO .. HI symbols.  Warps pull
+// tasks from one counter and work on their own.  One launch covers ten lengths
+// (a launch per length left most SMs idle for small dictionaries: every
+// launch ended in a tail of single long tasks).
+template <int LO, int HI, int EPI, bool TAB = false>
+__global__ void __launch_bounds__(kBlock, dp_min_blocks(HI)) nw_dp_kernel(const __grid_constant__ AlignParams P) {
+  extern __shared__ uint32_t s_dyn[];
+  __shared__ Terms s_terms[kWarpsPerBlock];
+  __shared__ AlignTask s_tasks[kWarpsPerBlock];
+  __shared__ uint32_t s_queue[kWarpsPerBlock][kQueueEntries];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr bool kHist = EPI == kEpiListsLaneHist;
+  const bool warp_hist = EPI == kEpiLists && P.hist_mode == kHistSmem;
+  const uint32_t hist_words = kHist ? P.nbins * 32u : (warp_hist ? P.nbins * kWarpsPerBlock : 0u);
+  // dynamic shared memory: substitution table, histogram, staged A symbols
+  // (symbol i of the chunk's word w at 32 * i + w)
   uint16_t* sTab = nullptr;
+  uint32_t* hist0 = s_dyn;
   if constexpr (TAB) {
-    sTab = reinterpret_cast<uint16_t*>(s_dyn + (size_t)kWarpsPerBlock * wstride +
-                                       (size_t)kWarpsPerBlock * 32u * (uint32_t)(LB + 1));
+    sTab = reinterpret_cast<uint16_t*>(s_dyn);
+    hist0 = s_dyn + kTabBytes / sizeof(uint32_t);
     const uint4* src = reinterpret_cast<const uint4*>(P.sim_tab);
     uint4* dst = reinterpret_cast<uint4*>(sTab);
-    for (int q = threadIdx.x; q < (int)(kTabBytes / sizeof(uint4)); q += blockDim.x) dst[q] = __ldg(src + q);
-    __syncthreads();
+    for (int q = tid; q < (int)(kTabBytes / sizeof(uint4)); q += kBlock) dst[q] = __ldg(src + q);
   }
-  if (smem_hist) {
-    for (uint32_t q = lane; q < wstride; q += 32) wh[q] = 0u;
-    __syncwarp();
-  }
-  uint64_t wpairs = 0;
+  uint32_t* wh = hist0 + (warp_hist ? (size_t)warp * P.nbins : 0);
+  uint32_t* sA = hist0 + hist_words + (size_t)warp * P.stage_syms;
+  for (uint32_t q = (uint32_t)tid; q < hist_words; q += kBlock) hist0[q] = 0u;
+  __syncthreads();
+  Terms& T = s_terms[warp];
+  AlignTask& Q = s_tasks[warp];
   uint32_t inserts = 0;
-  const int max_iters = P.dbg_insert_limit ? (int)(P.dbg_insert_limit - 1u) : kInsertMaxIters;
+  uint64_t hpairs = 0;
 
   for (;;) {
     unsigned long long t = 0;
     if (lane == 0) t = atomicAdd(P.counter, 1ull);
-    t = __shfl_sync(0xffffffffu, t, 0) + P.task_lo;
-    if (t >= P.task_hi) break;
-
-    const Seg S = P.segs[find_seg(P.segs, P.nsegs, t)];
-    const TaskGeom g = task_geom(S, t, P.TA);
-    TaskTerms T;
-    if constexpr (EPI == kEpiBatchLists) {
-      const DictTerms& D = P.terms[S.dict];
-      T = TaskTerms{D.a_enc, D.b_rec, D.A, D.B, D.C1, D.C2, D.match, D.mismatch, D.gap, D.key_lo, D.ib, D.imask};
-    } else {
-      T = TaskTerms{P.a_enc, P.b_rec, P.A, P.B, P.C1, P.C2, P.match, P.mismatch, P.gap, P.key_lo, P.ib, P.imask};
+    t = __shfl_sync(0xffffffffu, t, 0);
+    if (t >= P.ntasks) break;
+    const Seg* S = P.segs + find_seg(P.segs, P.nsegs, t);
+    const uint32_t d = S->dict;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(EPI == kEpiBatchLists ? P.terms + d : P.local + d);
+    __syncwarp();
+    for (int q = lane; q < (int)(sizeof(Terms) / 4); q += 32) reinterpret_cast<uint32_t*>(&T)[q] = src[q];
+    if (lane == 0) {
+      Q.g = task_geom(*S, t, P.TA);
+      Q.la = S->la;
+      Q.lb = (int)S->lb;
+      Q.mx = Q.lb;
+      Q.a_base = S->aenc_base + (Q.g.a0 - S->a_beg) * (uint32_t)Q.la;
+      Q.b_base = S->b_base + ((Q.g.b0 - S->b_beg) / 2u) * (uint32_t)(ceil4(Q.lb) / 4);
+      Q.check = Q.g.tri && Q.g.a1 > Q.g.b0;
     }
-    const bool listsA = kLists && T.A.slots != nullptr;
-    // (queries run without a histogram: the histogram kernels keep the lanes' own offers)
-    const bool serialA = EPI == kEpiLists && listsA && P.serial_a != 0u;
-    const bool listsB = kLists && T.B.slots != nullptr;
-    const uint32_t blo = g.b0 + 2u * lane;
-    const uint32_t bhi = blo + 1u;
-    const bool vlo = blo < g.bend;
-    const bool vhi = bhi < g.bend;
-    const bool check = g.tri && g.a1 > g.b0;  // the task straddles the diagonal: test a < b
-    const int la = S.la;
-    const int pconst = T.gap * (la + LB);  // score = G + pconst
-    const int hoff = pconst - P.hist_lo;   // histogram bin = G + hoff
-
-    // every bin this task can produce lies inside the histogram (proven
-    // bounds); checked once here instead of per pair
-    bool hist_on = (EPI == kEpiLists || EPI == kEpiListsLaneHist) && P.hist_mode != kHistNone;
-    if (hist_on) {
-      int lo, hi;
-      pair_score_bounds(T.match, T.mismatch, T.gap, la, LB, lo, hi);
-      if (lo < P.hist_lo || hi - P.hist_lo >= (int)P.nbins) {
-        if (lane == 0) atomicOr(P.err, kErrHistRange);
-        hist_on = false;
+    __syncwarp();
+    if ((EPI == kEpiLists || kHist) && P.hist_mode != kHistNone && !hist_covers(P, T, Q)) {
+      if (lane == 0) atomicOr(P.err, kErrHistRange);
+      continue;
+    }
+    dp_dispatch<LO, HI, EPI, TAB>(Q.lb, P, T, Q, wh, sA, sTab, s_queue[warp], inserts);
+    if (hist_words) {
+      hpairs += (uint64_t)(Q.g.a1 - Q.g.a0) * (uint32_t)kWarpB;
+      if (hpairs >= kHistFlushPairs) {
+        hist_flush(P, wh, lane);
+        hpairs = 0;
       }
-    }
-    uint32_t* hcol = wh + (ptrdiff_t)lane + (ptrdiff_t)hoff * 32;  // lane column shifted so bin = G
-
-    BRow<LB> brow;
-    if constexpr (LB > 0) {
-#pragma unroll
-      for (int j = 0; j < LB; ++j) brow.v[j] = 0xffffffffu;
-      if (vlo) load_brow<LB>(T.b_rec + S.brec_base + (size_t)(g.cb * (kWarpB / 2) + lane) * (ceil4(LB) / 4), brow);
-      if constexpr (TAB) {
-        // records hold ~code per half (unshifted codes): back to codes, and
-        // code 0 for halves without a word (their results are discarded)
-        const uint32_t keep = (vlo ? 0x0000ffffu : 0u) | (vhi ? 0xffff0000u : 0u);
-#pragma unroll
-        for (int j = 0; j < LB; ++j) brow.v[j] = ~brow.v[j] & keep;
-      }
-    }
-    const uint32_t ob_lo = vlo ? __ldg(T.B.perm + blo) : 0u;
-    const uint32_t ob_hi = vhi ? __ldg(T.B.perm + bhi) : 0u;
-    // B-side lists: cached smallest keys and their G-space candidate bounds
-    uint32_t thrB_lo = 0u, thrB_hi = 0u;
-    int tB_lo = INT_MAX, tB_hi = INT_MAX;
-    if (listsB) {
-      if (vlo) { thrB_lo = __ldcg(T.B.thr + blo); tB_lo = g_bound(P, T, thrB_lo, LB, pconst); }
-      if (vhi) { thrB_hi = __ldcg(T.B.thr + bhi); tB_hi = g_bound(P, T, thrB_hi, LB, pconst); }
-    }
-    // packed form of the B bounds for the prefilter, and the halves holding a word
-    uint32_t nB2 = neg_bound2(tB_lo, tB_hi);
-    const uint32_t okmask = (vlo ? 0x0000ffffu : 0u) | (vhi ? 0xffff0000u : 0u);
-
-    for (uint32_t c0 = g.a0; c0 < g.a1; c0 += 32u) {
-      // Stage 32 A words: lane l copies word c0 + l (la symbols) and its list
-      // bound; the warp then reads symbols as shared-memory broadcasts and the
-      // G-space bound by shuffle.
-      const uint32_t nA = g.a1 - c0 < 32u ? g.a1 - c0 : 32u;
-      const uint32_t my_a = c0 + (uint32_t)lane;
-      const bool have = (uint32_t)lane < nA;
-      const uint32_t my_orig = (EPI == kEpiMatrix && have) ? __ldg(T.A.perm + my_a) : 0u;
-      const uint32_t my_thr = (listsA && have) ? __ldcg(T.A.thr + my_a) : 0u;
-      const int my_tA = listsA ? g_bound(P, T, my_thr, LB, pconst) : INT_MAX;
-      const uint32_t my_nA2 = neg_bound2(my_tA, my_tA);
-      __syncwarp();
-      if (have) {
-        // asynchronous 4-byte copies: the word's symbol loads are in flight together
-        const uint32_t* src = T.a_enc + S.aenc_base + (size_t)(my_a - S.a_beg) * (uint32_t)la;
-        for (int i = 0; i < la; ++i) cp_async4(sA + 32 * i + lane, src + i);
-        sT[lane] = my_thr;
-      }
-      cp_async_wait_all();
-      __syncwarp();
-
-      for (uint32_t w = 0; w < nA; ++w) {
-        const uint32_t a = c0 + w;
-        const uint32_t res = dp_word_staged<LB, TAB>(sA + w, la, brow, T.C1, T.C2, sTab);
-        const int g_lo = (int)(res & 0xffffu);  // G >= 0
-        const int g_hi = (int)(res >> 16);
-        bool ok_lo = vlo, ok_hi = vhi;
-        if (check) {
-          ok_lo = ok_lo && a < blo;
-          ok_hi = ok_hi && a < bhi;
-        }
-
-        if constexpr (EPI == kEpiMatrix) {
-          const uint32_t oa = __shfl_sync(0xffffffffu, my_orig, (int)w);
-          if (ok_lo) {
-            const uint64_t i = oa < ob_lo ? oa : ob_lo, j = oa < ob_lo ? ob_lo : oa;
-            const uint64_t off = upper_offset(i, j, P.n);
-            if (off >= P.mat_lo && off < P.mat_hi) P.mat[off] = (int8_t)(g_lo + pconst);
-          }
-          if (ok_hi) {
-            const uint64_t i = oa < ob_hi ? oa : ob_hi, j = oa < ob_hi ? ob_hi : oa;
-            const uint64_t off = upper_offset(i, j, P.n);
-            if (off >= P.mat_lo && off < P.mat_hi) P.mat[off] = (int8_t)(g_hi + pconst);
-          }
-        } else {
-          if (hist_on) {
-            if constexpr (EPI == kEpiListsLaneHist) {
-              // lane columns are private to their lane: plain increments
-              if (ok_lo) hcol[32 * g_lo] += 1u;
-              if (ok_hi) hcol[32 * g_hi] += 1u;
-            } else {
-              if (ok_lo) hist_add(P, wh, lane, g_lo + hoff);
-              if (ok_hi) hist_add(P, wh, lane, g_hi + hoff);
-            }
-          }
-          // Both halves tested at once against the lower of the two lists'
-          // bounds (packed prefilter, exact: see neg_bound16); tasks on the
-          // diagonal, which must also test a < b, skip it.  Exact keys are
-          // formed only for the rare candidates.
-          const uint32_t nA2 = __shfl_sync(0xffffffffu, my_nA2, (int)w);
-          const bool pre = check || (__viaddmax_s16x2_relu(res, __vmaxs2(nB2, nA2), 0u) & okmask) != 0u;
-          uint32_t ka_lo = 0u, ka_hi = 0u;  // this lane's keys for the A word's list
-          if (pre) {
-            const uint32_t thrA = sT[w];
-            const int tA = listsA ? g_bound(P, T, thrA, LB, pconst) : INT_MAX;
-            const bool c_lo = ok_lo && g_lo >= min(tB_lo, tA);
-            const bool c_hi = ok_hi && g_hi >= min(tB_hi, tA);
-            if (c_lo || c_hi) {
-              const uint32_t oa = __ldg(T.A.perm + a);
-              if (c_lo) {
-                const int s = g_lo + pconst;
-                if (g_lo >= tB_lo) {  // the lane's word takes the A word as a neighbour
-                  const uint32_t key = list_key(P, T, s, LB, oa);
-                  if (key > thrB_lo) {
-                    const uint32_t nm = list_offer(T.B.slots + (size_t)blo * P.k, T.B.thr + blo, P.k, key, P.err, inserts, max_iters);
-                    if (nm > thrB_lo) {
-                      thrB_lo = nm;
-                      tB_lo = g_bound(P, T, nm, LB, pconst);
-                      nB2 = neg_bound2(tB_lo, tB_hi);
-                    }
-                  }
-                }
-                if (g_lo >= tA) {  // the A word takes the lane's word as a neighbour
-                  const uint32_t key = list_key(P, T, s, LB, ob_lo);
-                  if (key > thrA) {
-                    if (serialA) ka_lo = key;
-                    else list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, key, P.err, inserts, max_iters);
-                  }
-                }
-              }
-              if (c_hi) {
-                const int s = g_hi + pconst;
-                if (g_hi >= tB_hi) {
-                  const uint32_t key = list_key(P, T, s, LB, oa);
-                  if (key > thrB_hi) {
-                    const uint32_t nm = list_offer(T.B.slots + (size_t)bhi * P.k, T.B.thr + bhi, P.k, key, P.err, inserts, max_iters);
-                    if (nm > thrB_hi) {
-                      thrB_hi = nm;
-                      tB_hi = g_bound(P, T, nm, LB, pconst);
-                      nB2 = neg_bound2(tB_lo, tB_hi);
-                    }
-                  }
-                }
-                if (g_hi >= tA) {
-                  const uint32_t key = list_key(P, T, s, LB, ob_hi);
-                  if (key > thrA) {
-                    if (serialA) ka_hi = key;
-                    else list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, key, P.err, inserts, max_iters);
-                  }
-                }
-              }
-            }
-          }
-          if (serialA) {
-            // Every lane may hold keys for the same A word's list.  The warp
-            // offers them one at a time from the best down, each against the
-            // bound the previous offer returned, and stops at the first key
-            // below it: the lanes never race on that list, and a list that
-            // is already full costs one offer.
-            uint32_t best = ka_lo > ka_hi ? ka_lo : ka_hi;
-            uint32_t thrW = sT[w];
-            while (__any_sync(0xffffffffu, best > thrW)) {
-              const uint32_t m = __reduce_max_sync(0xffffffffu, best);
-              const int src = __ffs(__ballot_sync(0xffffffffu, best == m)) - 1;
-              uint32_t nm = 0u;
-              if (lane == src) {
-                nm = list_offer(T.A.slots + (size_t)a * P.k, T.A.thr + a, P.k, m, P.err, inserts, max_iters);
-                if (ka_lo == m) ka_lo = 0u; else ka_hi = 0u;
-                best = ka_lo > ka_hi ? ka_lo : ka_hi;
-              }
-              nm = __shfl_sync(0xffffffffu, nm, src);
-              thrW = nm > thrW ? nm : thrW;
-            }
-          }
-        }
-      }
-    }
-    if (smem_hist) {  // 32-bit shared counters: flush long before they could wrap
-      wpairs += (uint64_t)(g.a1 - g.a0) * 64u;
-      if (wpairs >= (1ull << 30)) { hist_flush(P, wh, lane); wpairs = 0; }
     }
   }
-
-  if (smem_hist) hist_flush(P, wh, lane);
+  if (hist_words) {
+    __syncthreads();
+    if (warp_hist || warp == 0) hist_flush(P, wh, lane);
+  }
   if (P.stats) {
     for (int o = 16; o > 0; o >>= 1) inserts += __shfl_xor_sync(0xffffffffu, inserts, o);
     if (lane == 0 && inserts) atomicAdd(P.stats, (unsigned long long)inserts);

@@ -1,4 +1,3 @@
-// Alignment kernels for the longer word length LB in [0, 10].
-#define NW_LB_LO 0
-#define NW_LB_HI 10
+// DPX alignment kernels for the longer word lengths 0 to 10.
+#define NW_DP_RANGE 0
 #include "nw_dp_inst.inc"

@@ -1,4 +1,3 @@
-// Alignment kernels for the longer word length LB in [11, 20].
-#define NW_LB_LO 11
-#define NW_LB_HI 20
+// DPX alignment kernels for the longer word lengths 11 to 20.
+#define NW_DP_RANGE 1
 #include "nw_dp_inst.inc"

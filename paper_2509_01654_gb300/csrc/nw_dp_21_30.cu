@@ -1,4 +1,3 @@
-// Alignment kernels for the longer word length LB in [21, 30].
-#define NW_LB_LO 21
-#define NW_LB_HI 30
+// DPX alignment kernels for the longer word lengths 21 to 30.
+#define NW_DP_RANGE 2
 #include "nw_dp_inst.inc"

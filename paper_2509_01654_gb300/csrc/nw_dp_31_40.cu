@@ -1,4 +1,3 @@
-// Alignment kernels for the longer word length LB in [31, 40].
-#define NW_LB_LO 31
-#define NW_LB_HI 40
+// DPX alignment kernels for the longer word lengths 31 to 40.
+#define NW_DP_RANGE 3
 #include "nw_dp_inst.inc"

@@ -1,19 +1,21 @@
-// Maps a length LB, and reduced steps (m, x), to their alignment kernels across
-// the instantiation units.
+// Maps a range of lengths, and reduced steps (m, x), to their alignment kernels
+// across the instantiation units.
 #include "nw_launch.h"
 
 namespace nw {
-const void* dp_kernel_range_0(int LB, int epi, bool tab);
-const void* dp_kernel_range_11(int LB, int epi, bool tab);
-const void* dp_kernel_range_21(int LB, int epi, bool tab);
-const void* dp_kernel_range_31(int LB, int epi, bool tab);
+const void* dp_kernel_range_0(int epi, bool tab);
+const void* dp_kernel_range_1(int epi, bool tab);
+const void* dp_kernel_range_2(int epi, bool tab);
+const void* dp_kernel_range_3(int epi, bool tab);
 
-const void* dp_kernel(int LB, int epi, bool tab) {
-  if (LB < 0 || LB > kMaxLen) return nullptr;
-  if (LB <= 10) return dp_kernel_range_0(LB, epi, tab);
-  if (LB <= 20) return dp_kernel_range_11(LB, epi, tab);
-  if (LB <= 30) return dp_kernel_range_21(LB, epi, tab);
-  return dp_kernel_range_31(LB, epi, tab);
+const void* dp_kernel(int range, int epi, bool tab) {
+  switch (range) {
+    case 0: return dp_kernel_range_0(epi, tab);
+    case 1: return dp_kernel_range_1(epi, tab);
+    case 2: return dp_kernel_range_2(epi, tab);
+    case 3: return dp_kernel_range_3(epi, tab);
+    default: return nullptr;
+  }
 }
 
 #define NW_BIT_ALL(F) F(1, 0) F(2, 1) F(3, 1) F(3, 2) F(4, 1) F(4, 3) F(5, 1) F(5, 2) F(5, 3) F(5, 4)

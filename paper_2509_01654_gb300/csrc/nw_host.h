@@ -46,28 +46,23 @@ struct WordSet {
   DevBuf perm, rank, slen, aoff, brec_w, a_enc, b_rec;
 };
 
-struct LaunchPlan {
-  int LB = 0;
-  int role = 0;  // 0: A and B from one set; 1: A = queries, B = dictionary; 2: A = dictionary, B = queries
-  uint32_t ta = 0;  // A words per task of this launch (0: the launch parameters' TA)
-  uint32_t bps = 0; // resident blocks per SM at most (0: as many as fit)
+// One alignment launch: a range of longer lengths of the DPX kernel, or the
+// bit-parallel kernel's length pairs of one step class.
+struct Launch {
+  int range = 0;            // DPX kernel: dp_range_of the longer length; -1: bit-parallel
+  int m = 0, x = 0;         // bit-parallel: the reduced steps
+  uint32_t alphabet = 0;    // bit-parallel: the largest of the launch's sets
+  uint32_t ta = 0;          // A words per task
+  uint32_t bps = 0;         // resident blocks per SM at most (0: as many as fit)
   uint32_t seg_first = 0, nsegs = 0;
   uint64_t ntasks = 0;
-  uint64_t pairs = 0, cells = 0;
+  uint32_t max_la = 0;      // longest A word
 };
 
 struct Plan {
   std::vector<Seg> segs;
-  std::vector<LaunchPlan> launches;
+  std::vector<Launch> launches;
   uint64_t pairs = 0, cells = 0;
-};
-
-// The plan of one bit-parallel launch: every length pair in one segment list.
-struct BitPlan {
-  std::vector<Seg> segs;
-  uint32_t ta = 0;      // A words per task
-  uint64_t ntasks = 0;
-  uint32_t max_la = 0;  // longest A word
 };
 
 }  // namespace
@@ -105,8 +100,7 @@ struct nw_dict {
   uint32_t alphabet = 0;
   int32_t score_lo = 0, score_hi = 0;
   Plan plan;
-  BitPlan bits;        // used instead of plan's launches when ss.bit_m > 0
-  DevBuf d_segs;       // the segments of the plan in use
+  DevBuf d_segs;       // the plan's segments
   bool subst = false;  // scored with a full similarity matrix (d_tab)
   DevBuf d_tab;        // kTabDim x kTabDim s'+ table
   uint64_t serial = 0;  // unique per loaded dictionary (caches keyed on it)
@@ -287,274 +281,225 @@ uint64_t brec_words(const Buckets& bk) {
 
 uint64_t cdiv(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 
-Seg make_seg(const Buckets& A, int La, uint32_t a_beg, uint32_t a_end, const Buckets& B, int LB,
-             uint32_t b_beg, uint32_t b_end, bool tri, uint32_t TA, uint64_t task0, uint64_t& ntasks) {
-  Seg s{};
-  s.a_beg = a_beg;
-  s.a_end = a_end;
-  s.b_beg = b_beg;
-  s.b_end = b_end;
-  s.aenc_base = A.aenc_base[La] + (a_beg - A.start[La]) * (uint32_t)La;
-  const uint32_t rb = b_beg - B.start[LB];
-  s.brec_base = (B.brec_word_base[LB] + (rb / 2) * (uint32_t)ceil4(LB)) / 4;
-  s.la = (uint16_t)La;
-  s.tri = tri ? 1 : 0;
-  s.nca = (uint32_t)cdiv(a_end - a_beg, TA);
-  s.task0 = task0;
-  ntasks = (uint64_t)s.nca * cdiv(b_end - b_beg, kWarpB);
-  return s;
+// ---------------------------------------------------------------------------
+// plans.  A call's pairs are listed as rectangles of buckets, the shorter
+// words on the A side; the kernel that scores them cuts them into segments and
+// tasks.
+
+// Words [a0, a1) of bucket La of set A against words [b0, b1) of bucket LB of
+// set B (relative to the buckets), La <= LB; tri: the same bucket, only pairs
+// a < b.  `dict` names the terms, dict_swapped those with the sides exchanged.
+struct Rect {
+  const Buckets* A;
+  const Buckets* B;
+  int La, LB;
+  uint32_t a0, a1, b0, b1;
+  bool tri;
+  uint32_t dict, dict_swapped;
+};
+using Rects = std::vector<Rect>;
+
+// Every unordered pair of one set, once.
+void rects_all(const Buckets& bk, uint32_t dict, Rects& out) {
+  for (int L = 0; L < kBuckets; ++L)
+    for (int s = 0; s <= L; ++s)
+      if (bk.count[s] && bk.count[L] && (s < L || bk.count[L] > 1))
+        out.push_back({&bk, &bk, s, L, 0, bk.count[s], 0, bk.count[L], s == L, dict, dict});
 }
 
-// Launches run in increasing longer length: a word of length L first meets
-// partners of its own length (the segment La == LB leads launch L), where its
-// best neighbours usually are, so list thresholds rise before the many
-// low-scoring pairs of very different lengths arrive.
-void order_launches(Plan& p) {
-  std::stable_sort(p.launches.begin(), p.launches.end(),
-                   [](const LaunchPlan& x, const LaunchPlan& y) { return x.LB < y.LB; });
+// Every (query, dictionary word) pair, once: terms dict where the queries are
+// the A words, dict + 1 where they are the B words.
+void rects_queries(const Buckets& qb, const Buckets& db, uint32_t dict, Rects& out) {
+  for (int lq = 0; lq < kBuckets; ++lq)
+    for (int ld = 0; ld < kBuckets; ++ld) {
+      if (!qb.count[lq] || !db.count[ld]) continue;
+      if (lq <= ld) out.push_back({&qb, &db, lq, ld, 0, qb.count[lq], 0, db.count[ld], false, dict, dict + 1});
+      else out.push_back({&db, &qb, ld, lq, 0, db.count[ld], 0, qb.count[lq], false, dict + 1, dict});
+    }
 }
 
-// Every unordered pair of one set, once: launch LB holds the pairs whose
-// longer word has length LB; inside it the same-length rectangle comes first,
-// then shorter A lengths in order of growing length difference.
-void plan_all_pairs(const Buckets& bk, uint32_t TA, Plan& out) {
-  out = Plan{};
-  if (TA == 0) TA = kDefaultTA;
-  TA = (TA + 1) & ~1u;  // A chunks start B chunks of the same bucket: keep them even
+// Shard `shard` of `nshards` of one set's pairs.  The partition: per longer
+// length LB a task list (same-length strips of 256 words first, then shorter
+// lengths in falling order; tasks of 256 A words by 64 B words, A chunks
+// fastest), each list cut into nshards contiguous ranges.  It is fixed,
+// whatever kernel scores the pairs and however it cuts them, so that shards
+// saved by one build combine with another's.
+constexpr uint32_t kShardTA = 256;
+void rects_shard(const Buckets& bk, uint32_t shard, uint32_t nshards, Rects& out) {
+  struct Block {
+    int La;
+    uint32_t a0, a1, b0, b1;
+    uint32_t nca, ncb;
+  };
   for (int LB = 0; LB < kBuckets; ++LB) {
     const uint32_t nB = bk.count[LB];
+    std::vector<Block> blocks;
+    uint64_t total = 0;
+    auto add = [&](int La, uint32_t a0, uint32_t a1, uint32_t b0) {
+      blocks.push_back({La, a0, a1, b0, nB, (uint32_t)cdiv(a1 - a0, kShardTA), (uint32_t)cdiv(nB - b0, kWarpB)});
+      total += (uint64_t)blocks.back().nca * blocks.back().ncb;
+    };
     if (nB == 0) continue;
-    LaunchPlan lp;
-    lp.LB = LB;
-    lp.role = 0;
-    lp.seg_first = (uint32_t)out.segs.size();
-    uint64_t task = 0;
-    for (int La = LB; La >= 0; --La) {
-      if (La == LB) {
-        if (nB < 2) continue;
-        const uint32_t s = bk.start[LB], e = s + nB;
-        for (uint32_t a_beg = s; a_beg < e; a_beg += TA) {
-          const uint32_t a_end = std::min(e, a_beg + TA);
-          if (e - a_beg < 2) continue;
-          uint64_t nt = 0;
-          out.segs.push_back(make_seg(bk, LB, a_beg, a_end, bk, LB, a_beg, e, true, TA, task, nt));
-          task += nt;
+    for (uint32_t a = 0; a + 1 < nB; a += kShardTA) add(LB, a, std::min(nB, a + kShardTA), a);
+    for (int La = LB - 1; La >= 0; --La)
+      if (bk.count[La]) add(La, 0, bk.count[La], 0);
+    const uint64_t lo = total * shard / nshards, hi = total * (shard + 1) / nshards;
+    uint64_t t0 = 0;
+    for (const Block& k : blocks) {
+      const uint64_t t1 = t0 + (uint64_t)k.nca * k.ncb, a = std::max(lo, t0), b = std::min(hi, t1);
+      if (a < b) {
+        // tasks [a, b): whole rows of B chunks, and parts of the first and last
+        auto rect = [&](uint32_t ca0, uint32_t ca1, uint32_t cb0, uint32_t cb1) {
+          if (ca0 >= ca1 || cb0 >= cb1) return;
+          out.push_back({&bk, &bk, k.La, LB, std::min(k.a1, k.a0 + ca0 * kShardTA), std::min(k.a1, k.a0 + ca1 * kShardTA),
+                         std::min(k.b1, k.b0 + cb0 * (uint32_t)kWarpB), std::min(k.b1, k.b0 + cb1 * (uint32_t)kWarpB),
+                         k.La == LB, 0u, 0u});
+        };
+        const uint32_t l0 = (uint32_t)((a - t0) / k.nca), c0 = (uint32_t)((a - t0) % k.nca);
+        const uint32_t l1 = (uint32_t)((b - t0) / k.nca), c1 = (uint32_t)((b - t0) % k.nca);
+        if (l0 == l1) {
+          rect(c0, c1, l0, l0 + 1);
+        } else {
+          rect(c0, k.nca, l0, l0 + 1);
+          rect(0, k.nca, l0 + 1, l1);
+          rect(0, c1, l1, l1 + 1);
         }
-        lp.pairs += (uint64_t)nB * (nB - 1) / 2;
-        lp.cells += (uint64_t)nB * (nB - 1) / 2 * (uint64_t)(LB * LB);
-      } else {
-        const uint32_t nA = bk.count[La];
-        if (nA == 0) continue;
-        uint64_t nt = 0;
-        out.segs.push_back(make_seg(bk, La, bk.start[La], bk.start[La] + nA, bk, LB, bk.start[LB],
-                                    bk.start[LB] + nB, false, TA, task, nt));
-        task += nt;
-        lp.pairs += (uint64_t)nA * nB;
-        lp.cells += (uint64_t)nA * nB * (uint64_t)(La * LB);
       }
-    }
-    lp.nsegs = (uint32_t)out.segs.size() - lp.seg_first;
-    lp.ntasks = task;
-    if (lp.nsegs) {
-      out.pairs += lp.pairs;
-      out.cells += lp.cells;
-      out.launches.push_back(lp);
+      t0 = t1;
     }
   }
-  order_launches(out);
 }
 
-// ---- plans of the bit-parallel kernel
+// Pairs and cells of whole-bucket rectangles.
+void count_rects(const Rects& rects, uint64_t& pairs, uint64_t& cells) {
+  for (const Rect& r : rects) {
+    const uint64_t na = r.a1 - r.a0, nb = r.b1 - r.b0, n = r.tri ? na * (na - 1) / 2 : na * nb;
+    pairs += n;
+    cells += n * (uint64_t)(r.La * r.LB);
+  }
+}
+
+// Smallest length difference first: a word's best neighbours mostly have
+// nearly its length, so its list bound rises before the many low-scoring pairs
+// arrive.  Within a difference the long words (the long tasks) come first.
+void order_rects(Rects& rects) {
+  std::stable_sort(rects.begin(), rects.end(), [](const Rect& x, const Rect& y) {
+    const int dx = x.LB - x.La, dy = y.LB - y.La;
+    return dx != dy ? dx < dy : x.LB > y.LB;
+  });
+}
+
+// Appends a rectangle to the launch's segments.  Same-bucket rectangles are
+// cut into strips of ta A words, each against the B words from its start on.
+void add_rect(Plan& p, Launch& l, const Rect& r) {
+  const bool bits = l.range < 0;
+  const uint32_t chunk = bits ? 32u * (uint32_t)bit_words_per_lane(r.LB) : (uint32_t)kWarpB;
+  auto seg = [&](uint32_t a0, uint32_t a1, uint32_t b0) {
+    if (a0 >= a1 || b0 >= r.b1 || (r.tri && a0 + 1 >= r.b1)) return;
+    Seg s{};
+    s.a_beg = r.A->start[r.La] + a0;
+    s.a_end = r.A->start[r.La] + a1;
+    s.b_beg = r.B->start[r.LB] + b0;
+    s.b_end = r.B->start[r.LB] + r.b1;
+    s.aenc_base = r.A->aenc_base[r.La] + a0 * (uint32_t)r.La;
+    // (b0 is even: bucket starts, and multiples of 64 and of the strip size)
+    s.b_base = bits ? r.B->aenc_base[r.LB] + b0 * (uint32_t)r.LB
+                    : (r.B->brec_word_base[r.LB] + (b0 / 2) * (uint32_t)ceil4(r.LB)) / 4;
+    s.la = (uint16_t)r.La;
+    s.lb = (uint32_t)r.LB;
+    s.tri = r.tri ? 1 : 0;
+    s.dict = r.dict;
+    s.nca = (uint32_t)cdiv(a1 - a0, l.ta);
+    s.task0 = l.ntasks;
+    l.ntasks += (uint64_t)s.nca * cdiv(r.b1 - b0, chunk);
+    l.max_la = std::max(l.max_la, (uint32_t)r.La);
+    p.segs.push_back(s);
+    ++l.nsegs;
+  };
+  if (!r.tri) return seg(r.a0, r.a1, r.b0);
+  for (uint32_t a = r.a0; a < r.a1; a += l.ta) seg(a, std::min(r.a1, a + l.ta), std::max(r.b0, a));
+}
+
+// The DPX launches of a pair list (in order_rects order), one per range of
+// longer lengths present, with `ta` A words per task.  Within a launch the
+// lengths come one after another, each smallest difference first: the loop
+// body of a length is several KB of instructions, and a mix of ten of them
+// ran out of the instruction cache.
+void plan_dp(Rects rects, uint32_t ta, Plan& p, int only_range = -1, uint32_t bps = 0) {
+  std::stable_sort(rects.begin(), rects.end(), [](const Rect& x, const Rect& y) { return x.LB < y.LB; });
+  for (int r = 0; r < kDpRanges; ++r) {
+    if (only_range >= 0 && r != only_range) continue;
+    Launch l;
+    l.range = r;
+    l.ta = ta;
+    l.bps = bps;
+    l.seg_first = (uint32_t)p.segs.size();
+    for (const Rect& x : rects)
+      if (dp_range_of(x.LB) == r) add_rect(p, l, x);
+    if (l.ntasks) p.launches.push_back(l);
+  }
+}
 
 // Estimated SM sub-partition cycles (per warp) of nA words of length a against
-// nB words of length b in the lanes: a row costs ~70 cycles for the lane's
-// words, an A word ~40, each of the lane's words ~12 to score and file, and
-// each task ~1500 to build its match masks.
+// nB words of length b in the lanes of the bit-parallel kernel: a row costs
+// ~70 cycles for the lane's words, an A word ~40, each of the lane's words ~12
+// to score and file, and each task ~1500 to build its match masks.
 uint64_t bit_cost(uint64_t nA, int a, uint64_t nB, int b, uint32_t ta) {
   const uint64_t K = (uint64_t)bit_words_per_lane(b);
   const uint64_t chunks = cdiv(nB, 32 * K), kk = std::min<uint64_t>(K, cdiv(nB, 32));
   return chunks * (nA * ((uint64_t)a * 70 + 40 + 12 * kk) + cdiv(nA, ta) * 1500);
 }
 
-// One rectangle of pairs for the bit-parallel kernel: words [a0, a1) of bucket
-// La of A (relative to the bucket) against [b0, b1) of bucket LB of B.
-struct BitRect {
-  int La, LB;
-  uint32_t a0, a1, b0, b1;
-  bool tri;
-  uint32_t dict;
-};
-
-void bit_add(BitPlan& p, const Buckets& A, const Buckets& B, const BitRect& r) {
-  if (r.a0 >= r.a1 || r.b0 >= r.b1) return;
-  Seg s{};
-  s.a_beg = A.start[r.La] + r.a0;
-  s.a_end = A.start[r.La] + r.a1;
-  s.b_beg = B.start[r.LB] + r.b0;
-  s.b_end = B.start[r.LB] + r.b1;
-  s.aenc_base = A.aenc_base[r.La] + r.a0 * (uint32_t)r.La;
-  s.brec_base = B.aenc_base[r.LB] + r.b0 * (uint32_t)r.LB;
-  s.la = (uint16_t)r.La;
-  s.lb = (uint32_t)r.LB;
-  s.tri = r.tri ? 1 : 0;
-  s.dict = r.dict;
-  s.nca = (uint32_t)cdiv(r.a1 - r.a0, p.ta);
-  s.task0 = p.ntasks;
-  p.ntasks += (uint64_t)s.nca * cdiv(r.b1 - r.b0, 32u * (uint32_t)bit_words_per_lane(r.LB));
-  p.max_la = std::max(p.max_la, (uint32_t)r.La);
-  p.segs.push_back(s);
-}
-
-// Every unordered pair of one set, once.  Same-length pairs are cut into
-// strips of ta A words against the words from the strip on; pairs of two
-// lengths take the cheaper of the two orientations.  Length differences come
-// in increasing order: a word's best neighbours mostly have nearly its
-// length, so its list bound rises before the many low-scoring pairs arrive.
-void bit_pairs(const Buckets& bk, uint32_t ta, uint32_t dict, BitPlan& p) {
-  p.ta = ta;
-  for (int diff = 0; diff < kBuckets; ++diff) {
-    for (int L = diff; L < kBuckets; ++L) {
-      const int s = L - diff;
-      const uint32_t nL = bk.count[L], ns = bk.count[s];
-      if (!nL || !ns) continue;
-      if (diff == 0) {
-        for (uint32_t a = 0; a + 1 < nL; a += ta)
-          bit_add(p, bk, bk, {L, L, a, std::min(nL, a + ta), a, nL, true, dict});
-      } else if (bit_cost(ns, s, nL, L, ta) <= bit_cost(nL, L, ns, s, ta)) {
-        bit_add(p, bk, bk, {s, L, 0, ns, 0, nL, false, dict});
-      } else {
-        bit_add(p, bk, bk, {L, s, 0, nL, 0, ns, false, dict});
-      }
+// The bit-parallel launch of a pair list.  Rectangles of two lengths take the
+// cheaper of the two orientations: short words in the lanes pack more densely.
+void plan_bits(const Rects& rects, int m, int x, uint32_t alphabet, uint32_t ta, Plan& p) {
+  Launch l;
+  l.range = -1;
+  l.m = m;
+  l.x = x;
+  l.alphabet = alphabet;
+  l.ta = ta;
+  l.seg_first = (uint32_t)p.segs.size();
+  for (Rect r : rects) {
+    if (!r.tri && bit_cost(r.b1 - r.b0, r.LB, r.a1 - r.a0, r.La, ta) < bit_cost(r.a1 - r.a0, r.La, r.b1 - r.b0, r.LB, ta)) {
+      std::swap(r.A, r.B);
+      std::swap(r.La, r.LB);
+      std::swap(r.a0, r.b0);
+      std::swap(r.a1, r.b1);
+      std::swap(r.dict, r.dict_swapped);
     }
+    add_rect(p, l, r);
   }
-}
-
-// Every (query, dictionary word) pair, once: terms dict0 where the queries
-// are the A words, dict0 + 1 where they are the lanes' words.
-void bit_queries(const Buckets& qb, const Buckets& db, uint32_t ta, uint32_t dict0, BitPlan& p) {
-  p.ta = ta;
-  for (int diff = 0; diff < kBuckets; ++diff)
-    for (int lq = 0; lq < kBuckets; ++lq)
-      for (int sign = -1; sign <= 1; sign += 2) {
-        const int ld = lq + sign * diff;
-        if (ld < 0 || ld >= kBuckets || (diff == 0 && sign > 0)) continue;
-        const uint32_t nq = qb.count[lq], nd = db.count[ld];
-        if (!nq || !nd) continue;
-        if (bit_cost(nq, lq, nd, ld, ta) <= bit_cost(nd, ld, nq, lq, ta))
-          bit_add(p, qb, db, {lq, ld, 0, nq, 0, nd, false, dict0});
-        else
-          bit_add(p, db, qb, {ld, lq, 0, nd, 0, nq, false, dict0 + 1});
-      }
+  if (l.ntasks) p.launches.push_back(l);
 }
 
 // The chunk of A words per task: 256, halved down to 16 while the plan has
-// fewer tasks than kBitMinTasks (several per resident block of a full GPU).
-constexpr uint64_t kBitMinTasks = 12288;
-constexpr uint32_t kBitMinTA = 16;
+// fewer tasks than these (several per resident block of the bit-parallel
+// kernel, several per resident warp of the DPX kernel, on a full GPU).
+constexpr uint64_t kBitMinTasks = 12288, kDpMinTasks = 40960;
+constexpr uint32_t kMinTA = 16;
 template <class Make>
-void bit_plan_sized(BitPlan& p, Make make) {
+void sized(Plan& p, uint64_t min_tasks, Make make) {
   for (uint32_t ta = kDefaultTA;; ta /= 2) {
-    p = BitPlan{};
+    p = Plan{};
     make(ta, p);
-    if (p.ntasks >= kBitMinTasks || ta <= kBitMinTA) return;
+    uint64_t n = 0;
+    for (const Launch& l : p.launches) n += l.ntasks;
+    if (n >= min_tasks || ta <= kMinTA) return;
   }
 }
 
-// The pairs that shard `shard` of `nshards` of the DPX plan holds (each
-// launch's task list cut into contiguous ranges), as rectangles of the same
-// buckets.  Shards keep this partition whatever kernel scores them, so
-// shards saved by one build combine with another's.
-void bit_shard(const Buckets& bk, const Plan& plan, uint32_t shard, uint32_t nshards, uint32_t ta, BitPlan& p) {
-  p.ta = ta;
-  for (const LaunchPlan& lp : plan.launches) {
-    const uint64_t lo = lp.ntasks * shard / nshards, hi = lp.ntasks * (shard + 1) / nshards;
-    for (uint32_t x = 0; x < lp.nsegs; ++x) {
-      const Seg& S = plan.segs[lp.seg_first + x];
-      const uint32_t ncb = (uint32_t)cdiv(S.b_end - S.b_beg, kWarpB);
-      const uint64_t t0 = S.task0, t1 = S.task0 + (uint64_t)S.nca * ncb;
-      const uint64_t a = std::max(lo, t0), b = std::min(hi, t1);
-      if (a >= b) continue;
-      // tasks [a, b) of the segment: chunk coordinates (ca fastest)
-      auto rect = [&](uint32_t ca0, uint32_t ca1, uint32_t cb0, uint32_t cb1) {
-        if (ca0 >= ca1 || cb0 >= cb1) return;
-        const uint32_t nA = S.a_end - S.a_beg, nB = S.b_end - S.b_beg, ao = S.a_beg - bk.start[S.la],
-                       bo = S.b_beg - bk.start[lp.LB];
-        BitRect r{(int)S.la, lp.LB, ao + std::min(nA, ca0 * kDefaultTA), ao + std::min(nA, ca1 * kDefaultTA),
-                  bo + std::min(nB, cb0 * (uint32_t)kWarpB), bo + std::min(nB, cb1 * (uint32_t)kWarpB), S.tri != 0, 0u};
-        if (!r.tri && bit_cost(r.b1 - r.b0, r.LB, r.a1 - r.a0, r.La, ta) < bit_cost(r.a1 - r.a0, r.La, r.b1 - r.b0, r.LB, ta)) {
-          std::swap(r.La, r.LB);
-          std::swap(r.a0, r.b0);
-          std::swap(r.a1, r.b1);
-        }
-        bit_add(p, bk, bk, r);
-      };
-      const uint32_t l0 = (uint32_t)((a - t0) / S.nca), c0 = (uint32_t)((a - t0) % S.nca);
-      const uint32_t l1 = (uint32_t)((b - t0) / S.nca), c1 = (uint32_t)((b - t0) % S.nca);
-      if (l0 == l1) {
-        rect(c0, c1, l0, l0 + 1);
-      } else {
-        rect(c0, S.nca, l0, l0 + 1);
-        rect(0, S.nca, l0 + 1, l1);
-        rect(0, c1, l1, l1 + 1);
-      }
-    }
-  }
-}
-
-// Tasks a query launch should have at least (a few per warp of a full GPU)
-// before its A chunks are cut below the default size.
-constexpr uint64_t kQueryMinTasks = 8192;
-
-// Every (query, dictionary word) pair once; the longer word goes to the lanes.
-// A launch whose B words are few (long dictionary words, or a small query
-// set in the lanes) has few tasks at TA A words per task: with min_tasks > 0
-// its chunk is halved, down to 32 words, until it has min_tasks tasks, and
-// the launch records the chunk in its ta.
-void plan_query(const Buckets& qb, const Buckets& db, uint32_t TA, Plan& out, uint64_t min_tasks = 0) {
-  out = Plan{};
-  for (int role = 1; role <= 2; ++role) {
-    for (int LB = 0; LB < kBuckets; ++LB) {
-      LaunchPlan lp;
-      lp.LB = LB;
-      lp.role = role;
-      lp.seg_first = (uint32_t)out.segs.size();
-      uint64_t task = 0;
-      const Buckets& Bset = role == 1 ? db : qb;
-      const Buckets& Aset = role == 1 ? qb : db;
-      const uint32_t nB = Bset.count[LB];
-      if (nB == 0) continue;
-      // role 1: query length La <= LB (dictionary length); role 2: dictionary length La < LB (query length)
-      const int La_hi = role == 1 ? LB : LB - 1;
-      uint32_t ta = TA;
-      if (min_tasks) {
-        auto tasks_at = [&](uint32_t t) {
-          uint64_t x = 0;
-          for (int La = La_hi; La >= 0; --La) x += cdiv(Aset.count[La], t) * cdiv(nB, kWarpB);
-          return x;
-        };
-        while (ta > 32 && tasks_at(ta) < min_tasks) ta /= 2;
-        lp.ta = ta;
-      }
-      for (int La = La_hi; La >= 0; --La) {
-        const uint32_t nA = Aset.count[La];
-        if (nA == 0) continue;
-        uint64_t nt = 0;
-        out.segs.push_back(make_seg(Aset, La, Aset.start[La], Aset.start[La] + nA, Bset, LB, Bset.start[LB],
-                                    Bset.start[LB] + nB, false, ta, task, nt));
-        task += nt;
-        lp.pairs += (uint64_t)nA * nB;
-        lp.cells += (uint64_t)nA * nB * (uint64_t)(La * LB);
-      }
-      lp.nsegs = (uint32_t)out.segs.size() - lp.seg_first;
-      lp.ntasks = task;
-      if (lp.nsegs) {
-        out.pairs += lp.pairs;
-        out.cells += lp.cells;
-        out.launches.push_back(lp);
-      }
-    }
-  }
-  order_launches(out);
+// The launches of a pair list for scoring ss and an alphabet; ta = 0 sizes
+// the tasks.
+void make_plan(Rects rects, const ShiftedScoring& ss, uint32_t alphabet, uint32_t ta, Plan& p) {
+  order_rects(rects);
+  auto make = [&](uint32_t t, Plan& q) {
+    if (ss.bit_m) plan_bits(rects, ss.bit_m, ss.bit_x, alphabet, t, q);
+    else plan_dp(rects, t, q);
+  };
+  if (ta) make(ta, p);
+  else sized(p, ss.bit_m ? kBitMinTasks : kDpMinTasks, make);
+  count_rects(rects, p.pairs, p.cells);
 }
 
 uint32_t index_bits(uint32_t n) {
@@ -784,73 +729,79 @@ struct Timer {
   }
 };
 
+// error flag, insert count, task counters: one per DPX range or bit-parallel launch
+constexpr size_t kCounterBytes = 64 + sizeof(unsigned long long) * 16;
+
 struct RunOut {
   uint32_t dp_launches = 0;
-  uint64_t pairs = 0, cells = 0;
 };
 
-// Launches the alignment kernels of `plan` (shard `shard` of `nshards` of each
-// launch's tasks) on `stream`.  The A and B sides of a launch come from the
-// per-role tables: role 0 = one set against itself, 1 = queries (A) against the
-// dictionary (B), 2 = dictionary (A) against queries (B).
-nw_status run_plan(nw_ctx* c, cudaStream_t stream, const Plan& plan, const Seg* d_segs, const DpParams& base,
-                   unsigned long long* counters, uint32_t shard, uint32_t nshards, Timer& tm, RunOut& ro,
-                   const uint32_t* const a_enc_by_role[3], const SideView* const A_by_role[3],
-                   const uint4* const b_rec_by_role[3], const SideView* const B_by_role[3]) {
-  for (size_t li = 0; li < plan.launches.size(); ++li) {
-    const LaunchPlan& lp = plan.launches[li];
-    const uint64_t lo = lp.ntasks * shard / nshards, hi = lp.ntasks * (shard + 1) / nshards;
-    if (lo >= hi) continue;
-    DpParams P = base;
-    P.dbg_insert_limit = c->dbg_insert_iters >= 0 ? (uint32_t)c->dbg_insert_iters + 1u : 0u;
-    P.segs = d_segs + lp.seg_first;
-    P.nsegs = lp.nsegs;
-    if (lp.ta) P.TA = lp.ta;
-    P.serial_a = lp.role == 1 ? 1u : 0u;  // query words are the A side
-    P.task_lo = lo;
-    P.task_hi = hi;
-    P.counter = counters + li;
-    P.a_enc = a_enc_by_role[lp.role];
-    P.A = *A_by_role[lp.role];
-    P.b_rec = b_rec_by_role[lp.role];
-    P.B = *B_by_role[lp.role];
-    const bool tab = P.sim_tab != nullptr;
-    const size_t smem = hist_smem_bytes(P.hist_mode, P.nbins) + dp_stage_bytes(lp.LB) + (tab ? kTabBytes : 0);
-    const int epi = P.terms ? kEpiBatchLists
-                            : (P.mode == kModeMatrix ? kEpiMatrix
-                                                     : (P.hist_mode == kHistLane ? kEpiListsLaneHist : kEpiLists));
-    const void* fn = dp_kernel(lp.LB, epi, tab);
-    if (!fn) return set_err(c, NW_EINVAL, "no kernel for length %d", lp.LB);
-    NW_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int occ = 0;
-    NW_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBlock, smem));
-    if (occ < 1) occ = 1;
-    if (lp.bps && occ > (int)lp.bps) occ = (int)lp.bps;
-    uint64_t grid = (uint64_t)c->sm_count * occ;
-    grid = std::min<uint64_t>(grid, cdiv(hi - lo, kWarpsPerBlock));
-    void* args[] = {&P};
-    cudaEvent_t e0 = nullptr;
-    tm.begin(true, e0);
-    NW_CK(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kBlock), args, smem, stream));
-    tm.end(true, e0);
-    ++ro.dp_launches;
-    ro.pairs += lp.pairs;  // whole-launch figures; exact for nshards == 1
-    ro.cells += lp.cells;
+// Launches one alignment launch of a plan on `stream`; `P` brings the terms,
+// the epilogue's settings and the counter.
+nw_status run_launch(nw_ctx* c, cudaStream_t stream, const Launch& l, const Seg* d_segs, int epi, AlignParams P,
+                     Timer& tm, RunOut& ro) {
+  const bool bits = l.range < 0;
+  const int warps = bits ? kBitWarps : kWarpsPerBlock;
+  P.segs = d_segs + l.seg_first;
+  P.nsegs = l.nsegs;
+  P.TA = l.ta;
+  P.ntasks = l.ntasks;
+  P.dbg_insert_limit = c->dbg_insert_iters >= 0 ? (uint32_t)c->dbg_insert_iters + 1u : 0u;
+  const bool tab = !bits && P.sim_tab != nullptr;
+  size_t smem = (epi == kEpiListsLaneHist || epi == kEpiLists ? hist_smem_words(P.hist_mode, P.nbins, warps) : 0) *
+                sizeof(uint32_t);
+  if (bits) {
+    P.sub = std::max<uint32_t>(1, std::min<uint32_t>(kBitSub, l.ta / kBitWarps));
+    P.mask_bytes = l.alphabet * kMaskRow;
+    P.stage_syms = (P.sub * l.max_la + 2 + 7) & ~7u;
+    smem += P.mask_bytes + (size_t)warps * P.stage_syms * sizeof(uint16_t);
+  } else {
+    P.stage_syms = 32u * std::max<uint32_t>(1, l.max_la);
+    smem += (size_t)warps * P.stage_syms * sizeof(uint32_t) + (tab ? kTabBytes : 0);
+  }
+  const void* fn = bits ? bit_kernel(l.m, l.x, epi) : dp_kernel(l.range, epi, tab);
+  if (!fn) return set_err(c, NW_EINVAL, "no alignment kernel for this launch");
+  const int block = bits ? kBitBlock : kBlock;
+  NW_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int occ = 0;
+  NW_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem));
+  if (occ < 1) occ = 1;
+  if (l.bps && occ > (int)l.bps) occ = (int)l.bps;
+  const uint64_t grid = std::min<uint64_t>((uint64_t)c->sm_count * occ, bits ? l.ntasks : cdiv(l.ntasks, kWarpsPerBlock));
+  void* args[] = {&P};
+  cudaEvent_t e0 = nullptr;
+  tm.begin(true, e0);
+  NW_CK(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), args, smem, stream));
+  tm.end(true, e0);
+  ++ro.dp_launches;
+  return NW_OK;
+}
+
+// All launches of a plan, in order; launch i takes counters[i].
+nw_status run_plan(nw_ctx* c, cudaStream_t stream, const Plan& plan, const Seg* d_segs, int epi, const AlignParams& base,
+                   unsigned long long* counters, Timer& tm, RunOut& ro) {
+  for (size_t i = 0; i < plan.launches.size(); ++i) {
+    AlignParams P = base;
+    P.counter = counters + i;
+    NW_TRY(run_launch(c, stream, plan.launches[i], d_segs, epi, P, tm, ro));
   }
   return NW_OK;
 }
 
-// One side of a bit-parallel launch's terms: scoring and key layout of `d`.
-BitTerms bit_terms(const nw_dict* d, const WordSet& a, const WordSet& b, SideView A, SideView B, int32_t key_lo,
-                   uint32_t ib) {
-  BitTerms T{};
+// Terms of dictionary `d`'s scoring between an A set and a B set.
+Terms make_terms(const nw_dict* d, const WordSet& a, const WordSet& b, SideView A, SideView B, int32_t key_lo,
+                 uint32_t ib) {
+  Terms T{};
   T.a_sym = a.a_enc.as<uint32_t>();
   T.b_sym = b.a_enc.as<uint32_t>();
+  T.b_rec = b.b_rec.as<uint4>();
   T.A = A;
   T.B = B;
   T.shift = d->ss.shift;
   T.alphabet = d->alphabet;
   T.coef = (uint32_t)d->ss.bit_coef;
+  T.C1 = d->ss.C1;
+  T.C2 = d->ss.C2;
   T.match = d->sc.match;
   T.mismatch = d->sc.mismatch;
   T.gap = d->sc.gap;
@@ -860,91 +811,24 @@ BitTerms bit_terms(const nw_dict* d, const WordSet& a, const WordSet& b, SideVie
   return T;
 }
 
-// Launches the bit-parallel kernel of steps (m, x) over a plan.  `P` brings
-// the terms, epilogue settings and counter; `alphabet` is the largest of the
-// launch's sets.
-nw_status run_bits(nw_ctx* c, cudaStream_t stream, int m, int x, int epi, uint32_t alphabet, const BitPlan& plan,
-                   const Seg* d_segs, BitParams P, Timer& tm, RunOut& ro, uint32_t bps = 0) {
-  if (plan.ntasks == 0) return NW_OK;
-  P.segs = d_segs;
-  P.nsegs = (uint32_t)plan.segs.size();
-  P.TA = plan.ta;
-  P.ntasks = plan.ntasks;
-  P.sub = std::max<uint32_t>(1, std::min<uint32_t>(kBitSub, plan.ta / kBitWarps));
-  P.mask_bytes = alphabet * kMaskRow;
-  P.stage_syms = (P.sub * plan.max_la + 2 + 7) & ~7u;
-  P.dbg_insert_limit = c->dbg_insert_iters >= 0 ? (uint32_t)c->dbg_insert_iters + 1u : 0u;
-  const void* fn = bit_kernel(m, x, epi);
-  if (!fn) return set_err(c, NW_EINVAL, "no kernel for steps (%d, %d)", m, x);
-  const size_t hist_words = epi == kEpiListsLaneHist                                ? (size_t)P.nbins * 32
-                            : epi == kEpiLists && P.hist_mode == kHistSmem ? (size_t)P.nbins * kBitWarps
-                                                                                    : 0;
-  const size_t smem = P.mask_bytes + hist_words * sizeof(uint32_t) + (size_t)kBitWarps * P.stage_syms * sizeof(uint16_t);
-  NW_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int occ = 0;
-  NW_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBitBlock, smem));
-  if (occ < 1) occ = 1;
-  if (bps && occ > (int)bps) occ = (int)bps;
-  const uint64_t grid = std::min<uint64_t>((uint64_t)c->sm_count * occ, plan.ntasks);
-  void* args[] = {&P};
-  cudaEvent_t e0 = nullptr;
-  tm.begin(true, e0);
-  NW_CK(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kBitBlock), args, smem, stream));
-  tm.end(true, e0);
-  ++ro.dp_launches;
-  return NW_OK;
-}
+int lists_epi(int hist_mode) { return hist_mode == kHistLane ? kEpiListsLaneHist : kEpiLists; }
 
-// The settings of a DPX launch that the bit-parallel kernel shares.
-BitParams bit_params(const DpParams& b, unsigned long long* counter) {
-  BitParams P{};
-  P.counter = counter;
-  P.mat = b.mat;
-  P.n = b.n;
-  P.mat_lo = b.mat_lo;
-  P.mat_hi = b.mat_hi;
-  P.k = b.k;
-  P.hist_mode = b.hist_mode;
-  P.hist = b.hist;
-  P.hist_lo = b.hist_lo;
-  P.nbins = b.nbins;
-  P.stats = b.stats;
-  P.err = b.err;
-  P.norm_rank = b.norm_rank;
-  P.norm_smin = b.norm_smin;
-  P.norm_lo = b.norm_lo;
-  return P;
-}
-
-int epi_for(int mode, int hist_mode) {
-  return mode == kModeMatrix ? kEpiMatrix : (hist_mode == kHistLane ? kEpiListsLaneHist : kEpiLists);
-}
-
-// The whole pair set of a dictionary (or one shard of it, through the
-// context's segment workspace) by whichever kernel its scoring takes.
-nw_status run_dict(nw_dict* d, const DpParams& base, SideView side, unsigned long long* counters, uint32_t shard,
+// The whole pair set of a dictionary, or one shard of it (planned on the spot
+// through the context's segment workspace).
+nw_status run_dict(nw_dict* d, int epi, const AlignParams& base, unsigned long long* counters, uint32_t shard,
                    uint32_t nshards, Timer& tm, RunOut& ro) {
   nw_ctx* c = d->ctx;
-  if (d->ss.bit_m == 0) {
-    const uint32_t* a_enc[3] = {d->ws.a_enc.as<uint32_t>(), nullptr, nullptr};
-    const uint4* b_rec[3] = {d->ws.b_rec.as<uint4>(), nullptr, nullptr};
-    const SideView* views[3] = {&side, nullptr, nullptr};
-    return run_plan(c, c->stream, d->plan, d->d_segs.as<Seg>(), base, counters, shard, nshards, tm, ro, a_enc, views,
-                    b_rec, views);
-  }
-  BitParams P = bit_params(base, counters);
-  P.local[0] = bit_terms(d, d->ws, d->ws, side, side, base.key_lo, base.ib);
-  const int epi = epi_for(base.mode, base.hist_mode);
-  if (nshards == 1)
-    return run_bits(c, c->stream, d->ss.bit_m, d->ss.bit_x, epi, d->alphabet, d->bits, d->d_segs.as<Seg>(), P, tm, ro);
-  BitPlan bp;
-  bit_plan_sized(bp, [&](uint32_t ta, BitPlan& p) { bit_shard(d->ws.bk, d->plan, shard, nshards, ta, p); });
-  NW_TRY(ctx_ensure(c, c->ws_segs, sizeof(Seg) * std::max<size_t>(1, bp.segs.size()), "shard segments"));
-  if (!bp.segs.empty()) {
-    NW_CK(cudaMemcpyAsync(c->ws_segs.p, bp.segs.data(), sizeof(Seg) * bp.segs.size(), cudaMemcpyHostToDevice, c->stream));
+  if (nshards == 1) return run_plan(c, c->stream, d->plan, d->d_segs.as<Seg>(), epi, base, counters, tm, ro);
+  Rects rects;
+  rects_shard(d->ws.bk, shard, nshards, rects);
+  Plan plan;
+  make_plan(std::move(rects), d->ss, d->alphabet, 0, plan);
+  NW_TRY(ctx_ensure(c, c->ws_segs, sizeof(Seg) * std::max<size_t>(1, plan.segs.size()), "shard segments"));
+  if (!plan.segs.empty()) {
+    NW_CK(cudaMemcpyAsync(c->ws_segs.p, plan.segs.data(), sizeof(Seg) * plan.segs.size(), cudaMemcpyHostToDevice, c->stream));
     NW_CK(cudaStreamSynchronize(c->stream));  // the host list goes out of scope
   }
-  return run_bits(c, c->stream, d->ss.bit_m, d->ss.bit_x, epi, d->alphabet, bp, c->ws_segs.as<Seg>(), P, tm, ro);
+  return run_plan(c, c->stream, plan, c->ws_segs.as<Seg>(), epi, base, counters, tm, ro);
 }
 
 nw_status check_device_flags(nw_ctx* c, const uint32_t* d_small) {
@@ -990,11 +874,9 @@ nw_status topk_impl(nw_dict* d, uint32_t shard, uint32_t nshards, uint32_t k, ui
   }
   const bool dev = flags & NW_DEVICE_PTRS;
   cudaStream_t s = c->stream;
-  const size_t nlaunch = d->plan.launches.size();
-
   NW_TRY(ctx_ensure(c, c->ws_slots, sizeof(uint32_t) * (size_t)n * k, "list slots"));
   NW_TRY(ctx_ensure(c, c->ws_thr, sizeof(uint32_t) * (size_t)n, "list thresholds"));
-  NW_TRY(ctx_ensure(c, c->ws_small, 64 + sizeof(unsigned long long) * (nlaunch + 1), "task counters"));
+  NW_TRY(ctx_ensure(c, c->ws_small, kCounterBytes, "task counters"));
   if (hist) NW_TRY(ctx_ensure(c, c->ws_hist, sizeof(unsigned long long) * need_bins, "histogram"));
   uint32_t* out_idx = nbr_idx;
   int16_t* out_score = nbr_score;
@@ -1016,19 +898,9 @@ nw_status topk_impl(nw_dict* d, uint32_t shard, uint32_t nshards, uint32_t k, ui
   NW_CK(cudaMemsetAsync(c->ws_thr.p, 0, sizeof(uint32_t) * (size_t)n, s));
   if (hist) NW_CK(cudaMemsetAsync(c->ws_hist.p, 0, sizeof(unsigned long long) * need_bins, s));
 
-  DpParams base{};
-  base.TA = kDefaultTA;
-  base.C1 = d->ss.C1;
-  base.C2 = d->ss.C2;
-  base.match = d->sc.match;
-  base.mismatch = d->sc.mismatch;
-  base.gap = d->sc.gap;
+  AlignParams base{};
   base.sim_tab = dict_tab(d);
-  base.mode = kModeLists;
   base.k = k;
-  base.ib = ib;
-  base.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
-  base.key_lo = key_lo;
   base.hist_mode = !hist ? kHistNone : hist_mode_for(need_bins);
   base.hist = hist ? c->ws_hist.as<unsigned long long>() : nullptr;
   base.hist_lo = d->score_lo;
@@ -1054,11 +926,12 @@ nw_status topk_impl(nw_dict* d, uint32_t shard, uint32_t nshards, uint32_t k, ui
     d_frac = reinterpret_cast<const int16_t*>(c->ws_norm.as<char>() + o_frac);
   }
   SideView side{d->ws.perm.as<uint32_t>(), c->ws_slots.as<uint32_t>(), c->ws_thr.as<uint32_t>()};
+  base.local[0] = make_terms(d, d->ws, d->ws, side, side, key_lo, ib);
   RunOut ro;
-  NW_TRY(run_dict(d, base, side, d_counters, shard, nshards, tm, ro));
+  NW_TRY(run_dict(d, lists_epi(base.hist_mode), base, d_counters, shard, nshards, tm, ro));
   cudaEvent_t e_fin = nullptr;
   tm.begin(false, e_fin);
-  NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), n, k, d->ws.perm.as<uint32_t>(), ib, base.imask, key_lo,
+  NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), n, k, d->ws.perm.as<uint32_t>(), ib, base.local[0].imask, key_lo,
                         out_idx, out_score, s, d_frac, d->ws.slen.as<uint8_t>(), d->ws.rank.as<uint32_t>()));
   tm.end(false, e_fin);
   if (hist && dev) NW_CK(cudaMemcpyAsync(hist, c->ws_hist.p, sizeof(int64_t) * need_bins, cudaMemcpyDeviceToDevice, s));

@@ -56,20 +56,20 @@ struct Buckets {
 };
 
 // A rectangle of pairs: A positions [a_beg, a_end) x B positions [b_beg, b_end),
-// all A words of length la and all B words of the launch's length LB.  With tri,
+// all A words of length la and all B words of length lb.  With tri,
 // A and B are the same bucket of the same set and only pairs a < b are scored.
 struct Seg {
   uint32_t a_beg, a_end;
   uint32_t b_beg, b_end;
   uint32_t aenc_base;   // a_enc index of word a_beg's first symbol
-  uint32_t brec_base;   // uint4 index into b_rec of the record holding b_beg
-                        // (b_beg - bucket start is even; records of bucket LB are ceil4(LB)/4 uint4 apart)
+  uint32_t b_base;      // DPX launches: uint4 index into b_rec of the record holding b_beg
+                        // (b_beg - bucket start is even; records of bucket LB are ceil4(LB)/4 uint4 apart);
+                        // bit-parallel launches: index of b_beg's first symbol in the B set's symbols
   uint16_t la;
   uint16_t tri;
-  uint32_t nca;         // A chunks (tasks = nca * ceil((b_end - b_beg) / kWarpB))
-  uint32_t dict;        // terms of the segment in a batched launch (else 0)
-  uint32_t lb;          // bit-parallel launches: the B words' length (brec_base is then the
-                        // index of b_beg's first symbol in the B set's symbols)
+  uint32_t nca;         // A chunks (tasks = nca * ceil((b_end - b_beg) / chunk))
+  uint32_t dict;        // index of the segment's terms
+  uint32_t lb;          // the B words' length
   uint64_t task0;       // first task of the segment within its launch
 };
 
@@ -80,18 +80,22 @@ struct SideView {
   uint32_t* thr;          // per-word lower bound of the k-th best key, or null
 };
 
-// Terms of one kind of segment in a batched launch (indexed by Seg::dict):
-// the A and B word sets with their lists and the scoring constants.  A
+// Word sets, lists and scoring of one kind of segment, named by Seg::dict: the
+// A and B word sets with their lists and the scoring constants.  A
 // dictionary's own pairs take A = B = the dictionary with its lists; a query
 // set against a dictionary takes the query words on one side (with the
 // queries' lists) and the dictionary on the other (no lists).
-struct DictTerms {
-  const uint32_t* a_enc;
-  const uint4* b_rec;
+struct Terms {
+  const uint32_t* a_sym;  // a_enc of the A side's set
+  const uint32_t* b_sym;  // a_enc of the B side's set (bit-parallel kernel)
+  const uint4* b_rec;     // pair records of the B side's set (DPX kernel)
   SideView A, B;
-  uint32_t C1, C2;
+  uint32_t shift;         // code shift of the symbols
+  uint32_t alphabet;
+  uint32_t coef;          // bit-parallel kernel: gcd of the steps, G = coef * (sum of the reduced steps)
+  uint32_t C1, C2;        // DPX kernel: packed (s'_m + 1) and max(s'_x, 0)
   int32_t match, mismatch, gap;
-  int32_t key_lo;
+  int32_t key_lo;         // list key = ((s - key_lo) << ib) | (imask - partner)
   uint32_t ib, imask;
 };
 
@@ -181,72 +185,45 @@ enum { kHistNone = 0, kHistSmem = 1, kHistGlobal = 2, kHistLane = 3 };
 // shrinks with LB (the lane keeps LB registers of B symbols and LB of DP row).
 __host__ __device__ constexpr int dp_min_blocks(int LB) { return LB <= 10 ? 4 : (LB <= 20 ? 3 : 2); }
 
-// Shared memory each block of the LB kernel stages A words in: every warp
-// holds 32 words of at most LB symbols and their 32 list bounds (after the
-// histogram area).
-__host__ __device__ constexpr size_t dp_stage_bytes(int LB) {
-  return (size_t)kWarpsPerBlock * 32u * (size_t)(LB + 1) * sizeof(uint32_t);
-}
+// The DPX kernel is instantiated for four ranges of the longer length, each a
+// launch of its own register budget: lengths dp_range_lo(r) .. dp_range_hi(r).
+constexpr int kDpRanges = 4;
+__host__ __device__ constexpr int dp_range_hi(int r) { return 10 * (r + 1); }
+__host__ __device__ constexpr int dp_range_lo(int r) { return r == 0 ? 0 : 10 * r + 1; }
+__host__ __device__ constexpr int dp_range_of(int LB) { return LB <= 10 ? 0 : (LB - 1) / 10; }
+static_assert(dp_range_of(kMaxLen) == kDpRanges - 1, "every length has a range");
+
+// What the warps of a block that work on one task share (the bit-parallel
+// kernel's block, or one warp of the DPX kernel).
+struct AlignTask {
+  TaskGeom g;
+  int K;                  // bit-parallel kernel: words per lane
+  int la, lb, mx;         // mx: the longer of the two
+  uint32_t a_base;        // index of A word g.a0's first symbol in a_sym
+  uint32_t b_base;        // bit-parallel: index of B word g.b0's first symbol in b_sym; DPX: its record in b_rec
+  bool check;             // same bucket, chunks overlap: test a < b
+};
+
+// Candidate queue of a warp (see file_candidates): entries waiting, up to 31
+// plus a warp's 32.
+constexpr uint32_t kQueueEntries = 64;
 
 // per-pair epilogue of the all-pairs kernel (a template parameter);
-// kEpiBatchLists takes word sets, lists and scoring per task from DpParams::terms
+// kEpiBatchLists reads the terms of a segment from AlignParams::terms
 enum { kEpiMatrix = 0, kEpiLists = 1, kEpiListsLaneHist = 2, kEpiBatchLists = 3, kEpiKinds = 4 };
 
-// Histogram accumulation mode for `nbins` bins and the dynamic shared memory
-// it needs per block: per-lane columns while they fit in 48 KiB, else one
-// shared array per warp, else global atomics.
+// Histogram accumulation mode for `nbins` bins: per-lane columns shared by a
+// block while they fit in 48 KiB (384 bins), else one shared array per warp,
+// else global atomics.
 inline int hist_mode_for(uint32_t nbins) {
-  if ((size_t)nbins * 32u * sizeof(uint32_t) * kWarpsPerBlock <= 48u * 1024u) return kHistLane;
+  if ((size_t)nbins * 32u * sizeof(uint32_t) <= 48u * 1024u) return kHistLane;
   if (nbins <= kHistSmemMaxBins) return kHistSmem;
   return kHistGlobal;
 }
-inline size_t hist_smem_bytes(int mode, uint32_t nbins) {
-  if (mode == kHistLane) return (size_t)kWarpsPerBlock * nbins * 32u * sizeof(uint32_t);
-  if (mode == kHistSmem) return (size_t)kWarpsPerBlock * nbins * sizeof(uint32_t);
-  return 0;
+// shared words of the histogram in a block of `warps` warps
+inline size_t hist_smem_words(int mode, uint32_t nbins, int warps) {
+  return mode == kHistLane ? (size_t)nbins * 32u : (mode == kHistSmem ? (size_t)nbins * warps : 0);
 }
-
-struct DpParams {
-  const Seg* segs;
-  uint32_t nsegs;
-  uint32_t TA;
-  uint64_t task_lo, task_hi;      // task slice handled by this launch
-  unsigned long long* counter;    // zeroed before the launch
-  const uint32_t* a_enc;          // A set
-  const uint4* b_rec;             // B set
-  SideView A, B;
-  uint32_t C1, C2;                // packed (s'_m + 1) and max(s'_x, 0), see the kernel
-  int32_t match, mismatch, gap;
-  int32_t mode;
-  int8_t* mat;                    // matrix mode: row-major upper triangle, entries [mat_lo, mat_hi) stored
-  uint64_t n;
-  uint64_t mat_lo, mat_hi;        // (mat points at the buffer holding entry mat_lo, minus mat_lo)
-  uint32_t k, ib, imask;          // list key = ((s - key_lo) << ib) | (imask - partner)
-  int32_t key_lo;
-  int32_t hist_mode;
-  unsigned long long* hist;
-  int32_t hist_lo;
-  uint32_t nbins;
-  unsigned long long* stats;      // [0] list inserts
-  uint32_t* err;
-  const DictTerms* terms;         // batched launches: per-dictionary terms (device), else null
-  // length-normalised ranking (null = raw scores): rank of s / max(la, lb) at
-  // norm_rank[(s - norm_lo) * kBuckets + m], and the smallest s reaching rank r
-  // for longer length m at norm_smin[r * kBuckets + m]
-  const uint16_t* norm_rank;
-  const int16_t* norm_smin;
-  int32_t norm_lo;
-  // substitution-matrix scoring (null = match / mismatch): kTabDim x kTabDim
-  // table of s'+(a, b) = max(sim(a, b) - 2p, 0), copied to shared memory
-  const uint16_t* sim_tab;
-  // debug setting: 0 = list insertions retry up to kInsertMaxIters times;
-  // otherwise they give up after dbg_insert_limit - 1 tries (NW_ETIMEOUT)
-  uint32_t dbg_insert_limit;
-  // nonzero: the A words' list offers of one A word go through the warp one at
-  // a time (A words that many tasks share, such as query words, whose lists
-  // the 64 lanes of a task would otherwise race on)
-  uint32_t serial_a;
-};
 
 // The substitution table of a dictionary scored with a full similarity
 // matrix: row a holds s'+(a, b) for b < kTabDim (zero past the alphabet).  A
@@ -282,42 +259,38 @@ __host__ __device__ constexpr int bit_pitch(int K) {
   return K == 8 ? 8 : K == 7 ? 9 : K == 6 ? 10 : K == 5 ? 12 : K == 4 ? 16 : K == 3 ? 21 : K == 2 ? 32 : 64;
 }
 
-// Word sets, lists and scoring of one kind of segment (indexed by Seg::dict).
-struct BitTerms {
-  const uint32_t* a_sym;  // a_enc of the A side's set
-  const uint32_t* b_sym;  // a_enc of the B side's set
-  SideView A, B;
-  uint32_t shift;         // code shift of the symbols
-  uint32_t alphabet;
-  uint32_t coef;          // gcd of the steps: G = coef * (sum of the reduced steps)
-  int32_t match, mismatch, gap, key_lo;
-  uint32_t ib, imask;
-};
-
-struct BitParams {
+struct AlignParams {
   const Seg* segs;
   uint32_t nsegs;
-  uint32_t TA;
+  uint32_t TA;                    // A words per task (at most 256)
   uint64_t ntasks;
   unsigned long long* counter;    // zeroed before the launch
-  BitTerms local[2];              // terms of segments 0 and 1 (single-dictionary launches)
-  const BitTerms* terms;          // batched launches: terms by segment (device)
-  uint32_t sub;                   // A words a warp takes at a time (1 .. kBitSub)
-  uint32_t mask_bytes;            // shared memory of the match masks
-  uint32_t stage_syms;            // symbols a warp has room to stage
-  int8_t* mat;                    // as in DpParams from here on
+  Terms local[2];                 // terms 0 and 1 of a single dictionary's launch
+  const Terms* terms;             // batched launches: terms by segment (device)
+  // shared memory: A words a warp stages at a time, room for their symbols,
+  // bit-parallel: bytes of the match masks
+  uint32_t sub, stage_syms, mask_bytes;
+  int8_t* mat;                    // matrix mode: row-major upper triangle, entries [mat_lo, mat_hi) stored
   uint64_t n;
-  uint64_t mat_lo, mat_hi;
+  uint64_t mat_lo, mat_hi;        // (mat points at the buffer holding entry mat_lo, minus mat_lo)
   uint32_t k;
   int32_t hist_mode;
   unsigned long long* hist;
   int32_t hist_lo;
   uint32_t nbins;
-  unsigned long long* stats;
+  unsigned long long* stats;      // [0] list inserts
   uint32_t* err;
+  // length-normalised ranking (null = raw scores): rank of s / max(la, lb) at
+  // norm_rank[(s - norm_lo) * kBuckets + m], and the smallest s reaching rank r
+  // for longer length m at norm_smin[r * kBuckets + m]
   const uint16_t* norm_rank;
   const int16_t* norm_smin;
   int32_t norm_lo;
+  // substitution-matrix scoring (null = match / mismatch): kTabDim x kTabDim
+  // table of s'+(a, b) = max(sim(a, b) - 2p, 0), copied to shared memory
+  const uint16_t* sim_tab;
+  // debug setting: 0 = list insertions retry up to kInsertMaxIters times;
+  // otherwise they give up after dbg_insert_limit - 1 tries (NW_ETIMEOUT)
   uint32_t dbg_insert_limit;
 };
 

@@ -8,9 +8,9 @@
 
 namespace nw {
 
-// alignment kernel for the longer length LB (0 .. kMaxLen), epilogue kind and
-// scoring (tab: substitution table); nullptr if there is none
-const void* dp_kernel(int LB, int epi, bool tab = false);
+// DPX alignment kernel for a range of longer lengths (dp_range_of), epilogue
+// kind and scoring (tab: substitution table); nullptr if there is none
+const void* dp_kernel(int range, int epi, bool tab = false);
 
 // bit-parallel alignment kernel for the reduced steps (m, x) and epilogue
 // kind; nullptr if there is none (kernels exist for gcd(m, x) = 1, x < m <=

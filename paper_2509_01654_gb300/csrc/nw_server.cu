@@ -77,7 +77,7 @@ struct Slot {
   Plan plan;
 };
 
-constexpr size_t kMaxSegs = 2u * kBuckets * kBuckets;  // plan_query makes at most one rectangle per (role, La, LB)
+constexpr size_t kMaxSegs = 2u * kBuckets * kBuckets;  // a plan has at most one segment per (query length, word length)
 
 // One batch in flight through the proposal: a private context, the model's
 // parameters copied into it, a non-owning view of the dictionary, and the
@@ -149,7 +149,7 @@ nw_status alloc_slot(nw_server* S, Slot& s) {
   NW_TRY(ctx_alloc(c, s.d_b_rec, sizeof(uint32_t) * brec_capacity_words(Q), "batch B records"));
   NW_TRY(ctx_alloc(c, s.d_slots, sizeof(uint32_t) * (size_t)Q * k, "batch list slots"));
   NW_TRY(ctx_alloc(c, s.d_thr, sizeof(uint32_t) * Q, "batch list bounds"));
-  NW_TRY(ctx_alloc(c, s.d_small, 64 + sizeof(unsigned long long) * (2 * kBuckets + 2), "batch counters"));
+  NW_TRY(ctx_alloc(c, s.d_small, kCounterBytes, "batch counters"));
   NW_TRY(ctx_alloc(c, s.d_segs, sizeof(Seg) * kMaxSegs, "batch segments"));
   NW_TRY(ctx_alloc(c, s.d_idx, sizeof(uint32_t) * (size_t)Q * k, "batch result indices"));
   NW_TRY(ctx_alloc(c, s.d_score, sizeof(int16_t) * (size_t)Q * k, "batch result scores"));
@@ -224,7 +224,10 @@ nw_status launch_batch(nw_server* S, Slot& s) {
   const int32_t key_lo = lo - 1;
   if ((uint64_t)(hi - key_lo) >= (1ull << (32 - ib)))
     return set_err(c, NW_ERANGE, "score range with %u dictionary words does not fit 32-bit list keys", d->ws.n);
-  plan_query(bk, d->ws.bk, kDefaultTA, s.plan, kQueryMinTasks);
+  Rects rects;
+  rects_queries(bk, d->ws.bk, 0, rects);
+  s.plan = Plan{};
+  make_plan(std::move(rects), d->ss, d->alphabet, 0, s.plan);
   if (s.plan.segs.size() > kMaxSegs) return set_err(c, NW_ERANGE, "batch plan too large");
   std::memcpy(s.h_segs, s.plan.segs.data(), sizeof(Seg) * s.plan.segs.size());
 
@@ -242,33 +245,23 @@ nw_status launch_batch(nw_server* S, Slot& s) {
   NW_CK(cudaMemsetAsync(s.d_slots.p, 0, sizeof(uint32_t) * (size_t)nq * k, st));
   NW_CK(cudaMemsetAsync(s.d_thr.p, 0, sizeof(uint32_t) * nq, st));
 
-  DpParams base{};
-  base.TA = kDefaultTA;
-  base.C1 = d->ss.C1;
-  base.C2 = d->ss.C2;
-  base.match = d->sc.match;
-  base.mismatch = d->sc.mismatch;
-  base.gap = d->sc.gap;
-  base.mode = kModeLists;
+  AlignParams base{};
   base.k = k;
-  base.ib = ib;
-  base.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
-  base.key_lo = key_lo;
   base.hist_mode = kHistNone;
   base.stats = reinterpret_cast<unsigned long long*>(s.d_small.as<char>() + 8);
   base.err = s.d_small.as<uint32_t>();
   SideView qside{s.d_perm.as<uint32_t>(), s.d_slots.as<uint32_t>(), s.d_thr.as<uint32_t>()};
   SideView dside{d->ws.perm.as<uint32_t>(), nullptr, nullptr};
-  const uint32_t* a_enc[3] = {nullptr, s.d_a_enc.as<uint32_t>(), d->ws.a_enc.as<uint32_t>()};
-  const uint4* b_rec[3] = {nullptr, d->ws.b_rec.as<uint4>(), s.d_b_rec.as<uint4>()};
-  const SideView* A_views[3] = {nullptr, &qside, &dside};
-  const SideView* B_views[3] = {nullptr, &dside, &qside};
+  WordSet q;  // the slot's buffers as a word set (nothing is owned here)
+  q.a_enc = s.d_a_enc;
+  q.b_rec = s.d_b_rec;
+  base.local[0] = make_terms(d, q, d->ws, qside, dside, key_lo, ib);
+  base.local[1] = make_terms(d, d->ws, q, dside, qside, key_lo, ib);
   Timer tm{c};
   RunOut ro;
-  NW_TRY(run_plan(c, st, s.plan, s.d_segs.as<Seg>(), base,
-                  reinterpret_cast<unsigned long long*>(s.d_small.as<char>() + 64), 0, 1, tm, ro, a_enc, A_views,
-                  b_rec, B_views));
-  NW_CK(launch_finalize(s.d_slots.as<uint32_t>(), nq, k, s.d_perm.as<uint32_t>(), ib, base.imask, key_lo,
+  NW_TRY(run_plan(c, st, s.plan, s.d_segs.as<Seg>(), kEpiLists, base,
+                  reinterpret_cast<unsigned long long*>(s.d_small.as<char>() + 64), tm, ro));
+  NW_CK(launch_finalize(s.d_slots.as<uint32_t>(), nq, k, s.d_perm.as<uint32_t>(), ib, base.local[0].imask, key_lo,
                         s.d_idx.as<uint32_t>(), s.d_score.as<int16_t>(), st));
   NW_CK(cudaMemcpyAsync(s.h_idx, s.d_idx.p, sizeof(uint32_t) * (size_t)nq * k, cudaMemcpyDeviceToHost, st));
   NW_CK(cudaMemcpyAsync(s.h_score, s.d_score.p, sizeof(int16_t) * (size_t)nq * k, cudaMemcpyDeviceToHost, st));
