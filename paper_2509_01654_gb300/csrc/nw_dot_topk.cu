@@ -371,6 +371,9 @@ struct DotArgs {
   // entries) and names the columns in the keys; row_ids places the output rows
   const uint32_t* col_ids;
   const uint32_t* row_ids;
+  // nullptr, or a word that has to be non-zero for the launch to run (without
+  // splits: for the CTA to run, together with its block's flag)
+  const uint32_t* gate;
   bool sorted;  // lists in descending key order (else in any order)
   uint32_t* out_idx;
   int32_t* out_val;
@@ -459,6 +462,443 @@ __device__ int compact_buffer(uint64_t* keys, int c, const uint64_t* other, int 
   return kept;
 }
 
+// ---- two-sweep path of the square product.  Most of the candidate kernel's
+// time at 100k rows went into values that reach a threshold still far below
+// the row's final C-th best: ~2,000 appends a row, their compactions, and the
+// epilogue threads waiting for them.  Two sweeps over the columns avoid that:
+//
+//   * kSweepMax keeps, per row, only the largest value of each group of
+//     columns.  The (C + 1)-th largest of a row's group maxima (row_bound_kernel)
+//     is reached by at least C other columns, one in each of C groups (the row
+//     itself can be the largest of one group), so it is at most the row's C-th
+//     best value: an exact lower bound.  With 3 C to 6 C groups and no relation
+//     between a column's position and its value, only 1.1 C to 1.25 C columns
+//     reach it.  This sweep takes the columns in the caller's own order, not
+//     the locality order: there a row's best columns would share a few groups.
+//     Ties: ranked by (maximum, lower position first), the (C + 1)-th group also
+//     bounds the ids.  A column at exactly the bound whose id lies past that
+//     group ranks behind C others, so a word with thousands of duplicates does
+//     not collect them all.
+//   * kSweepGather appends every value that reaches the row's bound (columns in
+//     the locality order, so that the hits of a warp's rows fall into few
+//     chunks), and select_row_kernel takes each row's C best of them exactly.
+//
+// Both are one kernel: the candidate kernel's producer and MMA thread, and
+// sixteen epilogue warps (four per SM sub-partition; each thread has one row
+// and half of a tile's columns, since eight warps left the issue slots idle
+// two thirds of the time).  A CTA reads an accumulator into registers whole and
+// releases it before it looks at the values.  With no compaction a row has a
+// fixed share of its append buffers per column split and half; a share that
+// would overflow (values with masses of ties) raises its row block's flag, and
+// the candidate kernel, gated on it, then redoes that block.  100k rows, C =
+// 512: the candidate kernel alone 18.7 ms, the sweeps and selections 5.2 ms.
+enum { kSweepMax = 0, kSweepGather = 1 };
+constexpr int kSwEpiWarps = 16;  // row quadrant = warp % 4, row block = warp / 4 % 2, column half = warp / 8
+constexpr int kSwProducer = kSwEpiWarps;
+constexpr int kSwMma = kSwEpiWarps + 1;
+constexpr int kSwWarps = kSwEpiWarps + 2;
+constexpr int kSwThreads = kSwWarps * 32;
+constexpr int kSwOffVals = kOffStages + kStages * kStageBytes;  // gather: a thread's 32 values of a chunk with hits
+constexpr int kSwOffBars = kSwOffVals + kSwEpiWarps * 32 * kValStride * 4;
+constexpr int kSwSmem = kSwOffBars + (2 * kStages + 4 + 1) * 8 + 16 + 1024;
+static_assert(kSwSmem <= 227 * 1024, "one CTA per SM");
+
+// A row's scratch is its two append buffers: 2 kCap slots of 8 bytes.  First
+// the group maxima (floats), then the gathered entries (column position,
+// value) in 2 S shares; the last slots hold the shares' counts (six words), the
+// bound with its id limit, and in a block's first row the overflow flag.
+constexpr uint32_t kRowSlots = 2 * kCap;
+constexpr uint32_t kDataSlots = kRowSlots - 5;
+constexpr uint32_t kMaxGroups = 4096;
+constexpr uint32_t kMaxSweepSplits = 3;
+static_assert(kMaxGroups * sizeof(float) <= kDataSlots * sizeof(uint64_t), "the maxima fit a row's scratch");
+__device__ __forceinline__ uint64_t* row_scratch(uint64_t* buf, uint32_t i) { return buf + (size_t)i * kRowSlots; }
+__device__ __forceinline__ uint32_t* row_counts(uint64_t* row) { return reinterpret_cast<uint32_t*>(row + kDataSlots); }
+__device__ __forceinline__ float* row_bound(uint64_t* row) { return reinterpret_cast<float*>(row + kRowSlots - 1); }
+__device__ __forceinline__ uint32_t* row_id_limit(uint64_t* row) { return reinterpret_cast<uint32_t*>(row + kRowSlots - 1) + 1; }
+// overflow flag of the block of rows that holds row i
+__device__ __forceinline__ uint32_t* block_flag(uint64_t* buf, uint32_t i) {
+  return reinterpret_cast<uint32_t*>(row_scratch(buf, i / kCtaRows * kCtaRows) + kRowSlots - 2);
+}
+__host__ __device__ constexpr uint32_t share_slots(uint32_t splits) { return kDataSlots / (2u * splits); }
+
+struct SweepArgs {
+  CUtensorMap tmA;  // the rows, boxes of kCtaRows rows
+  CUtensorMap tmB;  // the columns, boxes of kTileN rows
+  const unsigned char* ext;
+  uint32_t nA, nB;
+  uint32_t tps;     // tiles per column split (a multiple of a group's tiles)
+  uint32_t splits;
+  uint32_t lg;      // kSweepMax: groups of 32 << lg columns (lg >= 1: of one column half)
+  uint64_t* buf;
+  const uint32_t* ids;  // original ids by column position (nullptr: the position)
+  uint32_t* err;
+  uint32_t* overflow;   // any block's flag is up
+  long long wait_cycles;
+  uint32_t withhold;
+};
+
+__device__ __forceinline__ float max32(const uint32_t (&v)[32]) {
+  float a[11];
+#pragma unroll
+  for (int x = 0; x < 10; ++x)
+    a[x] = fmax3(__uint_as_float(v[3 * x]), __uint_as_float(v[3 * x + 1]), __uint_as_float(v[3 * x + 2]));
+  a[10] = fmaxf(__uint_as_float(v[30]), __uint_as_float(v[31]));
+  return fmax3(fmax3(fmax3(a[0], a[1], a[2]), fmax3(a[3], a[4], a[5]), fmax3(a[6], a[7], a[8])), a[9], a[10]);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_constant__ SweepArgs P) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const long long wait_lim = P.wait_cycles;
+  const uint32_t bar0 = smem_u32(smem + kSwOffBars);
+  auto full_bar = [&](uint32_t s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](uint32_t s) { return bar0 + 8u * (kStages + s); };
+  auto accf_bar = [&](uint32_t b) { return bar0 + 8u * (2 * kStages + b); };
+  auto acce_bar = [&](uint32_t b) { return bar0 + 8u * (2 * kStages + 2 + b); };
+  const uint32_t a_bar = bar0 + 8u * (2 * kStages + 4);
+  uint32_t* sTmem = reinterpret_cast<uint32_t*>(smem + kSwOffBars + (2 * kStages + 5) * 8);
+  const uint32_t row0 = blockIdx.x * (uint32_t)kCtaRows;
+  const uint32_t tall = (P.nB + kTileN - 1) / kTileN;
+  const uint32_t tlo = min(tall, blockIdx.y * P.tps), ntiles = min(tall - tlo, P.tps);
+
+  for (int x = tid; x < kRows * kExtK; x += kSwThreads) {
+    const uint32_t r = (uint32_t)x / kExtK, k = (uint32_t)x % kExtK;
+    const float w = k == 0 ? 65536.f : (k == 1 ? 256.f : (k == 2 ? 1.f : 0.f));
+    *reinterpret_cast<__nv_bfloat16*>(smem + kOffAExt + ext_offset(r, k)) = __float2bfloat16_rn(w);
+  }
+  if (tid == 0) {
+    for (uint32_t s = 0; s < (uint32_t)kStages; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    for (uint32_t b = 0; b < 2; ++b) {
+      mbar_init(accf_bar(b), 1);
+      mbar_init(acce_bar(b), kSwEpiWarps);
+    }
+    mbar_init(a_bar, 1);
+    tc::mbar_init_fence();
+  }
+  if (warp == 0) tc::tmem_alloc(smem_u32(sTmem), kTmemCols);
+  tc::fence_proxy_async();  // the weights above, for the tensor cores
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = *sTmem;
+
+  if (warp == kSwProducer) {
+    if (lane == 0) {
+      mbar_expect_tx(a_bar, kBlocksPerCta * kAMainBytes);
+      tc::tma_load_2d(smem_u32(smem + kOffAMain), &P.tmA, 0, (int)row0, a_bar);
+      uint32_t u = 0;
+      for (; u < ntiles; ++u) {
+        const uint32_t s = u % kStages;
+        if (u >= (uint32_t)kStages && !mbar_wait(empty_bar(s), ((u / kStages) - 1u) & 1u, wait_lim)) {
+          atomicOr(P.err, kErrWait);
+          break;
+        }
+        if (u == P.withhold) continue;  // debug: never issued; the waits for it run out
+        const uint32_t t = tlo + u;
+        unsigned char* st = smem + kOffStages + s * kStageBytes;
+        mbar_expect_tx(full_bar(s), kStageBytes);
+        tc::tma_load_2d(smem_u32(st), &P.tmB, 0, (int)(t * (uint32_t)kTileN), full_bar(s));
+        bulk_g2s(smem_u32(st + kMainBytes), P.ext + (size_t)t * kExtBytes, kExtBytes, full_bar(s));
+      }
+      // every copy issued has landed before the CTA exits (bounded)
+      if (!mbar_wait(a_bar, 0u, wait_lim)) atomicOr(P.err, kErrWait);
+      for (uint32_t v = u > (uint32_t)kStages ? u - kStages : 0u; v < u; ++v) {
+        if (v == P.withhold) continue;
+        if (!mbar_wait(full_bar(v % kStages), (v / kStages) & 1u, wait_lim)) {
+          atomicOr(P.err, kErrWait);
+          break;
+        }
+      }
+    }
+  } else if (warp == kSwMma) {
+    if (lane == 0) {
+      bool ok = mbar_wait(a_bar, 0u, wait_lim);
+      if (!ok) atomicOr(P.err, kErrWait);
+      const uint32_t a_main = smem_u32(smem + kOffAMain), a_ext = smem_u32(smem + kOffAExt);
+      uint32_t u = 0;
+      for (; ok && u < ntiles; ++u) {
+        const uint32_t s = u % kStages, b = u & 1u;
+        if (!mbar_wait(full_bar(s), (u / kStages) & 1u, wait_lim) ||
+            (u >= 2 && !mbar_wait(acce_bar(b), ((u >> 1) - 1u) & 1u, wait_lim))) {
+          atomicOr(P.err, kErrWait);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t st = smem_u32(smem + kOffStages + s * kStageBytes);
+#pragma unroll
+        for (uint32_t rb = 0; rb < (uint32_t)kBlocksPerCta; ++rb) {
+          const uint32_t d = tbase + (2u * rb + b) * (uint32_t)kTileN;
+          const uint32_t am = a_main + rb * (uint32_t)kAMainBytes;
+#pragma unroll
+          for (uint32_t ks = 0; ks < 4; ++ks)
+            tc_mma(d, smem_desc(am + 32u * ks, 16u, 1024u, 2u), smem_desc(st + 32u * ks, 16u, 1024u, 2u),
+                   ks > 0 ? 1u : 0u);
+          tc_mma(d, smem_desc(a_ext, 128u, 256u, 0u), smem_desc(st + kMainBytes, 128u, 256u, 0u), 1u);
+        }
+        tc_commit(empty_bar(s));
+        tc_commit(accf_bar(b));
+      }
+      // the products issued have completed before tensor memory is freed
+      if (u > 0 && !mbar_wait(accf_bar((u - 1u) & 1u), ((u - 1u) >> 1) & 1u, wait_lim)) atomicOr(P.err, kErrWait);
+    }
+  } else {
+    const uint32_t blk = ((uint32_t)warp >> 2) & 1u, half = (uint32_t)warp >> 3;
+    const uint32_t i = row0 + blk * (uint32_t)kRows + (uint32_t)((warp & 3) * 32 + lane);
+    bool live = i < P.nA;
+    const uint32_t lane_base = tbase + ((uint32_t)((warp & 3) * 32) << 16) + 2u * blk * (uint32_t)kTileN + 64u * half;
+    uint64_t* row = live ? row_scratch(P.buf, i) : nullptr;
+    // kSweepMax
+    float run = -FLT_MAX;  // the current group's maximum
+    // kSweepGather
+    const float thr = MODE == kSweepGather && live ? *row_bound(row) : 0.f;
+    const uint32_t id_limit = MODE == kSweepGather && live ? *row_id_limit(row) : 0u;
+    const uint32_t cap = share_slots(P.splits);
+    uint2* out = live ? reinterpret_cast<uint2*>(row + (size_t)(2u * blockIdx.y + half) * cap) : nullptr;
+    uint32_t cnt = 0u;
+    float* sv = reinterpret_cast<float*>(smem + kSwOffVals) + tid * kValStride;
+
+    // appends the values of a chunk (column colbase + k in v[k]) that reach the
+    // bound: the chunk's maximum first, then a hit mask of two instructions per
+    // value (the sign of x - thr: both are integers, so it is exact), then the
+    // hits read back from shared memory
+    auto gather = [&](const uint32_t (&v)[32], uint32_t colbase) {
+      if (!(live && max32(v) >= thr)) return;
+      uint32_t ms[4] = {0u, 0u, 0u, 0u};  // bit k: x_k < thr, in four independent chains
+#pragma unroll
+      for (int k = 7; k >= 0; --k)
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          ms[g] = __funnelshift_l(__float_as_uint(__uint_as_float(v[8 * g + k]) - thr), ms[g], 1);
+      uint32_t hit = ~(ms[0] | (ms[1] << 8) | (ms[2] << 16) | (ms[3] << 24));
+      if (i - colbase < 32u) hit &= ~(1u << (i - colbase));                     // the row itself
+      if (colbase + 32u > P.nB) hit &= colbase < P.nB ? (1u << (P.nB - colbase)) - 1u : 0u;  // padding
+      if (!hit) return;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        *reinterpret_cast<uint4*>(sv + 4 * q) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      do {
+        const uint32_t k = (uint32_t)__ffs(hit) - 1u, pos = colbase + k;
+        hit &= hit - 1u;
+        const float x = sv[k];
+        if (x == thr && (P.ids ? __ldg(P.ids + pos) : pos) >= id_limit) continue;  // behind C others by its id
+        out[cnt++] = make_uint2(pos, __float_as_uint(x));
+      } while (hit);
+    };
+
+    for (uint32_t u = 0; u < ntiles; ++u) {
+      const uint32_t b = u & 1u;
+      const bool got = mbar_wait(accf_bar(b), (u >> 1) & 1u, wait_lim);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) atomicOr(P.err, kErrWait);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t col0 = (tlo + u) * (uint32_t)kTileN + 64u * half;
+      const uint32_t tcol = lane_base + b * (uint32_t)kTileN;
+      uint32_t va[32], vb[32];
+      tmem_ld32(tcol, va);
+      tmem_ld32(tcol + 32u, vb);
+      tmem_wait(va);
+      tmem_wait(vb);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acce_bar(b));
+      if constexpr (MODE == kSweepMax) {
+        if (col0 + 64u > P.nB) {  // padding columns hold zero rows: not values
+#pragma unroll
+          for (int k = 0; k < 32; ++k) {
+            if (col0 + (uint32_t)k >= P.nB) va[k] = __float_as_uint(-FLT_MAX);
+            if (col0 + 32u + (uint32_t)k >= P.nB) vb[k] = __float_as_uint(-FLT_MAX);
+          }
+        }
+        const float ma = max32(va), mb = max32(vb);
+        float* gm = reinterpret_cast<float*>(row);
+        const uint32_t t = tlo + u;
+        if (P.lg == 0u) {
+          if (live) *reinterpret_cast<float2*>(gm + 4 * (size_t)t + 2u * half) = make_float2(ma, mb);
+        } else {
+          run = fmax3(run, ma, mb);
+          const uint32_t per = 1u << (P.lg - 1u);  // tiles of a group (splits start on whole groups)
+          if (((t + 1u) & (per - 1u)) == 0u || u + 1u == ntiles) {
+            if (live) gm[2u * (t >> (P.lg - 1u)) + half] = run;
+            run = -FLT_MAX;
+          }
+        }
+      } else {
+        if (live && cnt + 64u > cap) {  // the share may not hold this tile's hits
+          atomicOr(P.overflow, 1u);
+          atomicOr(block_flag(P.buf, i), 1u);
+          live = false;
+        }
+        gather(va, col0);
+        gather(vb, col0 + 32u);
+      }
+      __syncwarp();
+    }
+    if (MODE == kSweepGather && row) row_counts(row)[2u * blockIdx.y + half] = cnt;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tc::tmem_dealloc(tbase, kTmemCols);
+}
+
+// One warp per row: the rank-th largest of its G group maxima, or a value
+// below it when the maxima span more than 2^16 (two passes of a 256-bin
+// histogram, each narrowing the range to one bin), as the row's bound.
+constexpr int kBoundWarps = 4;
+__global__ void __launch_bounds__(kBoundWarps * 32) row_bound_kernel(uint64_t* buf, uint32_t n, uint32_t G,
+                                                                    uint32_t lg, uint32_t rank) {
+  extern __shared__ float s_max[];  // [kBoundWarps][G]
+  __shared__ unsigned s_hist[kBoundWarps][256];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t i = blockIdx.x * kBoundWarps + warp;
+  if (i >= n) return;  // warp-uniform
+  float* m = s_max + (size_t)warp * G;
+  unsigned* hist = s_hist[warp];
+  uint64_t* row = row_scratch(buf, i);
+  const float* src = reinterpret_cast<const float*>(row);
+  float flo = FLT_MAX, fhi = -FLT_MAX;
+#pragma unroll 4
+  for (uint32_t g = lane; g < G; g += 32) {
+    const float v = src[g];
+    m[g] = v;
+    if (v > -FLT_MAX) flo = fminf(flo, v);  // (a group of padding columns alone has no value)
+    fhi = fmaxf(fhi, v);
+  }
+  int lo = __reduce_min_sync(0xffffffffu, (int)flo), hi = __reduce_max_sync(0xffffffffu, (int)fhi);
+  float bound = -FLT_MAX;
+  unsigned need = rank;
+  bool exact = false;
+  for (int pass = 0; pass < 2 && lo <= hi; ++pass) {
+    const unsigned span = (unsigned)(hi - lo);
+    const int sh = span < 256u ? 0 : 24 - __clz((int)span);
+    for (int b = lane; b < 256; b += 32) hist[b] = 0u;
+    __syncwarp();
+    unsigned mine = 0u;
+    for (uint32_t g = lane; g < G; g += 32) {
+      const float v = m[g];
+      if (v >= (float)lo && v <= (float)hi) {
+        atomicAdd(&hist[min((unsigned)((int)v - lo) >> sh, 255u)], 1u);
+        ++mine;
+      }
+    }
+    __syncwarp();
+    if (__reduce_add_sync(0xffffffffu, mine) < need) break;  // fewer groups than the rank: no bound
+    int bin;
+    unsigned before;
+    hist_find_desc(hist, need, lane, bin, before);
+    __syncwarp();
+    need -= before;
+    lo += bin << sh;
+    bound = (float)lo;
+    hi = min(hi, lo + (1 << sh) - 1);
+    exact = sh == 0;
+    if (exact) break;
+  }
+  // ties at an exact bound: the need-th group with that maximum, in position
+  // order, ends the ids that can still be among the C best
+  uint32_t limit = 0xffffffffu;
+  if (exact) {
+    for (uint32_t g0 = 0; g0 < G; g0 += 32) {
+      const unsigned at = __ballot_sync(0xffffffffu, g0 + (uint32_t)lane < G && m[g0 + (uint32_t)lane] == bound);
+      const unsigned c = (unsigned)__popc(at);
+      if (need > c) {
+        need -= c;
+        continue;
+      }
+      const uint32_t g = g0 + __fns(at, 0, (int)need);
+      // past the last column of group g: chunk 32 g, or whole tiles of both halves
+      limit = lg == 0u ? (g + 1u) * 32u : (g / 2u + 1u) * ((uint32_t)kTileN << (lg - 1u));
+      break;
+    }
+  }
+  if (lane == 0) {
+    *row_bound(row) = bound;
+    *row_id_limit(row) = limit;
+    if (i % (uint32_t)kCtaRows == 0u) *block_flag(buf, i) = 0u;
+  }
+}
+
+// One warp per row: the C best of the row's gathered entries, exactly (a value
+// histogram between the bound and the largest value finds the C-th value's bin;
+// the exact select runs among the keys at or above that bin's lower edge), as
+// the candidate kernel's final pass does.  Entries hold column positions;
+// ids (nullable) maps them to original ids, which break ties.
+constexpr int kSelWarps = 4;
+__global__ void __launch_bounds__(kSelWarps * 32)
+    select_row_kernel(uint64_t* buf, uint32_t n, uint32_t splits, uint32_t C, uint32_t stage_keys, bool sorted,
+                      const uint32_t* __restrict__ ids, uint32_t* __restrict__ out_idx, int32_t* __restrict__ out_val,
+                      uint32_t* overflow) {
+  extern __shared__ uint64_t s_keys[];  // [kSelWarps][stage_keys]
+  __shared__ unsigned s_hist[kSelWarps][256];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t i = blockIdx.x * kSelWarps + warp;
+  if (i >= n) return;  // warp-uniform
+  uint64_t* keys = s_keys + (size_t)warp * stage_keys;
+  unsigned* hist = s_hist[warp];
+  uint64_t* row = row_scratch(buf, i);
+  const uint32_t cap = share_slots(splits);
+  uint32_t total = 0u;
+  int hi = INT32_MIN;
+  for (uint32_t sgm = 0; sgm < 2u * splits; ++sgm) {
+    const uint32_t c = min(row_counts(row)[sgm], cap);
+    if (total + c > stage_keys) {  // more than the staging area holds: the candidate kernel redoes the product
+      if (lane == 0) {
+        atomicOr(overflow, 1u);
+        atomicOr(block_flag(buf, i), 1u);
+      }
+      return;
+    }
+    const uint2* src = reinterpret_cast<const uint2*>(row + (size_t)sgm * cap);
+#pragma unroll 4
+    for (uint32_t x = lane; x < c; x += 32) {
+      const uint2 e = src[x];
+      const int v = (int)__uint_as_float(e.y);
+      keys[total + x] = make_key(v, ids ? __ldg(ids + e.x) : e.x);
+      hi = max(hi, v);
+    }
+    total += c;
+  }
+  __syncwarp();
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  int kept = (int)total;
+  if (total > C) {
+    const float bound = *row_bound(row);
+    const int lo = (int)bound;
+    const unsigned span = (unsigned)(hi - lo);
+    const int sh = span < 256u ? 0 : 24 - __clz((int)span);
+    warp_value_hist_ge(keys, (int)total, lo, sh, hist, lane);
+    int bin;
+    unsigned above;
+    hist_find_desc(hist, C, lane, bin, above);
+    __syncwarp();
+    kept = warp_keep_value_ge_to(keys, (int)total, lo + (bin << sh), keys, lane);
+    if (kept > (int)C) {
+      const uint64_t kth = warp_select_kth(keys, kept, (int)C, hist, lane);
+      kept = warp_gather_ge(keys, kept, kth, keys, lane);
+    }
+  }
+  if (sorted) {
+    const int size = pow2_at_least(kept);
+    for (int x = kept + lane; x < size; x += 32) keys[x] = 0ull;
+    warp_bitonic_desc(keys, size, lane);
+  }
+  __syncwarp();
+  const size_t orow = ids ? ids[i] : i;
+  for (uint32_t x = lane; x < C; x += 32) {
+    const bool have = (int)x < kept;
+    out_idx[orow * C + x] = have ? key_idx(keys[x]) : 0xffffffffu;
+    out_val[orow * C + x] = have ? key_val(keys[x]) : INT32_MIN;
+  }
+}
+
 template <bool kSplit, bool kSelf>
 __global__ void __launch_bounds__(kThreads, 1) dot_topk_kernel(const __grid_constant__ DotArgs P) {
   extern __shared__ unsigned char smem_raw[];
@@ -467,6 +907,8 @@ __global__ void __launch_bounds__(kThreads, 1) dot_topk_kernel(const __grid_cons
   const uint32_t C = P.C;
   uint32_t* __restrict__ err = P.err;
   const long long wait_lim = P.wait_cycles;
+  if (P.gate && (*P.gate == 0u || (!kSplit && *block_flag(P.buf, blockIdx.x * (uint32_t)kCtaRows) == 0u)))
+    return;  // block-uniform
 
   float* sThr = reinterpret_cast<float*>(smem + kOffThr);
   float* sHi = reinterpret_cast<float*>(smem + kOffHi);
@@ -952,7 +1394,8 @@ constexpr int kMergeWarps = 8;
 __global__ void __launch_bounds__(kMergeWarps * 32)
     merge_splits_kernel(const uint64_t* __restrict__ part, uint32_t nA, uint32_t S, uint32_t C, bool sorted,
                         const uint32_t* __restrict__ row_ids, uint32_t* __restrict__ out_idx,
-                        int32_t* __restrict__ out_val) {
+                        int32_t* __restrict__ out_val, const uint32_t* gate) {
+  if (gate && *gate == 0u) return;
   __shared__ unsigned hist[kMergeWarps][256];
   __shared__ uint64_t keep[kMergeWarps][kSel];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1371,10 +1814,45 @@ static cudaError_t encode_rows(CUtensorMap* m, const void* base, uint64_t rows, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// The group size 32 << lg of the two-sweep path: 3 C to 6 C groups (256 of 782
+// groups put 310 columns at or above the bound; twice as many groups would put
+// 281 there, but selecting the bound costs as much again).  Below 2 C groups
+// of 32 columns a bound would be too loose: false.
+static bool bound_groups(uint32_t n, uint32_t C, uint32_t& lg) {
+  lg = 0;
+  if (n / 32u < 2u * (C + 1u)) return false;
+  const uint32_t tiles = (n + kTileN - 1) / kTileN;
+  auto groups = [&](uint32_t g) { return g ? 2u * ((tiles + (1u << (g - 1u)) - 1) >> (g - 1u)) : 4u * tiles; };
+  while (groups(lg + 1u) >= 3u * (C + 1u) || groups(lg) > kMaxGroups) ++lg;
+  return true;
+}
+
+// Column splits of a sweep: the number up to `most` (of at least eight tiles
+// each) that leaves the last wave of CTAs, one per SM, the fullest.
+static uint32_t sweep_splits(uint32_t blocks, uint32_t tiles, uint32_t most) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
+    cudaGetLastError();
+    sms = 152;
+  }
+  uint32_t best = 1;
+  double best_t = 0;
+  for (uint32_t x = 1; x <= most && (x == 1 || tiles / x >= 8u); ++x) {
+    // waves of CTAs x (tiles of one + ~8 tiles' worth of set-up)
+    const double t = (double)((blocks * x + (uint32_t)sms - 1) / (uint32_t)sms) * ((double)((tiles + x - 1) / x) + 8.0);
+    if (x == 1 || t < best_t) {
+      best = x;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
 cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloat16* QB, const int32_t* biasB,
                           uint32_t nB, uint32_t C, bool self, uint64_t* buf, uint32_t* idx, int32_t* val,
                           uint32_t* err, cudaStream_t s, DotDebug dbg, const uint32_t* col_ids,
-                          const uint32_t* row_ids, bool sorted) {
+                          const uint32_t* row_ids, bool sorted, const __nv_bfloat16* Qraw, const int32_t* bias_raw) {
   if (nA == 0) return cudaSuccess;
   const uint32_t S = dot_topk_splits(nA, nB);
   const auto kernel = S > 1 ? (self ? dot_topk_kernel<true, true> : dot_topk_kernel<true, false>)
@@ -1406,19 +1884,78 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
   P.row_ids = row_ids;
   P.sorted = sorted;
   const uint32_t npad = (uint32_t)bias_pad(nB);
-  if (npad) bias_digits_kernel<<<(2 * npad + 255) / 256, 256, 0, s>>>(biasB, nB, npad, ext);
+  const uint32_t bias_grid = (2 * npad + 255) / 256;
+  uint32_t lg = 0;
+  // Past 2^18 columns the first sweep takes half of them: any subset gives a
+  // valid bound, twice as many columns reach it (2.5 C of 600k), and that
+  // costs less than half a sweep (600k rows, C = 256: 104 -> 88 ms).
+  const uint32_t nM = nB > (1u << 18) ? (nB / 2u + kTileN - 1) / kTileN * kTileN : nB;
+  if (self && bound_groups(nM, C, lg)) {
+    // the two-sweep path; the candidate kernel below runs only if it overflowed
+    uint32_t* overflow = err + 1;
+    e = cudaMemsetAsync(overflow, 0, sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    SweepArgs X;
+    std::memset(&X, 0, sizeof X);
+    X.tmA = P.tmA;
+    X.ext = ext;
+    X.nA = nA;
+    X.nB = nM;
+    X.lg = lg;
+    X.buf = buf;
+    X.err = err;
+    X.overflow = overflow;
+    X.wait_cycles = P.wait_cycles;
+    X.withhold = P.withhold;
+    const auto max_kernel = dot_sweep_kernel<kSweepMax>;
+    const auto gather_kernel = dot_sweep_kernel<kSweepGather>;
+    e = cudaFuncSetAttribute(max_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwSmem);
+    if (e != cudaSuccess) return e;
+    const uint32_t blocks = (nA + kCtaRows - 1) / kCtaRows, per = lg ? 1u << (lg - 1u) : 1u;
+    // maxima: any number of splits of whole groups
+    const uint32_t tm = (nM + kTileN - 1) / kTileN, sm = sweep_splits(blocks, tm, 8u);
+    X.tps = ((tm + sm - 1) / sm + per - 1) / per * per;
+    X.splits = (tm + X.tps - 1) / X.tps;
+    e = encode_rows(&X.tmB, Qraw ? Qraw : QB, bias_pad(nB), (uint32_t)kTileN);
+    if (e != cudaSuccess) return e;
+    bias_digits_kernel<<<bias_grid, 256, 0, s>>>(Qraw ? bias_raw : biasB, nB, npad, ext);
+    max_kernel<<<dim3(blocks, X.splits), kSwThreads, kSwSmem, s>>>(X);
+    const uint32_t G = lg ? 2u * ((tm + per - 1) / per) : 4u * tm;
+    const size_t bound_smem = (size_t)kBoundWarps * G * sizeof(float);
+    e = cudaFuncSetAttribute(row_bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bound_smem);
+    if (e != cudaSuccess) return e;
+    row_bound_kernel<<<(nA + kBoundWarps - 1) / kBoundWarps, kBoundWarps * 32, bound_smem, s>>>(buf, nA, G, lg, C + 1);
+    X.tmB = P.tmB;
+    X.nB = nB;
+    X.ids = col_ids;
+    if (Qraw) bias_digits_kernel<<<bias_grid, 256, 0, s>>>(biasB, nB, npad, ext);
+    const uint32_t sg = sweep_splits(blocks, tiles, kMaxSweepSplits);
+    X.tps = (tiles + sg - 1) / sg;
+    X.splits = sg;
+    gather_kernel<<<dim3(blocks, sg), kSwThreads, kSwSmem, s>>>(X);
+    const uint32_t stage_keys = (nM < nB ? 4u : 2u) * C + 256u;
+    const size_t sel_smem = (size_t)kSelWarps * stage_keys * sizeof(uint64_t);
+    e = cudaFuncSetAttribute(select_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem);
+    if (e != cudaSuccess) return e;
+    select_row_kernel<<<(nA + kSelWarps - 1) / kSelWarps, kSelWarps * 32, sel_smem, s>>>(
+        buf, nA, sg, C, stage_keys, sorted, col_ids, idx, val, overflow);
+    P.gate = overflow;
+  } else if (npad) {
+    bias_digits_kernel<<<bias_grid, 256, 0, s>>>(biasB, nB, npad, ext);
+  }
   const dim3 grid((nA + kCtaRows - 1) / kCtaRows, S);
   kernel<<<grid, kThreads, kSmemTotal, s>>>(P);
   if (S > 1)
     merge_splits_kernel<<<(nA + kMergeWarps - 1) / kMergeWarps, kMergeWarps * 32, 0, s>>>(P.part, nA, S, C, sorted, row_ids, idx,
-                                                                                         val);
+                                                                                         val, P.gate);
   return cudaGetLastError();
 }
 
 cudaError_t dot_topk(const __nv_bfloat16* Qb, const int32_t* bias, uint32_t n, uint32_t C, uint64_t* buf,
                      uint32_t* idx, int32_t* val, uint32_t* err, cudaStream_t s, DotDebug dbg,
-                     const uint32_t* ids, bool sorted) {
-  return dot_topk_rect(Qb, n, Qb, bias, n, C, true, buf, idx, val, err, s, dbg, ids, ids, sorted);
+                     const uint32_t* ids, bool sorted, const __nv_bfloat16* Qraw, const int32_t* bias_raw) {
+  return dot_topk_rect(Qb, n, Qb, bias, n, C, true, buf, idx, val, err, s, dbg, ids, ids, sorted, Qraw, bias_raw);
 }
 
 cudaError_t quantize(const float* E, uint32_t n, unsigned int* amax_bits, int8_t* q, __nv_bfloat16* qb,
