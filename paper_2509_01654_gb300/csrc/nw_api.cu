@@ -221,6 +221,7 @@ void nw_dict_free(nw_dict* d) {
   free_wordset(c, d->ws);
   ctx_free(c, d->d_segs);
   ctx_free(c, d->d_tab);
+  ctx_free(c, d->rec);
   c->dicts.erase(d);
   delete d;
 }
@@ -396,6 +397,9 @@ nw_status nw_score_pairs(nw_dict* d, const uint32_t* i, const uint32_t* j, size_
   P.C2 = d->ss.C2;
   P.gap = d->sc.gap;
   P.tab = dict_tab(d);
+  pairs_bits(d, P);
+  // (an eighth as many pairs as words repays making the records)
+  if (P.bit_m && (d->rec.p || m >= n / 8u)) P.rec = dict_records(d, s);
   P.out = dout;
   P.err = c->ws_small.as<uint32_t>();
   Timer tm{c};

@@ -879,8 +879,37 @@ __global__ void __launch_bounds__(kSelWarps * 32)
     unsigned above;
     hist_find_desc(hist, C, lane, bin, above);
     __syncwarp();
-    kept = warp_keep_value_ge_to(keys, (int)total, lo + (bin << sh), keys, lane);
-    if (kept > (int)C) {
+    const int edge = lo + (bin << sh);
+    const unsigned in_bin = hist[bin];
+    __syncwarp();
+    kept = warp_keep_value_ge_to(keys, (int)total, edge, keys, lane);
+    if (kept > (int)C && in_bin <= 64u) {
+      // the usual case: a few keys share the C-th's bin.  They move behind the
+      // others, and each finds its rank among them by counting
+      const int top = edge + (1 << sh) - 1;
+      const bool last = bin == 255;  // (the last bin also counts the values past it)
+      uint64_t* const edge_keys = reinterpret_cast<uint64_t*>(hist);  // 64 keys: half of the histogram's room
+      int base = 0, eb = 0;
+      for (int x0 = 0; x0 < kept; x0 += 32) {
+        const uint64_t k = x0 + lane < kept ? keys[x0 + lane] : 0ull;
+        const bool have = x0 + lane < kept, at_edge = have && (last || key_val(k) <= top);
+        const unsigned me = __ballot_sync(0xffffffffu, at_edge), mk = __ballot_sync(0xffffffffu, have && !at_edge);
+        if (at_edge) edge_keys[eb + __popc(me & ((1u << lane) - 1u))] = k;
+        if (have && !at_edge) keys[base + __popc(mk & ((1u << lane) - 1u))] = k;
+        eb += __popc(me);
+        base += __popc(mk);
+        __syncwarp();
+      }
+      const int need = (int)C - base;
+      for (int x = lane; x < eb; x += 32) {
+        const uint64_t k = edge_keys[x];
+        int rank = 0;
+        for (int y = 0; y < eb; ++y) rank += edge_keys[y] > k ? 1 : 0;
+        if (rank < need) keys[base + rank] = k;
+      }
+      kept = (int)C;
+      __syncwarp();
+    } else if (kept > (int)C) {
       const uint64_t kth = warp_select_kth(keys, kept, (int)C, hist, lane);
       kept = warp_gather_ge(keys, kept, kth, keys, lane);
     }

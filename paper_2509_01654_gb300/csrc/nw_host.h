@@ -104,6 +104,7 @@ struct nw_dict {
   bool subst = false;  // scored with a full similarity matrix (d_tab)
   DevBuf d_tab;        // kTabDim x kTabDim s'+ table
   uint64_t serial = 0;  // unique per loaded dictionary (caches keyed on it)
+  DevBuf rec;           // the words' 16-byte records, made at first use (dict_records)
 };
 
 namespace {
@@ -809,6 +810,36 @@ Terms make_terms(const nw_dict* d, const WordSet& a, const WordSet& b, SideView 
   T.ib = ib;
   T.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
   return T;
+}
+
+// The dictionary's word records, made on stream s at first use and kept with
+// it; null when there is no memory for them (the kernels then read symbols).
+const uint4* dict_records(nw_dict* d, cudaStream_t s) {
+  nw_ctx* c = d->ctx;
+  if (d->rec.p || d->ws.n == 0) return d->rec.as<uint4>();
+  const std::string err = c->err;
+  if (ctx_alloc(c, d->rec, (size_t)d->ws.n * 16, "word records") != NW_OK) {
+    c->err = err;
+    return nullptr;
+  }
+  if (launch_word_records(d->ws.rank.as<uint32_t>(), d->ws.slen.as<uint8_t>(), d->ws.aoff.as<uint32_t>(),
+                          d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, d->rec.as<uint4>(), s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess) {  // other streams may read them next
+    cudaGetLastError();
+    ctx_free(c, d->rec);
+    return nullptr;
+  }
+  return d->rec.as<uint4>();
+}
+
+// the bit-parallel part of a pair list's parameters
+void pairs_bits(const nw_dict* d, PairsParams& P) {
+  P.bit_m = d->ss.bit_m;
+  P.bit_x = d->ss.bit_x;
+  P.coef = d->ss.bit_coef;
+  P.shift = d->ss.shift;
+  P.alphabet = d->alphabet;
+  P.max_len = d->ws.max_len;
 }
 
 int lists_epi(int hist_mode) { return hist_mode == kHistLane ? kEpiListsLaneHist : kEpiLists; }

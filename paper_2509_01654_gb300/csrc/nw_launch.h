@@ -16,6 +16,13 @@ const void* dp_kernel(int range, int epi, bool tab = false);
 // kind; nullptr if there is none (kernels exist for gcd(m, x) = 1, x < m <=
 // kBitMaxStep)
 const void* bit_kernel(int m, int x, int epi);
+// the same for explicit pairs (wide: words of more than 32 symbols; blocks of
+// kBitPairsBlock) and for rescoring a row's candidates
+const void* bit_pairs(int m, int x, bool wide);
+const void* bit_rescore(int m, int x);
+constexpr int kBitPairsBlock = 128;
+// alphabets whose match masks fit the shared memory of those two
+constexpr uint32_t kBitPairsAlphabet = 128;
 
 // ingest: stable bucketing by length and encoding of a word set
 cudaError_t launch_ingest_count(const uint8_t* codes, const uint32_t* offsets, uint32_t n,
@@ -63,7 +70,15 @@ struct PairsParams {
   int16_t* out;
   uint32_t* err;
   const uint16_t* tab;  // substitution table (device, kTabDim x kTabDim) or null
+  // bit-parallel scoring (bit_m = 0: none)
+  int32_t bit_m, bit_x, coef;
+  uint32_t shift, alphabet, max_len;
+  const uint4* rec;  // word records by original index (launch_word_records), or null
 };
+// the 16-byte record of every word: length and up to 15 codes, or the offset
+// of a longer word's symbols
+cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const uint32_t* aoff, const uint32_t* sym,
+                                uint32_t shift, uint32_t n, uint4* rec, cudaStream_t s);
 cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s);
 
 // the all-pairs top-k reduction with every scratch buffer taken from a

@@ -3,6 +3,7 @@
 // (its own 16-bit half, copied into both halves), the shorter word is
 // streamed row by row, and the same shifted recurrence as the all-pairs
 // kernel is evaluated; the result is read from the low half.
+#include <algorithm>
 #include <cuda_runtime.h>
 
 #include "nw_dp.cuh"
@@ -156,6 +157,23 @@ cudaError_t select_topk(const uint32_t* cand, const int32_t* score, uint32_t n, 
 
 cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s) {
   if (p.m == 0) return cudaSuccess;
+  if (p.bit_m && p.alphabet <= kBitPairsAlphabet) {
+    const bool wide = p.max_len > 32u;
+    const void* fn = bit_pairs(p.bit_m, p.bit_x, wide);
+    if (!fn) return cudaErrorInvalidValue;
+    const size_t smem = (size_t)p.alphabet * kBitPairsBlock * (wide ? 8 : 4);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int occ = 0, dev = 0, sms = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBitPairsBlock, smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t blocks = (p.m + kBitPairsBlock - 1) / kBitPairsBlock;
+    const uint64_t resident = (uint64_t)std::max(1, occ) * (uint64_t)sms;
+    PairsParams arg = p;
+    void* args[] = {&arg};
+    return cudaLaunchKernel(fn, dim3((unsigned)std::min(blocks, resident)), dim3(kBitPairsBlock), args, smem, s);
+  }
   const uint32_t blk = 128;
   const uint64_t grid = (p.m + blk - 1) / blk;
   pairs_kernel<<<(unsigned)grid, blk, 0, s>>>(p);

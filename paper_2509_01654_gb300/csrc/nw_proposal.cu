@@ -10,6 +10,7 @@
 #include <cstring>
 #include <vector>
 
+#include "nw_bitpairs.cuh"
 #include "nw_cnn.h"
 #include "nw_host.h"
 #include "nw_proposal.h"
@@ -340,14 +341,73 @@ PairsParams pairs_params(const nw_dict* d, uint32_t* err) {
   P.C2 = d->ss.C2;
   P.gap = d->sc.gap;
   P.tab = dict_tab(d);
+  pairs_bits(d, P);
   P.err = err;
   return P;
+}
+
+// Whether the bit-parallel rescoring kernel takes a dictionary's candidates:
+// its scoring has a step class, the masks of its alphabet fit shared memory,
+// and scores in [lo, hi] fit 32-bit keys above the index bits.
+bool rescore_takes_bits(const nw_dict* d, uint32_t C, int32_t lo, int32_t hi, uint32_t ib) {
+  return d->ss.bit_m && d->alphabet <= kBitPairsAlphabet && C <= (uint32_t)NW_MAX_CANDIDATES &&
+         (uint64_t)((int64_t)hi - lo + 1) < (1ull << (32 - ib));
+}
+
+// The dictionary's word records: its own if it has them, else made in `scratch`
+// on stream s (a server slot's view of a dictionary owns no memory of it).
+nw_status rescore_records(nw_ctx* c, const nw_dict* d, DevBuf& scratch, const uint4** rec, cudaStream_t s) {
+  if (d->rec.p) {
+    *rec = d->rec.as<uint4>();
+    return NW_OK;
+  }
+  NW_TRY(ctx_ensure(c, scratch, std::max<size_t>(16, (size_t)d->ws.n * 16), "candidate word records"));
+  NW_CK(launch_word_records(d->ws.rank.as<uint32_t>(), d->ws.slen.as<uint8_t>(), d->ws.aoff.as<uint32_t>(),
+                            d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, scratch.as<uint4>(), s));
+  *rec = scratch.as<uint4>();
+  return NW_OK;
+}
+
+RescoreBits rescore_bits(const nw_dict* d, const uint32_t* cand, uint32_t rows, uint32_t C, uint32_t k, int32_t key_lo,
+                         uint32_t ib, const uint4* rec, uint32_t* out_idx, int16_t* out_score, uint32_t* err) {
+  RescoreBits R{};
+  R.cand = cand;
+  R.rows = rows;
+  R.C = C;
+  R.k = k;
+  R.nd = d->ws.n;
+  R.rec = rec;
+  R.d_sym = d->ws.a_enc.as<uint32_t>();
+  R.shift = d->ss.shift;
+  R.alphabet = d->alphabet;
+  R.coef = (uint32_t)d->ss.bit_coef;
+  R.gap = d->sc.gap;
+  R.key_lo = key_lo;
+  R.ib = ib;
+  R.imask = (uint32_t)(((uint64_t)1 << ib) - 1);
+  R.out_idx = out_idx;
+  R.out_score = out_score;
+  R.err = err;
+  return R;
 }
 
 // candidate rescoring + selection on the model's or context's buffers
 nw_status rescore_select(nw_ctx* c, nw_dict* d, const uint32_t* cand, uint32_t C, uint32_t k, DevBuf& score_buf,
                          uint32_t* out_idx, int16_t* out_score, uint32_t* err, cudaStream_t s) {
   const uint32_t n = d->ws.n;
+  const uint32_t ib = index_bits(std::max<uint32_t>(n, 2));
+  if (rescore_takes_bits(d, C, d->score_lo, d->score_hi, ib)) {
+    const uint4* rec = nullptr;
+    NW_TRY(rescore_records(c, d, score_buf, &rec, s));
+    RescoreBits R = rescore_bits(d, cand, n, C, k, d->score_lo - 1, ib, rec, out_idx, out_score, err);
+    R.self = true;
+    R.r_rank = d->ws.rank.as<uint32_t>();
+    R.r_slen = d->ws.slen.as<uint8_t>();
+    R.r_aoff = d->ws.aoff.as<uint32_t>();
+    R.r_sym = d->ws.a_enc.as<uint32_t>();
+    NW_CK(prop::rescore_topk_bits(R, d->ss.bit_m, d->ss.bit_x, c->sm_count, s));
+    return NW_OK;
+  }
   // scores, then the length-sorted candidates they belong to and the work lists
   NW_TRY(ctx_ensure(c, score_buf, prop::rescore_scratch_bytes(n, C), "candidate scores"));
   int32_t* score = score_buf.as<int32_t>();
@@ -616,6 +676,7 @@ nw_status nw_model_train(nw_model* M, nw_dict* d, const nw_train_config* cfg, co
     pd.long_thresh = (uint32_t)std::lround((double)cfg->long_fraction * (double)(1u << 20));
   }
   PairsParams pp = pairs_params(d, err_ptr(M));
+  if (pp.bit_m) pp.rec = dict_records(d, s);
   pp.pi = M->pi.as<uint32_t>();
   pp.pj = M->pj.as<uint32_t>();
   pp.m = m;
@@ -998,8 +1059,20 @@ nw_status proposal_query_impl(nw_model* M, nw_dict* d, const uint8_t* qcodes, co
     out_i = oi.as<uint32_t>();
     out_s = os.as<int16_t>();
   }
-  NW_CK(prop::cross_rescore(X, M->qcand.as<uint32_t>(), C, M->qscore.as<int32_t>(), s));
-  NW_CK(prop::select_topk(M->qcand.as<uint32_t>(), M->qscore.as<int32_t>(), nq, C, k, out_i, out_s, s));
+  const uint32_t ib = index_bits(std::max<uint32_t>(n, 2));
+  if (rescore_takes_bits(d, C, lo, hi, ib)) {
+    const uint4* rec = nullptr;
+    NW_TRY(rescore_records(c, d, M->qscore, &rec, s));
+    RescoreBits R = rescore_bits(d, M->qcand.as<uint32_t>(), nq, C, k, lo - 1, ib, rec, out_i, out_s, err_ptr(M));
+    R.r_rank = q.rank.as<uint32_t>();
+    R.r_slen = q.slen.as<uint8_t>();
+    R.r_aoff = q.aoff.as<uint32_t>();
+    R.r_sym = q.a_enc.as<uint32_t>();
+    NW_CK(prop::rescore_topk_bits(R, d->ss.bit_m, d->ss.bit_x, c->sm_count, s));
+  } else {
+    NW_CK(prop::cross_rescore(X, M->qcand.as<uint32_t>(), C, M->qscore.as<int32_t>(), s));
+    NW_CK(prop::select_topk(M->qcand.as<uint32_t>(), M->qscore.as<int32_t>(), nq, C, k, out_i, out_s, s));
+  }
   if (!dev) {
     NW_TRY(copy_out(c, nbr_idx, out_i, (size_t)nq * k, false, s));
     NW_TRY(copy_out(c, nbr_score, out_s, (size_t)nq * k, false, s));

@@ -12,6 +12,7 @@ struct nw_ctx;
 struct nw_model;
 
 namespace nw {
+struct RescoreBits;
 namespace prop {
 
 // the context a model was created on (its allocations, stream and error text)
@@ -121,6 +122,9 @@ struct CrossParams {
 // score[i * C + r] (INT32_MIN for UINT32_MAX entries; out-of-range
 // candidates raise kErrInput)
 cudaError_t cross_rescore(const CrossParams& X, const uint32_t* cand, uint32_t C, int32_t* score, cudaStream_t s);
+// Both in one bit-parallel kernel, for dictionaries of a step class (m, x);
+// R.rec: the word records of the candidates' set.
+cudaError_t rescore_topk_bits(const RescoreBits& R, int m, int x, int sms, cudaStream_t s);
 // each row's k best (score desc, index asc) of its C scored candidates
 cudaError_t select_topk(const uint32_t* cand, const int32_t* score, uint32_t n, uint32_t C, uint32_t k,
                         uint32_t* out_idx, int16_t* out_score, cudaStream_t s);

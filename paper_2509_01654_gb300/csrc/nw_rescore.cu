@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "nw_bitpairs.cuh"
 #include "nw_dp.cuh"
 #include "nw_launch.h"
 #include "nw_proposal.h"
@@ -297,7 +298,52 @@ __global__ void __launch_bounds__(128) rescore2_kernel(const PairsParams P, cons
 
 }  // namespace
 
+namespace {
+// word records of RescoreBits, one thread per word (original index)
+__global__ void __launch_bounds__(256) word_records_kernel(const uint32_t* __restrict__ rank,
+                                                           const uint8_t* __restrict__ slen,
+                                                           const uint32_t* __restrict__ aoff,
+                                                           const uint32_t* __restrict__ sym, uint32_t shift, uint32_t n,
+                                                           uint4* __restrict__ rec) {
+  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const uint32_t r = __ldg(rank + j), len = __ldg(slen + r), ao = __ldg(aoff + r);
+  uint32_t w[4] = {len, 0u, 0u, 0u};
+  if (len > (uint32_t)kRecCodes) {
+    w[1] = ao;
+  } else {
+#pragma unroll
+    for (int x = 0; x < kRecCodes; ++x)
+      if ((uint32_t)x < len) w[(x + 1) >> 2] |= ((__ldg(sym + ao + x) & 0xffffu) >> shift) << (8 * ((x + 1) & 3));
+  }
+  rec[j] = make_uint4(w[0], w[1], w[2], w[3]);
+}
+}  // namespace
+
+cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const uint32_t* aoff, const uint32_t* sym,
+                                uint32_t shift, uint32_t n, uint4* rec, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  word_records_kernel<<<(n + 255) / 256, 256, 0, s>>>(rank, slen, aoff, sym, shift, n, rec);
+  return cudaGetLastError();
+}
+
 namespace prop {
+
+cudaError_t rescore_topk_bits(const RescoreBits& R, int m, int x, int sms, cudaStream_t s) {
+  if (R.rows == 0) return cudaSuccess;
+  const void* fn = bit_rescore(m, x);
+  if (!fn) return cudaErrorInvalidValue;
+  const size_t smem = kRescoreWarps * rescore_warp_bytes(R.alphabet, R.C);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int occ = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kRescoreWarps * 32, smem);
+  if (e != cudaSuccess) return e;
+  const uint64_t blocks = (R.rows + kRescoreWarps - 1) / kRescoreWarps;
+  RescoreBits arg = R;
+  void* args[] = {&arg};
+  return cudaLaunchKernel(fn, dim3((unsigned)std::min<uint64_t>(blocks, (uint64_t)std::max(1, occ) * sms)),
+                          dim3(kRescoreWarps * 32), args, smem, s);
+}
 
 size_t rescore_scratch_bytes(uint32_t n, uint32_t C) {
   const size_t m = (size_t)n * ((C + 1) / 2);

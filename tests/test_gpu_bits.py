@@ -61,3 +61,37 @@ def test_largest_alphabet_and_matrix(ctx, oracle_mod):
     assert np.array_equal(d.all_pairs_matrix().astype(np.int32), oracle_mod.all_pairs(w, (1, -1, -1)))
     assert np.array_equal(d.all_pairs_matrix_chunked(10007).astype(np.int32), oracle_mod.all_pairs(w, (1, -1, -1)))
     d.free()
+
+
+# words of up to 15 symbols (whole in a record), 32 (one 32-bit column word) and 40; few pairs read no records
+@pytest.mark.parametrize("sc", SCORINGS[:10])
+@pytest.mark.parametrize("top", [15, 32, 40])
+@pytest.mark.parametrize("m", [30, 3001])
+def test_explicit_pairs(ctx, oracle_mod, sc, top, m):
+    lengths = np.concatenate([np.arange(top + 1), np.random.default_rng(7).integers(0, top + 1, 300)])
+    w = _words(lengths, 5, 8 + top)
+    d = ctx.load_dictionary(w.codes, w.offsets, w.alphabet, sc)
+    r = np.random.default_rng(m)
+    i, j = r.integers(0, w.n, m).astype(np.uint32), r.integers(0, w.n, m).astype(np.uint32)
+    assert np.array_equal(d.score_pairs(i, j).astype(np.int32), oracle_mod.score_pairs(w, i, j, sc))
+    d.free()
+
+
+@pytest.mark.parametrize("sc", SCORINGS[:10])
+@pytest.mark.parametrize("C,k", [(1, 1), (31, 40), (257, 10), (512, 128)])
+def test_rescoring_every_class(ctx, oracle_mod, sc, C, k):
+    w = _words(np.random.default_rng(9).integers(0, 41, 530), 4, 10)
+    d = ctx.load_dictionary(w.codes, w.offsets, w.alphabet, sc)
+    r = np.random.default_rng(C)
+    cand = np.array([r.permutation(np.delete(np.arange(w.n), row))[:C] for row in range(w.n)]).astype(np.uint32)
+    cand[r.random(cand.shape) < 0.1] = nw.MISSING_IDX
+    idx, score = nw.rescore_topk(d, cand, k)
+    full = np.zeros((w.n, w.n), np.int64)
+    full[np.triu_indices(w.n, 1)] = oracle_mod.all_pairs(w, sc)
+    full += full.T
+    for row in range(0, w.n, 13):
+        c = cand[row][cand[row] != nw.MISSING_IDX].astype(np.int64)
+        c = c[np.lexsort((c, -full[row, c]))][:k]
+        assert np.array_equal(idx[row, :c.size], c) and np.array_equal(score[row, :c.size], full[row, c])
+        assert (idx[row, c.size:] == nw.MISSING_IDX).all() and (score[row, c.size:] == nw.MISSING_SCORE).all()
+    d.free()
