@@ -697,18 +697,6 @@ __global__ void interleave_kernel(const uint32_t* pi, const uint32_t* pj, int m,
   widx[2 * p + 1] = pj[p];
 }
 
-__global__ void take_kernel(const uint32_t* src, uint32_t base, int count, uint32_t* out) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x < count) out[x] = src[base + (uint32_t)x];
-}
-
-__global__ void scatter_rows_kernel(const float* __restrict__ E, const uint32_t* widx, int Bw, float* dst) {
-  const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= (size_t)Bw * kOut) return;
-  const size_t w = x / kOut;
-  dst[(size_t)widx[w] * kOut + (x - w * kOut)] = E[x];
-}
-
 inline unsigned blocks_for(size_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
 
 // log2 of a channel count (32 or 128: the views index taps by shifts)
@@ -832,18 +820,6 @@ cudaError_t pair_targets(const int16_t* score, const uint32_t* pi, const uint32_
 cudaError_t interleave_pairs(const uint32_t* pi, const uint32_t* pj, int m, uint32_t* widx, cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   interleave_kernel<<<blocks_for(m, 256), 256, 0, s>>>(pi, pj, m, widx);
-  return cudaGetLastError();
-}
-
-cudaError_t take(const uint32_t* src, uint32_t base, int count, uint32_t* out, cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  take_kernel<<<blocks_for(count, 256), 256, 0, s>>>(src, base, count, out);
-  return cudaGetLastError();
-}
-
-cudaError_t scatter_rows(const float* E, const uint32_t* widx, int Bw, float* dst, cudaStream_t s) {
-  if (Bw <= 0) return cudaSuccess;
-  scatter_rows_kernel<<<blocks_for((size_t)Bw * kOut, 256), 256, 0, s>>>(E, widx, Bw, dst);
   return cudaGetLastError();
 }
 

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "nw_internal.cuh"
+
 namespace nw {
 namespace cnn {
 
@@ -139,10 +141,12 @@ cudaError_t draw_pairs(const PairDraw& d, uint32_t* pi, uint32_t* pj, uint32_t* 
 cudaError_t pair_targets(const int16_t* score, const uint32_t* pi, const uint32_t* pj, const uint32_t* rank,
                          const uint8_t* slen, int m, float raw_scale, float* target, cudaStream_t s);
 cudaError_t interleave_pairs(const uint32_t* pi, const uint32_t* pj, int m, uint32_t* widx, cudaStream_t s);
-// out[x] = src[base + x]
-cudaError_t take(const uint32_t* src, uint32_t base, int count, uint32_t* out, cudaStream_t s);
-// dst[widx[w] * 64 + d] = E[w * 64 + d]
-cudaError_t scatter_rows(const float* E, const uint32_t* widx, int Bw, float* dst, cudaStream_t s);
+// embeddings of all words of a set into out[original index][64], on at most
+// `sms` SMs; `pack` holds embed_pack_bytes() of scratch
+size_t embed_pack_bytes();
+cudaError_t embed_words(const float* params, const Layout& L, uint32_t alphabet, const Buckets& bk, const uint32_t* sym,
+                        const uint32_t* perm, uint32_t shift, void* pack, float* out, uint32_t* err, int sms,
+                        cudaStream_t s);
 
 }  // namespace cnn
 }  // namespace nw

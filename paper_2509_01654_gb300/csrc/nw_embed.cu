@@ -1,0 +1,423 @@
+// nw_embed.cu -- embeddings of a word set: the character CNN's whole forward pass
+// (embedding, three convolutions, mean, linear layer) in one kernel, on the
+// fifth-generation tensor cores.  Training keeps the layer-by-layer products of
+// nw_cnn.cu, whose activations its backward pass reads.
+//
+// Layer by layer, the float32 activations of 128 channels a position went
+// through memory between the products (600k words: 2.5 GB written and three
+// times that read), through registers into shared memory, and 128 x 128 tiles of
+// K = 96 or 384 were too short to hide it: 9.3 ms, 7 % of the tensor pipe.
+// Here a position's activations never leave the SM.
+//
+//   * Rows.  A block is 128 rows of one word length L: each word's L positions
+//     followed by one zero row, floor(129 / (L + 1)) words (at most 64).  The
+//     zero rows are the convolutions' padding, for both neighbours.
+//   * Activations are kept as bf16 in the canonical K-major layout without
+//     swizzle, in chunks of 8 channels: row r of a chunk at 16 (r + 1).  Rows are
+//     then 16 bytes apart everywhere, so the operand of the tap at t - 1, t or
+//     t + 1 is the same matrix from 0, 16 or 32 bytes in: no im2col copies.
+//     Every value is rounded to bf16 (nearest even) once, when it becomes an
+//     operand, as in the layer-by-layer products, and the products of an output
+//     are added in the same order, so the embeddings are the same bit for bit.
+//   * A CTA (one per SM, persistent) works on two blocks at a time, a layer of
+//     one and then the same layer of the other: each 8 KiB piece of weights
+//     (K = 32), streamed from L2 through a ring that holds one layer, feeds the
+//     products of both, and the products of one block run under the other's
+//     epilogue.  Four worker warps a block stage the embeddings, turn each
+//     layer's accumulator (tensor memory) into the next operand in place (bias,
+//     ReLU, zero rows), sum the last layer's positions in their order, and write
+//     the linear layer's outputs; one thread streams weights, one issues
+//     products.
+// Every wait is bounded; when one runs out the CTA sets kErrWait, waits (bounded)
+// for the copies and products it issued, frees its tensor memory and returns.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "nw_cnn.h"
+#include "nw_internal.cuh"
+#include "nw_tc.cuh"
+
+namespace nw {
+namespace cnn {
+namespace {
+
+constexpr int kRows = 128;                   // rows of a block
+constexpr int kChunkA = (kRows + 2) * 16;    // bytes of an activation chunk: rows -1 .. 128
+constexpr int kActBytes = (kCh / 8) * kChunkA;  // activations of a block
+constexpr int kPieceBytes = 8192;            // K = 32 of a layer's weights
+constexpr int kPieces1 = 3, kPieces2 = 12, kPiecesL = 2;
+constexpr int kPiecesTile = kPieces1 + 2 * kPieces2 + kPiecesL;
+constexpr int kRing = kPieces2;              // a whole layer: both blocks read a piece before it is replaced
+constexpr int kGroup = 128;                  // worker threads of a block
+constexpr int kThreads = 2 * kGroup + 64;
+constexpr int kMaxWords = 64;                // words of a block
+constexpr int kSliceStride = kRows + 1;      // pooling: floats between two channels of a 32-channel slice
+constexpr int kOffRing = 0;
+constexpr int kOffAct = kOffRing + kRing * kPieceBytes;  // two blocks
+// after the last convolution a block's activations give way to a slice of its
+// outputs and to the pooled operand, 64 rows (the product's other 64 rows read
+// what lies behind; their outputs are not used)
+constexpr int kOffPooled = 32 * kSliceStride * 4;
+constexpr int kPooledChunk = kMaxWords * 16;
+constexpr int kOffBias = kOffAct + 2 * kActBytes;        // b1, b2, b3, bl
+constexpr int kOffFirst = kOffBias + (3 * kCh + kOut) * 4;  // EmbedArgs::first, 64 entries
+constexpr int kOffBars = kOffFirst + 64 * 4;
+constexpr int kSmem = kOffBars + (2 * kRing + 4) * 8;
+static_assert(kOffPooled % 16 == 0 && kOffPooled + (kCh / 8) * kPooledChunk <= kActBytes, "the pooled operand fits");
+static_assert(kOffPooled + (kCh / 8) * kPooledChunk + 1024 <= kActBytes + (kSmem - kOffBias), "its unused rows are shared memory");
+static_assert(kMaxLen <= kRows && kBuckets <= 63, "a word fits a block; lengths in two ballots");
+static_assert(kSmem <= 227 * 1024 && kEmb == 32 && kCh == 128 && kOut == 64, "one CTA per SM, fixed shapes");
+constexpr long long kWaitCycles = 2000000000ll;  // about a second
+constexpr uint32_t kIdesc = tc::idesc_bf16(kRows, kCh), kIdescL = tc::idesc_bf16(kRows, kOut);
+constexpr uint32_t kTmemCols = 512;  // a block's accumulator at 128 b, its linear layer's at 256 + 64 b
+
+// the weights as the products read them, in the order of use: chunks of 8 K
+// values, [row][8] each (W1 12 chunks, W2 and W3 48, Wl 16 of 64 rows)
+constexpr size_t kPackBytes = (size_t)kPiecesTile * kPieceBytes;
+
+__global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restrict__ W, Layout L, __nv_bfloat16* out) {
+  const int x = blockIdx.x * 256 + threadIdx.x;
+  if (x >= (int)(kPackBytes / 2)) return;
+  constexpr int n1 = kCh * 3 * kEmb, n2 = kCh * 3 * kCh;
+  const float* src;
+  int K, rows, at;
+  if (x < n1) {
+    src = W + L.W1; K = 3 * kEmb; rows = kCh; at = x;
+  } else if (x < n1 + n2) {
+    src = W + L.W2; K = 3 * kCh; rows = kCh; at = x - n1;
+  } else if (x < n1 + 2 * n2) {
+    src = W + L.W3; K = 3 * kCh; rows = kCh; at = x - n1 - n2;
+  } else {
+    src = W + L.Wl; K = kCh; rows = kOut; at = x - n1 - 2 * n2;
+  }
+  const int chunk = at / (rows * 8), r = at / 8 % rows, k = chunk * 8 + at % 8;
+  out[x] = __float2bfloat16_rn(src[(size_t)r * K + k]);
+}
+
+struct EmbedArgs {
+  const float* params;
+  Layout L;
+  const __nv_bfloat16* pack;
+  const uint32_t* sym;   // the set's symbols (a_enc) and original indices by sorted position
+  const uint32_t* perm;
+  uint32_t shift, alphabet;
+  uint32_t nblocks;
+  // by length: first block, words, first sorted position, first symbol
+  uint32_t first[kBuckets + 1], count[kBuckets], start[kBuckets], base[kBuckets];
+  float* out;            // n x kOut, original order
+  uint32_t* err;
+};
+
+struct Block {
+  uint32_t L, words, pos, sym;  // length, words, first sorted position, first symbol
+};
+
+__host__ __device__ constexpr uint32_t block_words(uint32_t L) {
+  return 129u / (L + 1u) < (uint32_t)kMaxWords ? 129u / (L + 1u) : (uint32_t)kMaxWords;
+}
+
+// block b, by a whole warp; `first` is EmbedArgs::first padded to 64 entries
+__device__ __forceinline__ Block block_of(const EmbedArgs& P, const uint32_t* first, uint32_t b) {
+  Block k{0u, 0u, 0u, 0u};
+  if (b >= P.nblocks) return k;
+  const int lane = threadIdx.x & 31;
+  const uint32_t L = (uint32_t)__popc(__ballot_sync(~0u, b >= first[lane + 1])) +
+                     (uint32_t)__popc(__ballot_sync(~0u, lane < 31 && b >= first[(lane + 33) & 63]));
+  const uint32_t w0 = (b - first[L]) * block_words(L);
+  k.L = L;
+  k.words = min(block_words(L), P.count[L] - w0);
+  k.pos = P.start[L] + w0;
+  k.sym = P.base[L] + w0 * L;
+  return k;
+}
+
+// this block's worker threads agree on `ok`
+__device__ __forceinline__ bool group_and(int blk, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred.aligned q, %2, %3, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)ok), "r"(1 + blk), "n"(kGroup)
+      : "memory");
+  return r != 0u;
+}
+__device__ __forceinline__ void group_sync(int blk) {
+  asm volatile("barrier.cta.sync.aligned %0, %1;\n" ::"r"(1 + blk), "n"(kGroup) : "memory");
+}
+
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+__global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constant__ EmbedArgs P) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ uint32_t s_tmem;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* s_bias = reinterpret_cast<float*>(smem + kOffBias);
+  const uint32_t bar0 = tc::smem_u32(smem + kOffBars);
+  auto full_bar = [&](uint32_t s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](uint32_t s) { return bar0 + 8u * (kRing + s); };
+  // by block: an operand is staged (its warps); a layer's products are done
+  auto ready_bar = [&](uint32_t b) { return bar0 + 8u * (2 * kRing + b); };
+  auto acc_bar = [&](uint32_t b) { return bar0 + 8u * (2 * kRing + 2 + b); };
+  uint32_t* s_first = reinterpret_cast<uint32_t*>(smem + kOffFirst);
+  const uint32_t tiles = (P.nblocks + 1u) / 2u;
+  const float* W = P.params;
+  for (int x = tid; x < kCh; x += kThreads) {
+    s_bias[x] = W[P.L.b1 + x];
+    s_bias[kCh + x] = W[P.L.b2 + x];
+    s_bias[2 * kCh + x] = W[P.L.b3 + x];
+    if (x < kOut) s_bias[3 * kCh + x] = W[P.L.bl + x];
+    if (x < 64) s_first[x] = x <= kBuckets ? P.first[x] : ~0u;
+  }
+  if (tid == 0) {
+    for (uint32_t s = 0; s < (uint32_t)kRing; ++s) {
+      tc::mbar_init(full_bar(s), 1);
+      tc::mbar_init(empty_bar(s), 1);
+    }
+    for (uint32_t b = 0; b < 2u; ++b) {
+      tc::mbar_init(ready_bar(b), kGroup / 32);
+      tc::mbar_init(acc_bar(b), 1);
+    }
+    tc::mbar_init_fence();
+  }
+  if (warp == 0) tc::tmem_alloc(tc::smem_u32(&s_tmem), kTmemCols);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tbase = s_tmem;
+
+  if (warp == 2 * kGroup / 32) {
+    // ---- weights: every tile's pieces, in order, through the ring
+    if (lane == 0) {
+      uint32_t u = 0;  // pieces issued
+      bool ok = true;
+      for (uint32_t t = blockIdx.x; ok && t < tiles; t += gridDim.x)
+        for (uint32_t p = 0; p < (uint32_t)kPiecesTile; ++p, ++u) {
+          const uint32_t s = u % kRing;
+          if (u >= (uint32_t)kRing && !tc::mbar_wait(empty_bar(s), (u / kRing - 1u) & 1u, kWaitCycles)) {
+            atomicOr(P.err, kErrWait);
+            ok = false;
+            break;
+          }
+          tc::mbar_expect_tx(full_bar(s), kPieceBytes);
+          tc::bulk_g2s(tc::smem_u32(smem + kOffRing + s * kPieceBytes),
+                       reinterpret_cast<const unsigned char*>(P.pack) + (size_t)p * kPieceBytes, kPieceBytes, full_bar(s));
+        }
+      // every copy issued has landed before the CTA exits (bounded)
+      for (uint32_t v = u > (uint32_t)kRing ? u - kRing : 0u; v < u; ++v)
+        if (!tc::mbar_wait(full_bar(v % kRing), (v / kRing) & 1u, kWaitCycles)) {
+          atomicOr(P.err, kErrWait);
+          break;
+        }
+    }
+  } else if (warp == 2 * kGroup / 32 + 1) {
+    // ---- products
+    if (lane == 0) {
+      uint32_t u = 0, layers = 0;  // pieces of finished layers, finished layers
+      bool ok = true;
+      for (uint32_t t = blockIdx.x; ok && t < tiles; t += gridDim.x)
+        for (uint32_t layer = 0; ok && layer < 4u; ++layer) {
+          const uint32_t pieces = layer == 0u ? kPieces1 : (layer == 3u ? kPiecesL : kPieces2);
+          for (uint32_t b = 0; b < 2u; ++b) {
+            const uint32_t act = tc::smem_u32(smem + kOffAct + b * kActBytes), pooled = act + (uint32_t)kOffPooled;
+            ok = ok && tc::mbar_wait(ready_bar(b), layers & 1u, kWaitCycles);
+            for (uint32_t p = 0; ok && p < pieces; ++p) {
+              const uint32_t s = (u + p) % kRing;
+              if (b == 0u) ok = tc::mbar_wait(full_bar(s), ((u + p) / kRing) & 1u, kWaitCycles);
+              if (!ok) break;
+              tc::fence_after();
+              const uint32_t w = tc::smem_u32(smem + kOffRing + s * kPieceBytes);
+              if (layer < 3u) {
+                const uint32_t tap = layer == 0u ? p : p >> 2, chunk = layer == 0u ? 0u : (p & 3u) * 4u;
+#pragma unroll
+                for (uint32_t ks = 0; ks < 2u; ++ks)
+                  tc::mma(tbase + b * (uint32_t)kCh,
+                          tc::smem_desc(act + tap * 16u + (chunk + 2u * ks) * (uint32_t)kChunkA, (uint32_t)kChunkA, 128u, 0u),
+                          tc::smem_desc(w + ks * 2u * 2048u, 2048u, 128u, 0u), kIdesc, p + ks > 0u ? 1u : 0u);
+              } else {
+#pragma unroll
+                for (uint32_t ks = 0; ks < 4u; ++ks)
+                  tc::mma(tbase + 256u + b * (uint32_t)kOut,
+                          tc::smem_desc(pooled + (8u * p + 2u * ks) * (uint32_t)kPooledChunk, (uint32_t)kPooledChunk, 128u, 0u),
+                          tc::smem_desc(w + ks * 2u * 1024u, 1024u, 128u, 0u), kIdescL, p + ks > 0u ? 1u : 0u);
+              }
+              if (b == 1u) tc::commit(empty_bar(s));
+            }
+            // after a wait that ran out too, so that the exit can wait for what was issued
+            tc::commit(acc_bar(b));
+          }
+          u += pieces;
+          ++layers;
+        }
+      if (!ok) atomicOr(P.err, kErrWait);
+      // the products issued have completed before tensor memory is freed
+      if (layers)
+        for (uint32_t b = 0; b < 2u; ++b)
+          if (!tc::mbar_wait(acc_bar(b), (layers - 1u) & 1u, kWaitCycles)) atomicOr(P.err, kErrWait);
+    }
+  } else {
+    // ---- workers: thread = row `r` of block `blk`
+    const int blk = warp >> 2, r = tid & (kGroup - 1);
+    unsigned char* act = smem + kOffAct + blk * kActBytes;
+    const uint32_t lane_base = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+    uint32_t layers = 0;
+    bool ok = true;
+    auto publish = [&]() {  // this warp's part of an operand, for the tensor cores
+      tc::fence_proxy_async();
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(ready_bar((uint32_t)blk));
+    };
+    auto products_done = [&]() {
+      const bool got = tc::mbar_wait(acc_bar((uint32_t)blk), layers & 1u, kWaitCycles);
+      ++layers;
+      ok = group_and(blk, got);
+      if (!ok && r == 0) atomicOr(P.err, kErrWait);
+      tc::fence_after();
+      return ok;
+    };
+    for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+      const Block k = block_of(P, s_first, 2u * t + (uint32_t)blk);
+      const uint32_t w = (uint32_t)r / (k.L + 1u), at = (uint32_t)r % (k.L + 1u);
+      const bool real = w < k.words && at < k.L;
+      // embeddings, and the rows around the block (pooling has overwritten them)
+      {
+        uint4 q[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[c] = make_uint4(0u, 0u, 0u, 0u);
+        if (real) {
+          const uint32_t code = (__ldg(P.sym + k.sym + w * k.L + at) & 0xffffu) >> P.shift;
+          if (code >= P.alphabet) {
+            atomicOr(P.err, kErrInput);
+          } else {
+            const float4* e = reinterpret_cast<const float4*>(W + P.L.emb + (size_t)code * kEmb);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float4 a = __ldg(e + 2 * c), b = __ldg(e + 2 * c + 1);
+              q[c] = make_uint4(pack2(a.x, a.y), pack2(a.z, a.w), pack2(b.x, b.y), pack2(b.z, b.w));
+            }
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(act + c * kChunkA + (r + 1) * 16) = q[c];
+        if (r < 2 * (kCh / 8))
+          *reinterpret_cast<uint4*>(act + (r >> 1) * kChunkA + (r & 1) * (kRows + 1) * 16) = make_uint4(0u, 0u, 0u, 0u);
+      }
+      publish();
+      // layers 1 and 2: the accumulator becomes the next operand, in place
+#pragma unroll 1
+      for (int layer = 0; layer < 2; ++layer) {
+        if (!products_done()) break;
+        const float4* bias = reinterpret_cast<const float4*>(s_bias + layer * kCh);
+#pragma unroll 1
+        for (int c = 0; c < kCh; c += 32) {
+          uint32_t v[32];
+          tc::tmem_ld32(lane_base + (uint32_t)(blk * kCh + c), v);
+          tc::tmem_wait(v);
+#pragma unroll
+          for (int j = 0; j < 32; j += 8) {
+            const float4 b0 = bias[(c + j) >> 2], b1 = bias[((c + j) >> 2) + 1];
+            auto f = [&](int x, float b) { return real ? fmaxf(__uint_as_float(v[j + x]) + b, 0.f) : 0.f; };
+            *reinterpret_cast<uint4*>(act + ((c + j) >> 3) * kChunkA + (r + 1) * 16) =
+                make_uint4(pack2(f(0, b0.x), f(1, b0.y)), pack2(f(2, b0.z), f(3, b0.w)), pack2(f(4, b1.x), f(5, b1.y)),
+                           pack2(f(6, b1.z), f(7, b1.w)));
+          }
+        }
+        publish();
+      }
+      // layer 3: 32 channels at a time to shared memory, each word's positions
+      // added in their order (lane = channel), the mean as the linear layer's operand
+      if (!ok || !products_done()) break;
+      float* slice = reinterpret_cast<float*>(act);
+#pragma unroll 1
+      for (int c = 0; c < kCh; c += 32) {
+        uint32_t v[32];
+        tc::tmem_ld32(lane_base + (uint32_t)(blk * kCh + c), v);
+        tc::tmem_wait(v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          slice[j * kSliceStride + r] = fmaxf(__uint_as_float(v[j]) + s_bias[2 * kCh + c + j], 0.f);
+        group_sync(blk);
+        const int ch = c + lane;
+        unsigned char* dst = act + kOffPooled + (ch >> 3) * kPooledChunk + (ch & 7) * 2;
+#pragma unroll 1
+        for (uint32_t x = (uint32_t)(warp & 3); x < k.words; x += 4u) {
+          const float* y = slice + lane * kSliceStride + (int)(x * (k.L + 1u));
+          float acc = 0.f;
+#pragma unroll 4
+          for (uint32_t p = 0; p < k.L; ++p) acc += y[p];
+          *reinterpret_cast<__nv_bfloat16*>(dst + x * 16u) = __float2bfloat16_rn(k.L > 0u ? acc / (float)k.L : 0.f);
+        }
+        group_sync(blk);
+      }
+      publish();
+      if (!products_done()) break;
+      if (r < kMaxWords) {  // thread = word: its 64 outputs
+        const bool have = (uint32_t)r < k.words;
+        float* dst = have ? P.out + (size_t)__ldg(P.perm + k.pos + (uint32_t)r) * kOut : nullptr;
+#pragma unroll 1
+        for (int c = 0; c < kOut; c += 32) {
+          uint32_t v[32];
+          tc::tmem_ld32(lane_base + 256u + (uint32_t)(blk * kOut + c), v);
+          tc::tmem_wait(v);
+          if (have) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+              const float4 b = *reinterpret_cast<const float4*>(s_bias + 3 * kCh + c + j);
+              *reinterpret_cast<float4*>(dst + c + j) =
+                  make_float4(__uint_as_float(v[j]) + b.x, __uint_as_float(v[j + 1]) + b.y, __uint_as_float(v[j + 2]) + b.z,
+                              __uint_as_float(v[j + 3]) + b.w);
+            }
+          }
+          __syncwarp();
+        }
+      }
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (warp == 0) tc::tmem_dealloc(tbase, kTmemCols);
+}
+
+}  // namespace
+
+size_t embed_pack_bytes() { return kPackBytes; }
+
+cudaError_t embed_words(const float* params, const Layout& L, uint32_t alphabet, const Buckets& bk, const uint32_t* sym,
+                        const uint32_t* perm, uint32_t shift, void* pack, float* out, uint32_t* err, int sms,
+                        cudaStream_t s) {
+  EmbedArgs P{};
+  P.params = params;
+  P.L = L;
+  P.pack = static_cast<const __nv_bfloat16*>(pack);
+  P.sym = sym;
+  P.perm = perm;
+  P.shift = shift;
+  P.alphabet = alphabet;
+  P.out = out;
+  P.err = err;
+  for (int len = 0; len < kBuckets; ++len) {
+    P.first[len] = P.nblocks;
+    P.count[len] = bk.count[len];
+    P.start[len] = bk.start[len];
+    P.base[len] = bk.aenc_base[len];
+    P.nblocks += (bk.count[len] + block_words((uint32_t)len) - 1) / block_words((uint32_t)len);
+  }
+  P.first[kBuckets] = P.nblocks;
+  if (P.nblocks == 0) return cudaSuccess;
+  pack_weights_kernel<<<(unsigned)((kPackBytes / 2 + 255) / 256), 256, 0, s>>>(params, L, static_cast<__nv_bfloat16*>(pack));
+  cudaError_t e = cudaFuncSetAttribute(embed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  embed_kernel<<<std::min<unsigned>((P.nblocks + 1u) / 2u, (unsigned)sms), kThreads, kSmem, s>>>(P);
+  return cudaGetLastError();
+}
+
+}  // namespace cnn
+}  // namespace nw

@@ -32,7 +32,7 @@ struct nw_model {
   uint32_t cap_pairs = 0;
   DevBuf pi, pj, target, score16;
   // proposal path
-  DevBuf Eall, Qb, qbias, topbuf, cand, cand_dot, cand_score, nbr;
+  DevBuf Eall, Wpack, Qb, qbias, topbuf, cand, cand_dot, cand_score, nbr;
   // queries against a dictionary: its quantised rows, kept while the
   // dictionary (serial) and the parameters (gen) are unchanged
   uint64_t gen = 1, prep_serial = 0, prep_gen = 0;
@@ -56,8 +56,6 @@ prop::DotDebug dot_debug(const nw_ctx* c) {
   d.withhold = c->dbg_withhold_tile;
   return d;
 }
-
-constexpr int kMaxRowsPerPass = 1 << 20;  // packed positions per forward pass of nw_model_embed
 
 // codes of the dictionary's words from sorted position p0 on (contiguous in
 // a_enc: every symbol e(c) = c << shift replicated in both 16-bit halves)
@@ -107,7 +105,7 @@ void model_free_buffers(nw_model* M) {
                     &M->dYb, &M->dX0, &M->pi, &M->pj, &M->target, &M->score16, &M->Eall, &M->Qb,
                     &M->qbias, &M->topbuf, &M->cand, &M->cand_dot, &M->cand_score, &M->nbr,
                     &M->dQb, &M->dqbias, &M->prep_small, &M->qQb, &M->qcand, &M->qcand_dot, &M->qscore, &M->qbuf,
-                    &M->xcodes, &M->xoffs, &M->xidx, &M->xscore, &M->oQb, &M->obias, &M->operm, &M->oscratch};
+                    &M->xcodes, &M->xoffs, &M->xidx, &M->xscore, &M->oQb, &M->obias, &M->operm, &M->oscratch, &M->Wpack};
   for (DevBuf* b : bufs) ctx_free(c, *b);
 }
 
@@ -176,15 +174,15 @@ cnn::WordSrc word_src(const WordSet& ws, uint32_t shift, const uint32_t* widx) {
   return s;
 }
 
-// embeddings of Bw words of `ws` (M->widx), packed into at most Tmax rows, into M->E
-nw_status forward(nw_model* M, const WordSet& ws, uint32_t shift, int Bw, int Tmax, cudaStream_t s) {
+// embeddings of Bw words of the dictionary (M->widx), packed into at most Tmax rows, into M->E
+nw_status forward(nw_model* M, const nw_dict* d, int Bw, int Tmax, cudaStream_t s) {
   nw_ctx* c = M->ctx;
   const cnn::Layout& L = M->L;
   const float* W = fptr(M->params);
   const cnn::Packed pk = packed(M, Bw, Tmax);
   cnn::PackBufs pb{M->len.as<int>(), M->off.as<int>(), rows_ptr(M), M->rinfo.as<int>(), M->rword.as<int>(),
                    M->codes.as<int32_t>()};
-  NW_CK(cnn::pack_words(word_src(ws, shift, M->widx.as<uint32_t>()), Bw, Tmax, W + L.emb, pb, fptr(M->X0),
+  NW_CK(cnn::pack_words(word_src(d->ws, d->ss.shift, M->widx.as<uint32_t>()), Bw, Tmax, W + L.emb, pb, fptr(M->X0),
                         err_ptr(M), M->alphabet, s));
   cnn::Epi e;
   e.relu = true;
@@ -201,10 +199,6 @@ nw_status forward(nw_model* M, const WordSet& ws, uint32_t shift, int Bw, int Tm
   el.err = err_ptr(M);
   NW_CK(cnn::lin_fwd(fptr(M->P), cnn::kCh, W + L.Wl, cnn::kOut, Bw, fptr(M->E), el, s));
   return NW_OK;
-}
-
-nw_status forward(nw_model* M, const nw_dict* d, int Bw, int Tmax, cudaStream_t s) {
-  return forward(M, d->ws, d->ss.shift, Bw, Tmax, s);
 }
 
 // gradient of the pair loss (pairs = word slots 2p, 2p + 1; targets in M->target) into M->grads
@@ -284,44 +278,13 @@ uint64_t splitmix64_next(uint64_t& st) {
   return z ^ (z >> 31);
 }
 
-// embeddings of all n words into M->Eall (n x 64): chunks of consecutive
-// sorted positions (words of similar length), each at most kMaxRowsPerPass
-// packed rows, scattered back to original order
+// embeddings of all words of `ws` into M->Eall (n x 64, original order)
 nw_status embed_all(nw_model* M, const WordSet& ws, uint32_t shift, cudaStream_t s) {
   nw_ctx* c = M->ctx;
-  const uint32_t n = ws.n;
-  const Buckets& bk = ws.bk;
-  // chunk boundaries on the host from the bucket table
-  std::vector<std::pair<uint32_t, uint32_t>> chunks;  // (first sorted position, words)
-  int max_words = 1;
-  {
-    uint32_t p0 = 0;
-    uint64_t rows = 0;
-    for (int Lb = 0; Lb < kBuckets; ++Lb) {
-      for (uint32_t k = 0; k < bk.count[Lb]; ++k) {
-        const uint32_t p = bk.start[Lb] + k;
-        if (rows + (uint64_t)Lb > (uint64_t)kMaxRowsPerPass || p - p0 >= (uint32_t)kMaxRowsPerPass) {
-          chunks.push_back({p0, p - p0});
-          max_words = std::max<int>(max_words, (int)(p - p0));
-          p0 = p;
-          rows = 0;
-        }
-        rows += (uint64_t)Lb;
-      }
-    }
-    if (n > p0) {
-      chunks.push_back({p0, n - p0});
-      max_words = std::max<int>(max_words, (int)(n - p0));
-    }
-  }
-  NW_TRY(ensure_scratch(M, max_words, kMaxRowsPerPass));
-  NW_TRY(ctx_ensure(c, M->Eall, sizeof(float) * std::max<size_t>(1, (size_t)n * cnn::kOut), "embeddings"));
-  for (const auto& ch : chunks) {
-    const int Bw = (int)ch.second;
-    NW_CK(cnn::take(ws.perm.as<uint32_t>(), ch.first, Bw, M->widx.as<uint32_t>(), s));
-    NW_TRY(forward(M, ws, shift, Bw, kMaxRowsPerPass, s));
-    NW_CK(cnn::scatter_rows(fptr(M->E), M->widx.as<uint32_t>(), Bw, fptr(M->Eall), s));
-  }
+  NW_TRY(ctx_ensure(c, M->Eall, sizeof(float) * std::max<size_t>(1, (size_t)ws.n * cnn::kOut), "embeddings"));
+  NW_TRY(ctx_ensure(c, M->Wpack, cnn::embed_pack_bytes(), "packed weights"));
+  NW_CK(cnn::embed_words(fptr(M->params), M->L, M->alphabet, ws.bk, ws.a_enc.as<uint32_t>(), ws.perm.as<uint32_t>(),
+                         shift, M->Wpack.p, fptr(M->Eall), err_ptr(M), c->sm_count, s));
   return NW_OK;
 }
 
