@@ -23,11 +23,12 @@
 //     one and then the same layer of the other: each 8 KiB piece of weights
 //     (K = 32), streamed from L2 through a ring that holds one layer, feeds the
 //     products of both, and the products of one block run under the other's
-//     epilogue.  Four worker warps a block stage the embeddings, turn each
-//     layer's accumulator (tensor memory) into the next operand in place (bias,
-//     ReLU, zero rows), sum the last layer's positions in their order, and write
-//     the linear layer's outputs; one thread streams weights, one issues
-//     products.
+//     epilogue.  Eight worker warps a block (two for each row, half the channels
+//     each: four leave every warp waiting on its own chain, 0.97 ms for 200k
+//     words) stage the embeddings, turn each layer's accumulator (tensor memory)
+//     into the next operand in place (bias, ReLU, zero rows), sum the last
+//     layer's positions in their order, and write the linear layer's outputs; one
+//     thread streams weights, one issues products.
 // Every wait is bounded; when one runs out the CTA sets kErrWait, waits (bounded)
 // for the copies and products it issued, frees its tensor memory and returns.
 #include <cuda_bf16.h>
@@ -51,8 +52,9 @@ constexpr int kPieceBytes = 8192;            // K = 32 of a layer's weights
 constexpr int kPieces1 = 3, kPieces2 = 12, kPiecesL = 2;
 constexpr int kPiecesTile = kPieces1 + 2 * kPieces2 + kPiecesL;
 constexpr int kRing = kPieces2;              // a whole layer: both blocks read a piece before it is replaced
-constexpr int kGroup = 128;                  // worker threads of a block
-constexpr int kThreads = 2 * kGroup + 64;
+constexpr int kHalf = 128;                   // worker threads of half a block's channels
+constexpr int kWorkers = 4 * kHalf / 32;     // worker warps
+constexpr int kThreads = kWorkers * 32 + 64;
 constexpr int kMaxWords = 64;                // words of a block
 constexpr int kSliceStride = kRows + 1;      // pooling: floats between two channels of a 32-channel slice
 constexpr int kOffRing = 0;
@@ -65,8 +67,12 @@ constexpr int kPooledChunk = kMaxWords * 16;
 constexpr int kOffBias = kOffAct + 2 * kActBytes;        // b1, b2, b3, bl
 constexpr int kOffFirst = kOffBias + (3 * kCh + kOut) * 4;  // EmbedArgs::first, 64 entries
 constexpr int kOffBars = kOffFirst + 64 * 4;
-constexpr int kSmem = kOffBars + (2 * kRing + 4) * 8;
-static_assert(kOffPooled % 16 == 0 && kOffPooled + (kCh / 8) * kPooledChunk <= kActBytes, "the pooled operand fits");
+constexpr int kOffSlice = kOffBars + (2 * kRing + 4) * 8;   // the second halves' slices
+constexpr int kOffTable = kOffSlice + 2 * 32 * kSliceStride * 4;  // embeddings in bf16
+constexpr int kMaxAlphabet = 256;            // of a model
+constexpr int kTableRow = 5;                 // 16-byte units of an embedding (four, and one against bank conflicts)
+constexpr int kSmem = kOffTable + kMaxAlphabet * kTableRow * 16;
+static_assert(kOffPooled % 16 == 0 && kOffTable % 16 == 0 && kOffPooled + (kCh / 8) * kPooledChunk <= kActBytes, "the pooled operand fits");
 static_assert(kOffPooled + (kCh / 8) * kPooledChunk + 1024 <= kActBytes + (kSmem - kOffBias), "its unused rows are shared memory");
 static_assert(kMaxLen <= kRows && kBuckets <= 63, "a word fits a block; lengths in two ballots");
 static_assert(kSmem <= 227 * 1024 && kEmb == 32 && kCh == 128 && kOut == 64, "one CTA per SM, fixed shapes");
@@ -134,24 +140,29 @@ __device__ __forceinline__ Block block_of(const EmbedArgs& P, const uint32_t* fi
   return k;
 }
 
-// this block's worker threads agree on `ok`
-__device__ __forceinline__ bool group_and(int blk, bool ok) {
+// a block's worker threads agree on `ok`; a half's threads meet
+__device__ __forceinline__ bool block_and(int blk, bool ok) {
   uint32_t r;
   asm volatile(
       "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred.aligned q, %2, %3, p;\n"
       " selp.u32 %0, 1, 0, q;\n}\n"
       : "=r"(r)
-      : "r"((uint32_t)ok), "r"(1 + blk), "n"(kGroup)
+      : "r"((uint32_t)ok), "r"(1 + blk), "n"(2 * kHalf)
       : "memory");
   return r != 0u;
 }
-__device__ __forceinline__ void group_sync(int blk) {
-  asm volatile("barrier.cta.sync.aligned %0, %1;\n" ::"r"(1 + blk), "n"(kGroup) : "memory");
+__device__ __forceinline__ void half_sync(int blk, int half) {
+  asm volatile("barrier.cta.sync.aligned %0, %1;\n" ::"r"(3 + 2 * blk + half), "n"(kHalf) : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&v);
+}
+// ReLU of two sums rounded to bf16 (rounding keeps the order, so after it), or 0 (`keep` 0)
+__device__ __forceinline__ uint32_t relu2(float a, float b, uint32_t keep) {
+  const __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.f, 0.f));
+  return *reinterpret_cast<const uint32_t*>(&v) & keep;
 }
 
 __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constant__ EmbedArgs P) {
@@ -175,13 +186,19 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
     if (x < kOut) s_bias[3 * kCh + x] = W[P.L.bl + x];
     if (x < 64) s_first[x] = x <= kBuckets ? P.first[x] : ~0u;
   }
+  uint4* s_table = reinterpret_cast<uint4*>(smem + kOffTable);
+  for (uint32_t x = tid; x < P.alphabet * 4u; x += kThreads) {
+    const float4* e = reinterpret_cast<const float4*>(W + P.L.emb) + 2u * x;
+    const float4 a = __ldg(e), b = __ldg(e + 1);
+    s_table[(x >> 2) * kTableRow + (x & 3u)] = make_uint4(pack2(a.x, a.y), pack2(a.z, a.w), pack2(b.x, b.y), pack2(b.z, b.w));
+  }
   if (tid == 0) {
     for (uint32_t s = 0; s < (uint32_t)kRing; ++s) {
       tc::mbar_init(full_bar(s), 1);
       tc::mbar_init(empty_bar(s), 1);
     }
     for (uint32_t b = 0; b < 2u; ++b) {
-      tc::mbar_init(ready_bar(b), kGroup / 32);
+      tc::mbar_init(ready_bar(b), kWorkers / 2);
       tc::mbar_init(acc_bar(b), 1);
     }
     tc::mbar_init_fence();
@@ -192,7 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
   tc::fence_after();
   const uint32_t tbase = s_tmem;
 
-  if (warp == 2 * kGroup / 32) {
+  if (warp == kWorkers) {
     // ---- weights: every tile's pieces, in order, through the ring
     if (lane == 0) {
       uint32_t u = 0;  // pieces issued
@@ -216,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
           break;
         }
     }
-  } else if (warp == 2 * kGroup / 32 + 1) {
+  } else if (warp == kWorkers + 1) {
     // ---- products
     if (lane == 0) {
       uint32_t u = 0, layers = 0;  // pieces of finished layers, finished layers
@@ -262,9 +279,10 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
           if (!tc::mbar_wait(acc_bar(b), (layers - 1u) & 1u, kWaitCycles)) atomicOr(P.err, kErrWait);
     }
   } else {
-    // ---- workers: thread = row `r` of block `blk`
-    const int blk = warp >> 2, r = tid & (kGroup - 1);
+    // ---- workers: thread = row `r` of block `blk`, half its channels
+    const int blk = warp >> 3, half = (warp >> 2) & 1, r = tid & (kHalf - 1);
     unsigned char* act = smem + kOffAct + blk * kActBytes;
+    float* slice = reinterpret_cast<float*>(half ? smem + kOffSlice + blk * (32 * kSliceStride * 4) : act);
     const uint32_t lane_base = tbase + ((uint32_t)((warp & 3) * 32) << 16);
     uint32_t layers = 0;
     bool ok = true;
@@ -277,36 +295,39 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
     auto products_done = [&]() {
       const bool got = tc::mbar_wait(acc_bar((uint32_t)blk), layers & 1u, kWaitCycles);
       ++layers;
-      ok = group_and(blk, got);
+      ok = block_and(blk, got);
       if (!ok && r == 0) atomicOr(P.err, kErrWait);
       tc::fence_after();
       return ok;
     };
-    for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-      const Block k = block_of(P, s_first, 2u * t + (uint32_t)blk);
+    // the row of block (t, blk): whether it holds a symbol, and the symbol
+    Block k;
+    uint32_t sym = 0u;
+    auto row_of = [&](uint32_t t) {
+      k = block_of(P, s_first, 2u * t + (uint32_t)blk);
       const uint32_t w = (uint32_t)r / (k.L + 1u), at = (uint32_t)r % (k.L + 1u);
-      const bool real = w < k.words && at < k.L;
+      const bool have = w < k.words && at < k.L;
+      if (have) sym = __ldg(P.sym + k.sym + w * k.L + at);
+      return have;
+    };
+    bool real = row_of(blockIdx.x);
+    for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+      const uint32_t keep = real ? ~0u : 0u;
       // embeddings, and the rows around the block (pooling has overwritten them)
       {
-        uint4 q[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) q[c] = make_uint4(0u, 0u, 0u, 0u);
+        uint4 q[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
         if (real) {
-          const uint32_t code = (__ldg(P.sym + k.sym + w * k.L + at) & 0xffffu) >> P.shift;
+          const uint32_t code = (sym & 0xffffu) >> P.shift;
           if (code >= P.alphabet) {
             atomicOr(P.err, kErrInput);
           } else {
-            const float4* e = reinterpret_cast<const float4*>(W + P.L.emb + (size_t)code * kEmb);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const float4 a = __ldg(e + 2 * c), b = __ldg(e + 2 * c + 1);
-              q[c] = make_uint4(pack2(a.x, a.y), pack2(a.z, a.w), pack2(b.x, b.y), pack2(b.z, b.w));
-            }
+            q[0] = s_table[code * kTableRow + 2u * half];
+            q[1] = s_table[code * kTableRow + 2u * half + 1u];
           }
         }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(act + c * kChunkA + (r + 1) * 16) = q[c];
-        if (r < 2 * (kCh / 8))
+        for (int c = 0; c < 2; ++c) *reinterpret_cast<uint4*>(act + (2 * half + c) * kChunkA + (r + 1) * 16) = q[c];
+        if (half == 0 && r < 2 * (kCh / 8))
           *reinterpret_cast<uint4*>(act + (r >> 1) * kChunkA + (r & 1) * (kRows + 1) * 16) = make_uint4(0u, 0u, 0u, 0u);
       }
       publish();
@@ -316,17 +337,17 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
         if (!products_done()) break;
         const float4* bias = reinterpret_cast<const float4*>(s_bias + layer * kCh);
 #pragma unroll 1
-        for (int c = 0; c < kCh; c += 32) {
+        for (int c = half * (kCh / 2); c < (half + 1) * (kCh / 2); c += 32) {
           uint32_t v[32];
           tc::tmem_ld32(lane_base + (uint32_t)(blk * kCh + c), v);
           tc::tmem_wait(v);
 #pragma unroll
           for (int j = 0; j < 32; j += 8) {
             const float4 b0 = bias[(c + j) >> 2], b1 = bias[((c + j) >> 2) + 1];
-            auto f = [&](int x, float b) { return real ? fmaxf(__uint_as_float(v[j + x]) + b, 0.f) : 0.f; };
+            auto f = [&](int x) { return __uint_as_float(v[j + x]); };
             *reinterpret_cast<uint4*>(act + ((c + j) >> 3) * kChunkA + (r + 1) * 16) =
-                make_uint4(pack2(f(0, b0.x), f(1, b0.y)), pack2(f(2, b0.z), f(3, b0.w)), pack2(f(4, b1.x), f(5, b1.y)),
-                           pack2(f(6, b1.z), f(7, b1.w)));
+                make_uint4(relu2(f(0) + b0.x, f(1) + b0.y, keep), relu2(f(2) + b0.z, f(3) + b0.w, keep),
+                           relu2(f(4) + b1.x, f(5) + b1.y, keep), relu2(f(6) + b1.z, f(7) + b1.w, keep));
           }
         }
         publish();
@@ -334,49 +355,53 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
       // layer 3: 32 channels at a time to shared memory, each word's positions
       // added in their order (lane = channel), the mean as the linear layer's operand
       if (!ok || !products_done()) break;
-      float* slice = reinterpret_cast<float*>(act);
+      const Block kb = k;  // the next tile's row is read ahead
+      if (t + gridDim.x < tiles) real = row_of(t + gridDim.x);
 #pragma unroll 1
-      for (int c = 0; c < kCh; c += 32) {
+      for (int c = half * (kCh / 2); c < (half + 1) * (kCh / 2); c += 32) {
         uint32_t v[32];
         tc::tmem_ld32(lane_base + (uint32_t)(blk * kCh + c), v);
         tc::tmem_wait(v);
+        const float4* bias = reinterpret_cast<const float4*>(s_bias + 2 * kCh + c);
 #pragma unroll
-        for (int j = 0; j < 32; ++j)
-          slice[j * kSliceStride + r] = fmaxf(__uint_as_float(v[j]) + s_bias[2 * kCh + c + j], 0.f);
-        group_sync(blk);
+        for (int j = 0; j < 32; j += 4) {
+          const float4 b = bias[j >> 2];
+          slice[j * kSliceStride + r] = fmaxf(__uint_as_float(v[j]) + b.x, 0.f);
+          slice[(j + 1) * kSliceStride + r] = fmaxf(__uint_as_float(v[j + 1]) + b.y, 0.f);
+          slice[(j + 2) * kSliceStride + r] = fmaxf(__uint_as_float(v[j + 2]) + b.z, 0.f);
+          slice[(j + 3) * kSliceStride + r] = fmaxf(__uint_as_float(v[j + 3]) + b.w, 0.f);
+        }
+        half_sync(blk, half);
         const int ch = c + lane;
         unsigned char* dst = act + kOffPooled + (ch >> 3) * kPooledChunk + (ch & 7) * 2;
 #pragma unroll 1
-        for (uint32_t x = (uint32_t)(warp & 3); x < k.words; x += 4u) {
-          const float* y = slice + lane * kSliceStride + (int)(x * (k.L + 1u));
+        for (uint32_t x = (uint32_t)(warp & 3); x < kb.words; x += 4u) {
+          const float* y = slice + lane * kSliceStride + (int)(x * (kb.L + 1u));
           float acc = 0.f;
 #pragma unroll 4
-          for (uint32_t p = 0; p < k.L; ++p) acc += y[p];
-          *reinterpret_cast<__nv_bfloat16*>(dst + x * 16u) = __float2bfloat16_rn(k.L > 0u ? acc / (float)k.L : 0.f);
+          for (uint32_t p = 0; p < kb.L; ++p) acc += y[p];
+          *reinterpret_cast<__nv_bfloat16*>(dst + x * 16u) = __float2bfloat16_rn(kb.L > 0u ? acc / (float)kb.L : 0.f);
         }
-        group_sync(blk);
+        half_sync(blk, half);
       }
       publish();
       if (!products_done()) break;
-      if (r < kMaxWords) {  // thread = word: its 64 outputs
-        const bool have = (uint32_t)r < k.words;
-        float* dst = have ? P.out + (size_t)__ldg(P.perm + k.pos + (uint32_t)r) * kOut : nullptr;
-#pragma unroll 1
-        for (int c = 0; c < kOut; c += 32) {
-          uint32_t v[32];
-          tc::tmem_ld32(lane_base + 256u + (uint32_t)(blk * kOut + c), v);
-          tc::tmem_wait(v);
-          if (have) {
+      if (r < kMaxWords) {  // thread = word: 32 of its 64 outputs
+        const bool have = (uint32_t)r < kb.words;
+        uint32_t v[32];
+        tc::tmem_ld32(lane_base + 256u + (uint32_t)(blk * kOut + half * 32), v);
+        tc::tmem_wait(v);
+        if (have) {
+          float* dst = P.out + (size_t)__ldg(P.perm + kb.pos + (uint32_t)r) * kOut + half * 32;
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-              const float4 b = *reinterpret_cast<const float4*>(s_bias + 3 * kCh + c + j);
-              *reinterpret_cast<float4*>(dst + c + j) =
-                  make_float4(__uint_as_float(v[j]) + b.x, __uint_as_float(v[j + 1]) + b.y, __uint_as_float(v[j + 2]) + b.z,
-                              __uint_as_float(v[j + 3]) + b.w);
-            }
+          for (int j = 0; j < 32; j += 4) {
+            const float4 b = *reinterpret_cast<const float4*>(s_bias + 3 * kCh + half * 32 + j);
+            *reinterpret_cast<float4*>(dst + j) =
+                make_float4(__uint_as_float(v[j]) + b.x, __uint_as_float(v[j + 1]) + b.y, __uint_as_float(v[j + 2]) + b.z,
+                            __uint_as_float(v[j + 3]) + b.w);
           }
-          __syncwarp();
         }
+        __syncwarp();
       }
     }
   }
