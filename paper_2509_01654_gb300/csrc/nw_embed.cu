@@ -20,8 +20,8 @@
 //     operand, as in the layer-by-layer products, and the products of an output
 //     are added in the same order, so the embeddings are the same bit for bit.
 //   * A CTA (one per SM, persistent) works on two blocks at a time, a layer of
-//     one and then the same layer of the other: each 8 KiB piece of weights
-//     (K = 32), streamed from L2 through a ring that holds one layer, feeds the
+//     one and then the same layer of the other: each 24 KiB piece of weights
+//     (K = 96), streamed from L2 through a ring that holds one layer, feeds the
 //     products of both, and the products of one block run under the other's
 //     epilogue.  Eight worker warps a block (two for each row, half the channels
 //     each: four leave every warp waiting on its own chain, 0.97 ms for 200k
@@ -48,9 +48,11 @@ namespace {
 constexpr int kRows = 128;                   // rows of a block
 constexpr int kChunkA = (kRows + 2) * 16;    // bytes of an activation chunk: rows -1 .. 128
 constexpr int kActBytes = (kCh / 8) * kChunkA;  // activations of a block
-constexpr int kPieceBytes = 8192;            // K = 32 of a layer's weights
-constexpr int kPieces1 = 3, kPieces2 = 12, kPiecesL = 2;
-constexpr int kPiecesTile = kPieces1 + 2 * kPieces2 + kPiecesL;
+constexpr int kPieceBytes = 24576;           // K = 96 of a convolution's weights
+constexpr int kPieceSteps = 6;               // products of K = 16 in it
+constexpr int kLinBytes = kCh * kOut * 2;    // the linear layer's weights: one shorter piece
+constexpr int kPieces2 = 4;                  // layers 2 and 3; layer 1 and the linear layer have one each
+constexpr int kPiecesTile = 2 + 2 * kPieces2;
 constexpr int kRing = kPieces2;              // a whole layer: both blocks read a piece before it is replaced
 constexpr int kHalf = 128;                   // worker threads of half a block's channels
 constexpr int kWorkers = 4 * kHalf / 32;     // worker warps
@@ -82,7 +84,7 @@ constexpr uint32_t kTmemCols = 512;  // a block's accumulator at 128 b, its line
 
 // the weights as the products read them, in the order of use: chunks of 8 K
 // values, [row][8] each (W1 12 chunks, W2 and W3 48, Wl 16 of 64 rows)
-constexpr size_t kPackBytes = (size_t)kPiecesTile * kPieceBytes;
+constexpr size_t kPackBytes = (size_t)(kPiecesTile - 1) * kPieceBytes + kLinBytes;
 
 __global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restrict__ W, Layout L, __nv_bfloat16* out) {
   const int x = blockIdx.x * 256 + threadIdx.x;
@@ -222,9 +224,10 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
             ok = false;
             break;
           }
-          tc::mbar_expect_tx(full_bar(s), kPieceBytes);
+          const uint32_t bytes = p + 1u < (uint32_t)kPiecesTile ? kPieceBytes : kLinBytes;
+          tc::mbar_expect_tx(full_bar(s), bytes);
           tc::bulk_g2s(tc::smem_u32(smem + kOffRing + s * kPieceBytes),
-                       reinterpret_cast<const unsigned char*>(P.pack) + (size_t)p * kPieceBytes, kPieceBytes, full_bar(s));
+                       reinterpret_cast<const unsigned char*>(P.pack) + (size_t)p * kPieceBytes, bytes, full_bar(s));
         }
       // every copy issued has landed before the CTA exits (bounded)
       for (uint32_t v = u > (uint32_t)kRing ? u - kRing : 0u; v < u; ++v)
@@ -234,42 +237,67 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
         }
     }
   } else if (warp == kWorkers + 1) {
-    // ---- products
+    // ---- products.  One thread issues them all, so its own instructions are on
+    // the critical path: descriptors are constants added to four bases.
     if (lane == 0) {
       uint32_t u = 0, layers = 0;  // pieces of finished layers, finished layers
       bool ok = true;
+      const uint64_t wdesc = tc::smem_desc(tc::smem_u32(smem + kOffRing), 2048u, 128u, 0u);
+      const uint64_t ldesc = tc::smem_desc(tc::smem_u32(smem + kOffRing), 1024u, 128u, 0u);
+      auto piece_full = [&](uint32_t x) { return tc::mbar_wait(full_bar(x % kRing), (x / kRing) & 1u, kWaitCycles); };
       for (uint32_t t = blockIdx.x; ok && t < tiles; t += gridDim.x)
+#pragma unroll 1
         for (uint32_t layer = 0; ok && layer < 4u; ++layer) {
-          const uint32_t pieces = layer == 0u ? kPieces1 : (layer == 3u ? kPiecesL : kPieces2);
+#pragma unroll 1
           for (uint32_t b = 0; b < 2u; ++b) {
-            const uint32_t act = tc::smem_u32(smem + kOffAct + b * kActBytes), pooled = act + (uint32_t)kOffPooled;
+            const uint32_t act = tc::smem_u32(smem + kOffAct + b * kActBytes);
+            const uint64_t adesc = tc::smem_desc(act, (uint32_t)kChunkA, 128u, 0u);
+            const uint32_t acc = tbase + b * (uint32_t)kCh;
             ok = ok && tc::mbar_wait(ready_bar(b), layers & 1u, kWaitCycles);
-            for (uint32_t p = 0; ok && p < pieces; ++p) {
-              const uint32_t s = (u + p) % kRing;
-              if (b == 0u) ok = tc::mbar_wait(full_bar(s), ((u + p) / kRing) & 1u, kWaitCycles);
-              if (!ok) break;
-              tc::fence_after();
-              const uint32_t w = tc::smem_u32(smem + kOffRing + s * kPieceBytes);
-              if (layer < 3u) {
-                const uint32_t tap = layer == 0u ? p : p >> 2, chunk = layer == 0u ? 0u : (p & 3u) * 4u;
+            if (layer == 0u) {
+              if (b == 0u) ok = ok && piece_full(u);
+              if (ok) {
+                tc::fence_after();
+                const uint64_t wd = wdesc + (uint64_t)((u % kRing) * (kPieceBytes / 16));
 #pragma unroll
-                for (uint32_t ks = 0; ks < 2u; ++ks)
-                  tc::mma(tbase + b * (uint32_t)kCh,
-                          tc::smem_desc(act + tap * 16u + (chunk + 2u * ks) * (uint32_t)kChunkA, (uint32_t)kChunkA, 128u, 0u),
-                          tc::smem_desc(w + ks * 2u * 2048u, 2048u, 128u, 0u), kIdesc, p + ks > 0u ? 1u : 0u);
-              } else {
-#pragma unroll
-                for (uint32_t ks = 0; ks < 4u; ++ks)
-                  tc::mma(tbase + 256u + b * (uint32_t)kOut,
-                          tc::smem_desc(pooled + (8u * p + 2u * ks) * (uint32_t)kPooledChunk, (uint32_t)kPooledChunk, 128u, 0u),
-                          tc::smem_desc(w + ks * 2u * 1024u, 1024u, 128u, 0u), kIdescL, p + ks > 0u ? 1u : 0u);
+                for (int ks = 0; ks < kPieceSteps; ++ks)  // two a tap
+                  tc::mma(acc, adesc + (uint64_t)((ks >> 1) + (ks & 1) * 2 * (kChunkA / 16)), wd + (uint64_t)(ks * 256), kIdesc,
+                          ks > 0 ? 1u : 0u);
+                if (b == 1u) tc::commit(empty_bar(u % kRing));
               }
-              if (b == 1u) tc::commit(empty_bar(s));
+            } else if (layer < 3u) {
+#pragma unroll
+              for (int p = 0; p < kPieces2; ++p) {
+                if (b == 0u) ok = ok && piece_full(u + p);
+                if (ok) {
+                  tc::fence_after();
+                  const uint64_t wd = wdesc + (uint64_t)(((u + p) % kRing) * (kPieceBytes / 16));
+#pragma unroll
+                  for (int ks = 0; ks < kPieceSteps; ++ks) {
+                    const int step = p * kPieceSteps + ks;  // eight a tap
+                    tc::mma(acc, adesc + (uint64_t)((step >> 3) + (step & 7) * 2 * (kChunkA / 16)), wd + (uint64_t)(ks * 256),
+                            kIdesc, step > 0 ? 1u : 0u);
+                  }
+                  if (b == 1u) tc::commit(empty_bar((u + p) % kRing));
+                }
+              }
+            } else {
+              if (b == 0u) ok = ok && piece_full(u);
+              if (ok) {
+                tc::fence_after();
+                const uint64_t wd = ldesc + (uint64_t)((u % kRing) * (kPieceBytes / 16));
+                const uint64_t pd = tc::smem_desc(act + (uint32_t)kOffPooled, (uint32_t)kPooledChunk, 128u, 0u);
+#pragma unroll
+                for (int ks = 0; ks < kCh / 16; ++ks)
+                  tc::mma(tbase + 256u + b * (uint32_t)kOut, pd + (uint64_t)(ks * 2 * (kPooledChunk / 16)), wd + (uint64_t)(ks * 128),
+                          kIdescL, ks > 0 ? 1u : 0u);
+                if (b == 1u) tc::commit(empty_bar(u % kRing));
+              }
             }
             // after a wait that ran out too, so that the exit can wait for what was issued
             tc::commit(acc_bar(b));
           }
-          u += pieces;
+          u += layer == 1u || layer == 2u ? kPieces2 : 1;
           ++layers;
         }
       if (!ok) atomicOr(P.err, kErrWait);
@@ -374,13 +402,26 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
         half_sync(blk, half);
         const int ch = c + lane;
         unsigned char* dst = act + kOffPooled + (ch >> 3) * kPooledChunk + (ch & 7) * 2;
+        // four words at a time: four independent chains
 #pragma unroll 1
-        for (uint32_t x = (uint32_t)(warp & 3); x < kb.words; x += 4u) {
-          const float* y = slice + lane * kSliceStride + (int)(x * (kb.L + 1u));
-          float acc = 0.f;
-#pragma unroll 4
-          for (uint32_t p = 0; p < kb.L; ++p) acc += y[p];
-          *reinterpret_cast<__nv_bfloat16*>(dst + x * 16u) = __float2bfloat16_rn(kb.L > 0u ? acc / (float)kb.L : 0.f);
+        for (uint32_t x = (uint32_t)(warp & 3); x < kb.words; x += 16u) {
+          const float* y[4];
+          float acc[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            y[i] = slice + lane * kSliceStride + (int)(min(x + 4u * i, kb.words - 1u) * (kb.L + 1u));
+            acc[i] = 0.f;
+          }
+#pragma unroll 2
+          for (uint32_t p = 0; p < kb.L; ++p) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += y[i][p];
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (x + 4u * i < kb.words)
+              *reinterpret_cast<__nv_bfloat16*>(dst + (x + 4u * i) * 16u) =
+                  __float2bfloat16_rn(kb.L > 0u ? acc[i] / (float)kb.L : 0.f);
         }
         half_sync(blk, half);
       }
