@@ -134,6 +134,7 @@ void nw_destroy(nw_ctx* c) {
   ctx_free(c, c->ws_pairs);
   ctx_free(c, c->ws_segs);
   ctx_free(c, c->ws_norm);
+  while (!c->spare.empty()) ctx_drop_spare(c, c->spare.size() - 1);
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
@@ -445,11 +446,7 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   cudaStream_t s = c->stream;
 
   WordSet q;
-  struct QFree {
-    nw_ctx* c;
-    WordSet& q;
-    ~QFree() { free_wordset(c, q); }
-  } qfree{c, q};
+  CallBufs qbufs{c, wordset_bufs(q)};
   NW_TRY(ingest(c, qcodes, qoffsets, nq, d->alphabet, d->ss.shift, flags & NW_DEVICE_PTRS, q));
   int lo = INT32_MAX, hi = INT32_MIN;
   for (int La = 0; La < kBuckets; ++La)
@@ -516,8 +513,9 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
     NW_CK(cudaMemcpyAsync(nbr_score, out_score, sizeof(int16_t) * (size_t)nq * k, cudaMemcpyDeviceToHost, s));
   }
   tm.mark(c->profiling ? tm.get() : nullptr);
-  // the query set is freed on return, so the stream is always synchronised here
+  // the query set is released on return, so the stream is always synchronised here
   NW_TRY(check_device_flags(c, d_err));
+  qbufs.done = true;
   if (c->profiling) {
     tm.collect();
     unsigned long long ins = 0;

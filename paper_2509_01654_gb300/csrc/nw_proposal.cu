@@ -702,13 +702,7 @@ nw_status nw_quantize_embeddings(nw_ctx* c, const float* E, uint32_t n, int8_t* 
   cudaStream_t s = c->stream;
   const size_t cnt = (size_t)n * NW_EMBED_DIM;
   DevBuf dE, dq, db, dsmall;
-  struct Free {
-    nw_ctx* c;
-    DevBuf* b[4];
-    ~Free() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fr{c, {&dE, &dq, &db, &dsmall}};
+  CallBufs fr{c, {&dE, &dq, &db, &dsmall}};
   const float* srcE = E;
   int8_t* dstq = q;
   int32_t* dstb = bias;
@@ -730,6 +724,7 @@ nw_status nw_quantize_embeddings(nw_ctx* c, const float* E, uint32_t n, int8_t* 
   }
   NW_TRY(copy_out(c, scale, dscale, 1, dev, s));
   NW_CK(cudaStreamSynchronize(s));
+  fr.done = true;
   return NW_OK;
 }
 
@@ -743,13 +738,7 @@ nw_status nw_dot_topk(nw_ctx* c, const int8_t* q, const int32_t* bias, uint32_t 
   cudaStream_t s = c->stream;
   const size_t cnt = (size_t)n * NW_EMBED_DIM, outc = (size_t)n * C;
   DevBuf dq, db, qb, buf, oi, od;
-  struct Free {
-    nw_ctx* c;
-    DevBuf* b[6];
-    ~Free() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fr{c, {&dq, &db, &qb, &buf, &oi, &od}};
+  CallBufs fr{c, {&dq, &db, &qb, &buf, &oi, &od}};
   const int8_t* srcq = q;
   const int32_t* srcb = bias;
   if (!dev) {
@@ -768,13 +757,7 @@ nw_status nw_dot_topk(nw_ctx* c, const int8_t* q, const int32_t* bias, uint32_t 
   NW_TRY(ctx_alloc(c, buf, prop::dot_topk_buffer_bytes(n, C), "candidate buffers"));
   const bool locality = flags & NW_LOCALITY_ORDER;
   DevBuf oq, ob, op, osc;
-  struct FreeOrder {
-    nw_ctx* c;
-    DevBuf* b[4];
-    ~FreeOrder() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fro{c, {&oq, &ob, &op, &osc}};
+  CallBufs fro{c, {&oq, &ob, &op, &osc}};
   if (locality) {
     NW_TRY(ctx_alloc(c, oq, prop::dot_topk_qb_bytes(n), "bf16 embeddings in sweep order"));
     NW_TRY(ctx_alloc(c, ob, sizeof(int32_t) * n, "biases in sweep order"));
@@ -808,6 +791,7 @@ nw_status nw_dot_topk(nw_ctx* c, const int8_t* q, const int32_t* bias, uint32_t 
     NW_TRY(copy_out(c, val, out_v, outc, false, s));
   }
   NW_CK(cudaStreamSynchronize(s));
+  fr.done = fro.done = true;
   return NW_OK;
 }
 
@@ -826,13 +810,7 @@ nw_status nw_rescore_topk(nw_dict* d, const uint32_t* cand, uint32_t C, uint32_t
   const bool dev = flags & NW_DEVICE_PTRS;
   cudaStream_t s = c->stream;
   DevBuf dc, sc, oi, os, small;
-  struct Free {
-    nw_ctx* c;
-    DevBuf* b[5];
-    ~Free() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fr{c, {&dc, &sc, &oi, &os, &small}};
+  CallBufs fr{c, {&dc, &sc, &oi, &os, &small}};
   const uint32_t* srcc = cand;
   if (!dev) {
     NW_TRY(ctx_alloc(c, dc, sizeof(uint32_t) * (size_t)n * C, "candidates"));
@@ -855,6 +833,7 @@ nw_status nw_rescore_topk(nw_dict* d, const uint32_t* cand, uint32_t C, uint32_t
     NW_TRY(copy_out(c, nbr_score, out_s, (size_t)n * k, false, s));
   }
   NW_TRY(check_device_flags(c, small.as<uint32_t>()));
+  fr.done = true;
   return NW_OK;
 }
 
@@ -868,13 +847,7 @@ nw_status nw_dot_topk_cross(nw_ctx* c, const int8_t* qa, uint32_t na, const int8
   cudaStream_t s = c->stream;
   const size_t outc = (size_t)na * C;
   DevBuf dqa, dqb, db, qab, qbb, buf, oi, od;
-  struct Free {
-    nw_ctx* c;
-    DevBuf* b[8];
-    ~Free() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fr{c, {&dqa, &dqb, &db, &qab, &qbb, &buf, &oi, &od}};
+  CallBufs fr{c, {&dqa, &dqb, &db, &qab, &qbb, &buf, &oi, &od}};
   const int8_t* sa = qa;
   const int8_t* sb = qb;
   const int32_t* sbias = bias;
@@ -918,6 +891,7 @@ nw_status nw_dot_topk_cross(nw_ctx* c, const int8_t* qa, uint32_t na, const int8
     NW_TRY(copy_out(c, val, out_v, outc, false, s));
   }
   NW_CK(cudaStreamSynchronize(s));
+  fr.done = true;
   return NW_OK;
 }
 
@@ -941,11 +915,7 @@ nw_status proposal_query_impl(nw_model* M, nw_dict* d, const uint8_t* qcodes, co
   cudaStream_t s = M->stream;
 
   WordSet q;
-  struct QFree {
-    nw_ctx* c;
-    WordSet& q;
-    ~QFree() { free_wordset(c, q); }
-  } qfree{c, q};
+  CallBufs qbufs{c, wordset_bufs(q)};
   NW_TRY(ingest(c, qcodes, qoffsets, nq, d->alphabet, d->ss.shift, flags & NW_DEVICE_PTRS, q));
   int lo = INT32_MAX, hi = INT32_MIN;
   for (int La = 0; La < kBuckets; ++La)
@@ -1007,13 +977,7 @@ nw_status proposal_query_impl(nw_model* M, nw_dict* d, const uint8_t* qcodes, co
   X.nq = nq;
   X.nd = n;
   DevBuf oi, os;
-  struct Free {
-    nw_ctx* c;
-    DevBuf* b[2];
-    ~Free() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fr{c, {&oi, &os}};
+  CallBufs fr{c, {&oi, &os}};
   uint32_t* out_i = nbr_idx;
   int16_t* out_s = nbr_score;
   if (!dev) {
@@ -1041,6 +1005,7 @@ nw_status proposal_query_impl(nw_model* M, nw_dict* d, const uint8_t* qcodes, co
     NW_TRY(copy_out(c, nbr_score, out_s, (size_t)nq * k, false, s));
   }
   NW_TRY(check_err(M, s));
+  qbufs.done = fr.done = true;
   return NW_OK;
 }
 
@@ -1173,13 +1138,7 @@ nw_status nw_proposal_topk(nw_model* M, nw_dict* d, uint32_t C, uint32_t k, uint
     NW_TRY(ctx_ensure(c, M->oscratch, prop::sweep_order_bytes(n), "sweep order scratch"));
   }
   DevBuf oi, os;
-  struct Free {
-    nw_ctx* c;
-    DevBuf* b[2];
-    ~Free() {
-      for (DevBuf* x : b) ctx_free(c, *x);
-    }
-  } fr{c, {&oi, &os}};
+  CallBufs fr{c, {&oi, &os}};
   uint32_t* out_i = nbr_idx;
   int16_t* out_s = nbr_score;
   if (!dev) {
@@ -1242,6 +1201,7 @@ nw_status nw_proposal_topk(nw_model* M, nw_dict* d, uint32_t C, uint32_t k, uint
     prof->exact_ms = exact_ms;
     prof->total_ms = (double)ms[0] + ms[1] + ms[2] + ms[3] + exact_ms;
   }
+  fr.done = true;
   return NW_OK;
 }
 

@@ -1,0 +1,36 @@
+"""Buffers that a finished call leaves with its context: later calls of other
+sizes return what a fresh context returns, and the spare memory never makes a
+call exceed the budget that the call alone fits."""
+import numpy as np
+import pytest
+
+from paper_2509_01654_gb300 import nw, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("budget", [0, 300 << 20])
+def test_calls_of_changing_size_equal_a_fresh_context(budget):
+    rng = np.random.default_rng(5)
+    shared = nw.Context(0, mem_budget_bytes=budget)
+    w = synth.make_uniform_length_words(900, 30, 1.0, 0, 20, seed=3)
+    d = shared.load_dictionary(w.codes, w.offsets, 30, (1, -1, -1))
+    # 2,000 rows take 262 MB of candidate buffers, 1,000 rows 66 MB
+    for n in (2000, 1000, 2000, 37, 1990, 1000):
+        q = rng.integers(-128, 128, (n, 64), dtype=np.int8)
+        b = rng.integers(-5000, 5000, n, dtype=np.int32)
+        got = nw.dot_topk(shared, q, 32, bias=b)
+        fresh = nw.Context(0)
+        want = nw.dot_topk(fresh, q, 32, bias=b)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want)), n
+        qs = synth.make_uniform_length_words(1 + n % 41, 30, 1.0, 0, 30, seed=n)
+        got = d.query(qs.codes, qs.offsets, 7)
+        want = fresh.load_dictionary(w.codes, w.offsets, 30, (1, -1, -1)).query(qs.codes, qs.offsets, 7)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want)), n
+        fresh.close()
+    if budget:  # a call that does not fit by itself is still refused, and leaves the context usable
+        q = rng.integers(-128, 128, (4000, 64), dtype=np.int8)
+        with pytest.raises(nw.NwError):
+            nw.dot_topk(shared, q, 32)
+        assert nw.dot_topk(shared, q[:50], 8)[0].shape == (50, 8)
+    shared.close()
