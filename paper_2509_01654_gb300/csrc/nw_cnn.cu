@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "nw_cnn.h"
 #include "nw_internal.cuh"
 #include "nw_tc.cuh"
@@ -56,33 +58,6 @@ struct Im2col {
     const int pos = (info >> 8) + tap - 1;
     if (pos < 0 || pos >= (info & 255)) return make_float4(0.f, 0.f, 0.f, 0.f);
     return __ldg(reinterpret_cast<const float4*>(X + ((size_t)(t + tap - 1) << lg) + (k & ((1 << lg) - 1))));
-  }
-};
-
-// shifted output gradient: (t, tap * Co + o) = dY[t - tap + 1][o] when
-// position pos(t) - tap + 1 lies inside t's word
-struct Shift {
-  const float* dY;
-  const int* rinfo;
-  int lg;  // log2 Co
-  static constexpr bool kColFast = true;
-  __device__ __forceinline__ float4 vec4(int t, int k) const {
-    const int tap = k >> lg;
-    const int info = __ldg(rinfo + t);
-    const int pos = (info >> 8) - tap + 1;
-    if (pos < 0 || pos >= (info & 255)) return make_float4(0.f, 0.f, 0.f, 0.f);
-    return __ldg(reinterpret_cast<const float4*>(dY + ((size_t)(t - tap + 1) << lg) + (k & ((1 << lg) - 1))));
-  }
-};
-
-// W[Co][3][Ci] read as the (tap * Co + o, ch) matrix of the input gradient
-struct WTap {
-  const float* W;
-  int lgCo, Ci;
-  static constexpr bool kColFast = true;
-  __device__ __forceinline__ float4 vec4(int k, int ch) const {
-    const int tap = k >> lgCo, o = k & ((1 << lgCo) - 1);
-    return __ldg(reinterpret_cast<const float4*>(W + ((size_t)o * 3 + tap) * Ci + ch));
   }
 };
 
@@ -468,54 +443,64 @@ __global__ void word_len_kernel(WordSrc src, int Bw, int* len, uint32_t* err) {
 
 constexpr int kScanThreads = 1024;
 
-// off = exclusive prefix sum of len (one block), T = the total (at most Tmax)
-__global__ void __launch_bounds__(kScanThreads) scan_kernel(const int* len, int Bw, int* off, int* T, int Tmax,
-                                                            uint32_t* err) {
-  __shared__ int warp_sum[kScanThreads / 32];
+// off = exclusive prefix sum of len (one block), T = the total (at most Tmax);
+// poff and Tp: the same with one more row for every word that has any
+__global__ void __launch_bounds__(kScanThreads) scan_kernel(const int* len, int Bw, int* off, int* T, int* poff, int* Tp,
+                                                            int Tmax, uint32_t* err) {
+  __shared__ long long warp_sum[kScanThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = (Bw + kScanThreads - 1) / kScanThreads;
   const int w0 = min(Bw, tid * per), w1 = min(Bw, w0 + per);
-  int local = 0;
-  for (int w = w0; w < w1; ++w) local += len[w];
-  int incl = local;
+  auto item = [&](int w) {  // rows below, words with rows above
+    const int l = len[w];
+    return (long long)l | ((long long)(l > 0) << 32);
+  };
+  long long local = 0;
+  for (int w = w0; w < w1; ++w) local += item(w);
+  long long incl = local;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    const long long t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += t;
   }
   if (lane == 31) warp_sum[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    int ws = warp_sum[lane];
+    long long ws = warp_sum[lane];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, ws, o);
+      const long long t = __shfl_up_sync(0xffffffffu, ws, o);
       if (lane >= o) ws += t;
     }
     warp_sum[lane] = ws;  // inclusive over warps
   }
   __syncthreads();
-  int run = incl - local + (warp ? warp_sum[warp - 1] : 0);
+  long long run = incl - local + (warp ? warp_sum[warp - 1] : 0);
   for (int w = w0; w < w1; ++w) {
-    off[w] = run;
-    run += len[w];
+    off[w] = (int)run;
+    poff[w] = (int)run + (int)(run >> 32);
+    run += item(w);
   }
   if (tid == kScanThreads - 1) {
-    const int total = warp_sum[kScanThreads / 32 - 1];
+    const long long all = warp_sum[kScanThreads / 32 - 1];
+    const int total = (int)all;
     if (total > Tmax) atomicOr(err, kErrInput);
     *T = min(total, Tmax);
+    *Tp = min(total, Tmax) + (int)(all >> 32);
   }
 }
 
 // per-row tables: thread per word (rows past Tmax are dropped)
-__global__ void fill_rows_kernel(const int* len, const int* off, int Bw, int Tmax, int* rinfo, int* rword) {
+__global__ void fill_rows_kernel(const int* len, const int* off, const int* poff, int Bw, int Tmax, int* rinfo, int* rword,
+                                 int* prow) {
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= Bw) return;
-  const int L = len[w], o = off[w];
+  const int L = len[w], o = off[w], p = poff[w];
   for (int t = 0; t < L && o + t < Tmax; ++t) {
     rinfo[o + t] = (t << 8) | L;
     rword[o + t] = w;
   }
+  for (int t = 0; t < (L > 0 ? L + 1 : 0) && p + t < Tmax + Bw; ++t) prow[p + t] = t < L && o + t < Tmax ? o + t : -1;
 }
 
 // one warp per packed row: lane = embedding channel
@@ -548,15 +533,6 @@ __global__ void pool_kernel(const float* __restrict__ Y, const int* len, const i
   P[x] = L > 0 ? acc / (float)L : 0.f;
 }
 
-__global__ void pool_bwd_kernel(const float* __restrict__ dP, const float* __restrict__ Y, const int* len,
-                                const int* rword, const int* Tdev, int Tmax, float* dY) {
-  const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= (size_t)min(Tmax, *Tdev) * kCh) return;
-  const int row = (int)(x / kCh), ch = (int)(x - (size_t)row * kCh);
-  const int w = rword[row];
-  dY[x] = Y[x] > 0.f ? dP[(size_t)w * kCh + ch] / (float)len[w] : 0.f;
-}
-
 // one warp per pair: lanes hold dimensions lane and lane + 32.  The 64
 // outputs are 63 features and a bias (the last): pred = phi_a . phi_b + beta_a + beta_b
 __global__ void pair_loss_kernel(const float* __restrict__ E, const float* __restrict__ target, int m, float* dE,
@@ -584,9 +560,8 @@ __global__ void pair_loss_kernel(const float* __restrict__ E, const float* __res
 
 constexpr int kColSumRows = 256;
 
-__global__ void col_sum_kernel(const float* __restrict__ Y, int rows, const int* rows_dev, int cols, float* out) {
+__global__ void col_sum_kernel(const float* __restrict__ Y, int rows, int cols, float* out) {
   const int c = threadIdx.x;
-  if (rows_dev) rows = min(rows, *rows_dev);
   const int r0 = blockIdx.x * kColSumRows;
   const int r1 = min(rows, r0 + kColSumRows);
   if (c >= cols || r0 >= r1) return;
@@ -595,13 +570,39 @@ __global__ void col_sum_kernel(const float* __restrict__ Y, int rows, const int*
   atomicAdd(out + c, acc);
 }
 
+// demb[code] += the rows of dX0 with that code.  A batch has few codes and many
+// rows: an atomic a value meets 160k others on each of 1,280 addresses (136 us).
+// Here a warp adds its rows to its own table in shared memory (lane = channel),
+// a block adds its tables, and one atomic a value and block remains.
 __global__ void emb_scatter_kernel(const float* __restrict__ dX0, const int32_t* codes, const int* Tdev, int Tmax,
-                                   float* demb) {
-  const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= (size_t)min(Tmax, *Tdev) * kEmb) return;
-  const int row = (int)(x / kEmb), ch = (int)(x - (size_t)row * kEmb);
-  const int code = codes[row];
-  if (code >= 0) atomicAdd(demb + (size_t)code * kEmb + ch, dX0[x]);
+                                   int alphabet, float* demb) {
+  extern __shared__ float s_emb[];
+  const int warps = blockDim.x / 32, warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+  const int n = alphabet * kEmb;
+  for (int x = threadIdx.x; x < warps * n; x += blockDim.x) s_emb[x] = 0.f;
+  __syncthreads();
+  float* mine = s_emb + warp * n + lane;
+  const int T = min(Tmax, *Tdev), step = gridDim.x * warps;
+  constexpr int kAhead = 8;
+  for (int row = blockIdx.x * warps + warp; row < T; row += kAhead * step) {
+    float v[kAhead];
+    int code[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const bool in = row + (long long)i * step < T;
+      code[i] = in ? codes[row + i * step] : -1;
+      v[i] = in ? dX0[(size_t)(row + i * step) * kEmb + lane] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+      if (code[i] >= 0) mine[code[i] * kEmb] += v[i];
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < n; x += blockDim.x) {
+    float sum = 0.f;
+    for (int w = 0; w < warps; ++w) sum += s_emb[w * n + x];
+    if (sum != 0.f) atomicAdd(demb + x, sum);
+  }
 }
 
 // Adam with bias correction; the gradient is scaled by min(1, clip / |g|)
@@ -713,20 +714,6 @@ cudaError_t conv_fwd(const float* X, int Ci, const float* W, int Co, const Packe
   return run_gemm(Im2col{X, pk.rinfo, log2_ch(Ci)}, DenseT{W, 3 * Ci}, pk.Tmax, Co, 3 * Ci, Y, Co, e, 1, s, pk.T);
 }
 
-cudaError_t conv_dw(const float* dY, int Co, const float* X, int Ci, const Packed& pk, float* dW, int nsm,
-                    cudaStream_t s) {
-  Epi e;
-  e.atomic = true;
-  return run_gemm(DenseT{dY, Co}, Im2col{X, pk.rinfo, log2_ch(Ci)}, Co, 3 * Ci, pk.Tmax, dW, 3 * Ci, e,
-                  splits_for(Co, 3 * Ci, pk.Tmax, nsm), s, nullptr, pk.T);
-}
-
-cudaError_t conv_dx(const float* dY, int Co, const float* W, int Ci, const Packed& pk, float* dX, const Epi& e,
-                    cudaStream_t s) {
-  return run_gemm(Shift{dY, pk.rinfo, log2_ch(Co)}, WTap{W, log2_ch(Co), Ci}, pk.Tmax, Ci, 3 * Co, dX, Ci, e, 1, s,
-                  pk.T);
-}
-
 cudaError_t lin_fwd(const float* P, int Ci, const float* Wl, int Co, int B, float* E, const Epi& e, cudaStream_t s) {
   return run_gemm(Dense{P, Ci}, DenseT{Wl, Ci}, B, Co, Ci, E, Co, e, 1, s);
 }
@@ -743,10 +730,13 @@ cudaError_t lin_dx(const float* dE, int Co, const float* Wl, int Ci, int B, floa
 
 cudaError_t pack_words(const WordSrc& src, int Bw, int Tmax, const float* emb, const PackBufs& b, float* X0,
                        uint32_t* err, uint32_t alphabet, cudaStream_t s) {
-  if (Bw <= 0) return cudaMemsetAsync(b.T, 0, sizeof(int), s);
+  if (Bw <= 0) {
+    const cudaError_t e = cudaMemsetAsync(b.T, 0, sizeof(int), s);
+    return e != cudaSuccess ? e : cudaMemsetAsync(b.Tp, 0, sizeof(int), s);
+  }
   word_len_kernel<<<blocks_for(Bw, 256), 256, 0, s>>>(src, Bw, b.len, err);
-  scan_kernel<<<1, kScanThreads, 0, s>>>(b.len, Bw, b.off, b.T, Tmax, err);
-  fill_rows_kernel<<<blocks_for(Bw, 256), 256, 0, s>>>(b.len, b.off, Bw, Tmax, b.rinfo, b.rword);
+  scan_kernel<<<1, kScanThreads, 0, s>>>(b.len, Bw, b.off, b.T, b.poff, b.Tp, Tmax, err);
+  fill_rows_kernel<<<blocks_for(Bw, 256), 256, 0, s>>>(b.len, b.off, b.poff, Bw, Tmax, b.rinfo, b.rword, b.prow);
   gather_kernel<<<blocks_for((size_t)Tmax, 8), 256, 0, s>>>(src, b.T, Tmax, emb, b.rinfo, b.rword, b.codes, X0, err,
                                                              alphabet);
   return cudaGetLastError();
@@ -758,27 +748,27 @@ cudaError_t mean_pool(const float* Y, const Packed& pk, float* P, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t mean_pool_bwd(const float* dP, const float* Y, const Packed& pk, float* dY, cudaStream_t s) {
-  if (pk.Tmax <= 0) return cudaSuccess;
-  pool_bwd_kernel<<<blocks_for((size_t)pk.Tmax * kCh, 256), 256, 0, s>>>(dP, Y, pk.len, pk.rword, pk.T, pk.Tmax, dY);
-  return cudaGetLastError();
-}
-
 cudaError_t pair_loss(const float* E, const float* target, int m, float* dE, float* loss_acc, cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   pair_loss_kernel<<<blocks_for(m, 8), 256, 0, s>>>(E, target, m, dE, loss_acc);
   return cudaGetLastError();
 }
 
-cudaError_t col_sum(const float* Y, int rows, const int* rows_dev, int cols, float* out, cudaStream_t s) {
+cudaError_t col_sum(const float* Y, int rows, int cols, float* out, cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
-  col_sum_kernel<<<blocks_for(rows, kColSumRows), cols <= 64 ? 64 : 128, 0, s>>>(Y, rows, rows_dev, cols, out);
+  col_sum_kernel<<<blocks_for(rows, kColSumRows), cols <= 64 ? 64 : 128, 0, s>>>(Y, rows, cols, out);
   return cudaGetLastError();
 }
 
-cudaError_t emb_scatter(const float* dX0, const int32_t* codes, const Packed& pk, float* demb, cudaStream_t s) {
+cudaError_t emb_scatter(const float* dX0, const int32_t* codes, const Packed& pk, int alphabet, float* demb, int sms,
+                        cudaStream_t s) {
   if (pk.Tmax <= 0) return cudaSuccess;
-  emb_scatter_kernel<<<blocks_for((size_t)pk.Tmax * kEmb, 256), 256, 0, s>>>(dX0, codes, pk.T, pk.Tmax, demb);
+  const int table = alphabet * kEmb * (int)sizeof(float);  // at most 32 KiB
+  const int warps = std::max(1, std::min(16, 192 * 1024 / table));
+  const cudaError_t e = cudaFuncSetAttribute(emb_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 * 1024);
+  if (e != cudaSuccess) return e;
+  emb_scatter_kernel<<<std::min(sms, (pk.Tmax + warps - 1) / warps), warps * 32, warps * table, s>>>(dX0, codes, pk.T, pk.Tmax,
+                                                                                                  alphabet, demb);
   return cudaGetLastError();
 }
 

@@ -56,6 +56,10 @@ struct Packed {
   const int* T;      // device: rows in use
   const int* rinfo;  // per row: (position << 8) | word length
   const int* rword;  // per row: word
+  // the same rows with one empty row after every word that has any: a padded
+  // row's packed row, or -1 (Tmax + Bw entries), and the padded rows in use
+  const int* prow;
+  const int* Tp;
   int Bw, Tmax;
 };
 
@@ -74,8 +78,8 @@ struct Epi {
 // [Co][3][Ci], Wl is [Co][Ci]; Ci and Co of a convolution are powers of
 // two; activations of a packed batch have pk.T rows.
 //   conv_fwd: Y[T][Co]  = im2col(X[T][Ci]) . W^T            (epilogue e)
-//   conv_dw:  dW[Co][3Ci] += dY^T . im2col(X)               (split over rows, atomic)
-//   conv_dx:  dX[T][Ci] = sum_tap shift_tap(dY) . W[.][tap]  (col2im folded in; epilogue e)
+//   conv_bwd: dW[Co][3Ci] += dY^T . im2col(X), db[Co] += column sums of dY and
+//             dX[T][Ci] = sum_tap shift_tap(dY) . W[.][tap], x (X > 0) for layers 2 and 3
 //   lin_fwd:  E[B][Co]  = P[B][Ci] . Wl^T                   (epilogue e)
 //   lin_dw:   dWl[Co][Ci] += dE^T . P                       (split over B, atomic)
 //   lin_dx:   dP[B][Ci] = dE[B][Co] . Wl
@@ -83,10 +87,12 @@ struct Epi {
 // pos(t) + tap - 1 lies inside t's word, else 0 (the zero padding).
 cudaError_t conv_fwd(const float* X, int Ci, const float* W, int Co, const Packed& pk, float* Y, const Epi& e,
                      cudaStream_t s);
-cudaError_t conv_dw(const float* dY, int Co, const float* X, int Ci, const Packed& pk, float* dW, int nsm,
-                    cudaStream_t s);
-cudaError_t conv_dx(const float* dY, int Co, const float* W, int Ci, const Packed& pk, float* dX, const Epi& e,
-                    cudaStream_t s);
+// layer 3 takes its output gradient from the mean's (dP) and its output Ytop,
+// layers 2 and 1 from dY; `pack` holds pack_bwd's bwd_pack_bytes() of weights
+size_t bwd_pack_bytes();
+cudaError_t pack_bwd(const float* params, const Layout& L, void* pack, cudaStream_t s);
+cudaError_t conv_bwd(int layer, const float* dY, const float* Ytop, const float* dP, const float* X, const Packed& pk,
+                     const void* pack, float* dX, float* dW, float* db, uint32_t* err, int sms, cudaStream_t s);
 cudaError_t lin_fwd(const float* P, int Ci, const float* Wl, int Co, int B, float* E, const Epi& e, cudaStream_t s);
 cudaError_t lin_dw(const float* dE, int Co, const float* P, int Ci, int B, float* dWl, int nsm, cudaStream_t s);
 cudaError_t lin_dx(const float* dE, int Co, const float* Wl, int Ci, int B, float* dP, cudaStream_t s);
@@ -99,18 +105,21 @@ struct PackBufs {
   int* T;
   int* rinfo;
   int* rword;
+  int* poff;  // Bw first padded rows
+  int* prow;
+  int* Tp;
   int32_t* codes;
 };
 cudaError_t pack_words(const WordSrc& src, int Bw, int Tmax, const float* emb, const PackBufs& b, float* X0,
                        uint32_t* err, uint32_t alphabet, cudaStream_t s);
 cudaError_t mean_pool(const float* Y, const Packed& pk, float* P, cudaStream_t s);
-cudaError_t mean_pool_bwd(const float* dP, const float* Y, const Packed& pk, float* dY, cudaStream_t s);
 // pairs are word slots (2p, 2p + 1), pred = phi . phi + beta + beta (outputs
 // 0..62 features, 63 bias); loss_acc += sum (pred - y)^2 / m (if non-null)
 cudaError_t pair_loss(const float* E, const float* target, int m, float* dE, float* loss_acc, cudaStream_t s);
-// out += column sums of Y's first rows (rows: a host count, or the device count *rows_dev when non-null)
-cudaError_t col_sum(const float* Y, int rows, const int* rows_dev, int cols, float* out, cudaStream_t s);
-cudaError_t emb_scatter(const float* dX0, const int32_t* codes, const Packed& pk, float* demb, cudaStream_t s);
+// out += column sums of Y's rows
+cudaError_t col_sum(const float* Y, int rows, int cols, float* out, cudaStream_t s);
+cudaError_t emb_scatter(const float* dX0, const int32_t* codes, const Packed& pk, int alphabet, float* demb, int sms,
+                        cudaStream_t s);
 struct AdamCfg {
   float lr, lr_final, b1, b2, eps;
   float clip;        // > 0: scale the gradient to norm <= clip

@@ -27,7 +27,7 @@ struct nw_model {
   DevBuf params, grads, adam_m, adam_v, small;  // small: step counter, loss accumulator, error flags, amax
   // forward/backward scratch for cap_words words packed into cap_rows rows
   int cap_words = 0, cap_rows = 0;
-  DevBuf widx, len, off, rinfo, rword, codes, X0, Y1, Y2, Y3, P, E, dE, dP, dYa, dYb, dX0;
+  DevBuf widx, len, off, poff, rinfo, rword, prow, Wbwd, codes, X0, Y1, Y2, Y3, P, E, dE, dP, dYa, dYb, dX0;
   // training pairs
   uint32_t cap_pairs = 0;
   DevBuf pi, pj, target, score16;
@@ -96,6 +96,7 @@ float* loss_ptr(nw_model* M) { return reinterpret_cast<float*>(M->small.as<char>
 uint32_t* err_ptr(nw_model* M) { return reinterpret_cast<uint32_t*>(M->small.as<char>() + 8); }
 unsigned int* amax_ptr(nw_model* M) { return reinterpret_cast<unsigned int*>(M->small.as<char>() + 12); }
 int* rows_ptr(nw_model* M) { return reinterpret_cast<int*>(M->small.as<char>() + 16); }
+int* padded_rows_ptr(nw_model* M) { return reinterpret_cast<int*>(M->small.as<char>() + 24); }
 float* sumsq_ptr(nw_model* M) { return reinterpret_cast<float*>(M->small.as<char>() + 20); }
 
 void model_free_buffers(nw_model* M) {
@@ -105,7 +106,8 @@ void model_free_buffers(nw_model* M) {
                     &M->dYb, &M->dX0, &M->pi, &M->pj, &M->target, &M->score16, &M->Eall, &M->Qb,
                     &M->qbias, &M->topbuf, &M->cand, &M->cand_dot, &M->cand_score, &M->nbr,
                     &M->dQb, &M->dqbias, &M->prep_small, &M->qQb, &M->qcand, &M->qcand_dot, &M->qscore, &M->qbuf,
-                    &M->xcodes, &M->xoffs, &M->xidx, &M->xscore, &M->oQb, &M->obias, &M->operm, &M->oscratch, &M->Wpack};
+                    &M->xcodes, &M->xoffs, &M->xidx, &M->xscore, &M->oQb, &M->obias, &M->operm, &M->oscratch,
+                    &M->Wpack, &M->poff, &M->prow, &M->Wbwd};
   for (DevBuf* b : bufs) ctx_free(c, *b);
 }
 
@@ -120,6 +122,9 @@ nw_status ensure_scratch(nw_model* M, int Bw, int Tmax) {
   NW_TRY(ctx_ensure(c, M->widx, sizeof(uint32_t) * W, "model word indices"));
   NW_TRY(ctx_ensure(c, M->len, sizeof(int) * W, "model word lengths"));
   NW_TRY(ctx_ensure(c, M->off, sizeof(int) * W, "model word offsets"));
+  NW_TRY(ctx_ensure(c, M->poff, sizeof(int) * W, "model word offsets"));
+  NW_TRY(ctx_ensure(c, M->prow, sizeof(int) * (T + W), "model row tables"));
+  NW_TRY(ctx_ensure(c, M->Wbwd, cnn::bwd_pack_bytes(), "packed weights"));
   NW_TRY(ctx_ensure(c, M->rinfo, sizeof(int) * T, "model row tables"));
   NW_TRY(ctx_ensure(c, M->rword, sizeof(int) * T, "model row tables"));
   NW_TRY(ctx_ensure(c, M->codes, sizeof(int32_t) * T, "model codes"));
@@ -157,6 +162,8 @@ cnn::Packed packed(nw_model* M, int Bw, int Tmax) {
   pk.T = rows_ptr(M);
   pk.rinfo = M->rinfo.as<int>();
   pk.rword = M->rword.as<int>();
+  pk.prow = M->prow.as<int>();
+  pk.Tp = padded_rows_ptr(M);
   pk.Bw = Bw;
   pk.Tmax = Tmax;
   return pk;
@@ -180,8 +187,8 @@ nw_status forward(nw_model* M, const nw_dict* d, int Bw, int Tmax, cudaStream_t 
   const cnn::Layout& L = M->L;
   const float* W = fptr(M->params);
   const cnn::Packed pk = packed(M, Bw, Tmax);
-  cnn::PackBufs pb{M->len.as<int>(), M->off.as<int>(), rows_ptr(M), M->rinfo.as<int>(), M->rword.as<int>(),
-                   M->codes.as<int32_t>()};
+  cnn::PackBufs pb{M->len.as<int>(),  M->off.as<int>(),  rows_ptr(M),        M->rinfo.as<int>(),    M->rword.as<int>(),
+                   M->poff.as<int>(), M->prow.as<int>(), padded_rows_ptr(M), M->codes.as<int32_t>()};
   NW_CK(cnn::pack_words(word_src(d->ws, d->ss.shift, M->widx.as<uint32_t>()), Bw, Tmax, W + L.emb, pb, fptr(M->X0),
                         err_ptr(M), M->alphabet, s));
   cnn::Epi e;
@@ -213,26 +220,17 @@ nw_status backward(nw_model* M, int m, int Tmax, cudaStream_t s) {
   NW_CK(cudaMemsetAsync(G, 0, sizeof(float) * L.total, s));
   NW_CK(cnn::pair_loss(fptr(M->E), fptr(M->target), m, fptr(M->dE), loss_ptr(M), s));
   NW_CK(cnn::lin_dw(fptr(M->dE), cnn::kOut, fptr(M->P), cnn::kCh, Bw, G + L.Wl, nsm, s));
-  NW_CK(cnn::col_sum(fptr(M->dE), Bw, nullptr, cnn::kOut, G + L.bl, s));
+  NW_CK(cnn::col_sum(fptr(M->dE), Bw, cnn::kOut, G + L.bl, s));
   NW_CK(cnn::lin_dx(fptr(M->dE), cnn::kOut, W + L.Wl, cnn::kCh, Bw, fptr(M->dP), s));
-  NW_CK(cnn::mean_pool_bwd(fptr(M->dP), fptr(M->Y3), pk, fptr(M->dYa), s));
-  // layer 3: dYa = dY3
-  NW_CK(cnn::conv_dw(fptr(M->dYa), cnn::kCh, fptr(M->Y2), cnn::kCh, pk, G + L.W3, nsm, s));
-  NW_CK(cnn::col_sum(fptr(M->dYa), Tmax, pk.T, cnn::kCh, G + L.b3, s));
-  cnn::Epi e;
-  e.gate = fptr(M->Y2);
-  NW_CK(cnn::conv_dx(fptr(M->dYa), cnn::kCh, W + L.W3, cnn::kCh, pk, fptr(M->dYb), e, s));
-  // layer 2: dYb = dY2
-  NW_CK(cnn::conv_dw(fptr(M->dYb), cnn::kCh, fptr(M->Y1), cnn::kCh, pk, G + L.W2, nsm, s));
-  NW_CK(cnn::col_sum(fptr(M->dYb), Tmax, pk.T, cnn::kCh, G + L.b2, s));
-  e.gate = fptr(M->Y1);
-  NW_CK(cnn::conv_dx(fptr(M->dYb), cnn::kCh, W + L.W2, cnn::kCh, pk, fptr(M->dYa), e, s));
-  // layer 1: dYa = dY1
-  NW_CK(cnn::conv_dw(fptr(M->dYa), cnn::kCh, fptr(M->X0), cnn::kEmb, pk, G + L.W1, nsm, s));
-  NW_CK(cnn::col_sum(fptr(M->dYa), Tmax, pk.T, cnn::kCh, G + L.b1, s));
-  e.gate = nullptr;
-  NW_CK(cnn::conv_dx(fptr(M->dYa), cnn::kCh, W + L.W1, cnn::kEmb, pk, fptr(M->dX0), e, s));
-  NW_CK(cnn::emb_scatter(fptr(M->dX0), M->codes.as<int32_t>(), pk, G + L.emb, s));
+  NW_CK(cnn::pack_bwd(W, L, M->Wbwd.p, s));
+  // dYb = dY2, dYa = dY1
+  NW_CK(cnn::conv_bwd(3, nullptr, fptr(M->Y3), fptr(M->dP), fptr(M->Y2), pk, M->Wbwd.p, fptr(M->dYb), G + L.W3, G + L.b3,
+                      err_ptr(M), nsm, s));
+  NW_CK(cnn::conv_bwd(2, fptr(M->dYb), nullptr, nullptr, fptr(M->Y1), pk, M->Wbwd.p, fptr(M->dYa), G + L.W2, G + L.b2,
+                      err_ptr(M), nsm, s));
+  NW_CK(cnn::conv_bwd(1, fptr(M->dYa), nullptr, nullptr, fptr(M->X0), pk, M->Wbwd.p, fptr(M->dX0), G + L.W1, G + L.b1,
+                      err_ptr(M), nsm, s));
+  NW_CK(cnn::emb_scatter(fptr(M->dX0), M->codes.as<int32_t>(), pk, (int)M->alphabet, G + L.emb, nsm, s));
   return NW_OK;
 }
 
