@@ -1,7 +1,6 @@
-// nw_cnn.cu -- kernels of the proposal network: bf16 tensor-core matrix
-// products (float32 accumulation) whose operand loaders gather convolution windows directly from the packed
-// activations (no im2col buffer, no padding rows), and the elementwise steps
-// around them.
+// nw_cnn.cu -- kernels of the proposal network's training around its
+// convolutions (nw_conv.cu): the linear layer's bf16 tensor-core products
+// (float32 accumulation) and the elementwise steps.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -29,9 +28,6 @@ struct Dense {  // row-major
   __device__ __forceinline__ float4 vec4(int r, int c) const {
     return __ldg(reinterpret_cast<const float4*>(p + (size_t)r * ld + c));
   }
-  // the same, with the row's table entry read ahead (none for a dense view)
-  __device__ __forceinline__ int row_info(int) const { return 0; }
-  __device__ __forceinline__ float4 vec4r(int r, int c, int) const { return vec4(r, c); }
 };
 
 struct DenseT {  // transpose of a row-major matrix
@@ -40,24 +36,6 @@ struct DenseT {  // transpose of a row-major matrix
   static constexpr bool kColFast = false;
   __device__ __forceinline__ float4 vec4(int r, int c) const {
     return __ldg(reinterpret_cast<const float4*>(p + (size_t)c * ld + r));
-  }
-};
-
-// im2col of packed X[T][Ci]: (t, tap * Ci + ch) = X[t + tap - 1][ch] when
-// position pos(t) + tap - 1 lies inside t's word (rinfo: (pos << 8) | len)
-struct Im2col {
-  const float* X;
-  const int* rinfo;
-  int lg;  // log2 Ci
-  static constexpr bool kColFast = true;
-  __device__ __forceinline__ float4 vec4(int t, int k) const { return vec4r(t, k, row_info(t)); }
-  // the same with row t's table entry given (a kernel that keeps its rows' entries at hand)
-  __device__ __forceinline__ int row_info(int t) const { return __ldg(rinfo + t); }
-  __device__ __forceinline__ float4 vec4r(int t, int k, int info) const {
-    const int tap = k >> lg;
-    const int pos = (info >> 8) + tap - 1;
-    if (pos < 0 || pos >= (info & 255)) return make_float4(0.f, 0.f, 0.f, 0.f);
-    return __ldg(reinterpret_cast<const float4*>(X + ((size_t)(t + tap - 1) << lg) + (k & ((1 << lg) - 1))));
   }
 };
 
@@ -119,19 +97,16 @@ struct TileMap {
   __device__ __forceinline__ static int off(int o, int k) { return KFast ? o * LDK + k : k * LDM + o; }
 };
 
-// C[M][N] = A[M][K] . B[K][N] over the K range of blockIdx.z.  Mlim / Klim
-// (device, may be null) lower M / K below the launch's bounds.
+// C[M][N] = A[M][K] . B[K][N] over the K range of blockIdx.z
 template <class AV, class BV>
 __global__ void __launch_bounds__(NT, 2) gemm_kernel(AV A, BV B, int M, int N, int K, int kchunk, float* C, int ldc,
-                                                  Epi e, const int* Mlim, const int* Klim) {
+                                                  Epi e) {
   constexpr bool kAK = AV::kColFast;   // A contiguous along k
   constexpr bool kBK = !BV::kColFast;  // B contiguous along k
   using MA = TileMap<kAK>;
   using MB = TileMap<kBK>;
   __shared__ __align__(16) __nv_bfloat16 As[2][kTileHalfs];
   __shared__ __align__(16) __nv_bfloat16 Bs[2][kTileHalfs];
-  if (Mlim) M = min(M, *Mlim);
-  if (Klim) K = min(K, *Klim);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wm = warp >> 2, wn = warp & 3, g = lane >> 2, t4 = lane & 3;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -227,16 +202,13 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(AV A, BV B, int M, int N, i
             continue;
           }
           if (e.bias) v += __ldg(e.bias + n);
-          if (e.relu) v = fmaxf(v, 0.f);
-          if (e.gate && !(__ldg(e.gate + (size_t)m * ldc + n) > 0.f)) v = 0.f;
           *dst = v;
         }
     }
 }
 
 // ---- the same products on the fifth-generation tensor cores, for operands
-// that are both contiguous along K (the forward convolutions and the linear
-// layer).  One CTA of 256 threads computes a 128 x 128 output tile into a
+// that are both contiguous along K (the linear layer forward).  One CTA of 256 threads computes a 128 x 128 output tile into a
 // 128-column tensor-memory accumulator.  K advances 32 at a time through two
 // shared stages in the canonical K-major layout (8-row x 16-byte core
 // matrices, no swizzle): each thread loads its four 16-byte vectors of each
@@ -255,14 +227,11 @@ constexpr uint32_t kTcIdesc = tc::idesc_bf16(BM, BN);
 constexpr long long kTcWaitCycles = 2000000000ll;  // about a second
 
 template <class AV, class BV>
-__global__ void __launch_bounds__(NT, 4) gemm_tc_kernel(AV A, BV B, int M, int N, int K, float* C, int ldc, Epi e,
-                                                     const int* Mlim) {
+__global__ void __launch_bounds__(NT, 4) gemm_tc_kernel(AV A, BV B, int M, int N, int K, float* C, int ldc, Epi e) {
   static_assert(AV::kColFast && !BV::kColFast, "both operands contiguous along K");
   __shared__ __align__(1024) unsigned char sm[2][2][kTcTileBytes];  // [stage][A, B]
   __shared__ __align__(8) unsigned long long bars[2];
   __shared__ uint32_t tmem_base;
-  __shared__ int rows_info[BM];  // the A view's table entries of the tile's rows, read once
-  if (Mlim) M = min(M, *Mlim);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   if (m0 >= M) return;  // block-uniform, before any barrier or allocation
@@ -273,21 +242,17 @@ __global__ void __launch_bounds__(NT, 4) gemm_tc_kernel(AV A, BV B, int M, int N
     tc::mbar_init_fence();
   }
   if (warp == 0) tc::tmem_alloc(tc::smem_u32(&tmem_base), BN);
-  if (tid < BM) rows_info[tid] = m0 + tid < M ? A.row_info(m0 + tid) : 0;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tbase = tmem_base;
-  int info[4];  // this thread's four A rows (fixed for the whole K loop)
-#pragma unroll
-  for (int q = 0; q < 4; ++q) info[q] = rows_info[(tid + q * NT) >> 3];
 
   float4 ra[4], rb[4];
   auto load = [&](int k0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int x = tid + q * NT, o = x >> 3, k = (x & 7) * 4;
-      ra[q] = (m0 + o < M && k0 + k < K) ? A.vec4r(m0 + o, k0 + k, info[q]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      ra[q] = (m0 + o < M && k0 + k < K) ? A.vec4(m0 + o, k0 + k) : make_float4(0.f, 0.f, 0.f, 0.f);
       rb[q] = (n0 + o < N && k0 + k < K) ? B.vec4(k0 + k, n0 + o) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
@@ -360,19 +325,6 @@ __global__ void __launch_bounds__(NT, 4) gemm_tc_kernel(AV A, BV B, int M, int N
             r.z += __ldg(e.bias + min(n + 2, N - 1));
             r.w += __ldg(e.bias + min(n + 3, N - 1));
           }
-          if (e.relu) {
-            r.x = fmaxf(r.x, 0.f);
-            r.y = fmaxf(r.y, 0.f);
-            r.z = fmaxf(r.z, 0.f);
-            r.w = fmaxf(r.w, 0.f);
-          }
-          if (e.gate) {
-            const float* gp = e.gate + (size_t)m * ldc;
-            if (!(__ldg(gp + n) > 0.f)) r.x = 0.f;
-            if (!(__ldg(gp + min(n + 1, N - 1)) > 0.f)) r.y = 0.f;
-            if (!(__ldg(gp + min(n + 2, N - 1)) > 0.f)) r.z = 0.f;
-            if (!(__ldg(gp + min(n + 3, N - 1)) > 0.f)) r.w = 0.f;
-          }
           float* dst = C + (size_t)m * ldc + n;
           if (n + 4 <= N) {
             *reinterpret_cast<float4*>(dst) = r;
@@ -393,8 +345,7 @@ __global__ void __launch_bounds__(NT, 4) gemm_tc_kernel(AV A, BV B, int M, int N
 }
 
 template <class AV, class BV>
-cudaError_t run_gemm(AV A, BV B, int M, int N, int K, float* C, int ldc, const Epi& e, int splits, cudaStream_t s,
-                     const int* Mlim = nullptr, const int* Klim = nullptr) {
+cudaError_t run_gemm(AV A, BV B, int M, int N, int K, float* C, int ldc, const Epi& e, int splits, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   // the operands are read in 16-byte vectors along their contiguous axes
   if ((AV::kColFast ? K : M) % 4 != 0 || (BV::kColFast ? N : K) % 4 != 0) return cudaErrorInvalidValue;
@@ -409,12 +360,12 @@ cudaError_t run_gemm(AV A, BV B, int M, int N, int K, float* C, int ldc, const E
   if (K <= 0) gz = 1;
   if constexpr (AV::kColFast && !BV::kColFast) {
     // both operands contiguous along K: the tcgen05 kernel, when nothing is split or accumulated
-    if (gz == 1 && !e.atomic && !Klim && K > 0 && ldc % 4 == 0) {
-      gemm_tc_kernel<AV, BV><<<dim3(gx, gy), NT, 0, s>>>(A, B, M, N, K, C, ldc, e, Mlim);
+    if (gz == 1 && !e.atomic && K > 0 && ldc % 4 == 0) {
+      gemm_tc_kernel<AV, BV><<<dim3(gx, gy), NT, 0, s>>>(A, B, M, N, K, C, ldc, e);
       return cudaGetLastError();
     }
   }
-  gemm_kernel<AV, BV><<<dim3(gx, gy, gz), NT, 0, s>>>(A, B, M, N, K, kchunk, C, ldc, e, Mlim, Klim);
+  gemm_kernel<AV, BV><<<dim3(gx, gy, gz), NT, 0, s>>>(A, B, M, N, K, kchunk, C, ldc, e);
   return cudaGetLastError();
 }
 
@@ -700,19 +651,7 @@ __global__ void interleave_kernel(const uint32_t* pi, const uint32_t* pj, int m,
 
 inline unsigned blocks_for(size_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
 
-// log2 of a channel count (32 or 128: the views index taps by shifts)
-inline int log2_ch(int c) {
-  int l = 0;
-  while ((1 << l) < c) ++l;
-  return l;
-}
-
 }  // namespace
-
-cudaError_t conv_fwd(const float* X, int Ci, const float* W, int Co, const Packed& pk, float* Y, const Epi& e,
-                     cudaStream_t s) {
-  return run_gemm(Im2col{X, pk.rinfo, log2_ch(Ci)}, DenseT{W, 3 * Ci}, pk.Tmax, Co, 3 * Ci, Y, Co, e, 1, s, pk.T);
-}
 
 cudaError_t lin_fwd(const float* P, int Ci, const float* Wl, int Co, int B, float* E, const Epi& e, cudaStream_t s) {
   return run_gemm(Dense{P, Ci}, DenseT{Wl, Ci}, B, Co, Ci, E, Co, e, 1, s);

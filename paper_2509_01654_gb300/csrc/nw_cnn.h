@@ -63,12 +63,10 @@ struct Packed {
   int Bw, Tmax;
 };
 
-// GEMM epilogue: out = acc (+ bias[n]) (ReLU) (x (gate[m][n] > 0)), or
-// atomicAdd of acc (split-K accumulation into a zeroed C).
+// GEMM epilogue: out = acc (+ bias[n]), or atomicAdd of acc (split-K
+// accumulation into a zeroed C).
 struct Epi {
   const float* bias = nullptr;
-  bool relu = false;
-  const float* gate = nullptr;   // same layout as C
   bool atomic = false;
   uint32_t* err = nullptr;       // receives kErrWait if a tensor-core pipeline wait runs out (may be null)
 };
@@ -77,7 +75,7 @@ struct Epi {
 // to bf16 (nearest even) as they are loaded, float32 accumulation.  W is
 // [Co][3][Ci], Wl is [Co][Ci]; Ci and Co of a convolution are powers of
 // two; activations of a packed batch have pk.T rows.
-//   conv_fwd: Y[T][Co]  = im2col(X[T][Ci]) . W^T            (epilogue e)
+//   conv_fwd: Y[T][Co]  = max(im2col(X[T][Ci]) . W^T + bias, 0)
 //   conv_bwd: dW[Co][3Ci] += dY^T . im2col(X), db[Co] += column sums of dY and
 //             dX[T][Ci] = sum_tap shift_tap(dY) . W[.][tap], x (X > 0) for layers 2 and 3
 //   lin_fwd:  E[B][Co]  = P[B][Ci] . Wl^T                   (epilogue e)
@@ -85,10 +83,13 @@ struct Epi {
 //   lin_dx:   dP[B][Ci] = dE[B][Co] . Wl
 // im2col(X) row t, column tap * Ci + c, is X[t + tap - 1][c] when position
 // pos(t) + tap - 1 lies inside t's word, else 0 (the zero padding).
-cudaError_t conv_fwd(const float* X, int Ci, const float* W, int Co, const Packed& pk, float* Y, const Epi& e,
-                     cudaStream_t s);
+// conv_fwd takes pack_fwd's weights (fwd_pack_bytes()), conv_bwd pack_bwd's (bwd_pack_bytes())
+size_t fwd_pack_bytes();
+cudaError_t pack_fwd(const float* params, const Layout& L, void* pack, cudaStream_t s);
+cudaError_t conv_fwd(int layer, const float* X, const Packed& pk, const void* pack, const float* bias, float* Y,
+                     uint32_t* err, int sms, cudaStream_t s);
 // layer 3 takes its output gradient from the mean's (dP) and its output Ytop,
-// layers 2 and 1 from dY; `pack` holds pack_bwd's bwd_pack_bytes() of weights
+// layers 2 and 1 from dY
 size_t bwd_pack_bytes();
 cudaError_t pack_bwd(const float* params, const Layout& L, void* pack, cudaStream_t s);
 cudaError_t conv_bwd(int layer, const float* dY, const float* Ytop, const float* dP, const float* X, const Packed& pk,
@@ -151,8 +152,7 @@ cudaError_t pair_targets(const int16_t* score, const uint32_t* pi, const uint32_
                          const uint8_t* slen, int m, float raw_scale, float* target, cudaStream_t s);
 cudaError_t interleave_pairs(const uint32_t* pi, const uint32_t* pj, int m, uint32_t* widx, cudaStream_t s);
 // embeddings of all words of a set into out[original index][64], on at most
-// `sms` SMs; `pack` holds embed_pack_bytes() of scratch
-size_t embed_pack_bytes();
+// `sms` SMs; `pack` holds fwd_pack_bytes() of scratch
 cudaError_t embed_words(const float* params, const Layout& L, uint32_t alphabet, const Buckets& bk, const uint32_t* sym,
                         const uint32_t* perm, uint32_t shift, void* pack, float* out, uint32_t* err, int sms,
                         cudaStream_t s);

@@ -454,7 +454,12 @@ __global__ void __launch_bounds__(kThreads, 1) embed_kernel(const __grid_constan
 
 }  // namespace
 
-size_t embed_pack_bytes() { return kPackBytes; }
+size_t fwd_pack_bytes() { return kPackBytes; }
+
+cudaError_t pack_fwd(const float* params, const Layout& L, void* pack, cudaStream_t s) {
+  pack_weights_kernel<<<(unsigned)((kPackBytes / 2 + 255) / 256), 256, 0, s>>>(params, L, static_cast<__nv_bfloat16*>(pack));
+  return cudaGetLastError();
+}
 
 cudaError_t embed_words(const float* params, const Layout& L, uint32_t alphabet, const Buckets& bk, const uint32_t* sym,
                         const uint32_t* perm, uint32_t shift, void* pack, float* out, uint32_t* err, int sms,
@@ -478,8 +483,9 @@ cudaError_t embed_words(const float* params, const Layout& L, uint32_t alphabet,
   }
   P.first[kBuckets] = P.nblocks;
   if (P.nblocks == 0) return cudaSuccess;
-  pack_weights_kernel<<<(unsigned)((kPackBytes / 2 + 255) / 256), 256, 0, s>>>(params, L, static_cast<__nv_bfloat16*>(pack));
-  cudaError_t e = cudaFuncSetAttribute(embed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  cudaError_t e = pack_fwd(params, L, pack, s);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(embed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) return e;
   embed_kernel<<<std::min<unsigned>((P.nblocks + 1u) / 2u, (unsigned)sms), kThreads, kSmem, s>>>(P);
   return cudaGetLastError();

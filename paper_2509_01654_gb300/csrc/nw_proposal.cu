@@ -124,6 +124,7 @@ nw_status ensure_scratch(nw_model* M, int Bw, int Tmax) {
   NW_TRY(ctx_ensure(c, M->off, sizeof(int) * W, "model word offsets"));
   NW_TRY(ctx_ensure(c, M->poff, sizeof(int) * W, "model word offsets"));
   NW_TRY(ctx_ensure(c, M->prow, sizeof(int) * (T + W), "model row tables"));
+  NW_TRY(ctx_ensure(c, M->Wpack, cnn::fwd_pack_bytes(), "packed weights"));
   NW_TRY(ctx_ensure(c, M->Wbwd, cnn::bwd_pack_bytes(), "packed weights"));
   NW_TRY(ctx_ensure(c, M->rinfo, sizeof(int) * T, "model row tables"));
   NW_TRY(ctx_ensure(c, M->rword, sizeof(int) * T, "model row tables"));
@@ -191,15 +192,11 @@ nw_status forward(nw_model* M, const nw_dict* d, int Bw, int Tmax, cudaStream_t 
                    M->poff.as<int>(), M->prow.as<int>(), padded_rows_ptr(M), M->codes.as<int32_t>()};
   NW_CK(cnn::pack_words(word_src(d->ws, d->ss.shift, M->widx.as<uint32_t>()), Bw, Tmax, W + L.emb, pb, fptr(M->X0),
                         err_ptr(M), M->alphabet, s));
-  cnn::Epi e;
-  e.relu = true;
-  e.err = err_ptr(M);
-  e.bias = W + L.b1;
-  NW_CK(cnn::conv_fwd(fptr(M->X0), cnn::kEmb, W + L.W1, cnn::kCh, pk, fptr(M->Y1), e, s));
-  e.bias = W + L.b2;
-  NW_CK(cnn::conv_fwd(fptr(M->Y1), cnn::kCh, W + L.W2, cnn::kCh, pk, fptr(M->Y2), e, s));
-  e.bias = W + L.b3;
-  NW_CK(cnn::conv_fwd(fptr(M->Y2), cnn::kCh, W + L.W3, cnn::kCh, pk, fptr(M->Y3), e, s));
+  NW_CK(cnn::pack_fwd(W, L, M->Wpack.p, s));
+  float* X[] = {fptr(M->X0), fptr(M->Y1), fptr(M->Y2), fptr(M->Y3)};
+  const uint64_t bias[] = {L.b1, L.b2, L.b3};
+  for (int l = 1; l <= 3; ++l)
+    NW_CK(cnn::conv_fwd(l, X[l - 1], pk, M->Wpack.p, W + bias[l - 1], X[l], err_ptr(M), c->sm_count, s));
   NW_CK(cnn::mean_pool(fptr(M->Y3), pk, fptr(M->P), s));
   cnn::Epi el;
   el.bias = W + L.bl;
@@ -280,7 +277,7 @@ uint64_t splitmix64_next(uint64_t& st) {
 nw_status embed_all(nw_model* M, const WordSet& ws, uint32_t shift, cudaStream_t s) {
   nw_ctx* c = M->ctx;
   NW_TRY(ctx_ensure(c, M->Eall, sizeof(float) * std::max<size_t>(1, (size_t)ws.n * cnn::kOut), "embeddings"));
-  NW_TRY(ctx_ensure(c, M->Wpack, cnn::embed_pack_bytes(), "packed weights"));
+  NW_TRY(ctx_ensure(c, M->Wpack, cnn::fwd_pack_bytes(), "packed weights"));
   NW_CK(cnn::embed_words(fptr(M->params), M->L, M->alphabet, ws.bk, ws.a_enc.as<uint32_t>(), ws.perm.as<uint32_t>(),
                          shift, M->Wpack.p, fptr(M->Eall), err_ptr(M), c->sm_count, s));
   return NW_OK;
