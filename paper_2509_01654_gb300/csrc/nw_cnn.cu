@@ -400,14 +400,19 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int* len, int 
                                                             int Tmax, uint32_t* err) {
   __shared__ long long warp_sum[kScanThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int per = (Bw + kScanThreads - 1) / kScanThreads;
+  const int per = ((Bw + kScanThreads - 1) / kScanThreads + 3) & ~3;  // whole groups of four words
   const int w0 = min(Bw, tid * per), w1 = min(Bw, w0 + per);
-  auto item = [&](int w) {  // rows below, words with rows above
-    const int l = len[w];
-    return (long long)l | ((long long)(l > 0) << 32);
+  auto item = [](int l) { return (long long)l | ((long long)(l > 0) << 32); };  // rows below, words with rows above
+  auto four = [&](int w) {
+    if (w + 4 <= w1) return *reinterpret_cast<const int4*>(len + w);
+    return make_int4(len[w], w + 1 < w1 ? len[w + 1] : 0, w + 2 < w1 ? len[w + 2] : 0, 0);
   };
   long long local = 0;
-  for (int w = w0; w < w1; ++w) local += item(w);
+#pragma unroll 4
+  for (int w = w0; w < w1; w += 4) {
+    const int4 l = four(w);
+    local += item(l.x) + item(l.y) + item(l.z) + item(l.w);
+  }
   long long incl = local;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -427,10 +432,26 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int* len, int 
   }
   __syncthreads();
   long long run = incl - local + (warp ? warp_sum[warp - 1] : 0);
-  for (int w = w0; w < w1; ++w) {
-    off[w] = (int)run;
-    poff[w] = (int)run + (int)(run >> 32);
-    run += item(w);
+#pragma unroll 4
+  for (int w = w0; w < w1; w += 4) {
+    const int4 l = four(w);
+    const int v[4] = {l.x, l.y, l.z, l.w};
+    int o[4], p[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      o[i] = (int)run;
+      p[i] = (int)run + (int)(run >> 32);
+      run += item(v[i]);
+    }
+    if (w + 4 <= w1) {
+      *reinterpret_cast<int4*>(off + w) = make_int4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<int4*>(poff + w) = make_int4(p[0], p[1], p[2], p[3]);
+    } else {
+      for (int i = 0; w + i < w1; ++i) {
+        off[w + i] = o[i];
+        poff[w + i] = p[i];
+      }
+    }
   }
   if (tid == kScanThreads - 1) {
     const long long all = warp_sum[kScanThreads / 32 - 1];
@@ -457,8 +478,8 @@ __global__ void fill_rows_kernel(const int* len, const int* off, const int* poff
 // one warp per packed row: lane = embedding channel
 __global__ void gather_kernel(WordSrc src, const int* Tdev, int Tmax, const float* __restrict__ emb, const int* rinfo,
                               const int* rword, int32_t* codes, float* X0, uint32_t* err, uint32_t alphabet) {
-  const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
+  const int row = blockIdx.x * (blockDim.x / 8) + threadIdx.x / 8;  // eight lanes a row
+  const int lane = threadIdx.x & 7;
   if (row >= min(Tmax, *Tdev)) return;
   const int w = rword[row], t = rinfo[row] >> 8;
   const uint32_t pos = __ldg(src.rank + src.widx[w]);
@@ -469,7 +490,8 @@ __global__ void gather_kernel(WordSrc src, const int* Tdev, int Tmax, const floa
     code = -1;
   }
   if (lane == 0) codes[row] = code;
-  X0[(size_t)row * kEmb + lane] = code >= 0 ? __ldg(emb + (size_t)code * kEmb + lane) : 0.f;
+  reinterpret_cast<float4*>(X0 + (size_t)row * kEmb)[lane] =
+      code >= 0 ? __ldg(reinterpret_cast<const float4*>(emb + (size_t)code * kEmb) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // P[w] = mean of word w's rows (0 for an empty word)
@@ -482,6 +504,20 @@ __global__ void pool_kernel(const float* __restrict__ Y, const int* len, const i
   float acc = 0.f;
   for (int t = 0; t < L; ++t) acc += Y[((size_t)o + t) * kCh + ch];
   P[x] = L > 0 ? acc / (float)L : 0.f;
+}
+
+__global__ void mean_grad_kernel(float* dP, const int* len, int Bw) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;  // four channels
+  if (x >= Bw * (kCh / 4)) return;
+  const int L = len[x / (kCh / 4)];
+  if (L <= 1) return;
+  float4 v = reinterpret_cast<float4*>(dP)[x];
+  const float f = (float)L;
+  v.x /= f;
+  v.y /= f;
+  v.z /= f;
+  v.w /= f;
+  reinterpret_cast<float4*>(dP)[x] = v;
 }
 
 // one warp per pair: lanes hold dimensions lane and lane + 32.  The 64
@@ -509,7 +545,7 @@ __global__ void pair_loss_kernel(const float* __restrict__ E, const float* __res
   if (lane == 0 && loss_acc) atomicAdd(loss_acc, diff * diff / (float)m);
 }
 
-constexpr int kColSumRows = 256;
+constexpr int kColSumRows = 64;
 
 __global__ void col_sum_kernel(const float* __restrict__ Y, int rows, int cols, float* out) {
   const int c = threadIdx.x;
@@ -676,7 +712,7 @@ cudaError_t pack_words(const WordSrc& src, int Bw, int Tmax, const float* emb, c
   word_len_kernel<<<blocks_for(Bw, 256), 256, 0, s>>>(src, Bw, b.len, err);
   scan_kernel<<<1, kScanThreads, 0, s>>>(b.len, Bw, b.off, b.T, b.poff, b.Tp, Tmax, err);
   fill_rows_kernel<<<blocks_for(Bw, 256), 256, 0, s>>>(b.len, b.off, b.poff, Bw, Tmax, b.rinfo, b.rword, b.prow);
-  gather_kernel<<<blocks_for((size_t)Tmax, 8), 256, 0, s>>>(src, b.T, Tmax, emb, b.rinfo, b.rword, b.codes, X0, err,
+  gather_kernel<<<blocks_for((size_t)Tmax, 32), 256, 0, s>>>(src, b.T, Tmax, emb, b.rinfo, b.rword, b.codes, X0, err,
                                                              alphabet);
   return cudaGetLastError();
 }
@@ -684,6 +720,12 @@ cudaError_t pack_words(const WordSrc& src, int Bw, int Tmax, const float* emb, c
 cudaError_t mean_pool(const float* Y, const Packed& pk, float* P, cudaStream_t s) {
   if (pk.Bw <= 0) return cudaSuccess;
   pool_kernel<<<blocks_for((size_t)pk.Bw * kCh, 256), 256, 0, s>>>(Y, pk.len, pk.off, pk.Bw, pk.Tmax, P);
+  return cudaGetLastError();
+}
+
+cudaError_t mean_grad(float* dP, const Packed& pk, cudaStream_t s) {
+  if (pk.Bw <= 0) return cudaSuccess;
+  mean_grad_kernel<<<blocks_for((size_t)pk.Bw * (kCh / 4), 256), 256, 0, s>>>(dP, pk.len, pk.Bw);
   return cudaGetLastError();
 }
 

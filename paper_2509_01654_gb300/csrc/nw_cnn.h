@@ -88,8 +88,8 @@ size_t fwd_pack_bytes();
 cudaError_t pack_fwd(const float* params, const Layout& L, void* pack, cudaStream_t s);
 cudaError_t conv_fwd(int layer, const float* X, const Packed& pk, const void* pack, const float* bias, float* Y,
                      uint32_t* err, int sms, cudaStream_t s);
-// layer 3 takes its output gradient from the mean's (dP) and its output Ytop,
-// layers 2 and 1 from dY
+// layer 3 takes its output gradient from the mean's (mean_grad's dP) and its
+// output Ytop, layers 2 and 1 from dY
 size_t bwd_pack_bytes();
 cudaError_t pack_bwd(const float* params, const Layout& L, void* pack, cudaStream_t s);
 cudaError_t conv_bwd(int layer, const float* dY, const float* Ytop, const float* dP, const float* X, const Packed& pk,
@@ -114,6 +114,8 @@ struct PackBufs {
 cudaError_t pack_words(const WordSrc& src, int Bw, int Tmax, const float* emb, const PackBufs& b, float* X0,
                        uint32_t* err, uint32_t alphabet, cudaStream_t s);
 cudaError_t mean_pool(const float* Y, const Packed& pk, float* P, cudaStream_t s);
+// dP[w] /= the word's length (the gradient of each of its rows)
+cudaError_t mean_grad(float* dP, const Packed& pk, cudaStream_t s);
 // pairs are word slots (2p, 2p + 1), pred = phi . phi + beta + beta (outputs
 // 0..62 features, 63 bias); loss_acc += sum (pred - y)^2 / m (if non-null)
 cudaError_t pair_loss(const float* E, const float* target, int m, float* dE, float* loss_acc, cudaStream_t s);

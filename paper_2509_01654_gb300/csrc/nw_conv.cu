@@ -62,9 +62,8 @@ static_assert(kWarps * 2 * 4 == kRows && kWarps * kCh * 4 <= kAct, "four rows a 
 
 struct BwdArgs {
   const float* dY;      // output gradient, or (top layer) null:
-  const float* Ytop;    //   the layer's output, its gradient the mean's: Y > 0 ? dP[word] / length : 0
+  const float* Ytop;    //   the layer's output, its gradient the mean's: Y > 0 ? dP[word] : 0
   const float* dP;
-  const int* rinfo;
   const int* rword;
   const float* X;       // the layer's input
   const int* prow;
@@ -195,12 +194,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_bwd_kernel(const __grid_cons
 #pragma unroll
     for (int q = 0; q < 5; ++q) row[q] = nrow[q];
     if (kTop) {
-      int word[5], info[5];
+      int word[5];
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        word[q] = row[q] >= 0 ? __ldg(P.rword + row[q]) : 0;
-        info[q] = row[q] >= 0 ? __ldg(P.rinfo + row[q]) : 1;
-      }
+      for (int q = 0; q < 5; ++q) word[q] = row[q] >= 0 ? __ldg(P.rword + row[q]) : 0;
 #pragma unroll
       for (int q0 = 0; q0 < 5; q0 += 3) {  // (three rows of both operands at a time: registers)
         float4 y[6], d[6];
@@ -216,9 +212,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_bwd_kernel(const __grid_cons
         }
 #pragma unroll
         for (int i = 0; i < 3 && q0 + i < 5; ++i) {
-          const float len = (float)(info[q0 + i] & 255);
-          auto f = [&](float yv, float dv) { return yv > 0.f ? dv / len : 0.f; };
           const float4 ya = y[2 * i], yb = y[2 * i + 1], da = d[2 * i], e = d[2 * i + 1];
+          auto f = [](float yv, float dv) { return yv > 0.f ? dv : 0.f; };
           add_dy(q0 + i, make_float4(f(ya.x, da.x), f(ya.y, da.y), f(ya.z, da.z), f(ya.w, da.w)),
                  make_float4(f(yb.x, e.x), f(yb.y, e.y), f(yb.z, e.z), f(yb.w, e.w)));
         }
@@ -533,7 +528,6 @@ cudaError_t conv_bwd(int layer, const float* dY, const float* Ytop, const float*
   P.dY = dY;
   P.Ytop = Ytop;
   P.dP = dP;
-  P.rinfo = pk.rinfo;
   P.rword = pk.rword;
   P.X = X;
   P.prow = pk.prow;

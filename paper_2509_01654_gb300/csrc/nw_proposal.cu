@@ -219,6 +219,7 @@ nw_status backward(nw_model* M, int m, int Tmax, cudaStream_t s) {
   NW_CK(cnn::lin_dw(fptr(M->dE), cnn::kOut, fptr(M->P), cnn::kCh, Bw, G + L.Wl, nsm, s));
   NW_CK(cnn::col_sum(fptr(M->dE), Bw, cnn::kOut, G + L.bl, s));
   NW_CK(cnn::lin_dx(fptr(M->dE), cnn::kOut, W + L.Wl, cnn::kCh, Bw, fptr(M->dP), s));
+  NW_CK(cnn::mean_grad(fptr(M->dP), pk, s));
   NW_CK(cnn::pack_bwd(W, L, M->Wbwd.p, s));
   // dYb = dY2, dYa = dY1
   NW_CK(cnn::conv_bwd(3, nullptr, fptr(M->Y3), fptr(M->dP), fptr(M->Y2), pk, M->Wbwd.p, fptr(M->dYb), G + L.W3, G + L.b3,
