@@ -13,13 +13,20 @@
 //
 // Match masks.  A block (four warps) keeps the masks of its B words in shared
 // memory, masks[code][lane] (256 bytes a code), built once per task; the
-// warps share them and take 16 A words at a time each.  A row costs one
-// broadcast read of the A symbol's table offset and one conflict-free 8-byte
-// read.
+// warps share them and take P.sub A words (kBitSub, fewer in small tasks) at a
+// time each.  A row costs one broadcast read of the A symbol's code and one
+// conflict-free 8-byte read.
 //
 // Score.  G = g * (sum of the word's h) = g * (sum of the planes' bit counts);
 // for m >= 3 the planes are first recoded to binary digits, so that a word
 // takes two or three bit counts.
+//
+// What bounds it: the logic pipe.  A row of (1, -1, -1), steps (3, 1), is 17
+// logic and add instructions per 32 columns, 34 a lane for up to 48 cells
+// where the DPX cell takes 3 for 2.  600k words, top-10 and histogram: 1,129
+// ms on the DPX kernel, 390 here, of which the row logic at the measured LOP3
+// rate is about 280, lists that move about 25 and the histogram's shared
+// additions 13 to 20.
 #pragma once
 
 #include "nw_bitrow.cuh"
@@ -195,7 +202,7 @@ __device__ __forceinline__ void bit_task(const AlignParams& P, const Terms& T, c
 #pragma unroll
             for (int i = 1; i < KP; ++i) G = (w >> 1) == i ? res[i] : G;
             G = (w & 1) ? G >> 16 : G & 0xffffu;
-            filed |= queue_candidate(P, T, Q, queue, waiting, inserts, cand != 0u,
+            filed |= queue_candidate<kFileAhead<EPI>>(P, T, Q, queue, waiting, inserts, cand != 0u,
                                      (G << 16) | ((a - g.a0) << 8) | (32u * (uint32_t)w + (uint32_t)lane));
             cand &= cand - 1u;
           }
@@ -210,7 +217,7 @@ __device__ __forceinline__ void bit_task(const AlignParams& P, const Terms& T, c
   if constexpr (kLists) {
     if (waiting) {
       __syncwarp();
-      inserts += file_candidates(P, T, Q, queue, waiting);
+      inserts += file_candidates<kFileAhead<EPI>>(P, T, Q, queue, waiting);
     }
   }
 }
