@@ -6,7 +6,7 @@
 // code shift.  The pair lists of all dictionaries and query sets are planned
 // together, each rectangle tagged with its terms (3d for dictionary d's own
 // pairs, 3d + 1 for its queries as A words, 3d + 2 for its queries as B words);
-// the kernels (epilogue kEpiBatchLists) read those terms' word sets, lists and
+// the kernels (epilogue kEpiOtherLists) read those terms' word sets, lists and
 // scoring per task.  Dictionaries whose scoring the bit-parallel kernel takes
 // share one launch per step class, on a second stream; the others share one
 // DPX launch per range of longer lengths, whose A-chunk size is a tile-shape
@@ -97,7 +97,7 @@ nw_status issue_lists(nw_batch* B, const Plan& plan) {
   for (size_t i = 0; i < plan.launches.size() && st == NW_OK; ++i) {
     AlignParams P = batch_params(B);
     P.counter = reinterpret_cast<unsigned long long*>(B->d_small.as<char>() + 64) + i;
-    st = run_launch(c, plan.launches[i].range < 0 ? B->side : s, plan.launches[i], B->d_segs.as<Seg>(), kEpiBatchLists,
+    st = run_launch(c, plan.launches[i].range < 0 ? B->side : s, plan.launches[i], B->d_segs.as<Seg>(), kEpiOtherLists,
                     P, tm, ro);
   }
   NW_CK(cudaEventRecord(B->joined, B->side));

@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kBitBlock, kBitMinBlocks) nw_bit_kernel(const 
     const Seg* S = P.segs + s_seg[buf];
     {
       const uint32_t d = S->dict;
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(EPI == kEpiBatchLists ? P.terms + d : P.local + d);
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(EPI == kEpiOtherLists && P.terms ? P.terms + d : P.local + d);
       if (tid < (int)(sizeof(Terms) / 4)) reinterpret_cast<uint32_t*>(&T)[tid] = src[tid];
     }
     if (tid == kBitBlock - 1) {

@@ -28,8 +28,7 @@
 // so G[i-1][j-1] + s'_x < 0 + G[i-1][j-1] <= G[i-1][j] whenever s'_x < 0 and
 // raising the mismatch term to 0 changes no maximum; it keeps f >= 0, so the
 // packed add never carries between halves (G + f <= s'_m * LB < 2^15).
-// Per two cells: one LOP3, one add and two DPX instructions; rows go two at
-// a time so the two rows' dependency chains interleave.
+// Per two cells: one LOP3, one add and two DPX instructions.
 //
 // Substitution-matrix scoring (TAB): the lane holds its B words' codes
 // (lo / hi halves) and the per-cell term is read from the table row of the A
@@ -318,10 +317,11 @@ __device__ __forceinline__ uint32_t neg_bound2(int t_lo, int t_hi) {
 // have lists the best of a warp's candidates is offered first (a query's empty
 // list is offered to by hundreds of warps at once).  One query against 100k
 // words 251 -> 183 us, 4,096 against 600k 14.2 -> 12.3 ms, 16 dictionaries 8.97
-// -> 8.13 ms.  The histogram kernels, whose lists belong to both sides, lose by
-// it (600k 390 -> 418 ms): there it is compiled out.
+// -> 8.13 ms.  The all-pairs kernels, whose lists belong to both sides, lose by
+// it at 600k words (390 -> 418 ms with histogram, 380 -> 410 normalised): there
+// it is compiled out.
 template <int EPI>
-constexpr bool kFileAhead = EPI != kEpiListsLaneHist;
+constexpr bool kFileAhead = EPI == kEpiOtherLists;
 template <bool kAhead>
 __device__ __forceinline__ uint32_t file_candidates(const AlignParams& P, const Terms& T, const AlignTask& Q,
                                                     const uint32_t* queue, uint32_t n) {
@@ -391,8 +391,8 @@ __device__ __forceinline__ bool queue_candidate(const AlignParams& P, const Term
 // LB.  TAB selects substitution-matrix scoring; EPI the per-pair epilogue:
 // kEpiMatrix writes the int8 upper triangle, kEpiLists updates neighbour lists
 // (and a shared or global histogram), kEpiListsLaneHist lists and the lane
-// columns of the shared histogram, kEpiBatchLists the lists named by the
-// segment's terms in a launch spanning many dictionaries.
+// columns of the shared histogram, kEpiOtherLists the lists of queries and of
+// batches (named by the segment's terms in a launch spanning dictionaries).
 template <int LB, int EPI, bool TAB>
 __device__ __forceinline__ void dp_task(const AlignParams& P, const Terms& T, const AlignTask& Q, uint32_t* wh,
                                         uint32_t* sA, const uint16_t* sTab, uint32_t* queue, uint32_t& inserts) {
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(kBlock, dp_min_blocks(HI)) nw_dp_kernel(const 
     if (t >= P.ntasks) break;
     const Seg* S = P.segs + find_seg(P.segs, P.nsegs, t);
     const uint32_t d = S->dict;
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(EPI == kEpiBatchLists ? P.terms + d : P.local + d);
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(EPI == kEpiOtherLists && P.terms ? P.terms + d : P.local + d);
     __syncwarp();
     for (int q = lane; q < (int)(sizeof(Terms) / 4); q += 32) reinterpret_cast<uint32_t*>(&T)[q] = src[q];
     if (lane == 0) {

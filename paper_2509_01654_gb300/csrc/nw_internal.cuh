@@ -209,8 +209,10 @@ struct AlignTask {
 constexpr uint32_t kQueueEntries = 64;
 
 // per-pair epilogue of the all-pairs kernel (a template parameter);
-// kEpiBatchLists reads the terms of a segment from AlignParams::terms
-enum { kEpiMatrix = 0, kEpiLists = 1, kEpiListsLaneHist = 2, kEpiBatchLists = 3, kEpiKinds = 4 };
+// kEpiOtherLists: lists without a histogram for queries and batches, whose
+// candidates are filed another way (kFileAhead), with a segment's terms from
+// AlignParams::terms if given
+enum { kEpiMatrix = 0, kEpiLists = 1, kEpiListsLaneHist = 2, kEpiOtherLists = 3, kEpiKinds = 4 };
 
 // Histogram accumulation mode for `nbins` bins: per-lane columns shared by a
 // block while they fit in 48 KiB (384 bins), else one shared array per warp,
