@@ -4,7 +4,7 @@
 One step = the whole path over one synthetic dictionary of 600,000 words
 (lengths round(N(8, 3)) on [1, 25], 40 codes with Zipf(1.1) usage, index =
 frequency rank): ingest and length bucketing on the device, every one of the
-179,999,700,000 upper-triangle pairs scored by the DPX alignment kernel, the
+179,999,700,000 upper-triangle pairs scored by the bit-parallel alignment kernel, the
 on-device per-word top-10 and score histogram, list finalisation.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--sharded]
@@ -44,15 +44,40 @@ L2_FLUSH_BYTES = 512 << 20
 # workload, from an ncu capture of dram__bytes_read.sum + dram__bytes_write.sum
 # (summarised under profiles/); valid only while the kernel sources hash to
 # kernel_sha, and reported as null otherwise
-TRAFFIC = {"kernel_sha": "e8027e6a77ddc0f4", "bytes_per_step": 441.6e6}
+TRAFFIC = {"kernel_sha": "df755f379759f5ef", "bytes_per_step": 98.5e6}
 
 
 def kernel_sha() -> str:
     h = hashlib.sha256()
-    for f in ("nw_dp.cuh", "nw_internal.cuh"):
+    for f in ("nw_bitrow.cuh", "nw_bits.cuh", "nw_dp.cuh", "nw_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2509_01654_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
+
+
+def bit_words_per_lane(b: int) -> int:
+    """Words of length b that share a lane's 64 columns in the bit-parallel kernel."""
+    return 8 if b <= 8 else 7 if b == 9 else 6 if b == 10 else 5 if b <= 12 else 4 if b <= 16 else \
+        3 if b <= 21 else 2 if b <= 32 else 1
+
+
+# logic and add instructions of one row of 64 columns for the reduced steps
+# (3, 1) of the scoring (1, -1, -1): 14 LOP3 and 3 additions per 32 columns
+ROW_OPS = 34
+
+
+def row_ops_per_set(lengths) -> float:
+    """Lane instructions of the bit-parallel rows of every unordered pair of
+    words of these lengths, each pair of lengths the cheaper way round: the
+    least work of that kernel's formulation, without scores, lists or histogram."""
+    import numpy as np
+    cnt = np.bincount(np.asarray(lengths, dtype=np.int64))
+    rows = 0.0
+    for a in range(len(cnt)):
+        for b in range(a, len(cnt)):
+            pairs = cnt[a] * cnt[b] if a < b else cnt[a] * (cnt[a] - 1) / 2
+            rows += float(pairs) * min(a / bit_words_per_lane(b), b / bit_words_per_lane(a))
+    return ROW_OPS * rows
 
 
 def tensor_roofline(flops: float, ms: float, peaks_path: str = os.path.join(ROOT, "MEASURED_PEAKS.json")) -> dict:
@@ -324,12 +349,13 @@ def run_ours(args, rank, world, local_rank):
     value = copies * pairs * args.steps / (total_ms / 1e3)
     e2e_value = copies * pairs * len(e2e_times) / (total_e2e / 1e3)
 
-    # roofline of the alignment kernel: algorithmic cells over its launches' event time
+    # roofline of the alignment kernel: algorithmic cells over its launches' event time,
+    # against the bit-parallel rows alone at the measured LOP3 rate
     # (a shard holds 1/world of the cells: the planner cuts each launch into equal task ranges)
     dp_avg_ms = statistics.mean(dp_ms)
     achieved = (cells / world if sharded else cells) / (dp_avg_ms / 1e3) / 1e9
-    c_min = 3.0  # packed instructions per two cells in the fewest-instruction cell update
-    peak = 2.0 * rates["viaddmax_s16x2"] / c_min / 1e9
+    row_ops = row_ops_per_set(w.lengths)
+    peak = cells / (row_ops / rates["lop3"]) / 1e9
     sha = kernel_sha()
     traffic = TRAFFIC["bytes_per_step"] if TRAFFIC["kernel_sha"] == sha and args.n == 600_000 else None
 
@@ -427,7 +453,7 @@ def run_ours(args, rank, world, local_rank):
     # issue width implied by the measured rate at the SM clock nvidia-smi reported under load
     lanes_note = ""
     if clocks and clocks.get("sm_mhz"):
-        lanes = rates["viaddmax_s16x2"] / (rates["sm_count"] * clocks["sm_mhz"] * 1e6)
+        lanes = rates["lop3"] / (rates["sm_count"] * clocks["sm_mhz"] * 1e6)
         lanes_note = f", {lanes:.1f} lanes/clk/SM at the {clocks['sm_mhz']:.0f} MHz median SM clock under load"
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -438,11 +464,12 @@ def run_ours(args, rank, world, local_rank):
         "dp_kernel_ms_per_step": dp_avg_ms,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "GCUPS",
                      "frac": achieved / peak, "traffic": traffic,
-                     "traffic_basis": "DRAM bytes of one step's alignment launches (all 22), ncu, 600k words",
-                     "peak_basis": f"2 cells x measured __viaddmax_s16x2 rate ({rates['viaddmax_s16x2']:.4g}/s "
-                                   f"over {rates['sm_count']} SMs{lanes_note}) / {c_min:g} "
-                                   f"packed instructions per cell pair; cell-mix microbenchmark "
-                                   f"{2 * rates['nw_cell_mix'] / 1e9:.0f} GCUPS",
+                     "traffic_basis": "DRAM bytes of one step's alignment launch, ncu, 600k words",
+                     "peak_basis": f"bit-parallel rows alone ({ROW_OPS} logic and add instructions a lane for 64 "
+                                   f"columns, {row_ops:.4g} lane instructions) at the measured lop3 rate "
+                                   f"({rates['lop3']:.4g}/s over {rates['sm_count']} SMs{lanes_note}); the DPX cell "
+                                   f"(3 packed instructions for 2 cells) would peak at "
+                                   f"{2 * rates['viaddmax_s16x2'] / 3 / 1e9:.0f} GCUPS",
                      "rates_per_s": {key: rates[key] for key in ("viaddmax_s16x2", "vimax3_s16x2",
                                                                   "vimax_s16x2_relu", "iadd3", "lop3")}},
         "cpu_baseline": cpu,

@@ -247,9 +247,9 @@ nw_status nw_query(nw_dict *dict, const uint8_t *qcodes, const uint32_t *qoffset
  * set of its own size and lengths (Section 6's search for similar-sounding
  * words, nw_query), answered in the same launch.  nw_batch_create loads every
  * dictionary and query set, plans all their pairs together (one alignment
- * launch per longer length covering every dictionary and query set),
- * optionally autotunes the tile shape (A words per task) of each launch by
- * timing candidates on the batch itself, and captures the whole reduction --
+ * launch per class of scorings or range of ten longer lengths, covering every
+ * dictionary and query set), optionally autotunes the tile shapes of the
+ * latter by timing candidates on the batch itself, and captures the whole reduction --
  * list resets, alignment launches, list finalisation -- into a CUDA graph.
  * nw_batch_run / nw_batch_run_queries replay the graph and copy the lists
  * out.  Results equal nw_all_pairs_topk run on each dictionary alone and
@@ -451,7 +451,7 @@ nw_status nw_debug_enumerate_pairs(const uint32_t *lengths, uint32_t n, uint32_t
 /* Host-only: the (query, dictionary word) pairs that nw_query's kernels
  * would score for query words of lengths q_lengths[0..nq) against dictionary
  * words of lengths d_lengths[0..nd), with at most `ta` A words per task (0 =
- * the default; a launch with few tasks takes smaller chunks, down to 32
+ * the default; a launch with few tasks takes smaller chunks, down to 16
  * words, as nw_query plans it), as original-index pairs (q[p], d[p]).
  * Writes at most `cap` pairs and sets *count to the total.  Runs the same
  * query planner and task-to-pair mapping as the kernels, on the CPU, so tests

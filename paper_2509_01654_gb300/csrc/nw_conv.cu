@@ -6,8 +6,9 @@
 // As separate products (forward with gathered windows; dW split over rows with
 // atomics, dX, column sums) each read the 128 float32 channels of every row
 // again, three times for the taps, through registers: 64 us a layer forward and
-// 364 us backward for 164k rows, where moving each operand once is 170 MB
-// (25 us) and 250 MB (37 us).
+// 364 us backward for 132k rows, where moving each operand once is 135 MB
+// (20 us) and 200 MB (30 us).  Here: 28 to 39 us a layer forward, 42 to 79
+// backward; a CTA's reads, products and stores of a tile overlap only in part.
 //
 //   * Rows are taken in padded order (Packed::prow): every word's rows, then one
 //     zero row.  A tile is 128 padded rows and one on either side.  With the zero
