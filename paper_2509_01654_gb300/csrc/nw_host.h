@@ -166,11 +166,12 @@ nw_status ctx_alloc(nw_ctx* c, DevBuf& b, size_t bytes, const char* what) {
   if (c->budget && c->used + bytes > c->budget)
     return set_err(c, NW_ENOMEM, "memory budget exceeded: %s needs %zu bytes, %zu of %zu in use", what,
                    bytes, c->used, c->budget);
-  // the smallest spare block that holds it and is not much larger
+  // the smallest spare block that holds it and is not much larger (under a
+  // budget only one of the same size: what fitted it before still fits)
   size_t best = c->spare.size();
   for (size_t i = 0; i < c->spare.size(); ++i) {
     const size_t have = c->spare[i].bytes;
-    if (have < bytes || have > bytes + bytes / 4 + 4096 || (c->budget && c->used + have > c->budget)) continue;
+    if (have < bytes || have > (c->budget ? bytes : bytes + bytes / 4 + 4096)) continue;
     if (best == c->spare.size() || have < c->spare[best].bytes) best = i;
   }
   if (best < c->spare.size()) {
