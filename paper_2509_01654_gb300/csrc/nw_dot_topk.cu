@@ -55,6 +55,7 @@
 #include <stdint.h>
 
 #include "nw_internal.cuh"
+#include "nw_launch.h"
 #include "nw_proposal.h"
 #include "nw_proposal_internal.h"
 #include "nw_tc.cuh"
@@ -1975,7 +1976,7 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
     max_kernel<<<dim3(blocks, X.splits), kSwThreads, kSwSmem, s>>>(X);
     const uint32_t G = lg ? 2u * ((tm + per - 1) / per) : 4u * tm;
     const size_t bound_smem = (size_t)kBoundWarps * G * sizeof(float);
-    e = cudaFuncSetAttribute(row_bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bound_smem);
+    e = allow_shared(reinterpret_cast<const void*>(row_bound_kernel));
     if (e != cudaSuccess) return e;
     row_bound_kernel<<<(nA + kBoundWarps - 1) / kBoundWarps, kBoundWarps * 32, bound_smem, s>>>(buf, nA, G, lg, C + 1);
     X.tmB = P.tmB;
@@ -1988,7 +1989,7 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
     gather_kernel<<<dim3(blocks, sg), kSwThreads, kSwSmem, s>>>(X);
     const uint32_t stage_keys = (nM < nB ? 4u : 2u) * C + 256u;
     const size_t sel_smem = (size_t)kSelWarps * stage_keys * sizeof(uint64_t);
-    e = cudaFuncSetAttribute(select_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem);
+    e = allow_shared(reinterpret_cast<const void*>(select_row_kernel));
     if (e != cudaSuccess) return e;
     select_row_kernel<<<(nA + kSelWarps - 1) / kSelWarps, kSelWarps * 32, sel_smem, s>>>(
         buf, nA, sg, C, stage_keys, sorted, col_ids, idx, val, overflow);

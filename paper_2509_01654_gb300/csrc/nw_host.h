@@ -826,7 +826,7 @@ nw_status run_launch(nw_ctx* c, cudaStream_t stream, const Launch& l, const Seg*
   const void* fn = bits ? bit_kernel(l.m, l.x, epi) : dp_kernel(l.range, epi, tab);
   if (!fn) return set_err(c, NW_EINVAL, "no alignment kernel for this launch");
   const int block = bits ? kBitBlock : kBlock;
-  NW_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  NW_CK(allow_shared(fn));
   int occ = 0;
   NW_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem));
   if (occ < 1) occ = 1;

@@ -8,6 +8,12 @@
 
 namespace nw {
 
+// Lets `fn` ask for as much dynamic shared memory as the device has beside its
+// static shared memory, once per function and device.  The limit belongs to the
+// process's function, not to a context: a limit set to one call's need refused
+// the launch of another host thread whose need was larger.
+cudaError_t allow_shared(const void* fn);
+
 // DPX alignment kernel for a range of longer lengths (dp_range_of), epilogue
 // kind and scoring (tab: substitution table); nullptr if there is none
 const void* dp_kernel(int range, int epi, bool tab = false);

@@ -162,7 +162,7 @@ cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s) {
     const void* fn = bit_pairs(p.bit_m, p.bit_x, wide);
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = (size_t)p.alphabet * kBitPairsBlock * (wide ? 8 : 4);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(fn);
     int occ = 0, dev = 0, sms = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBitPairsBlock, smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);

@@ -334,7 +334,7 @@ cudaError_t rescore_topk_bits(const RescoreBits& R, int m, int x, int sms, cudaS
   const void* fn = bit_rescore(m, x);
   if (!fn) return cudaErrorInvalidValue;
   const size_t smem = kRescoreWarps * rescore_warp_bytes(R.alphabet, R.C);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(fn);
   int occ = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kRescoreWarps * 32, smem);
   if (e != cudaSuccess) return e;
