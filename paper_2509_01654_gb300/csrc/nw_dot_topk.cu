@@ -1818,7 +1818,7 @@ uint32_t dot_topk_splits(uint32_t nA, uint32_t nB) {
 }
 
 // scratch layout: [row buffers: nA x S x 2 x kCap keys][column bias digits:
-// bias_pad(nB) x 32 B][error word: 16 B][split lists: nA x S x C keys]
+// bias_pad(nB) x 32 B][error word, overflow flag: 16 B][split lists: nA x S x C keys]
 static size_t ext_offset_bytes(uint32_t nA, uint32_t nB) {
   return (size_t)nA * dot_topk_splits(nA, nB) * 2 * kCap * sizeof(uint64_t);
 }
@@ -1945,7 +1945,7 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
   const uint32_t nM = nB > (1u << 18) ? (nB / 2u + kTileN - 1) / kTileN * kTileN : nB;
   if (self && bound_groups(nM, C, lg)) {
     // the two-sweep path; the candidate kernel below runs only if it overflowed
-    uint32_t* overflow = err + 1;
+    uint32_t* overflow = dot_topk_err_word(buf, nA, nB) + 1;  // (a caller's err may be any single word)
     e = cudaMemsetAsync(overflow, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     SweepArgs X;

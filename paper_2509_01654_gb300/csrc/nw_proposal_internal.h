@@ -37,12 +37,12 @@ cudaError_t quantize(const float* E, uint32_t n, unsigned int* amax_bits, int8_t
 cudaError_t widen(const int8_t* q, uint32_t n, __nv_bfloat16* qb, cudaStream_t s);
 // bf16 rows: row-major rows of 64 values, zero-padded to whole 256-row tiles
 size_t dot_topk_qb_bytes(uint32_t n);
-// scratch of a launch over nA rows, nB columns and C candidates (the err
-// word must follow the returned layout: use dot_topk_err_word)
+// scratch of a launch over nA rows, nB columns and C candidates
 uint32_t dot_topk_splits(uint32_t nA, uint32_t nB);
 size_t dot_topk_buffer_bytes(uint32_t nA, uint32_t nB, uint32_t C);
 inline size_t dot_topk_buffer_bytes(uint32_t n, uint32_t C) { return dot_topk_buffer_bytes(n, n, C); }
-// the device error word inside a dot_topk buffer (zero it before a launch)
+// a device error word inside a dot_topk buffer (zero it before a launch); a
+// launch's err may be it or any other word of the caller's
 uint32_t* dot_topk_err_word(uint64_t* buf, uint32_t nA, uint32_t nB);
 inline uint32_t* dot_topk_err_word(uint64_t* buf, uint32_t n) { return dot_topk_err_word(buf, n, n); }
 // debug settings of the candidate kernel: wait_cycles < 0 keeps the kernel's
