@@ -151,6 +151,25 @@ __device__ __forceinline__ void bit_row31_first(W (&H)[2], const W M, const W NL
   H[1] = M & ~U3;
 }
 
+// One row of the steps (2, 1), the general row with its terms written out: 9
+// logic operations and two additions.  (As an instance of bit_row the compiler
+// spilled 700 to 880 bytes a thread in every alignment kernel of this class: top-10
+// lists and histogram of 20,000 words of 24 symbols, 128 codes, 8.5 ms, of 40
+// symbols, 256 codes, 46.8 ms, slower than the DPX kernel's 28.2; written out 3.5
+// and 12.5 ms.)
+template <bool Split, class W>
+__device__ __forceinline__ void bit_row21(W (&H)[2], const W M, const W NL) {
+  const W h1 = H[0], h2 = H[1];
+  const W z = ~h1 & NL;
+  const W g = M & z;
+  const W U2 = add_cols<Split>(z, g) ^ (z & ~g);  // v' = 2
+  const W v1 = (((M | U2) & ~h2) | ~h1) & NL;     // v >= 1
+  const W U1 = add_cols<Split>(v1, v1);
+  const W q = M | h2;
+  H[0] = (q & ~U2) | ~U1;
+  H[1] = q & ~U1;
+}
+
 // The state recoded to binary digits: h = sum over d of 2^d * D[d].
 __host__ __device__ constexpr int bit_digits(int m) { return m == 1 ? 1 : (m <= 3 ? 2 : 3); }
 template <int MM, int XX, class W>
@@ -177,7 +196,13 @@ __device__ __forceinline__ void bit_digit_planes(const W (&H)[bit_planes(MM, XX)
   }
 }
 
-// row 1 from nothing, and any later row
+// any later row, and row 1 from nothing
+template <int MM, int XX, bool Split, class W>
+__device__ __forceinline__ void bit_next(W (&H)[bit_planes(MM, XX)], const W M, const W NL) {
+  if constexpr (MM == 3 && XX == 1) bit_row31<Split>(H, M, NL);
+  else if constexpr (MM == 2) bit_row21<Split>(H, M, NL);
+  else bit_row<MM, XX, Split>(H, M, NL);
+}
 template <int MM, int XX, bool Split, class W>
 __device__ __forceinline__ void bit_first(W (&H)[bit_planes(MM, XX)], const W M, const W NL) {
   if constexpr (MM == 3 && XX == 1) {
@@ -185,13 +210,8 @@ __device__ __forceinline__ void bit_first(W (&H)[bit_planes(MM, XX)], const W M,
   } else {
 #pragma unroll
     for (int a = 0; a < MM; ++a) H[a] = W{};  // folds most of the row away
-    bit_row<MM, XX, Split>(H, M, NL);
+    bit_next<MM, XX, Split>(H, M, NL);
   }
-}
-template <int MM, int XX, bool Split, class W>
-__device__ __forceinline__ void bit_next(W (&H)[bit_planes(MM, XX)], const W M, const W NL) {
-  if constexpr (MM == 3 && XX == 1) bit_row31<Split>(H, M, NL);
-  else bit_row<MM, XX, Split>(H, M, NL);
 }
 
 // bits of a word's field [w * pitch, (w + 1) * pitch) in the two halves
