@@ -50,3 +50,12 @@ def test_shards_hold_the_same_pairs_as_the_dpx_plan(lib, nshards):
         a, b = nw.debug_enumerate_bit_pairs(lengths, shard=s, nshards=nshards)
         x, y = nw.debug_enumerate_pairs(lengths, s, nshards)
         assert np.array_equal(np.sort(_codes(a, b, n)), np.sort(_codes(x, y, n)))
+
+
+@pytest.mark.parametrize("length", [2, 8, 16, 24, 32])
+@pytest.mark.parametrize("queries", [64, 256, 1000])
+def test_queries_of_one_length_are_the_a_words(lib, length, queries):
+    """Cold query lists: the pairs of a task run over the dictionary's words first, whatever a few percent of rows say."""
+    q, w = nw.debug_enumerate_bit_pairs([length] * 4100, [length] * queries)
+    assert q.size == 4100 * queries
+    assert (q[:32] == q[0]).all() and np.unique(w[:32]).size == 32
