@@ -20,6 +20,16 @@ __device__ __forceinline__ B64 cols_below<B64>(int n) {
   const uint64_t v = (1ull << n) - 1ull;  // n <= kMaxLen
   return {(uint32_t)v, (uint32_t)(v >> 32)};
 }
+// the columns of a mask as C: all of them, or the first 32
+template <class C>
+__device__ __forceinline__ C cols_of(B32 x) {
+  return x;
+}
+template <class C>
+__device__ __forceinline__ C cols_of(B64 x) {
+  if constexpr (sizeof(C) == 4) return {x.lo};
+  else return x;
+}
 __device__ __forceinline__ int cols_count(B32 x) { return __popc(x.lo); }
 __device__ __forceinline__ int cols_count(B64 x) { return __popc(x.lo) + __popc(x.hi); }
 // sets column j of a mask in shared memory that only this thread touches (an
@@ -28,11 +38,46 @@ __device__ __forceinline__ void set_col(B32* x, int j) { atomicOr(&x->lo, 1u << 
 __device__ __forceinline__ void set_col(B64* x, int j) { atomicOr(j < 32 ? &x->lo : &x->hi, 1u << (j & 31)); }
 
 // A word's 16-byte record: byte 0 its length, then up to 15 codes; a longer
-// word has its offset in the symbols in the second 32 bits.
+// word has its offset in the symbols in the second 32 bits and that of its pair
+// record, with its half, in the third.
 constexpr int kRecCodes = 15;
 __device__ __forceinline__ uint32_t rec_byte(const uint4& r, int b) {  // b a compile-time constant
   const uint32_t w = b < 4 ? r.x : (b < 8 ? r.y : (b < 12 ? r.z : r.w));
   return (w >> (8 * (b & 3))) & 0xffu;
+}
+
+// Sixteen codes of a word, a byte each, from its first on.
+struct Codes16 {
+  uint32_t w[4];
+};
+__device__ __forceinline__ Codes16 rec_codes(const uint4& r) {
+  return {{__funnelshift_r(r.x, r.y, 8), __funnelshift_r(r.y, r.z, 8), __funnelshift_r(r.z, r.w, 8), r.w >> 8}};
+}
+// The same for symbols at .. at + 15 (at a multiple of 16) of a word of len symbols in
+// the pair records (`word`: brec_w of it): four symbols a load, all loads in flight.
+__device__ __forceinline__ Codes16 brec_codes(const uint32_t* __restrict__ b_rec, uint32_t word, uint32_t shift, int at,
+                                              int len) {
+  const uint4* src = reinterpret_cast<const uint4*>(b_rec + (word & ~3u) + at);
+  uint4 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = at + 4 * q < len ? __ldg(src + q) : make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t sh = (word & 1u) * 16u + shift, mask = 0x7fu;  // (alphabets of up to 128)
+  Codes16 c;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    c.w[q] = ((~v[q].x >> sh) & mask) | (((~v[q].y >> sh) & mask) << 8) | (((~v[q].z >> sh) & mask) << 16) |
+           (((~v[q].w >> sh) & mask) << 24);
+  return c;
+}
+__device__ __forceinline__ uint32_t code_at(const Codes16& c, int x) {  // x a compile-time constant
+  return (c.w[x >> 2] >> (8 * (x & 3))) & 0xffu;
+}
+__device__ __forceinline__ uint32_t next_code(Codes16& c) {  // takes the first code off
+  const uint32_t code = c.w[0] & 0xffu;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) c.w[q] = __funnelshift_r(c.w[q], c.w[q + 1], 8);
+  c.w[3] >>= 8;
+  return code;
 }
 
 // ---- explicit pairs: one thread per pair, the longer word in the thread's
@@ -42,19 +87,33 @@ __device__ __forceinline__ uint32_t rec_byte(const uint4& r, int b) {  // b a co
 // set from the longer word and cleared again after the pair.  A thread loops
 // over its own word lengths, so a warp of mixed lengths runs one code path;
 // the DPX kernel it replaces ran one unrolled body per length present in the
-// warp.  What bounds it then is L1: every lane reads other words, so a 4-byte
-// load takes 32 tag look-ups.  With the words' records (P.rec) a pair takes two
-// 16-byte loads instead of about 35 loads.  1,000,003 random pairs of 100k
-// words: 381 us DPX, 193 reading symbols, 66 with records.
+// warp.  What bounds it then is L1: every lane reads other words, so a load
+// takes 32 tag look-ups whatever its width.  With the words' records (P.rec) a pair
+// of words of up to 15 symbols takes two 16-byte loads; other words are read 16
+// symbols at a time from the pair records, four a load, and a pair's first loads are
+// issued together.  (Symbol by symbol a word of 24 took 72 loads.)  1,000,003 random
+// pairs of 100k words, whole calls: lengths N(8, 3) 397 us DPX, 62 with records, 76
+// without; all of 16 symbols 126, 67 (symbol by symbol 300); of 24, 164, 90 (412); of
+// 40, 398, 174.
 template <int MM, int XX, class W>
 __global__ void __launch_bounds__(kBitPairsBlock) bit_pairs_kernel(const PairsParams P) {
   extern __shared__ __align__(16) unsigned char s_pairs[];
-  constexpr bool kSplit = sizeof(W) == 4;  // (64 columns: a word may straddle bit 32)
   W* tab = reinterpret_cast<W*>(s_pairs) + threadIdx.x;
-  for (uint32_t c = 0; c < P.alphabet; ++c) tab[c * kBitPairsBlock] = W{};
-  auto symbol = [&](uint32_t at) { return (__ldg(P.a_enc + at) & 0xffffu) >> P.shift; };
-  for (uint64_t p = (uint64_t)blockIdx.x * kBitPairsBlock + threadIdx.x; p < P.m; p += (uint64_t)gridDim.x * kBitPairsBlock) {
-    const uint32_t i = P.pi[p], j = P.pj[p];
+  const uint32_t pitch = blockDim.x;
+  const uint64_t step = (uint64_t)gridDim.x * pitch;
+  uint64_t p = (uint64_t)blockIdx.x * pitch + threadIdx.x, next = 0;
+  uint32_t i = 0u, j = 0u, ni = 0u, nj = 0u;  // this pair, and the next one read ahead
+  if (p < P.m) {
+    i = P.pi[p];
+    j = P.pj[p];
+  }
+  for (uint32_t c = 0; c < P.alphabet; ++c) tab[c * pitch] = W{};
+  for (; p < P.m; p = next, i = ni, j = nj) {
+    next = p + step;
+    if (next < P.m) {
+      ni = P.pi[next];
+      nj = P.pj[next];
+    }
     if (i >= P.n || j >= P.n) {
       atomicOr(P.err, kErrInput);
       P.out[p] = INT16_MIN;
@@ -67,12 +126,12 @@ __global__ void __launch_bounds__(kBitPairsBlock) bit_pairs_kernel(const PairsPa
       rb = __ldg(P.rec + j);
       la = (int)(ra.x & 0xffu);
       lb = (int)(rb.x & 0xffu);
-    } else {  // few pairs of a large set: offsets, as for words too long for a record
+    } else {  // few pairs: the pair records' offsets, as for words too long for a record
       const uint32_t pa = __ldg(P.rank + i), pb = __ldg(P.rank + j);
       la = __ldg(P.slen + pa);
       lb = __ldg(P.slen + pb);
-      ra.y = __ldg(P.aoff + pa);
-      rb.y = __ldg(P.aoff + pb);
+      ra.z = __ldg(P.brec_w + pa);
+      rb.z = __ldg(P.brec_w + pb);
     }
     if (la > lb) {
       const uint4 t = ra;
@@ -84,42 +143,52 @@ __global__ void __launch_bounds__(kBitPairsBlock) bit_pairs_kernel(const PairsPa
     }
     int g = 0;
     if (la > 0) {
-      const bool rec_a = P.rec && la <= kRecCodes, rec_b = P.rec && lb <= kRecCodes;
-      if (rec_b) {
+      auto first = [&](const uint4& r, int len) {
+        return P.rec && len <= kRecCodes ? rec_codes(r) : brec_codes(P.b_rec, r.z, P.shift, 0, len);
+      };
+      const Codes16 b0 = first(rb, lb);
+      Codes16 c = first(ra, la);
+      auto each_column = [&](auto f) {
 #pragma unroll
-        for (int x = 0; x < kRecCodes; ++x)
-          if (x < lb) set_col(tab + rec_byte(rb, x + 1) * kBitPairsBlock, x);
-      } else {
-        for (int x = 0; x < lb; ++x) set_col(tab + symbol(rb.y + (uint32_t)x) * kBitPairsBlock, x);
-      }
-      const W NL = cols_below<W>(lb - 1);
-      W H[bit_planes(MM, XX)];
-      if (rec_a) {
-        bit_first<MM, XX, kSplit>(H, tab[rec_byte(ra, 1) * kBitPairsBlock], NL);
-        uint64_t lo = ((uint64_t)ra.y << 16) | (ra.x >> 16), hi = ((uint64_t)ra.w << 16) | (ra.z >> 16);
-        lo |= (uint64_t)(ra.z & 0xffffu) << 48;  // codes 1 .. 14 as one shifted run of bytes
-        for (int r = 1; r < la; ++r) {
-          const W M = tab[((uint32_t)lo & 0xffu) * kBitPairsBlock];
-          lo = (lo >> 8) | (hi << 56);
-          hi >>= 8;
-          bit_next<MM, XX, kSplit>(H, M, NL);
+        for (int x = 0; x < 16; ++x)
+          if (x < lb) f(tab + code_at(b0, x) * pitch, x);
+#pragma unroll 1
+        for (int at = 16; at < lb; at += 16) {
+          const Codes16 b = brec_codes(P.b_rec, rb.z, P.shift, at, lb);
+#pragma unroll
+          for (int x = 0; x < 16; ++x)
+            if (at + x < lb) f(tab + code_at(b, x) * pitch, at + x);
         }
-      } else {
-        bit_first<MM, XX, kSplit>(H, tab[symbol(ra.y) * kBitPairsBlock], NL);
-        for (int r = 1; r < la; ++r) bit_next<MM, XX, kSplit>(H, tab[symbol(ra.y + (uint32_t)r) * kBitPairsBlock], NL);
-      }
-      W D[bit_digits(MM)];
-      bit_digit_planes<MM, XX>(H, D);
-      const W F = cols_below<W>(lb);
+      };
+      each_column([](W* t, int x) { set_col(t, x); });
+      auto rows = [&](auto kind) {
+        using V = decltype(kind);
+        constexpr bool kSplit = sizeof(V) == 4;  // (64 columns: a word may straddle bit 32)
+        auto next_mask = [&]() { return cols_of<V>(tab[next_code(c) * pitch]); };
+        const V NL = cols_below<V>(lb - 1);
+        V H[bit_planes(MM, XX)];
+        bit_first<MM, XX, kSplit>(H, next_mask(), NL);
+#pragma unroll 1
+        for (int r = 1;;) {
+          const int end = la < (r | 15) + 1 ? la : (r | 15) + 1;
+#pragma unroll 1
+          for (; r < end; ++r) bit_next<MM, XX, kSplit>(H, next_mask(), NL);
+          if (r == la) break;
+          c = brec_codes(P.b_rec, ra.z, P.shift, r, la);  // r a multiple of 16
+        }
+        V D[bit_digits(MM)];
+        bit_digit_planes<MM, XX>(H, D);
+        const V F = cols_below<V>(lb);
 #pragma unroll
-      for (int d = 0; d < bit_digits(MM); ++d) g += cols_count(D[d] & F) << d;
-      if (rec_b) {
-#pragma unroll
-        for (int x = 0; x < kRecCodes; ++x)
-          if (x < lb) tab[rec_byte(rb, x + 1) * kBitPairsBlock] = W{};
+        for (int d = 0; d < bit_digits(MM); ++d) g += cols_count(D[d] & F) << d;
+      };
+      if constexpr (sizeof(W) == 8) {
+        if (__any_sync(__activemask(), lb > 32)) rows(B64{});
+        else rows(B32{});  // (a list in order of length)
       } else {
-        for (int x = 0; x < lb; ++x) tab[symbol(rb.y + (uint32_t)x) * kBitPairsBlock] = W{};
+        rows(B32{});
       }
+      each_column([](W* t, int) { *t = W{}; });
     }
     P.out[p] = (int16_t)(g * P.coef + P.gap * (la + lb));
   }

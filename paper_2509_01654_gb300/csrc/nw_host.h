@@ -907,7 +907,7 @@ const uint4* dict_records(nw_dict* d, cudaStream_t s) {
     return nullptr;
   }
   if (launch_word_records(d->ws.rank.as<uint32_t>(), d->ws.slen.as<uint8_t>(), d->ws.aoff.as<uint32_t>(),
-                          d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, d->rec.as<uint4>(), s) != cudaSuccess ||
+                          d->ws.brec_w.as<uint32_t>(), d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, d->rec.as<uint4>(), s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {  // other streams may read them next
     cudaGetLastError();
     ctx_free(c, d->rec);
@@ -923,6 +923,7 @@ void pairs_bits(const nw_dict* d, PairsParams& P) {
   P.coef = d->ss.bit_coef;
   P.shift = d->ss.shift;
   P.alphabet = d->alphabet;
+  P.min_len = d->ws.min_len;
   P.max_len = d->ws.max_len;
 }
 

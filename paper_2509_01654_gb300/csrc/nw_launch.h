@@ -78,13 +78,14 @@ struct PairsParams {
   const uint16_t* tab;  // substitution table (device, kTabDim x kTabDim) or null
   // bit-parallel scoring (bit_m = 0: none)
   int32_t bit_m, bit_x, coef;
-  uint32_t shift, alphabet, max_len;
+  uint32_t shift, alphabet, min_len, max_len;
   const uint4* rec;  // word records by original index (launch_word_records), or null
 };
-// the 16-byte record of every word: length and up to 15 codes, or the offset
-// of a longer word's symbols
-cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const uint32_t* aoff, const uint32_t* sym,
-                                uint32_t shift, uint32_t n, uint4* rec, cudaStream_t s);
+// the 16-byte record of every word: length and up to 15 codes, or the offsets
+// of a longer word's symbols and pair record
+cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const uint32_t* aoff,
+                                const uint32_t* brec_w, const uint32_t* sym, uint32_t shift, uint32_t n, uint4* rec,
+                                cudaStream_t s);
 cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s);
 
 // the all-pairs top-k reduction with every scratch buffer taken from a

@@ -157,22 +157,33 @@ cudaError_t select_topk(const uint32_t* cand, const int32_t* score, uint32_t n, 
 
 cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s) {
   if (p.m == 0) return cudaSuccess;
-  if (p.bit_m && p.alphabet <= kBitPairsAlphabet) {
-    const bool wide = p.max_len > 32u;
+  // Words of one length above 32 and many codes stay with the DPX kernel: its warps
+  // then run one body, and 64-column masks of that alphabet leave few threads on an
+  // SM (128 codes, 1,000,003 pairs of 33 symbols, steps (5, 2): 371 us, DPX 262;
+  // lengths 1 .. 40: 396, DPX 16,500; 40 codes, 33 symbols: 248).
+  const bool wide = p.max_len > 32u, one_body = wide && p.min_len == p.max_len && p.alphabet > 48u;
+  if (p.bit_m && p.alphabet <= kBitPairsAlphabet && !one_body) {
     const void* fn = bit_pairs(p.bit_m, p.bit_x, wide);
     if (!fn) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)p.alphabet * kBitPairsBlock * (wide ? 8 : 4);
+    // A thread's masks are alphabet x 4 or 8 bytes, so large alphabets leave few
+    // threads on an SM; of blocks of 128, 64 and 32 the largest that holds the most
+    const size_t each = (size_t)p.alphabet * (wide ? 8 : 4);
+    auto resident = [&](int b) { return (int)std::min<size_t>((227 * 1024) / (each * b + 1024), 32) * b; };
+    int block = kBitPairsBlock;
+    for (int b : {64, 32})
+      if (resident(b) > resident(block)) block = b;
+    const size_t smem = each * block;
     cudaError_t e = allow_shared(fn);
     int occ = 0, dev = 0, sms = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kBitPairsBlock, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const uint64_t blocks = (p.m + kBitPairsBlock - 1) / kBitPairsBlock;
-    const uint64_t resident = (uint64_t)std::max(1, occ) * (uint64_t)sms;
+    const uint64_t blocks = (p.m + block - 1) / block;
+    const uint64_t fit = (uint64_t)std::max(1, occ) * (uint64_t)sms;
     PairsParams arg = p;
     void* args[] = {&arg};
-    return cudaLaunchKernel(fn, dim3((unsigned)std::min(blocks, resident)), dim3(kBitPairsBlock), args, smem, s);
+    return cudaLaunchKernel(fn, dim3((unsigned)std::min(blocks, fit)), dim3(block), args, smem, s);
   }
   const uint32_t blk = 128;
   const uint64_t grid = (p.m + blk - 1) / blk;

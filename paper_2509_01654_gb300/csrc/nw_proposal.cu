@@ -322,7 +322,7 @@ nw_status rescore_records(nw_ctx* c, const nw_dict* d, DevBuf& scratch, const ui
   }
   NW_TRY(ctx_ensure(c, scratch, std::max<size_t>(16, (size_t)d->ws.n * 16), "candidate word records"));
   NW_CK(launch_word_records(d->ws.rank.as<uint32_t>(), d->ws.slen.as<uint8_t>(), d->ws.aoff.as<uint32_t>(),
-                            d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, scratch.as<uint4>(), s));
+                            d->ws.brec_w.as<uint32_t>(), d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, scratch.as<uint4>(), s));
   *rec = scratch.as<uint4>();
   return NW_OK;
 }

@@ -303,6 +303,7 @@ namespace {
 __global__ void __launch_bounds__(256) word_records_kernel(const uint32_t* __restrict__ rank,
                                                            const uint8_t* __restrict__ slen,
                                                            const uint32_t* __restrict__ aoff,
+                                                           const uint32_t* __restrict__ brec_w,
                                                            const uint32_t* __restrict__ sym, uint32_t shift, uint32_t n,
                                                            uint4* __restrict__ rec) {
   const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(256) word_records_kernel(const uint32_t* __res
   uint32_t w[4] = {len, 0u, 0u, 0u};
   if (len > (uint32_t)kRecCodes) {
     w[1] = ao;
+    w[2] = __ldg(brec_w + r);
   } else {
 #pragma unroll
     for (int x = 0; x < kRecCodes; ++x)
@@ -320,10 +322,10 @@ __global__ void __launch_bounds__(256) word_records_kernel(const uint32_t* __res
 }
 }  // namespace
 
-cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const uint32_t* aoff, const uint32_t* sym,
-                                uint32_t shift, uint32_t n, uint4* rec, cudaStream_t s) {
+cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const uint32_t* aoff,
+                                const uint32_t* brec_w, const uint32_t* sym, uint32_t shift, uint32_t n, uint4* rec, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  word_records_kernel<<<(n + 255) / 256, 256, 0, s>>>(rank, slen, aoff, sym, shift, n, rec);
+  word_records_kernel<<<(n + 255) / 256, 256, 0, s>>>(rank, slen, aoff, brec_w, sym, shift, n, rec);
   return cudaGetLastError();
 }
 

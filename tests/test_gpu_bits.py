@@ -95,3 +95,19 @@ def test_rescoring_every_class(ctx, oracle_mod, sc, C, k):
         assert np.array_equal(idx[row, :c.size], c) and np.array_equal(score[row, :c.size], full[row, c])
         assert (idx[row, c.size:] == nw.MISSING_IDX).all() and (score[row, c.size:] == nw.MISSING_SCORE).all()
     d.free()
+
+
+# words read 16 symbols at a time, blocks of 128, 64 and 32 threads by the size of the masks, and one length above 32
+@pytest.mark.parametrize("alphabet", [7, 60, 97, 128])
+@pytest.mark.parametrize("lengths", [[0, 1, 15, 16, 17, 31, 32], [0, 1, 15, 16, 17, 31, 32, 33, 40], [33]])
+@pytest.mark.parametrize("sc", [(1, -1, -1), (0, -1, -1), (3, 0, -1)])
+@pytest.mark.parametrize("m", [20, 2000])
+def test_explicit_pairs_at_chunk_edges(ctx, oracle_mod, alphabet, lengths, sc, m):
+    w = _words(np.random.default_rng(11).choice(lengths, 300), alphabet, alphabet)
+    d = ctx.load_dictionary(w.codes, w.offsets, alphabet, sc)
+    r = np.random.default_rng(m)
+    i, j = r.integers(0, w.n, m).astype(np.uint32), r.integers(0, w.n, m).astype(np.uint32)
+    by_length = np.argsort(np.maximum(w.lengths[i], w.lengths[j]), kind="stable")
+    for p in (np.arange(m), by_length):
+        assert np.array_equal(d.score_pairs(i[p], j[p]).astype(np.int32), oracle_mod.score_pairs(w, i[p], j[p], sc))
+    d.free()
