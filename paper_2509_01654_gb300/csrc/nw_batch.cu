@@ -328,7 +328,7 @@ nw_status create_impl(nw_batch* B, const nw_batch_dict* dicts, uint32_t ndicts, 
     terms[term_index(d, 0)] = make_terms(D, D->ws, D->ws, dict_side, dict_side, D->score_lo - 1, ib);
     terms[term_index(d, 1)] = make_terms(D, Q, D->ws, query_side, dict_nolists, B->q_key_lo[d], ib);
     terms[term_index(d, 2)] = make_terms(D, D->ws, Q, dict_nolists, query_side, B->q_key_lo[d], ib);
-    Rects* rects = &B->dp_rects;
+    Rects* rects = &B->dp_rects;  // of the dictionary's pairs, those that are not taken out for the DPX launches
     if (D->ss.bit_m) {
       auto g = std::find_if(groups.begin(), groups.end(),
                             [&](const Group& x) { return x.m == D->ss.bit_m && x.x == D->ss.bit_x; });
@@ -340,12 +340,18 @@ nw_status create_impl(nw_batch* B, const nw_batch_dict* dicts, uint32_t ndicts, 
     if (B->self[d]) rects_all(D->ws.bk, term_index(d, 0), own);
     if (Q.n) rects_queries(Q.bk, D->ws.bk, term_index(d, 1), queries);
     count_rects(queries, B->query_pairs, B->query_cells);
-    for (const Rects* list : {&own, &queries})
-      for (const Rect& r : *list) {
-        rects->push_back(r);
-        B->has_len[r.LB] = true;
-        if (!D->ss.bit_m) B->dp_len[r.LB] = true;
+    for (Rects* list : {&own, &queries}) {
+      const Rects dpx = D->ss.bit_m ? take_long(*list, D->ss) : std::move(*list);
+      if (D->ss.bit_m)
+        for (const Rect& r : *list) {
+          rects->push_back(r);
+          B->has_len[r.LB] = true;
+        }
+      for (const Rect& r : dpx) {
+        B->dp_rects.push_back(r);
+        B->has_len[r.LB] = B->dp_len[r.LB] = true;
       }
+    }
   }
   NW_TRY(ctx_alloc(c, B->d_terms, sizeof(Terms) * terms.size(), "batch terms"));
   NW_CK(cudaMemcpyAsync(B->d_terms.p, terms.data(), sizeof(Terms) * terms.size(), cudaMemcpyHostToDevice, B->stream));
@@ -360,11 +366,7 @@ nw_status create_impl(nw_batch* B, const nw_batch_dict* dicts, uint32_t ndicts, 
     order_rects(g.rects);
     Plan p;
     sized(p, kBitMinTasks, [&](uint32_t ta, Plan& q) { plan_bits(g.rects, g.m, g.x, g.alphabet, ta, q); });
-    for (Launch& l : p.launches) {
-      l.seg_first += (uint32_t)B->plan.segs.size();
-      B->plan.launches.push_back(l);
-    }
-    B->plan.segs.insert(B->plan.segs.end(), p.segs.begin(), p.segs.end());
+    append_plan(B->plan, p);
     count_rects(g.rects, B->plan.pairs, B->plan.cells);
   }
   NW_TRY(upload_plan(B, B->plan));

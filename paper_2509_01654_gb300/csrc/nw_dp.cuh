@@ -1,8 +1,9 @@
 // nw_dp.cuh -- the DPX alignment kernel (sm_103a), whose inner loop is unrolled
 // for the length LB of the longer word of a pair, and the list and histogram
 // updates it shares with the bit-parallel kernel (nw_bits.cuh).  It scores
-// substitution-matrix dictionaries and the match / mismatch scorings that the
-// bit-parallel kernel does not take.
+// substitution-matrix dictionaries, the match / mismatch scorings that the
+// bit-parallel kernel does not take, and the long words of its dearest classes
+// (take_long).
 //
 // Recurrence.  Algorithm 1 of the paper fills H[i][j] = max(H[i-1][j-1] +
 // sim(A[i-1], B[j-1]), H[i-1][j] + p, H[i][j-1] + p) from H[i][0] = p*i and

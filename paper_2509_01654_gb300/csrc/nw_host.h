@@ -574,17 +574,58 @@ void sized(Plan& p, uint64_t min_tasks, Make make) {
   }
 }
 
+// Takes out of a step class's pair list what the DPX kernel scores faster: pairs of
+// words of more than 32 symbols, one to a lane in the bit-parallel kernel, for the
+// classes with the dearest rows (m >= 4 with x <= m - 2: (4,1), (5,1), (5,2), (5,3)),
+// when there are enough of them to pay for another launch.  Top-10 lists and
+// histogram of 20,000 words of 33 / 40 symbols: (5,1) 31.1 / 37.6 ms, (5,3) 23.9 / 28.8,
+// (4,1) 22.5 / 27.1, the DPX kernel 18.1 / 25.4 whatever the scoring, (5,4) 18.7 / 22.4
+// and every other class less; of 3,000 words (4.5M pairs) of 33 symbols (4,1) 0.70, DPX
+// 0.64, of 2,000 0.40 and 0.41; 1,024 queries against 4,500 words of 33 symbols (4,1)
+// 0.68, DPX 0.67.  (5,1) at 17, 18 and 22 to 25 symbols would gain up to 12 % too.
+constexpr uint64_t kLongPairs = (uint64_t)1 << 22;
+Rects take_long(Rects& rects, const ShiftedScoring& ss) {
+  Rects taken;
+  if (ss.bit_m < 4 || ss.bit_x > ss.bit_m - 2) return taken;
+  auto is_long = [](const Rect& r) { return bit_words_per_lane(std::min(r.La, r.LB)) == 1; };
+  uint64_t pairs = 0;
+  for (const Rect& r : rects)
+    if (is_long(r)) {
+      const uint64_t na = r.a1 - r.a0, nb = r.b1 - r.b0;
+      pairs += r.tri ? na * nb / 2 : na * nb;
+    }
+  if (pairs < kLongPairs) return taken;
+  const auto at = std::stable_partition(rects.begin(), rects.end(), [&](const Rect& r) { return !is_long(r); });
+  taken.assign(at, rects.end());
+  rects.erase(at, rects.end());
+  return taken;
+}
+
+// Appends a plan's launches and segments (not its counts).
+void append_plan(Plan& to, const Plan& p) {
+  for (Launch l : p.launches) {
+    l.seg_first += (uint32_t)to.segs.size();
+    to.launches.push_back(l);
+  }
+  to.segs.insert(to.segs.end(), p.segs.begin(), p.segs.end());
+}
+
 // The launches of a pair list for scoring ss and an alphabet; ta = 0 sizes
 // the tasks.
 void make_plan(Rects rects, const ShiftedScoring& ss, uint32_t alphabet, uint32_t ta, Plan& p) {
   order_rects(rects);
-  auto make = [&](uint32_t t, Plan& q) {
-    if (ss.bit_m) plan_bits(rects, ss.bit_m, ss.bit_x, alphabet, t, q);
-    else plan_dp(rects, t, q);
-  };
-  if (ta) make(ta, p);
-  else sized(p, ss.bit_m ? kBitMinTasks : kDpMinTasks, make);
+  p = Plan{};
   count_rects(rects, p.pairs, p.cells);
+  const Rects dpx = ss.bit_m ? take_long(rects, ss) : std::move(rects);
+  auto add = [&](uint64_t min_tasks, auto make) {
+    Plan part;
+    if (ta) make(ta, part);
+    else sized(part, min_tasks, make);
+    append_plan(p, part);
+  };
+  if (ss.bit_m && !rects.empty())
+    add(kBitMinTasks, [&](uint32_t t, Plan& q) { plan_bits(rects, ss.bit_m, ss.bit_x, alphabet, t, q); });
+  if (!dpx.empty()) add(kDpMinTasks, [&](uint32_t t, Plan& q) { plan_dp(dpx, t, q); });
 }
 
 uint32_t index_bits(uint32_t n) {

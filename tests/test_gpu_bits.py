@@ -111,3 +111,32 @@ def test_explicit_pairs_at_chunk_edges(ctx, oracle_mod, alphabet, lengths, sc, m
     for p in (np.arange(m), by_length):
         assert np.array_equal(d.score_pairs(i[p], j[p]).astype(np.int32), oracle_mod.score_pairs(w, i[p], j[p], sc))
     d.free()
+
+
+# classes whose pairs of words above 32 symbols go to the DPX kernel when there are many: 4.9M such pairs do, the
+# parts of a sharded run (at most 1.7M each) and small query sets do not
+@pytest.mark.parametrize("sc", [(2, -1, -1), (3, -1, -1), (3, 0, -1), (3, 1, -1)])
+def test_long_words_of_the_dearest_classes(ctx, oracle_mod, sc):
+    r = np.random.default_rng(13)
+    w = _words(np.concatenate([r.integers(33, 41, 3150), r.integers(0, 33, 400)])[r.permutation(3550)], 6, 14)
+    d = ctx.load_dictionary(w.codes, w.offsets, w.alphabet, sc)
+    idx, score, hist, lo = d.all_pairs_topk(6)
+    rows = r.integers(0, w.n, 12)
+    wi, ws = oracle_mod.topk_rows(w, rows, 6, sc)
+    assert np.array_equal(idx[rows], wi) and np.array_equal(score[rows].astype(np.int32), ws)
+    parts = [d.all_pairs_topk(6, shard=(g, 3)) for g in range(3)]
+    mi, ms = nw.topk_merge([p[:2] for p in parts], 6)
+    assert np.array_equal(idx, mi) and np.array_equal(score, ms)
+    assert np.array_equal(hist, sum(p[2] for p in parts)) and hist.sum() == w.n * (w.n - 1) // 2
+    q = _words(r.integers(30, 41, 1900), 6, 15)
+    qi, qs = d.query(q.codes, q.offsets, 6)
+    for a in range(0, q.n, 500):
+        part = q.subset(np.arange(a, min(q.n, a + 500)))
+        pi, ps = d.query(part.codes, part.offsets, 6)
+        assert np.array_equal(qi[a:a + 500], pi) and np.array_equal(qs[a:a + 500], ps)
+    with nw.Context(0) as c:
+        batch = nw.Batch(c, [(w.codes, w.offsets, 6, sc, (q.codes, q.offsets)), (q.codes, q.offsets, 6, (1, -1, -1))], k=6)
+        (bi, bs), _ = batch.run_queries()[0]
+        assert np.array_equal(bi, idx) and np.array_equal(bs, score)
+        assert np.array_equal(batch.run_queries()[1][0][0], qi)
+    d.free()
