@@ -497,15 +497,20 @@ __device__ int compact_buffer(uint64_t* keys, int c, const uint64_t* other, int 
 //     itself can be the largest of one group), so it is at most the row's C-th
 //     best value: an exact lower bound.  With 3 C to 6 C groups and no relation
 //     between a column's position and its value, only 1.1 C to 1.25 C columns
-//     reach it.  This sweep takes the columns in the caller's own order, not
-//     the locality order: there a row's best columns would share a few groups.
-//     Ties: ranked by (maximum, lower position first), the (C + 1)-th group also
-//     bounds the ids.  A column at exactly the bound whose id lies past that
-//     group ranks behind C others, so a word with thousands of duplicates does
-//     not collect them all.
+//     reach it.  Neither the locality order nor a caller's own has that property
+//     (in an alphabetical dictionary a word's best columns share a few groups: up
+//     to 12 C reached the bound, and the candidate kernel redid most blocks), so
+//     this sweep reads the columns through a fixed pseudo-random permutation
+//     (shuffle_kernel).  100,003 clustered rows, C = 256: 14.9 ms in the caller's
+//     order, 5.13 shuffled, rows in no order 5.12 and 5.14; 300,000 alphabetical
+//     words, C = 256, the whole proposal: 73.4 and 31.5 ms, in no order 28.7 and 29.0.
 //   * kSweepGather appends every value that reaches the row's bound (columns in
 //     the locality order, so that the hits of a warp's rows fall into few
 //     chunks), and select_row_kernel takes each row's C best of them exactly.
+//     Ties at the bound can be thousands (duplicate words).  If the bound is the
+//     (C + 1)-th maximum by value and m of the C + 1 groups have exactly that
+//     value, at most m tied columns are among the C best, those of the lowest ids;
+//     so each thread keeps only the m lowest ids of its tied columns.
 //
 // Both are one kernel: the candidate kernel's producer and MMA thread, and
 // sixteen epilogue warps (four per SM sub-partition; each thread has one row
@@ -513,9 +518,9 @@ __device__ int compact_buffer(uint64_t* keys, int c, const uint64_t* other, int 
 // two thirds of the time).  A CTA reads an accumulator into registers whole and
 // releases it before it looks at the values.  With no compaction a row has a
 // fixed share of its append buffers per column split and half; a share that
-// would overflow (values with masses of ties) raises its row block's flag, and
-// the candidate kernel, gated on it, then redoes that block.  100k rows, C =
-// 512: the candidate kernel alone 18.7 ms, the sweeps and selections 5.2 ms.
+// would overflow raises its row block's flag, and the candidate kernel, gated on
+// it, then redoes that block.  100k rows, C = 512: the candidate kernel alone 18.7
+// ms, the sweeps and selections 5.2 ms.
 enum { kSweepMax = 0, kSweepGather = 1 };
 constexpr int kSwEpiWarps = 16;  // row quadrant = warp % 4, row block = warp / 4 % 2, column half = warp / 8
 constexpr int kSwProducer = kSwEpiWarps;
@@ -528,18 +533,23 @@ constexpr int kSwSmem = kSwOffBars + (2 * kStages + 4 + 1) * 8 + 16 + 1024;
 static_assert(kSwSmem <= 227 * 1024, "one CTA per SM");
 
 // A row's scratch is its two append buffers: 2 kCap slots of 8 bytes.  First
-// the group maxima (floats), then the gathered entries (column position,
-// value) in 2 S shares; the last slots hold the shares' counts (six words), the
-// bound with its id limit, and in a block's first row the overflow flag.
+// the group maxima (floats) and, in the scratch of row t, the shuffled column tile t
+// of kSweepMax; then the gathered entries in 2 S shares, from the front (column
+// position, value), from the back the ties (id); the last slots hold the shares'
+// counts (six words: entries, ties << 16), the bound with the ties to keep, and in a
+// block's first row the overflow flag.
 constexpr uint32_t kRowSlots = 2 * kCap;
 constexpr uint32_t kDataSlots = kRowSlots - 5;
-constexpr uint32_t kMaxGroups = 4096;
+constexpr uint32_t kMaxGroups = 3840;
+constexpr uint32_t kShuffledOffset = kMaxGroups * sizeof(float);
 constexpr uint32_t kMaxSweepSplits = 3;
-static_assert(kMaxGroups * sizeof(float) <= kDataSlots * sizeof(uint64_t), "the maxima fit a row's scratch");
+static_assert(kShuffledOffset + kMainBytes <= kDataSlots * sizeof(uint64_t) && kShuffledOffset % 1024 == 0,
+              "the maxima and a tile fit a row's scratch");
+static_assert(kDataSlots < 65536, "two counts in a word");
 __device__ __forceinline__ uint64_t* row_scratch(uint64_t* buf, uint32_t i) { return buf + (size_t)i * kRowSlots; }
 __device__ __forceinline__ uint32_t* row_counts(uint64_t* row) { return reinterpret_cast<uint32_t*>(row + kDataSlots); }
 __device__ __forceinline__ float* row_bound(uint64_t* row) { return reinterpret_cast<float*>(row + kRowSlots - 1); }
-__device__ __forceinline__ uint32_t* row_id_limit(uint64_t* row) { return reinterpret_cast<uint32_t*>(row + kRowSlots - 1) + 1; }
+__device__ __forceinline__ uint32_t* row_ties(uint64_t* row) { return reinterpret_cast<uint32_t*>(row + kRowSlots - 1) + 1; }
 // overflow flag of the block of rows that holds row i
 __device__ __forceinline__ uint32_t* block_flag(uint64_t* buf, uint32_t i) {
   return reinterpret_cast<uint32_t*>(row_scratch(buf, i / kCtaRows * kCtaRows) + kRowSlots - 2);
@@ -548,7 +558,7 @@ __host__ __device__ constexpr uint32_t share_slots(uint32_t splits) { return kDa
 
 struct SweepArgs {
   CUtensorMap tmA;  // the rows, boxes of kCtaRows rows
-  CUtensorMap tmB;  // the columns, boxes of kTileN rows
+  CUtensorMap tmB;  // the columns, boxes of kTileN rows (kSweepMax: the shuffled tiles)
   const unsigned char* ext;
   uint32_t nA, nB;
   uint32_t tps;     // tiles per column split (a multiple of a group's tiles)
@@ -627,7 +637,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_c
         const uint32_t t = tlo + u;
         unsigned char* st = smem + kOffStages + s * kStageBytes;
         mbar_expect_tx(full_bar(s), kStageBytes);
-        tc::tma_load_2d(smem_u32(st), &P.tmB, 0, (int)(t * (uint32_t)kTileN), full_bar(s));
+        if constexpr (MODE == kSweepMax) tc::tma_load_3d(smem_u32(st), &P.tmB, 0, 0, (int)t, full_bar(s));
+        else tc::tma_load_2d(smem_u32(st), &P.tmB, 0, (int)(t * (uint32_t)kTileN), full_bar(s));
         bulk_g2s(smem_u32(st + kMainBytes), P.ext + (size_t)t * kExtBytes, kExtBytes, full_bar(s));
       }
       // every copy issued has landed before the CTA exits (bounded)
@@ -681,10 +692,37 @@ __global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_c
     float run = -FLT_MAX;  // the current group's maximum
     // kSweepGather
     const float thr = MODE == kSweepGather && live ? *row_bound(row) : 0.f;
-    const uint32_t id_limit = MODE == kSweepGather && live ? *row_id_limit(row) : 0u;
+    const uint32_t keep = MODE == kSweepGather && live ? *row_ties(row) : 0u;
     const uint32_t cap = share_slots(P.splits);
     uint2* out = live ? reinterpret_cast<uint2*>(row + (size_t)(2u * blockIdx.y + half) * cap) : nullptr;
-    uint32_t cnt = 0u;
+    uint32_t cnt = 0u, ties = 0u, cut = 0xffffffffu;  // a tied column of an id >= cut is behind `keep` others
+    // a column tied with the bound: among the `keep` lowest ids of this thread's so far
+    auto tie = [&](uint32_t id) {
+      if (id >= cut) return;
+      uint2* const last = out + cap - 1;  // tie t at last[-t]
+      if (ties < keep) {
+        last[-(int)ties] = make_uint2(id, 0u);
+        if (++ties < keep) return;
+      }
+      // the largest id kept, and the one below it; a new id takes the largest's place
+      uint32_t top = 0u, below = 0u, at = 0u;
+#pragma unroll 4
+      for (uint32_t t = 0; t < keep; ++t) {
+        const uint32_t v = last[-(int)t].x;
+        if (v >= top) {
+          below = top;
+          top = v;
+          at = t;
+        } else {
+          below = max(below, v);
+        }
+      }
+      if (cut != 0xffffffffu) {
+        last[-(int)at] = make_uint2(id, 0u);
+        top = max(below, id);
+      }
+      cut = top;
+    };
     float* sv = reinterpret_cast<float*>(smem + kSwOffVals) + tid * kValStride;
 
     // appends the values of a chunk (column colbase + k in v[k]) that reach the
@@ -710,8 +748,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_c
         const uint32_t k = (uint32_t)__ffs(hit) - 1u, pos = colbase + k;
         hit &= hit - 1u;
         const float x = sv[k];
-        if (x == thr && (P.ids ? __ldg(P.ids + pos) : pos) >= id_limit) continue;  // behind C others by its id
-        out[cnt++] = make_uint2(pos, __float_as_uint(x));
+        if (x == thr) tie(P.ids ? __ldg(P.ids + pos) : pos);
+        else out[cnt++] = make_uint2(pos, __float_as_uint(x));
       } while (hit);
     };
 
@@ -755,7 +793,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_c
           }
         }
       } else {
-        if (live && cnt + 64u > cap) {  // the share may not hold this tile's hits
+        if (live && cnt + ties + 64u > cap) {  // the share may not hold this tile's hits
           atomicOr(P.overflow, 1u);
           atomicOr(block_flag(P.buf, i), 1u);
           live = false;
@@ -765,7 +803,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_c
       }
       __syncwarp();
     }
-    if (MODE == kSweepGather && row) row_counts(row)[2u * blockIdx.y + half] = cnt;
+    if (MODE == kSweepGather && row) row_counts(row)[2u * blockIdx.y + half] = cnt | (ties << 16);
   }
   tc_fence_before();
   __syncthreads();
@@ -778,7 +816,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) dot_sweep_kernel(const __grid_c
 // histogram, each narrowing the range to one bin), as the row's bound.
 constexpr int kBoundWarps = 4;
 __global__ void __launch_bounds__(kBoundWarps * 32) row_bound_kernel(uint64_t* buf, uint32_t n, uint32_t G,
-                                                                    uint32_t lg, uint32_t rank) {
+                                                                    uint32_t rank) {
   extern __shared__ float s_max[];  // [kBoundWarps][G]
   __shared__ unsigned s_hist[kBoundWarps][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -799,7 +837,6 @@ __global__ void __launch_bounds__(kBoundWarps * 32) row_bound_kernel(uint64_t* b
   int lo = __reduce_min_sync(0xffffffffu, (int)flo), hi = __reduce_max_sync(0xffffffffu, (int)fhi);
   float bound = -FLT_MAX;
   unsigned need = rank;
-  bool exact = false;
   for (int pass = 0; pass < 2 && lo <= hi; ++pass) {
     const unsigned span = (unsigned)(hi - lo);
     const int sh = span < 256u ? 0 : 24 - __clz((int)span);
@@ -823,29 +860,11 @@ __global__ void __launch_bounds__(kBoundWarps * 32) row_bound_kernel(uint64_t* b
     lo += bin << sh;
     bound = (float)lo;
     hi = min(hi, lo + (1 << sh) - 1);
-    exact = sh == 0;
-    if (exact) break;
-  }
-  // ties at an exact bound: the need-th group with that maximum, in position
-  // order, ends the ids that can still be among the C best
-  uint32_t limit = 0xffffffffu;
-  if (exact) {
-    for (uint32_t g0 = 0; g0 < G; g0 += 32) {
-      const unsigned at = __ballot_sync(0xffffffffu, g0 + (uint32_t)lane < G && m[g0 + (uint32_t)lane] == bound);
-      const unsigned c = (unsigned)__popc(at);
-      if (need > c) {
-        need -= c;
-        continue;
-      }
-      const uint32_t g = g0 + __fns(at, 0, (int)need);
-      // past the last column of group g: chunk 32 g, or whole tiles of both halves
-      limit = lg == 0u ? (g + 1u) * 32u : (g / 2u + 1u) * ((uint32_t)kTileN << (lg - 1u));
-      break;
-    }
+    if (sh == 0) break;
   }
   if (lane == 0) {
     *row_bound(row) = bound;
-    *row_id_limit(row) = limit;
+    *row_ties(row) = need;  // rank - need groups lie above the bound (or its bin), so at most need ties count
     if (i % (uint32_t)kCtaRows == 0u) *block_flag(buf, i) = 0u;
   }
 }
@@ -858,8 +877,7 @@ __global__ void __launch_bounds__(kBoundWarps * 32) row_bound_kernel(uint64_t* b
 constexpr int kSelWarps = 4;
 __global__ void __launch_bounds__(kSelWarps * 32)
     select_row_kernel(uint64_t* buf, uint32_t n, uint32_t splits, uint32_t C, uint32_t stage_keys, bool sorted,
-                      const uint32_t* __restrict__ ids, uint32_t* __restrict__ out_idx, int32_t* __restrict__ out_val,
-                      uint32_t* overflow) {
+                      const uint32_t* __restrict__ ids, uint32_t* __restrict__ out_idx, int32_t* __restrict__ out_val) {
   extern __shared__ uint64_t s_keys[];  // [kSelWarps][stage_keys]
   __shared__ unsigned s_hist[kSelWarps][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -871,31 +889,46 @@ __global__ void __launch_bounds__(kSelWarps * 32)
   const uint32_t cap = share_slots(splits);
   uint32_t total = 0u;
   int hi = INT32_MIN;
-  for (uint32_t sgm = 0; sgm < 2u * splits; ++sgm) {
-    const uint32_t c = min(row_counts(row)[sgm], cap);
-    if (total + c > stage_keys) {  // more than the staging area holds: the candidate kernel redoes the product
-      if (lane == 0) {
-        atomicOr(overflow, 1u);
-        atomicOr(block_flag(buf, i), 1u);
+  // stages c keys, key x from get(x); a full staging area is cut to its C best first
+  auto stage = [&](uint32_t c, auto get) {
+    for (uint32_t x0 = 0; x0 < c;) {
+      if (total == stage_keys) {
+        __syncwarp();
+        const uint64_t kth = warp_select_kth(keys, (int)total, (int)C, hist, lane);
+        total = (uint32_t)warp_gather_ge(keys, (int)total, kth, keys, lane);
       }
-      return;
-    }
-    const uint2* src = reinterpret_cast<const uint2*>(row + (size_t)sgm * cap);
+      const uint32_t take = min(c - x0, stage_keys - total);
 #pragma unroll 4
-    for (uint32_t x = lane; x < c; x += 32) {
+      for (uint32_t x = lane; x < take; x += 32) keys[total + x] = get(x0 + x);
+      total += take;
+      x0 += take;
+    }
+  };
+  const int bound_val = (int)*row_bound(row);
+  uint32_t above = 0u;
+  for (uint32_t sgm = 0; sgm < 2u * splits; ++sgm) {
+    const uint32_t c = min(row_counts(row)[sgm] & 0xffffu, cap);
+    const uint2* src = reinterpret_cast<const uint2*>(row + (size_t)sgm * cap);
+    above += c;
+    stage(c, [&](uint32_t x) {
       const uint2 e = src[x];
       const int v = (int)__uint_as_float(e.y);
-      keys[total + x] = make_key(v, ids ? __ldg(ids + e.x) : e.x);
       hi = max(hi, v);
+      return make_key(v, ids ? __ldg(ids + e.x) : e.x);
+    });
+  }
+  if (above < C) {  // the ties count only where the values above the bound are too few
+    hi = max(hi, bound_val);
+    for (uint32_t sgm = 0; sgm < 2u * splits; ++sgm) {
+      const uint2* last = reinterpret_cast<const uint2*>(row + (size_t)(sgm + 1u) * cap) - 1;
+      stage(min(row_counts(row)[sgm] >> 16, cap), [&](uint32_t x) { return make_key(bound_val, last[-(int)x].x); });
     }
-    total += c;
   }
   __syncwarp();
   hi = __reduce_max_sync(0xffffffffu, hi);
   int kept = (int)total;
   if (total > C) {
-    const float bound = *row_bound(row);
-    const int lo = (int)bound;
+    const int lo = bound_val;
     const unsigned span = (unsigned)(hi - lo);
     const int sh = span < 256u ? 0 : 24 - __clz((int)span);
     warp_value_hist_ge(keys, (int)total, lo, sh, hist, lane);
@@ -1524,6 +1557,13 @@ __global__ void widen_kernel(const int8_t* __restrict__ q, uint32_t n, uint32_t 
   qb[qb_index(r, (int)(x - r * kDim))] = __float2bfloat16_rn(r < n ? (float)q[x] : 0.f);
 }
 
+// a bias as its three bf16 digits and five zeros
+__device__ __forceinline__ uint4 bias_digits(int32_t b) {
+  const __nv_bfloat162 hi = __floats2bfloat162_rn((float)(b >> 16), (float)((b >> 8) & 255));
+  const __nv_bfloat162 lo = __floats2bfloat162_rn((float)(b & 255), 0.f);
+  return make_uint4(*reinterpret_cast<const uint32_t*>(&hi), *reinterpret_cast<const uint32_t*>(&lo), 0u, 0u);
+}
+
 // one thread per (column, K half) of the padded columns: the bias digits
 // (b >> 16, (b >> 8) & 255, b & 255 at K = 0, 1, 2; zero elsewhere and past n)
 __global__ void bias_digits_kernel(const int32_t* __restrict__ bias, uint32_t n, uint32_t npad, unsigned char* ext) {
@@ -1531,15 +1571,41 @@ __global__ void bias_digits_kernel(const int32_t* __restrict__ bias, uint32_t n,
   if (x >= 2u * npad) return;
   const uint32_t j = x >> 1, h = x & 1u;
   const int32_t b = (bias && j < n) ? bias[j] : 0;
-  __nv_bfloat16 v[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) v[e] = __float2bfloat16_rn(0.f);
-  if (h == 0) {
-    v[0] = __float2bfloat16_rn((float)(b >> 16));
-    v[1] = __float2bfloat16_rn((float)((b >> 8) & 255));
-    v[2] = __float2bfloat16_rn((float)(b & 255));
+  *reinterpret_cast<uint4*>(ext + ext_offset(j, 8u * h)) = h == 0 ? bias_digits(b) : make_uint4(0u, 0u, 0u, 0u);
+}
+
+// A fixed pseudo-random permutation of 0 .. n - 1: bijections of b bits (odd factors,
+// xor shifts), repeated while the image is past the end.
+__device__ __forceinline__ uint32_t shuffled(uint32_t x, uint32_t n, int b) {
+  const uint32_t mask = (uint32_t)((1ull << b) - 1ull);
+  const int h = (b + 1) / 2;
+  do {
+    x = (x + 0x7f4a7c15u) & mask;
+    x = (x * 0x9e3779b1u) & mask;
+    x ^= x >> h;
+    x = (x * 0x85ebca77u) & mask;
+    x ^= x >> h;
+  } while (x >= n);
+  return x;
+}
+
+// one thread per (position, 16-byte chunk) of the shuffled columns' tiles: row
+// shuffled(position), zero from `cols` on, and its bias digits (ext: see bias_digits_kernel)
+__global__ void __launch_bounds__(256) shuffle_kernel(const __nv_bfloat16* __restrict__ Q,
+                                                      const int32_t* __restrict__ bias, uint32_t n, uint32_t cols,
+                                                      uint32_t npos, uint64_t* buf, unsigned char* ext) {
+  const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x, pos = x >> 3, ch = x & 7u;
+  if (pos >= npos) return;
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  int32_t b = 0;
+  if (pos < cols) {
+    const uint32_t r = shuffled(pos, n, 32 - __clz((int)(n - 1u)));
+    v = __ldg(reinterpret_cast<const uint4*>(Q + (size_t)r * kDim) + ch);
+    if (ch == 0u && bias) b = __ldg(bias + r);
   }
-  *reinterpret_cast<uint4*>(ext + ext_offset(j, 8u * h)) = *reinterpret_cast<const uint4*>(v);
+  unsigned char* tile = reinterpret_cast<unsigned char*>(row_scratch(buf, pos / kTileN)) + kShuffledOffset;
+  reinterpret_cast<uint4*>(tile + (pos % kTileN) * kRowBytes)[ch] = v;
+  if (ch < 2u) *reinterpret_cast<uint4*>(ext + ext_offset(pos, 8u * ch)) = ch == 0u ? bias_digits(b) : make_uint4(0u, 0u, 0u, 0u);
 }
 
 size_t bias_pad(uint32_t n) { return ((size_t)n + kPadRows - 1) / kPadRows * kPadRows; }
@@ -1774,8 +1840,8 @@ __global__ void __launch_bounds__(1024) key_scan_kernel(unsigned* cnt) { block_e
 
 __global__ void __launch_bounds__(256) order_scatter_kernel(const uint32_t* __restrict__ key, uint32_t n,
                                                             unsigned* cursor, uint32_t* perm) {
-  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) perm[atomicAdd(&cursor[key[r]], 1u)] = r;
+  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+    perm[atomicAdd(&cursor[key[r]], 1u)] = r;
 }
 
 // one thread per (position, 16-byte chunk) of the padded rows: row perm[p]
@@ -1867,6 +1933,20 @@ static cudaError_t encode_rows(CUtensorMap* m, const void* base, uint64_t rows, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// `tiles` tiles of 128 such rows, tile t in the scratch of row t (base: of row 0)
+static cudaError_t encode_tiles(CUtensorMap* m, const void* base, uint32_t tiles) {
+  const EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return cudaErrorNotSupported;
+  const cuuint64_t dims[3] = {(cuuint64_t)kDim, (cuuint64_t)kTileN, (cuuint64_t)tiles};
+  const cuuint64_t strides[2] = {(cuuint64_t)kRowBytes, (cuuint64_t)kRowSlots * sizeof(uint64_t)};
+  const cuuint32_t box[3] = {(cuuint32_t)kDim, (cuuint32_t)kTileN, 1};
+  const cuuint32_t elem[3] = {1, 1, 1};
+  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // The group size 32 << lg of the two-sweep path: 3 C to 6 C groups (256 of 782
 // groups put 310 columns at or above the bound; twice as many groups would put
 // 281 there, but selecting the bound costs as much again).  Below 2 C groups
@@ -1905,7 +1985,7 @@ static uint32_t sweep_splits(uint32_t blocks, uint32_t tiles, uint32_t most) {
 cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloat16* QB, const int32_t* biasB,
                           uint32_t nB, uint32_t C, bool self, uint64_t* buf, uint32_t* idx, int32_t* val,
                           uint32_t* err, cudaStream_t s, DotDebug dbg, const uint32_t* col_ids,
-                          const uint32_t* row_ids, bool sorted, const __nv_bfloat16* Qraw, const int32_t* bias_raw) {
+                          const uint32_t* row_ids, bool sorted) {
   if (nA == 0) return cudaSuccess;
   const uint32_t S = dot_topk_splits(nA, nB);
   const auto kernel = S > 1 ? (self ? dot_topk_kernel<true, true> : dot_topk_kernel<true, false>)
@@ -1970,19 +2050,19 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
     const uint32_t tm = (nM + kTileN - 1) / kTileN, sm = sweep_splits(blocks, tm, 8u);
     X.tps = ((tm + sm - 1) / sm + per - 1) / per * per;
     X.splits = (tm + X.tps - 1) / X.tps;
-    e = encode_rows(&X.tmB, Qraw ? Qraw : QB, bias_pad(nB), (uint32_t)kTileN);
+    e = encode_tiles(&X.tmB, reinterpret_cast<unsigned char*>(buf) + kShuffledOffset, tm);
     if (e != cudaSuccess) return e;
-    bias_digits_kernel<<<bias_grid, 256, 0, s>>>(Qraw ? bias_raw : biasB, nB, npad, ext);
+    shuffle_kernel<<<(8u * tm * kTileN + 255u) / 256u, 256, 0, s>>>(QB, biasB, nB, nM, tm * kTileN, buf, ext);
     max_kernel<<<dim3(blocks, X.splits), kSwThreads, kSwSmem, s>>>(X);
     const uint32_t G = lg ? 2u * ((tm + per - 1) / per) : 4u * tm;
     const size_t bound_smem = (size_t)kBoundWarps * G * sizeof(float);
     e = allow_shared(reinterpret_cast<const void*>(row_bound_kernel));
     if (e != cudaSuccess) return e;
-    row_bound_kernel<<<(nA + kBoundWarps - 1) / kBoundWarps, kBoundWarps * 32, bound_smem, s>>>(buf, nA, G, lg, C + 1);
+    row_bound_kernel<<<(nA + kBoundWarps - 1) / kBoundWarps, kBoundWarps * 32, bound_smem, s>>>(buf, nA, G, C + 1);
     X.tmB = P.tmB;
     X.nB = nB;
     X.ids = col_ids;
-    if (Qraw) bias_digits_kernel<<<bias_grid, 256, 0, s>>>(biasB, nB, npad, ext);
+    bias_digits_kernel<<<bias_grid, 256, 0, s>>>(biasB, nB, npad, ext);
     const uint32_t sg = sweep_splits(blocks, tiles, kMaxSweepSplits);
     X.tps = (tiles + sg - 1) / sg;
     X.splits = sg;
@@ -1992,7 +2072,7 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
     e = allow_shared(reinterpret_cast<const void*>(select_row_kernel));
     if (e != cudaSuccess) return e;
     select_row_kernel<<<(nA + kSelWarps - 1) / kSelWarps, kSelWarps * 32, sel_smem, s>>>(
-        buf, nA, sg, C, stage_keys, sorted, col_ids, idx, val, overflow);
+        buf, nA, sg, C, stage_keys, sorted, col_ids, idx, val);
     P.gate = overflow;
   } else if (npad) {
     bias_digits_kernel<<<bias_grid, 256, 0, s>>>(biasB, nB, npad, ext);
@@ -2007,8 +2087,8 @@ cudaError_t dot_topk_rect(const __nv_bfloat16* QA, uint32_t nA, const __nv_bfloa
 
 cudaError_t dot_topk(const __nv_bfloat16* Qb, const int32_t* bias, uint32_t n, uint32_t C, uint64_t* buf,
                      uint32_t* idx, int32_t* val, uint32_t* err, cudaStream_t s, DotDebug dbg,
-                     const uint32_t* ids, bool sorted, const __nv_bfloat16* Qraw, const int32_t* bias_raw) {
-  return dot_topk_rect(Qb, n, Qb, bias, n, C, true, buf, idx, val, err, s, dbg, ids, ids, sorted, Qraw, bias_raw);
+                     const uint32_t* ids, bool sorted) {
+  return dot_topk_rect(Qb, n, Qb, bias, n, C, true, buf, idx, val, err, s, dbg, ids, ids, sorted);
 }
 
 cudaError_t quantize(const float* E, uint32_t n, unsigned int* amax_bits, int8_t* q, __nv_bfloat16* qb,
@@ -2064,7 +2144,10 @@ cudaError_t sweep_order(const __nv_bfloat16* Qb, const int32_t* bias, const uint
     proj_buckets_kernel<<<1, 1024, 0, s>>>(hist, n);
     order_key_kernel<<<grid, 256, 0, s>>>(proj, n, range, hist, rank, slen, key, cnt);
     key_scan_kernel<<<1, 1024, 0, s>>>(cnt);
-    order_scatter_kernel<<<grid, 256, 0, s>>>(key, n, cnt, perm);
+    // 4,096 rows at a time: rows of one key (duplicate words) then come about in the
+    // order of their ids, and the gather sweep's tie lists fill with the lowest first
+    // (600k words, C = 512: 113.5 ms against 116.5 for all rows at once)
+    order_scatter_kernel<<<std::min(grid, 16u), 256, 0, s>>>(key, n, cnt, perm);
   }
   if (npad)
     order_gather_kernel<<<(unsigned)(((size_t)npad * 8 + 255) / 256), 256, 0, s>>>(Qb, bias, n, npad, perm, Qp, bp);

@@ -775,8 +775,7 @@ nw_status nw_dot_topk(nw_ctx* c, const int8_t* q, const int32_t* bias, uint32_t 
     NW_CK(prop::sweep_order(qb.as<__nv_bfloat16>(), srcb, nullptr, nullptr, n, osc.p, op.as<uint32_t>(),
                             oq.as<__nv_bfloat16>(), srcb ? ob.as<int32_t>() : nullptr, s));
     NW_CK(prop::dot_topk(oq.as<__nv_bfloat16>(), srcb ? ob.as<int32_t>() : nullptr, n, C, buf.as<uint64_t>(), out_i,
-                         out_v, derr, s, dot_debug(c), op.as<uint32_t>(),
-                         true, qb.as<__nv_bfloat16>(), srcb));
+                         out_v, derr, s, dot_debug(c), op.as<uint32_t>()));
   } else {
     NW_CK(prop::dot_topk(qb.as<__nv_bfloat16>(), srcb, n, C, buf.as<uint64_t>(), out_i, out_v, derr, s,
                          dot_debug(c)));
@@ -1170,7 +1169,7 @@ nw_status nw_proposal_topk(nw_model* M, nw_dict* d, uint32_t C, uint32_t k, uint
                             M->oQb.as<__nv_bfloat16>(), M->obias.as<int32_t>(), s));
     NW_CK(prop::dot_topk(M->oQb.as<__nv_bfloat16>(), M->obias.as<int32_t>(), n, C, M->topbuf.as<uint64_t>(),
                          M->cand.as<uint32_t>(), M->cand_dot.as<int32_t>(), err_ptr(M), s, dot_debug(c),
-                         M->operm.as<uint32_t>(), /*sorted=*/false, M->Qb.as<__nv_bfloat16>(), M->qbias.as<int32_t>()));
+                         M->operm.as<uint32_t>(), /*sorted=*/false));
   } else {
     NW_CK(prop::dot_topk(M->Qb.as<__nv_bfloat16>(), M->qbias.as<int32_t>(), n, C, M->topbuf.as<uint64_t>(),
                          M->cand.as<uint32_t>(), M->cand_dot.as<int32_t>(), err_ptr(M), s, dot_debug(c), nullptr,
