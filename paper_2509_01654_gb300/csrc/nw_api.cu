@@ -209,7 +209,7 @@ nw_status nw_dict_info_get(const nw_dict* d, nw_dict_info* out) {
   i.nbins = (uint32_t)(d->score_hi - d->score_lo + 1);
   i.pairs = d->plan.pairs;
   i.cells = d->plan.cells;
-  i.device_bytes = wordset_bytes(d->ws) + d->d_segs.bytes;
+  i.device_bytes = wordset_bytes(d->ws) + d->d_segs.bytes + d->rec.bytes;
   *out = i;
   return NW_OK;
 }
@@ -399,8 +399,7 @@ nw_status nw_score_pairs(nw_dict* d, const uint32_t* i, const uint32_t* j, size_
   P.gap = d->sc.gap;
   P.tab = dict_tab(d);
   pairs_bits(d, P);
-  // (an eighth as many pairs as words repays making the records)
-  if (P.bit_m && (d->rec.p || m >= n / 8u)) P.rec = dict_records(d, s);
+  P.rec = pair_records(d, P, m, !((flags & NW_ASYNC) && dev), s);
   P.out = dout;
   P.err = c->ws_small.as<uint32_t>();
   Timer tm{c};

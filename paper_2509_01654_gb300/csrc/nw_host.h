@@ -109,7 +109,8 @@ struct nw_dict {
   bool subst = false;  // scored with a full similarity matrix (d_tab)
   DevBuf d_tab;        // kTabDim x kTabDim s'+ table
   uint64_t serial = 0;  // unique per loaded dictionary (caches keyed on it)
-  DevBuf rec;           // the words' 16-byte records, made at first use (dict_records)
+  DevBuf rec;           // the words' 16-byte records, once they repay their making (pair_records)
+  uint64_t pairs_scored = 0;  // by the calls that could have read them
 };
 
 namespace {
@@ -937,11 +938,26 @@ Terms make_terms(const nw_dict* d, const WordSet& a, const WordSet& b, SideView 
   return T;
 }
 
-// The dictionary's word records, made on stream s at first use and kept with
-// it; null when there is no memory for them (the kernels then read symbols).
-const uint4* dict_records(nw_dict* d, cudaStream_t s) {
+// The word records for a call that scores m pairs on stream s, or null (the
+// kernel then reads the pair records).  Making them takes an allocation, a kernel
+// and a wait for it, about 100 us from 65,536 words on, and saves 15 to 40 us a
+// million pairs (1,000,003 pairs of 100k words, 40 / 128 codes: 76 / 101 us without,
+// 62 / 68 with), so they are made once the dictionary has met kRecordPairs pairs: no
+// program pays for them much more than they have saved it.  None are made for pairs
+// that another kernel scores, for a call that does not wait for its stream
+// (may_wait), and a call that is being captured reads none: the memory may go.
+constexpr uint64_t kRecordPairs = (uint64_t)3 << 20;
+const uint4* pair_records(nw_dict* d, const PairsParams& P, uint64_t m, bool may_wait, cudaStream_t s) {
   nw_ctx* c = d->ctx;
-  if (d->rec.p || d->ws.n == 0) return d->rec.as<uint4>();
+  if (!pairs_take_bits(P) || d->ws.n == 0) return nullptr;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (d->rec.p) return d->rec.as<uint4>();
+  d->pairs_scored += m;
+  if (!may_wait || d->pairs_scored < kRecordPairs) return nullptr;
   const std::string err = c->err;
   if (ctx_alloc(c, d->rec, (size_t)d->ws.n * 16, "word records") != NW_OK) {
     c->err = err;

@@ -87,6 +87,8 @@ cudaError_t launch_word_records(const uint32_t* rank, const uint8_t* slen, const
                                 const uint32_t* brec_w, const uint32_t* sym, uint32_t shift, uint32_t n, uint4* rec,
                                 cudaStream_t s);
 cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s);
+// whether launch_pairs takes the bit-parallel kernel, which reads P.rec
+bool pairs_take_bits(const PairsParams& p);
 
 // the all-pairs top-k reduction with every scratch buffer taken from a
 // caller-supplied device region; `provide` is called with the dictionary's

@@ -155,14 +155,19 @@ cudaError_t select_topk(const uint32_t* cand, const int32_t* score, uint32_t n, 
 
 }  // namespace prop
 
+// Words of one length above 32 and many codes stay with the DPX kernel: its warps
+// then run one body, and 64-column masks of that alphabet leave few threads on an
+// SM (128 codes, 1,000,003 pairs of 33 symbols, steps (5, 2): 371 us, DPX 262;
+// lengths 1 .. 40: 396, DPX 16,500; 40 codes, 33 symbols: 248).
+bool pairs_take_bits(const PairsParams& p) {
+  const bool one_body = p.max_len > 32u && p.min_len == p.max_len && p.alphabet > 48u;
+  return p.bit_m && p.alphabet <= kBitPairsAlphabet && !one_body;
+}
+
 cudaError_t launch_pairs(const PairsParams& p, cudaStream_t s) {
   if (p.m == 0) return cudaSuccess;
-  // Words of one length above 32 and many codes stay with the DPX kernel: its warps
-  // then run one body, and 64-column masks of that alphabet leave few threads on an
-  // SM (128 codes, 1,000,003 pairs of 33 symbols, steps (5, 2): 371 us, DPX 262;
-  // lengths 1 .. 40: 396, DPX 16,500; 40 codes, 33 symbols: 248).
-  const bool wide = p.max_len > 32u, one_body = wide && p.min_len == p.max_len && p.alphabet > 48u;
-  if (p.bit_m && p.alphabet <= kBitPairsAlphabet && !one_body) {
+  if (pairs_take_bits(p)) {
+    const bool wide = p.max_len > 32u;
     const void* fn = bit_pairs(p.bit_m, p.bit_x, wide);
     if (!fn) return cudaErrorInvalidValue;
     // A thread's masks are alphabet x 4 or 8 bytes, so large alphabets leave few

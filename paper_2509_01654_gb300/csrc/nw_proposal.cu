@@ -635,7 +635,7 @@ nw_status nw_model_train(nw_model* M, nw_dict* d, const nw_train_config* cfg, co
     pd.long_thresh = (uint32_t)std::lround((double)cfg->long_fraction * (double)(1u << 20));
   }
   PairsParams pp = pairs_params(d, err_ptr(M));
-  if (pp.bit_m) pp.rec = dict_records(d, s);
+  pp.rec = pair_records(d, pp, (uint64_t)m * cfg->steps, true, s);
   pp.pi = M->pi.as<uint32_t>();
   pp.pj = M->pj.as<uint32_t>();
   pp.m = m;

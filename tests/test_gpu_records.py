@@ -1,0 +1,57 @@
+"""The word records that a dictionary keeps for long pair lists: when they are made, that scores are the same with and
+without them, and that they never stand in the way of a call that fits without them."""
+import numpy as np
+import pytest
+
+from paper_2509_01654_gb300 import nw, synth
+
+pytestmark = pytest.mark.gpu
+
+MANY = 3 << 20  # pairs after which a dictionary makes its records
+
+
+def _dictionary(ctx, alphabet, hi, n=600, sc=(1, -1, -1)):
+    w = synth.make_uniform_length_words(n, alphabet, 1.0, 0, hi, seed=alphabet + hi)
+    return w, ctx.load_dictionary(w.codes, w.offsets, alphabet, sc)
+
+
+@pytest.mark.parametrize("alphabet,hi,makes", [(5, 15, True), (40, 40, True), (128, 25, True), (129, 25, False)])
+def test_records_after_many_pairs_and_equal_scores(oracle_mod, alphabet, hi, makes):
+    import torch
+    with nw.Context(0) as ctx:
+        w, d = _dictionary(ctx, alphabet, hi)
+        r = np.random.default_rng(1)
+        i, j = r.integers(0, w.n, (2, 3000)).astype(np.uint32)
+        bare = d.info()["device_bytes"]
+        want = oracle_mod.score_pairs(w, i, j, (1, -1, -1))
+        assert np.array_equal(d.score_pairs(i, j).astype(np.int32), want)
+        assert d.info()["device_bytes"] == bare  # a short list does not repay them
+        p = torch.randint(0, w.n, (MANY,), device="cuda", dtype=torch.int32)
+        d.score_pairs(p, p.flip(0))
+        more = d.info()["device_bytes"] - bare
+        assert more >= 16 * w.n if makes else more == 0
+        assert np.array_equal(d.score_pairs(i, j).astype(np.int32), want)
+
+
+@pytest.mark.parametrize("warm", [10, MANY])
+def test_pairs_in_a_captured_graph(warm):
+    """A call on a stream that is being captured neither allocates nor waits, and replays after the records have gone
+    or come."""
+    import torch
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream), nw.Context(0, stream=stream.cuda_stream) as ctx:
+        w, d = _dictionary(ctx, 20, 30)
+        i = torch.randint(0, w.n, (5000,), device="cuda", dtype=torch.int32)
+        j = torch.randint(0, w.n, (5000,), device="cuda", dtype=torch.int32)
+        p = torch.randint(0, w.n, (warm,), device="cuda", dtype=torch.int32)
+        d.score_pairs(p, p)
+        out = torch.zeros(5000, device="cuda", dtype=torch.int16)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            d.score_pairs(i, j, out=out, async_=True)
+        p = torch.randint(0, w.n, (MANY,), device="cuda", dtype=torch.int32)
+        d.score_pairs(p, p)
+        graph.replay()
+        stream.synchronize()
+        assert torch.equal(out, d.score_pairs(i, j))
