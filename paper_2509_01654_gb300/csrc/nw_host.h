@@ -159,12 +159,17 @@ void ctx_drop_spare(nw_ctx* c, size_t at) {
   c->spare.erase(c->spare.begin() + (std::ptrdiff_t)at);
 }
 
-nw_status ctx_alloc(nw_ctx* c, DevBuf& b, size_t bytes, const char* what) {
+bool ctx_drop_records(nw_ctx* c);
+
+// give_up: what is kept only for speed (spare blocks, word records) is released
+// before the allocation is refused.
+nw_status ctx_alloc(nw_ctx* c, DevBuf& b, size_t bytes, const char* what, bool give_up = true) {
   if (bytes == 0) bytes = 16;
   if (c->fail_countdown) {
     if (--c->fail_countdown == 0)
       return set_err(c, NW_ENOMEM, "injected allocation failure for %s (%zu bytes)", what, bytes);
   }
+  if (c->budget && c->used + bytes > c->budget && give_up) ctx_drop_records(c);
   if (c->budget && c->used + bytes > c->budget)
     return set_err(c, NW_ENOMEM, "memory budget exceeded: %s needs %zu bytes, %zu of %zu in use", what,
                    bytes, c->used, c->budget);
@@ -191,6 +196,10 @@ nw_status ctx_alloc(nw_ctx* c, DevBuf& b, size_t bytes, const char* what) {
     ctx_drop_spare(c, 0);
     e = cudaMalloc(&p, bytes);
   }
+  if (e != cudaSuccess && give_up && ctx_drop_records(c)) {
+    cudaGetLastError();
+    e = cudaMalloc(&p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return set_err(c, NW_ENOMEM, "cudaMalloc(%zu) for %s failed: %s", bytes, what, cudaGetErrorString(e));
@@ -207,6 +216,21 @@ void ctx_free(nw_ctx* c, DevBuf& b) {
     c->used -= b.bytes;
   }
   b = DevBuf{};
+}
+
+// Frees the word records of the context's dictionaries; they are made again once
+// as many pairs have been scored as the first time.  A call takes its records after
+// its last allocation.
+bool ctx_drop_records(nw_ctx* c) {
+  bool any = false;
+  for (nw_dict* d : c->dicts) {
+    if (!d->rec.p) continue;
+    if (!any) cudaStreamSynchronize(c->stream);  // an asynchronous call may still read them
+    ctx_free(c, d->rec);
+    d->pairs_scored = 0;
+    any = true;
+  }
+  return any;
 }
 
 // For a buffer that no work in flight uses.
@@ -959,7 +983,7 @@ const uint4* pair_records(nw_dict* d, const PairsParams& P, uint64_t m, bool may
   d->pairs_scored += m;
   if (!may_wait || d->pairs_scored < kRecordPairs) return nullptr;
   const std::string err = c->err;
-  if (ctx_alloc(c, d->rec, (size_t)d->ws.n * 16, "word records") != NW_OK) {
+  if (ctx_alloc(c, d->rec, (size_t)d->ws.n * 16, "word records", /*give_up=*/false) != NW_OK) {
     c->err = err;
     return nullptr;
   }

@@ -555,6 +555,7 @@ nw_status nw_server_create_proposal(nw_dict* dict, nw_model* model, uint32_t C, 
     }
     sp->view = new nw_dict(*dict);  // the dictionary's device data, owned by the caller's context
     sp->view->ctx = sp->ctx;
+    sp->view->rec = DevBuf{};  // (its context may release them at any time)
     S->pslots.push_back(std::move(sp));
   }
   for (auto& sp : S->pslots) sp->th = std::thread(proposal_slot_main, S, sp.get());

@@ -55,3 +55,32 @@ def test_pairs_in_a_captured_graph(warm):
         graph.replay()
         stream.synchronize()
         assert torch.equal(out, d.score_pairs(i, j))
+
+
+def test_records_give_way_under_a_memory_budget():
+    """A call that fits the budget before a long pair list fits it after."""
+    import torch
+    n, k = 20_000, 10
+    w = synth.make_uniform_length_words(n, 30, 1.0, 1, 15, seed=9)
+    idx = torch.empty((n, k), dtype=torch.int32, device="cuda")
+    score = torch.empty((n, k), dtype=torch.int16, device="cuda")
+    p = torch.randint(0, n, (MANY,), device="cuda", dtype=torch.int32)
+
+    def run(budget, pairs):
+        with nw.Context(0, mem_budget_bytes=budget) as ctx:
+            d = ctx.load_dictionary(w.codes, w.offsets, 30, (1, -1, -1))
+            if pairs:
+                bare = d.info()["device_bytes"]
+                d.score_pairs(p, p.flip(0))
+                assert d.info()["device_bytes"] >= bare + 16 * n  # (there was room)
+            d.all_pairs_topk(k, idx, score, hist=False)
+
+    lo, hi = 0, 64 << 20
+    while hi - lo > 1024:  # the least budget that the lists alone fit
+        mid = (lo + hi) // 2
+        try:
+            run(mid, False)
+            hi = mid
+        except nw.NwError:
+            lo = mid
+    run(hi, True)
