@@ -313,6 +313,25 @@ bool rescore_takes_bits(const nw_dict* d, uint32_t C, int32_t lo, int32_t hi, ui
          (uint64_t)((int64_t)hi - lo + 1) < (1ull << (32 - ib));
 }
 
+// Room for rescoring `rows` rows of C candidates with scores in [lo, hi]: for the
+// bit-parallel kernel (*bits) that of the dictionary's word records unless it has
+// them, else `general` bytes of scores.  Where the records do not fit and the scores
+// do, the scores' kernels take the call.  (The last allocation before the rescoring:
+// a later one may release the dictionary's records.)
+nw_status rescore_room(nw_ctx* c, const nw_dict* d, uint32_t C, int32_t lo, int32_t hi, uint32_t ib, size_t general,
+                       DevBuf& scratch, bool* bits) {
+  *bits = rescore_takes_bits(d, C, lo, hi, ib);
+  const size_t records = std::max<size_t>(16, (size_t)d->ws.n * 16);
+  if (*bits && d->rec.p) return NW_OK;
+  if (*bits) {
+    const nw_status st = ctx_ensure(c, scratch, records, "candidate word records");
+    if (st == NW_OK || records <= general) return st;
+    c->err.clear();
+  }
+  *bits = false;
+  return ctx_ensure(c, scratch, general, "candidate scores");
+}
+
 // The dictionary's word records: its own if it has them, else made in `scratch`
 // on stream s (a server slot's view of a dictionary owns no memory of it).
 nw_status rescore_records(nw_ctx* c, const nw_dict* d, DevBuf& scratch, const uint4** rec, cudaStream_t s) {
@@ -320,7 +339,7 @@ nw_status rescore_records(nw_ctx* c, const nw_dict* d, DevBuf& scratch, const ui
     *rec = d->rec.as<uint4>();
     return NW_OK;
   }
-  NW_TRY(ctx_ensure(c, scratch, std::max<size_t>(16, (size_t)d->ws.n * 16), "candidate word records"));
+  if (!scratch.p) return set_err(c, NW_EINVAL, "no room for word records");
   NW_CK(launch_word_records(d->ws.rank.as<uint32_t>(), d->ws.slen.as<uint8_t>(), d->ws.aoff.as<uint32_t>(),
                             d->ws.brec_w.as<uint32_t>(), d->ws.a_enc.as<uint32_t>(), d->ss.shift, d->ws.n, scratch.as<uint4>(), s));
   *rec = scratch.as<uint4>();
@@ -350,12 +369,20 @@ RescoreBits rescore_bits(const nw_dict* d, const uint32_t* cand, uint32_t rows, 
   return R;
 }
 
+// rescore_room for all rows of the dictionary
+nw_status rescore_self_room(nw_ctx* c, const nw_dict* d, uint32_t C, DevBuf& score_buf, bool* bits) {
+  return rescore_room(c, d, C, d->score_lo, d->score_hi, index_bits(std::max<uint32_t>(d->ws.n, 2)),
+                      prop::rescore_scratch_bytes(d->ws.n, C), score_buf, bits);
+}
+
 // candidate rescoring + selection on the model's or context's buffers
 nw_status rescore_select(nw_ctx* c, nw_dict* d, const uint32_t* cand, uint32_t C, uint32_t k, DevBuf& score_buf,
                          uint32_t* out_idx, int16_t* out_score, uint32_t* err, cudaStream_t s) {
   const uint32_t n = d->ws.n;
   const uint32_t ib = index_bits(std::max<uint32_t>(n, 2));
-  if (rescore_takes_bits(d, C, d->score_lo, d->score_hi, ib)) {
+  bool bits = false;
+  NW_TRY(rescore_self_room(c, d, C, score_buf, &bits));
+  if (bits) {
     const uint4* rec = nullptr;
     NW_TRY(rescore_records(c, d, score_buf, &rec, s));
     RescoreBits R = rescore_bits(d, cand, n, C, k, d->score_lo - 1, ib, rec, out_idx, out_score, err);
@@ -368,7 +395,6 @@ nw_status rescore_select(nw_ctx* c, nw_dict* d, const uint32_t* cand, uint32_t C
     return NW_OK;
   }
   // scores, then the length-sorted candidates they belong to and the work lists
-  NW_TRY(ctx_ensure(c, score_buf, prop::rescore_scratch_bytes(n, C), "candidate scores"));
   int32_t* score = score_buf.as<int32_t>();
   uint32_t* sorted = nullptr;
   NW_CK(prop::rescore_sorted(pairs_params(d, err), cand, C, (int)d->ws.max_len, score, &sorted, s));
@@ -948,7 +974,6 @@ nw_status proposal_query_impl(nw_model* M, nw_dict* d, const uint8_t* qcodes, co
   NW_TRY(ctx_ensure(c, M->qbuf, prop::dot_topk_buffer_bytes(nq, n, C), "candidate buffers"));
   NW_TRY(ctx_ensure(c, M->qcand, sizeof(uint32_t) * outc, "candidate lists"));
   NW_TRY(ctx_ensure(c, M->qcand_dot, sizeof(int32_t) * outc, "candidate lists"));
-  NW_TRY(ctx_ensure(c, M->qscore, sizeof(int32_t) * outc, "candidate scores"));
   uint32_t* derr = prop::dot_topk_err_word(M->qbuf.as<uint64_t>(), nq, n);
   NW_CK(cudaMemsetAsync(derr, 0, sizeof(uint32_t), s));
   NW_CK(prop::dot_topk_rect(M->qQb.as<__nv_bfloat16>(), nq, M->dQb.as<__nv_bfloat16>(), M->dqbias.as<int32_t>(), n,
@@ -982,7 +1007,9 @@ nw_status proposal_query_impl(nw_model* M, nw_dict* d, const uint8_t* qcodes, co
     out_s = os.as<int16_t>();
   }
   const uint32_t ib = index_bits(std::max<uint32_t>(n, 2));
-  if (rescore_takes_bits(d, C, lo, hi, ib)) {
+  bool bits = false;
+  NW_TRY(rescore_room(c, d, C, lo, hi, ib, sizeof(int32_t) * outc, M->qscore, &bits));
+  if (bits) {
     const uint4* rec = nullptr;
     NW_TRY(rescore_records(c, d, M->qscore, &rec, s));
     RescoreBits R = rescore_bits(d, M->qcand.as<uint32_t>(), nq, C, k, lo - 1, ib, rec, out_i, out_s, err_ptr(M));
@@ -1144,7 +1171,8 @@ nw_status nw_proposal_topk(nw_model* M, nw_dict* d, uint32_t C, uint32_t k, uint
   }
   // scratch sized before the timed stages
   NW_TRY(ctx_ensure(c, M->Eall, sizeof(float) * (size_t)n * cnn::kOut, "embeddings"));
-  NW_TRY(ctx_ensure(c, M->cand_score, sizeof(int32_t) * outc, "candidate scores"));
+  bool bits = false;
+  NW_TRY(rescore_self_room(c, d, C, M->cand_score, &bits));
   cudaEvent_t ev[5];
   for (auto& e : ev) NW_CK(cudaEventCreate(&e));
   struct FreeEv {

@@ -57,6 +57,19 @@ def test_pairs_in_a_captured_graph(warm):
         assert torch.equal(out, d.score_pairs(i, j))
 
 
+def _least(run):
+    """The least budget, to 1 KiB, that run(budget) fits."""
+    lo, hi = 0, 4 << 30
+    while hi - lo > 1024:
+        mid = (lo + hi) // 2
+        try:
+            run(mid)
+            hi = mid
+        except nw.NwError:
+            lo = mid
+    return hi
+
+
 def test_records_give_way_under_a_memory_budget():
     """A call that fits the budget before a long pair list fits it after."""
     import torch
@@ -75,12 +88,22 @@ def test_records_give_way_under_a_memory_budget():
                 assert d.info()["device_bytes"] >= bare + 16 * n  # (there was room)
             d.all_pairs_topk(k, idx, score, hist=False)
 
-    lo, hi = 0, 64 << 20
-    while hi - lo > 1024:  # the least budget that the lists alone fit
-        mid = (lo + hi) // 2
-        try:
-            run(mid, False)
-            hi = mid
-        except nw.NwError:
-            lo = mid
-    run(hi, True)
+    run(_least(lambda budget: run(budget, False)), True)
+
+
+def test_rescoring_takes_no_more_memory_than_without_records():
+    """Queries and lists through the proposal fit the budget that they fit with a scoring that uses no records."""
+    n, C, k = 20_000, 16, 5
+    w = synth.make_uniform_length_words(n, 30, 1.0, 1, 15, seed=9)
+    q = synth.make_uniform_length_words(2, 30, 1.0, 1, 15, seed=10)
+
+    def run(budget, sc, lists):
+        with nw.Context(0, mem_budget_bytes=budget) as ctx:
+            d = ctx.load_dictionary(w.codes, w.offsets, 30, sc)
+            model = nw.Model(ctx, 30, seed=1)
+            return model.proposal_topk(d, C, k)[:2] if lists else model.query(d, q.codes, q.offsets, C, k)
+
+    for lists in (False, True):
+        budget = _least(lambda b: run(b, (4, -1, -1), lists)) + (64 << 10)
+        got, want = run(budget, (1, -1, -1), lists), run(0, (1, -1, -1), lists)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
