@@ -118,6 +118,13 @@ void nw_destroy(nw_ctx *ctx);
  * nw_create on this thread. */
 const char *nw_last_error(const nw_ctx *ctx);
 
+/* Releases the device memory that the context keeps only to make its next calls
+ * faster: the buffers of finished calls (at most 4 GiB over all contexts of a
+ * device) and its dictionaries' word records.  The library's own allocations
+ * release it by themselves before they fail; a program calls this before it
+ * needs the memory elsewhere. */
+nw_status nw_trim(nw_ctx *ctx);
+
 /* Turns per-call event timing on or off (off by default). */
 nw_status nw_set_profiling(nw_ctx *ctx, int enable);
 

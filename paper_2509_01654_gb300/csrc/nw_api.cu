@@ -134,13 +134,20 @@ void nw_destroy(nw_ctx* c) {
   ctx_free(c, c->ws_pairs);
   ctx_free(c, c->ws_segs);
   ctx_free(c, c->ws_norm);
-  while (!c->spare.empty()) ctx_drop_spare(c, c->spare.size() - 1);
+  spare_drop_owner(c);
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
 
 const char* nw_last_error(const nw_ctx* c) { return c ? c->err.c_str() : g_create_error.c_str(); }
+
+nw_status nw_trim(nw_ctx* c) {
+  NW_ENTER(c);
+  spare_drop_owner(c);
+  ctx_drop_records(c);
+  return NW_OK;
+}
 
 nw_status nw_set_profiling(nw_ctx* c, int enable) {
   if (!c) return NW_EINVAL;

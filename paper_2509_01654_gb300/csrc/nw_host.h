@@ -25,6 +25,7 @@
 #include "nw_proposal.h"
 #include "nw_internal.cuh"
 #include "nw_launch.h"
+#include "nw_spare.h"
 
 using namespace nw;
 
@@ -90,10 +91,6 @@ struct nw_ctx {
   std::atomic<int> busy{0};
   // grow-only workspace
   DevBuf ws_slots, ws_thr, ws_hist, ws_small, ws_out_idx, ws_out_score, ws_mat, ws_pairs, ws_segs, ws_norm;
-  // blocks that finished calls gave back (ctx_release), oldest first: at most
-  // kSpareBytes in kSpareBlocks blocks, not part of `used`
-  std::vector<DevBuf> spare;
-  size_t spare_bytes = 0;
   std::vector<cudaEvent_t> events;
 };
 
@@ -142,23 +139,6 @@ nw_status cuda_fail(nw_ctx* c, cudaError_t e, const char* what) {
     if (s_ != NW_OK) return s_;             \
   } while (0)
 
-// Memory that lives for one call.  cudaMalloc and cudaFree map and unmap pages
-// and wait for the device: 3.3 GB of candidate buffers cost 2.7 ms of an 8.1 ms
-// call for 100,000 rows, and sixteen small buffers 200 us of a 290 us query.  A
-// call that has synchronised its stream therefore hands its buffers to the
-// context (ctx_release), whose next allocations take them.  The spare blocks are
-// bounded, they are released before an allocation is refused for the budget or
-// for want of device memory, and with the context.  A call that fails frees its
-// buffers (CallBufs): its stream may still be using them.
-constexpr size_t kSpareBytes = (size_t)4 << 30;
-constexpr size_t kSpareBlocks = 64;
-
-void ctx_drop_spare(nw_ctx* c, size_t at) {
-  cudaFree(c->spare[at].p);
-  c->spare_bytes -= c->spare[at].bytes;
-  c->spare.erase(c->spare.begin() + (std::ptrdiff_t)at);
-}
-
 bool ctx_drop_records(nw_ctx* c);
 
 // give_up: what is kept only for speed (spare blocks, word records) is released
@@ -173,27 +153,21 @@ nw_status ctx_alloc(nw_ctx* c, DevBuf& b, size_t bytes, const char* what, bool g
   if (c->budget && c->used + bytes > c->budget)
     return set_err(c, NW_ENOMEM, "memory budget exceeded: %s needs %zu bytes, %zu of %zu in use", what,
                    bytes, c->used, c->budget);
-  // the smallest spare block that holds it and is not much larger (under a
-  // budget only one of the same size: what fitted it before still fits)
-  size_t best = c->spare.size();
-  for (size_t i = 0; i < c->spare.size(); ++i) {
-    const size_t have = c->spare[i].bytes;
-    if (have < bytes || have > (c->budget ? bytes : bytes + bytes / 4 + 4096)) continue;
-    if (best == c->spare.size() || have < c->spare[best].bytes) best = i;
-  }
-  if (best < c->spare.size()) {
-    b = c->spare[best];
-    c->spare_bytes -= b.bytes;
-    c->spare.erase(c->spare.begin() + (std::ptrdiff_t)best);
-    c->used += b.bytes;
+  // a spare block that is not much larger (under a budget only one of the same
+  // size: what fitted it before still fits)
+  size_t have = 0;
+  if (void* p = spare_take(c, bytes, c->budget ? bytes : bytes + bytes / 4 + 4096, &have)) {
+    b.p = p;
+    b.bytes = have;
+    c->used += have;
     return NW_OK;
   }
-  while (c->budget && !c->spare.empty() && c->used + c->spare_bytes + bytes > c->budget) ctx_drop_spare(c, 0);
+  while (c->budget && c->used + spare_held(c) + bytes > c->budget && spare_drop_oldest(c)) {
+  }
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
-  while (e != cudaSuccess && !c->spare.empty()) {
+  if (e != cudaSuccess && spare_drop_device(c->device)) {
     cudaGetLastError();
-    ctx_drop_spare(c, 0);
     e = cudaMalloc(&p, bytes);
   }
   if (e != cudaSuccess && give_up && ctx_drop_records(c)) {
@@ -233,18 +207,17 @@ bool ctx_drop_records(nw_ctx* c) {
   return any;
 }
 
-// For a buffer that no work in flight uses.
+// For a buffer that no work in flight uses: kept for the next call (nw_spare.h).
 void ctx_release(nw_ctx* c, DevBuf& b) {
-  if (!b.p || b.bytes > kSpareBytes) return ctx_free(c, b);
-  while (!c->spare.empty() && (c->spare.size() >= kSpareBlocks || c->spare_bytes + b.bytes > kSpareBytes))
-    ctx_drop_spare(c, 0);
-  c->used -= b.bytes;
-  c->spare_bytes += b.bytes;
-  c->spare.push_back(b);
+  if (b.p) {
+    c->used -= b.bytes;
+    spare_give(c, c->device, b.p, b.bytes);
+  }
   b = DevBuf{};
 }
 
-// RAII: a call's own buffers; `done` once the call has synchronised its stream.
+// RAII: a call's own buffers; `done` once the call has synchronised its stream
+// (a call that fails frees them: its stream may still be using them).
 struct CallBufs {
   nw_ctx* c;
   std::vector<DevBuf*> bufs;

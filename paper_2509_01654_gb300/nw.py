@@ -28,7 +28,7 @@ MISSING_IDX = 0xFFFFFFFF
 MISSING_SCORE = -32768
 
 EXPORTED = [
-    "nw_create", "nw_destroy", "nw_last_error", "nw_set_profiling", "nw_last_profile",
+    "nw_create", "nw_destroy", "nw_last_error", "nw_trim", "nw_set_profiling", "nw_last_profile",
     "nw_load_dictionary", "nw_dict_info_get", "nw_dict_free", "nw_all_pairs_matrix",
     "nw_all_pairs_topk", "nw_all_pairs_topk_shard", "nw_topk_merge", "nw_topk_merge_device", "nw_score_pairs",
     "nw_query",
@@ -139,6 +139,7 @@ def load_library(path: str = LIB_PATH):
     L.nw_last_error.argtypes = [vp]
     L.nw_last_error.restype = ctypes.c_char_p
     L.nw_set_profiling.argtypes = [vp, ctypes.c_int]
+    L.nw_trim.argtypes = [vp]
     L.nw_last_profile.argtypes = [vp, ctypes.POINTER(Profile)]
     L.nw_load_dictionary.argtypes = [vp, vp, vp, u32, u32, ctypes.POINTER(Scoring), u32, ctypes.POINTER(vp)]
     L.nw_dict_info_get.argtypes = [vp, ctypes.POINTER(DictInfo)]
@@ -280,6 +281,10 @@ class Context:
 
     def set_profiling(self, on: bool = True):
         _check(self.handle, load_library().nw_set_profiling(self.handle, int(on)))
+
+    def trim(self):
+        """nw_trim: releases the memory that the context keeps for its next calls."""
+        _check(self.handle, load_library().nw_trim(self.handle))
 
     def last_profile(self) -> dict:
         p = Profile()

@@ -34,3 +34,23 @@ def test_calls_of_changing_size_equal_a_fresh_context(budget):
             nw.dot_topk(shared, q, 32)
         assert nw.dot_topk(shared, q[:50], 8)[0].shape == (50, 8)
     shared.close()
+
+
+def test_another_context_can_have_the_memory():
+    """What one context keeps for its next call does not refuse another's, and a program can have it back."""
+    import torch
+    q = np.random.default_rng(1).integers(-128, 128, (20_000, 64), dtype=np.int8)
+    with nw.Context(0) as a, nw.Context(0) as b:
+        want = nw.dot_topk(a, q, 32)  # leaves more than a gigabyte of buffers
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        hog = torch.empty(free - (1 << 30), dtype=torch.uint8, device="cuda")
+        got = nw.dot_topk(b, q, 32)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
+        held = torch.cuda.mem_get_info()[0]
+        b.trim()
+        assert torch.cuda.mem_get_info()[0] - held > 1 << 30
+        del hog
+        torch.cuda.empty_cache()
+        got = nw.dot_topk(a, q, 32)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
