@@ -508,7 +508,7 @@ nw_status query_impl(nw_dict* d, const uint8_t* qcodes, const uint32_t* qoffsets
   base.local[0] = make_terms(d, q, d->ws, qside, dside, key_lo, ib);
   base.local[1] = make_terms(d, d->ws, q, dside, qside, key_lo, ib);
   RunOut ro;
-  NW_TRY(run_plan(c, s, plan, c->ws_segs.as<Seg>(), query_epi(d), base, d_counters, tm, ro));
+  NW_TRY(run_plan(c, s, plan, c->ws_segs.as<Seg>(), kEpiOtherLists, base, d_counters, tm, ro));
   cudaEvent_t e_fin = nullptr;
   tm.begin(false, e_fin);
   NW_CK(launch_finalize(c->ws_slots.as<uint32_t>(), nq, k, q.perm.as<uint32_t>(), ib, base.local[0].imask, key_lo, out_idx,

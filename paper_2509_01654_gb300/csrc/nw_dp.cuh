@@ -205,6 +205,39 @@ __device__ __forceinline__ uint32_t list_offer(uint32_t* row, uint32_t* thr, uin
   return 0xffffffffu;
 }
 
+// Offers the lanes' keys (0: none) to one list of k <= 32 slots, the warp together:
+// lane s holds slot s, the largest key takes the place of the smallest slot until none
+// is larger, and each slot that changed is swapped in memory.  A failed swap means that
+// another warp changed that slot: its key is offered again (bounded).  With j slots
+// m_1 < .. < m_j given up, the j keys taken and the k - j slots left (slots only grow)
+// are k keys above m_j, so each of them is rightly dropped whatever the other swaps do;
+// a key is rejected only against k slots above it.
+__device__ __forceinline__ void list_offer_warp(uint32_t* row, uint32_t* thr, uint32_t k, uint32_t key, uint32_t* err,
+                                                uint32_t& inserts, int max_iters) {
+  const uint32_t lane = threadIdx.x & 31u;
+  for (int it = 0; it < max_iters; ++it) {
+    const uint32_t old = lane < k ? __ldcg(row + lane) : 0xffffffffu;
+    uint32_t now = old, low;
+    for (;;) {
+      low = __reduce_min_sync(0xffffffffu, now);
+      const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+      if (top <= low) break;
+      if ((uint32_t)(__ffs(__ballot_sync(0xffffffffu, now == low)) - 1) == lane) now = top;
+      if (key == top) key = 0u;  // (keys of one list are distinct)
+    }
+    key = 0u;
+    if (now != old) {
+      if (atomicCAS(row + lane, old, now) == old) ++inserts;
+      else key = now;
+    }
+    if (!__any_sync(0xffffffffu, key != 0u)) {
+      if (lane == 0u) atomicMax(thr, low);
+      return;
+    }
+  }
+  if (lane == 0u) atomicOr(err, kErrRetry);
+}
+
 // global -> shared 4-byte asynchronous copy (cp.async.ca; 4-byte aligned)
 __device__ __forceinline__ void cp_async4(uint32_t* dst, const uint32_t* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
@@ -315,12 +348,15 @@ __device__ __forceinline__ uint32_t neg_bound2(int t_lo, int t_hi) {
 //
 // Files n <= 32 queued pairs in their words' lists; returns the lane's inserts.
 // kAhead: the slots of a list are read eight at a time, and where only A words
-// have lists the best of a warp's candidates is offered first (a query's empty
-// list is offered to by hundreds of warps at once).  One query against 100k
-// words 251 -> 183 us, 4,096 against 600k 14.2 -> 12.3 ms, 16 dictionaries 8.97
-// -> 8.13 ms.  The all-pairs kernels, whose lists belong to both sides, lose by
-// it at 600k words (390 -> 418 ms with histogram, 380 -> 410 normalised): there
-// it is compiled out.
+// have lists (queries) a warp's candidates for one list are offered together
+// (list_offer_warp; above 32 slots one by one, the best first): a list that starts
+// empty takes k candidates of each of the first warps, and one by one each was four
+// trips to L2.  One by one, 16 queries of 12 symbols against 2,000 words took 388 us
+// on the DPX kernel (269 before the queue) and 672 with a similarity matrix, whose
+// kernels had no such epilogue (296); together 199 and 206.  Bit-parallel: one query against
+// 600k words 196 -> 139 us, 4,096 11.8 -> 10.8 ms.  The all-pairs kernels, whose lists
+// belong to both sides, lose by reading ahead at 600k words (390 -> 418 ms with
+// histogram, 380 -> 410 normalised): there it is compiled out.
 template <int EPI>
 constexpr bool kFileAhead = EPI == kEpiOtherLists;
 template <bool kAhead>
@@ -348,8 +384,17 @@ __device__ __forceinline__ uint32_t file_candidates(const AlignParams& P, const 
       key = list_key(P, T, s, Q.mx, ob);
       if (key <= __ldcg(T.A.thr + a)) key = 0u;
     }
-    const uint32_t group = __match_any_sync(0xffffffffu, a);
     uint32_t todo;
+    if (kAhead && !T.B.slots && P.k <= 32u) {  // one list at a time, its candidates together
+      while ((todo = __ballot_sync(0xffffffffu, key != 0u)) != 0u) {
+        const uint32_t a0 = __shfl_sync(0xffffffffu, a, __ffs(todo) - 1);
+        const bool mine = key != 0u && a == a0;
+        list_offer_warp(T.A.slots + (size_t)a0 * P.k, T.A.thr + a0, P.k, mine ? key : 0u, P.err, inserts, max_iters);
+        if (mine) key = 0u;
+      }
+      return inserts;
+    }
+    const uint32_t group = __match_any_sync(0xffffffffu, a);
     while ((todo = __ballot_sync(0xffffffffu, key != 0u)) != 0u) {
       bool lead = (uint32_t)(__ffs(todo & group) - 1) == lane;
       if constexpr (kAhead) {

@@ -981,9 +981,6 @@ void pairs_bits(const nw_dict* d, PairsParams& P) {
   P.max_len = d->ws.max_len;
 }
 
-// queries; similarity matrices have no kEpiOtherLists kernel
-int query_epi(const nw_dict* d) { return d->subst ? kEpiLists : kEpiOtherLists; }
-
 int lists_epi(int hist_mode) { return hist_mode == kHistLane ? kEpiListsLaneHist : kEpiLists; }
 
 // The whole pair set of a dictionary, or one shard of it (planned on the spot

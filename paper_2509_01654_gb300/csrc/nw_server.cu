@@ -259,7 +259,7 @@ nw_status launch_batch(nw_server* S, Slot& s) {
   base.local[1] = make_terms(d, d->ws, q, dside, qside, key_lo, ib);
   Timer tm{c};
   RunOut ro;
-  NW_TRY(run_plan(c, st, s.plan, s.d_segs.as<Seg>(), query_epi(d), base,
+  NW_TRY(run_plan(c, st, s.plan, s.d_segs.as<Seg>(), kEpiOtherLists, base,
                   reinterpret_cast<unsigned long long*>(s.d_small.as<char>() + 64), tm, ro));
   NW_CK(launch_finalize(s.d_slots.as<uint32_t>(), nq, k, s.d_perm.as<uint32_t>(), ib, base.local[0].imask, key_lo,
                         s.d_idx.as<uint32_t>(), s.d_score.as<int16_t>(), st));

@@ -140,3 +140,20 @@ def test_long_words_of_the_dearest_classes(ctx, oracle_mod, sc):
         assert np.array_equal(bi, idx) and np.array_equal(bs, score)
         assert np.array_equal(batch.run_queries()[1][0][0], qi)
     d.free()
+
+
+# query lists of one slot, of a warp's width and past it, which start empty under many warps at once; the similarity
+# matrix of the second scoring has to give its lists
+@pytest.mark.parametrize("k", [1, 7, 32, 33, 128])
+@pytest.mark.parametrize("length,n,nq", [(6, 4000, 40), (12, 900, 300), (35, 300, 5)])
+def test_query_lists_of_every_width(ctx, oracle_mod, k, length, n, nq):
+    w, q = _words([length] * n, 5, n), _words([length] * nq, 5, nq)
+    for sc in ((1, -1, -1), (4, -1, -1)):
+        d = ctx.load_dictionary(w.codes, w.offsets, 5, sc)
+        got = d.query(q.codes, q.offsets, k)
+        wi, ws = oracle_mod.query_topk(q, w, k, sc)
+        assert np.array_equal(got[0], wi) and np.array_equal(got[1].astype(np.int32), ws)
+        d.free()
+    d = ctx.load_dictionary_sim(w.codes, w.offsets, 5, np.where(np.eye(5, dtype=bool), 4, -1).astype(np.int32), -1)
+    assert all(np.array_equal(x, y) for x, y in zip(d.query(q.codes, q.offsets, k), got))
+    d.free()
