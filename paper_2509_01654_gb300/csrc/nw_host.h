@@ -15,7 +15,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
 #include <set>
 #include <string>
 #include <utility>
@@ -534,13 +533,15 @@ void plan_bits(const Rects& rects, int m, int x, uint32_t alphabet, uint32_t ta,
   l.alphabet = alphabet;
   l.ta = ta;
   l.seg_first = (uint32_t)p.segs.size();
-  std::map<std::pair<uint32_t, int>, uint64_t> met;  // words met so far, by query set and length
+  uint32_t sets = 0;
+  for (const Rect& r : rects) sets = std::max(sets, std::min(r.dict, r.dict_swapped) + 1);
+  std::vector<uint64_t> met((size_t)sets * kBuckets, 0);  // words met so far, by query set and length
   for (Rect r : rects) {
     const uint32_t na = r.a1 - r.a0, nb = r.b1 - r.b0;
     uint64_t cost = bit_cost(na, r.La, nb, r.LB, ta), swapped = bit_cost(nb, r.LB, na, r.La, ta);
     if (r.dict != r.dict_swapped) {
       const bool a_queries = r.dict < r.dict_swapped;  // (rects_queries)
-      uint64_t& m = met[{std::min(r.dict, r.dict_swapped), a_queries ? r.La : r.LB}];
+      uint64_t& m = met[(size_t)std::min(r.dict, r.dict_swapped) * kBuckets + (size_t)(a_queries ? r.La : r.LB)];
       if (m < kColdWords) (a_queries ? swapped : cost) *= kColdFactor;
       m += a_queries ? nb : na;
     }
@@ -563,12 +564,16 @@ constexpr uint64_t kBitMinTasks = 12288, kDpMinTasks = 40960;
 constexpr uint32_t kMinTA = 16;
 template <class Make>
 void sized(Plan& p, uint64_t min_tasks, Make make) {
-  for (uint32_t ta = kDefaultTA;; ta /= 2) {
+  for (uint32_t ta = kDefaultTA;;) {
     p = Plan{};
     make(ta, p);
     uint64_t n = 0;
     for (const Launch& l : p.launches) n += l.ntasks;
     if (n >= min_tasks || ta <= kMinTA) return;
+    do {  // (half the chunk makes at most twice the tasks: sizes that cannot suffice are skipped)
+      ta /= 2;
+      n *= 2;
+    } while (n < min_tasks && ta > kMinTA);
   }
 }
 
