@@ -152,10 +152,11 @@ nw_status ctx_alloc(nw_ctx* c, DevBuf& b, size_t bytes, const char* what, bool g
   if (c->budget && c->used + bytes > c->budget)
     return set_err(c, NW_ENOMEM, "memory budget exceeded: %s needs %zu bytes, %zu of %zu in use", what,
                    bytes, c->used, c->budget);
-  // a spare block that is not much larger (under a budget only one of the same
-  // size: what fitted it before still fits)
+  // a spare block that is not much larger (under a budget only an own one of the
+  // same size: what fitted it before still fits)
   size_t have = 0;
-  if (void* p = spare_take(c, bytes, c->budget ? bytes : bytes + bytes / 4 + 4096, &have)) {
+  if (void* p = spare_take(c->budget ? c : nullptr, c->device, bytes, c->budget ? bytes : bytes + bytes / 4 + 4096,
+                           &have)) {
     b.p = p;
     b.bytes = have;
     c->used += have;

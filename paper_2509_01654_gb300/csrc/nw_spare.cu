@@ -40,12 +40,12 @@ bool drop(Pick pick, size_t most) {
 
 }  // namespace
 
-void* spare_take(const void* owner, size_t bytes, size_t most, size_t* have) {
+void* spare_take(const void* owner, int device, size_t bytes, size_t most, size_t* have) {
   std::lock_guard<std::mutex> lock(mu);
   size_t best = blocks.size();
   for (size_t i = 0; i < blocks.size(); ++i) {
     const Block& b = blocks[i];
-    if (b.owner != owner || b.bytes < bytes || b.bytes > most) continue;
+    if (b.device != device || (owner && b.owner != owner) || b.bytes < bytes || b.bytes > most) continue;
     if (best == blocks.size() || b.bytes < blocks[best].bytes) best = i;
   }
   if (best == blocks.size()) return nullptr;

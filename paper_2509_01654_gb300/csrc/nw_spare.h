@@ -1,14 +1,14 @@
-// nw_spare.h -- device blocks that finished calls gave back, kept for their
-// context's next calls.
+// nw_spare.h -- device blocks that finished calls gave back, kept for the next
+// calls.
 //
 // cudaMalloc and cudaFree map and unmap pages and wait for the device: 3.3 GB of
 // candidate buffers cost 2.7 ms of an 8.1 ms call for 100,000 rows, and sixteen small
 // buffers 200 us of a 290 us query.  A call that has synchronised its stream
-// therefore gives its buffers here, and its context's next allocations take them, on
-// any stream.  A context takes its own blocks only (they count against its budget),
-// but all contexts share one list per process: it is bounded for a device as a
-// whole, and an allocation that fails for want of device memory releases every
-// context's blocks before it is refused.
+// therefore gives its buffers here, and the next allocations take them, of any context
+// and on any stream; a context with a memory budget takes its own only, which count
+// against it.  The list is bounded for a device as a whole (two contexts that call in
+// turn use the same blocks), and an allocation that fails for want of device memory
+// releases all of it before it is refused.
 #pragma once
 
 #include <stddef.h>
@@ -18,8 +18,9 @@ namespace nw {
 constexpr size_t kSpareBytes = (size_t)4 << 30;  // of a device, over all contexts
 constexpr size_t kSpareBlocks = 64;              // of a context
 
-// the smallest of the owner's blocks of `bytes` to `most` bytes; its size in *have
-void* spare_take(const void* owner, size_t bytes, size_t most, size_t* have);
+// the smallest block of the device (with an owner: of its own) of `bytes` to `most`
+// bytes; its size in *have
+void* spare_take(const void* owner, int device, size_t bytes, size_t most, size_t* have);
 // keeps a block that no work in flight uses; older blocks of the device make room
 void spare_give(const void* owner, int device, void* p, size_t bytes);
 size_t spare_held(const void* owner);

@@ -54,3 +54,23 @@ def test_another_context_can_have_the_memory():
         torch.cuda.empty_cache()
         got = nw.dot_topk(a, q, 32)
         assert all(np.array_equal(x, y) for x, y in zip(got, want))
+
+
+def test_two_contexts_in_turn_keep_their_speed():
+    """Calls of two contexts, one after the other, do not allocate each time."""
+    import time
+
+    import torch
+    q = torch.randint(-128, 128, (60_000, 64), dtype=torch.int8, device="cuda")  # about 2 GB of buffers a call
+    with nw.Context(0) as a, nw.Context(0) as b:
+        took = {}
+        for name, contexts in (("one", [a, a]), ("two", [a, b])):
+            times = []
+            for _ in range(8):
+                for c in contexts:
+                    torch.cuda.synchronize()
+                    t0 = time.perf_counter()
+                    nw.dot_topk(c, q, 64)
+                    times.append(time.perf_counter() - t0)
+            took[name] = np.median(times[4:])
+    assert took["two"] < 1.3 * took["one"], took
