@@ -118,11 +118,12 @@ void nw_destroy(nw_ctx *ctx);
  * nw_create on this thread. */
 const char *nw_last_error(const nw_ctx *ctx);
 
-/* Releases the device memory that the context keeps only to make its next calls
- * faster: the buffers of finished calls (at most 4 GiB over all contexts of a
- * device) and its dictionaries' word records.  The library's own allocations
- * release it by themselves before they fail; a program calls this before it
- * needs the memory elsewhere. */
+/* Releases the device memory that is kept only to make the next calls faster:
+ * the buffers of finished calls (at most 4 GiB over all contexts of the
+ * device, which share them) and the context's dictionaries' word records.  The
+ * library's own allocations release it by themselves before they fail, and the
+ * last context of a device releases the buffers; a program calls this before
+ * it needs the memory elsewhere. */
 nw_status nw_trim(nw_ctx *ctx);
 
 /* Turns per-call event timing on or off (off by default). */
@@ -282,12 +283,13 @@ typedef struct {
 /* nw_batch_create flag: time tile-shape candidates per launch.  Per range of
  * ten longer lengths, the A words per task of the DPX kernel's launch are
  * chosen from {64, 128, 256}, then the resident blocks per SM from {2, 3, as
- * many as fit} at that size, by timing whole launches on the batch.  (The
- * bit-parallel kernel's launches follow a rule on their number of tasks.)  (A task's B chunk is 64 words: two words per
- * lane in the kernel's int16x2 registers, fixed at compile time.)  The
- * choices are cached for the life of the process, keyed by the device's SM
- * count, k, and every dictionary's and query set's length histogram, scoring
- * and flags: a batch of the same shape is not timed again (tune_cached = 1). */
+ * many as fit} at that size, by timing whole launches on the batch.  (A
+ * task's B chunk is 64 words: two words per lane in the kernel's int16x2
+ * registers, fixed at compile time.)  The bit-parallel kernel's launches
+ * follow a rule on their number of tasks instead.  The choices are cached for
+ * the life of the process, keyed by the device's SM count, k, and every
+ * dictionary's and query set's length histogram, scoring and flags: a batch
+ * of the same shape is not timed again (tune_cached = 1). */
 #define NW_BATCH_AUTOTUNE 0x10u
 
 typedef struct {

@@ -112,6 +112,7 @@ nw_status nw_create(nw_ctx** out, int device, size_t mem_budget_bytes, void* cud
     }
     c->own_stream = true;
   }
+  spare_open(device);
   *out = c;
   return NW_OK;
 }
@@ -134,7 +135,7 @@ void nw_destroy(nw_ctx* c) {
   ctx_free(c, c->ws_pairs);
   ctx_free(c, c->ws_segs);
   ctx_free(c, c->ws_norm);
-  spare_drop_owner(c);
+  spare_close(c, c->device);
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
@@ -144,7 +145,7 @@ const char* nw_last_error(const nw_ctx* c) { return c ? c->err.c_str() : g_creat
 
 nw_status nw_trim(nw_ctx* c) {
   NW_ENTER(c);
-  spare_drop_owner(c);
+  spare_drop_device(c->device);
   ctx_drop_records(c);
   return NW_OK;
 }

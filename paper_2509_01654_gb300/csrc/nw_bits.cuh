@@ -21,12 +21,14 @@
 // for m >= 3 the planes are first recoded to binary digits, so that a word
 // takes two or three bit counts.
 //
-// What bounds it: the logic pipe.  A row of (1, -1, -1), steps (3, 1), is 17
-// logic and add instructions per 32 columns, 34 a lane for up to 48 cells
-// where the DPX cell takes 3 for 2.  600k words, top-10 and histogram: 1,129
-// ms on the DPX kernel, 390 here, of which the row logic at the measured LOP3
-// rate is about 280, lists that move about 25 and the histogram's shared
-// additions 13 to 20.
+// What bounds it: the logic pipe.  A row of (1, -1, -1), steps (3, 1), is 14
+// logic operations and 3 additions per 32 columns, 34 instructions a lane for up
+// to 48 cells where the DPX cell takes 3 for 2.  600k words, top-10 and histogram:
+// 1,129 ms on the DPX kernel, 390 here, of which the logic operations at the
+// measured LOP3 rate are 272 (the additions have a second pipe: 100 lanes a clock
+// against 64), lists that move about 25 and the histogram's shared additions 13 to
+// 20; the rest is issue slots and stalls (at 100k words the logic pipe is 70.5 %
+// active, issue 65.8 %).
 #pragma once
 
 #include "nw_bitrow.cuh"

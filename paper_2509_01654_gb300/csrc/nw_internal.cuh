@@ -178,7 +178,6 @@ __host__ __device__ inline void merge_ranked_row(uint32_t nparts, uint32_t k, At
   }
 }
 
-enum { kModeMatrix = 0, kModeLists = 1 };
 enum { kHistNone = 0, kHistSmem = 1, kHistGlobal = 2, kHistLane = 3 };
 
 // Blocks per SM the alignment kernel is compiled for: the register budget
@@ -248,7 +247,7 @@ constexpr int kBitBlock = 128;
 constexpr int kBitWarps = kBitBlock / 32;
 constexpr uint32_t kMaskRow = 256;   // bytes of one code's match masks: 32 lanes x 64 columns
 constexpr uint32_t kBitSub = 32;     // A words a warp stages at a time (at most 32)
-constexpr int kBitMaxStep = 5;       // largest reduced match step with a kernel
+constexpr int kBitMaxStep = 5;       // largest reduced match step with a kernel (the classes' times: take_long)
 
 // Words of length b held in a lane's 64 columns, and the columns each gets
 // (fixed by that number, so that the score extraction knows every field at

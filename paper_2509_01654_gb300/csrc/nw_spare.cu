@@ -2,6 +2,7 @@
 // cudaFree may wait for the device.
 #include <cuda_runtime.h>
 
+#include <map>
 #include <mutex>
 #include <vector>
 
@@ -18,6 +19,7 @@ struct Block {
 };
 std::mutex mu;
 std::vector<Block> blocks;  // oldest first
+std::map<int, int> contexts;  // by device
 
 // takes out what `pick` says, at most `most` blocks, and frees it
 template <class Pick>
@@ -87,11 +89,24 @@ size_t spare_held(const void* owner) {
 bool spare_drop_oldest(const void* owner) {
   return drop([&](const Block& b) { return b.owner == owner; }, 1);
 }
-bool spare_drop_owner(const void* owner) {
-  return drop([&](const Block& b) { return b.owner == owner; }, (size_t)-1);
-}
 bool spare_drop_device(int device) {
   return drop([&](const Block& b) { return b.device == device; }, (size_t)-1);
+}
+
+
+void spare_open(int device) {
+  std::lock_guard<std::mutex> lock(mu);
+  ++contexts[device];
+}
+void spare_close(const void* owner, int device) {
+  bool last = false;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    last = --contexts[device] <= 0;
+    for (Block& b : blocks)
+      if (b.owner == owner) b.owner = nullptr;
+  }
+  if (last) spare_drop_device(device);
 }
 
 }  // namespace nw

@@ -7,8 +7,11 @@
 // therefore gives its buffers here, and the next allocations take them, of any context
 // and on any stream; a context with a memory budget takes its own only, which count
 // against it.  The list is bounded for a device as a whole (two contexts that call in
-// turn use the same blocks), and an allocation that fails for want of device memory
-// releases all of it before it is refused.
+// turn use the same blocks).  It is released when an allocation fails for want of
+// device memory, before that is refused; by nw_trim; and with the device's last
+// context (a program that makes a context for each piece of work keeps the blocks:
+// the first candidate lists of 100,003 rows 5.4 ms, 6.7 where the context before had
+// freed them).
 #pragma once
 
 #include <stddef.h>
@@ -24,9 +27,11 @@ void* spare_take(const void* owner, int device, size_t bytes, size_t most, size_
 // keeps a block that no work in flight uses; older blocks of the device make room
 void spare_give(const void* owner, int device, void* p, size_t bytes);
 size_t spare_held(const void* owner);
-// the oldest of the owner's blocks, all of them, or all of a device: false if there is none
+// frees the oldest of the owner's blocks, or all of a device: false if there is none
 bool spare_drop_oldest(const void* owner);
-bool spare_drop_owner(const void* owner);
 bool spare_drop_device(int device);
+// a context of the device comes, and goes: its blocks stay for the others
+void spare_open(int device);
+void spare_close(const void* owner, int device);
 
 }  // namespace nw

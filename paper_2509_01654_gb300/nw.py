@@ -283,7 +283,7 @@ class Context:
         _check(self.handle, load_library().nw_set_profiling(self.handle, int(on)))
 
     def trim(self):
-        """nw_trim: releases the memory that the context keeps for its next calls."""
+        """nw_trim: releases the memory that is kept for the next calls."""
         _check(self.handle, load_library().nw_trim(self.handle))
 
     def last_profile(self) -> dict:

@@ -74,3 +74,29 @@ def test_two_contexts_in_turn_keep_their_speed():
                     times.append(time.perf_counter() - t0)
             took[name] = np.median(times[4:])
     assert took["two"] < 1.3 * took["one"], took
+
+
+LAST = """
+import torch
+from paper_2509_01654_gb300 import nw
+q = torch.randint(-128, 128, (20_000, 64), dtype=torch.int8, device="cuda")
+for _ in range(2):
+    a, b = nw.Context(0), nw.Context(0)
+    want = nw.dot_topk(a, q, 32)
+    a.close()
+    got = nw.dot_topk(b, q, 32)  # with the blocks that a left
+    assert all(torch.equal(x, y) for x, y in zip(got, want))
+    before = torch.cuda.mem_get_info()[0]
+    b.close()
+    assert torch.cuda.mem_get_info()[0] - before > 1 << 30
+"""
+
+
+def test_the_last_context_gives_the_memory_back():
+    """In a process of its own: no other context may be alive."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", LAST], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
