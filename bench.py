@@ -44,7 +44,7 @@ L2_FLUSH_BYTES = 512 << 20
 # workload, from an ncu capture of dram__bytes_read.sum + dram__bytes_write.sum
 # (summarised under profiles/); valid only while the kernel sources hash to
 # kernel_sha, and reported as null otherwise
-TRAFFIC = {"kernel_sha": "df755f379759f5ef", "bytes_per_step": 98.5e6}
+TRAFFIC = {"kernel_sha": "0cf576aa0fe39c99", "bytes_per_step": 99.5e6}
 
 
 def kernel_sha() -> str:
@@ -61,15 +61,15 @@ def bit_words_per_lane(b: int) -> int:
         3 if b <= 21 else 2 if b <= 32 else 1
 
 
-# logic and add instructions of one row of 64 columns for the reduced steps
+# logic operations and additions of one row of 64 columns for the reduced steps
 # (3, 1) of the scoring (1, -1, -1): 14 LOP3 and 3 additions per 32 columns
-ROW_OPS = 34
+ROW_LOGIC, ROW_ADDS = 28, 6
 
 
-def row_ops_per_set(lengths) -> float:
-    """Lane instructions of the bit-parallel rows of every unordered pair of
-    words of these lengths, each pair of lengths the cheaper way round: the
-    least work of that kernel's formulation, without scores, lists or histogram."""
+def rows_per_set(lengths) -> float:
+    """Rows of 64 columns (a lane's) of every unordered pair of words of these
+    lengths, each pair of lengths the cheaper way round: the least work of the
+    bit-parallel formulation, without scores, lists or histogram."""
     import numpy as np
     cnt = np.bincount(np.asarray(lengths, dtype=np.int64))
     rows = 0.0
@@ -77,7 +77,14 @@ def row_ops_per_set(lengths) -> float:
         for b in range(a, len(cnt)):
             pairs = cnt[a] * cnt[b] if a < b else cnt[a] * (cnt[a] - 1) / 2
             rows += float(pairs) * min(a / bit_words_per_lane(b), b / bit_words_per_lane(a))
-    return ROW_OPS * rows
+    return rows
+
+
+def row_seconds(rates: dict) -> float:
+    """Least time of a row at the measured lane-instruction rates: the logic
+    operations on their pipe, or all of it at the rate of additions, which have
+    a second pipe (IADD3 measures more lanes a clock than LOP3)."""
+    return max(ROW_LOGIC / rates["lop3"], (ROW_LOGIC + ROW_ADDS) / rates["iadd3"])
 
 
 def tensor_roofline(flops: float, ms: float, peaks_path: str = os.path.join(ROOT, "MEASURED_PEAKS.json")) -> dict:
@@ -350,12 +357,12 @@ def run_ours(args, rank, world, local_rank):
     e2e_value = copies * pairs * len(e2e_times) / (total_e2e / 1e3)
 
     # roofline of the alignment kernel: algorithmic cells over its launches' event time,
-    # against the bit-parallel rows alone at the measured LOP3 rate
+    # against the bit-parallel rows alone at the measured LOP3 and IADD3 rates
     # (a shard holds 1/world of the cells: the planner cuts each launch into equal task ranges)
     dp_avg_ms = statistics.mean(dp_ms)
     achieved = (cells / world if sharded else cells) / (dp_avg_ms / 1e3) / 1e9
-    row_ops = row_ops_per_set(w.lengths)
-    peak = cells / (row_ops / rates["lop3"]) / 1e9
+    lane_rows = rows_per_set(w.lengths)
+    peak = cells / (lane_rows * row_seconds(rates)) / 1e9
     sha = kernel_sha()
     traffic = TRAFFIC["bytes_per_step"] if TRAFFIC["kernel_sha"] == sha and args.n == 600_000 else None
 
@@ -465,9 +472,10 @@ def run_ours(args, rank, world, local_rank):
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "GCUPS",
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_basis": "DRAM bytes of one step's alignment launch, ncu, 600k words",
-                     "peak_basis": f"bit-parallel rows alone ({ROW_OPS} logic and add instructions a lane for 64 "
-                                   f"columns, {row_ops:.4g} lane instructions) at the measured lop3 rate "
-                                   f"({rates['lop3']:.4g}/s over {rates['sm_count']} SMs{lanes_note}); the DPX cell "
+                     "peak_basis": f"bit-parallel rows alone ({ROW_LOGIC} logic operations a lane for 64 columns, "
+                                   f"{lane_rows:.4g} rows) at the measured lop3 rate "
+                                   f"({rates['lop3']:.4g}/s over {rates['sm_count']} SMs{lanes_note}), the "
+                                   f"{ROW_ADDS} additions beside them (iadd3 {rates['iadd3']:.4g}/s); the DPX cell "
                                    f"(3 packed instructions for 2 cells) would peak at "
                                    f"{2 * rates['viaddmax_s16x2'] / 3 / 1e9:.0f} GCUPS",
                      "rates_per_s": {key: rates[key] for key in ("viaddmax_s16x2", "vimax3_s16x2",
