@@ -87,11 +87,12 @@ __device__ __forceinline__ uint32_t next_code(Codes16& c) {  // takes the first 
 // set from the longer word and cleared again after the pair.  A thread loops
 // over its own word lengths, so a warp of mixed lengths runs one code path;
 // the DPX kernel it replaces ran one unrolled body per length present in the
-// warp.  What bounds it then is L1: every lane reads other words, so a load
-// takes 32 tag look-ups whatever its width.  With the words' records (P.rec) a pair
-// of words of up to 15 symbols takes two 16-byte loads; other words are read 16
-// symbols at a time from the pair records, four a load, and a pair's first loads are
-// issued together.  (Symbol by symbol a word of 24 took 72 loads.)  1,000,003 random
+// warp.  Every lane reads other words, so a load takes 32 tag look-ups whatever its
+// width.  With the words' records (P.rec) a pair of words of up to 15 symbols takes
+// two 16-byte loads; other words are read 16 symbols at a time from the pair records,
+// four a load, and a pair's first loads are issued together.  (Symbol by symbol a word
+// of 24 took 72 loads.)  With records its own instructions bound it (ALU pipe 63 %, L1
+// 47 %), without them L1 (70 %): 31 and 51 us in the kernel.  1,000,003 random
 // pairs of 100k words, whole calls: lengths N(8, 3) 397 us DPX, 62 with records, 76
 // without; all of 16 symbols 126, 67 (symbol by symbol 300); of 24, 164, 90 (412); of
 // 40, 398, 174.
